@@ -80,7 +80,7 @@ static int upload_as(DevBuf<T>& dst, const std::vector<double>& v) {
 // ---------------------------------------------------------------------------------------------
 struct Plan {
   int p = 0, P = 0;
-  DevBuf<double> T0, T1, T2, A, cs, wsin, wsq;
+  DevBuf<double> T0, T1, T2, At, cs, wsin, wsq;
   DevBuf<float> T0f, csf;
   DevBuf<dff> csdf;
   template <typename R>
@@ -145,7 +145,6 @@ struct bie_ctx {
   std::mutex mu;
   std::map<std::pair<int, int>, std::unique_ptr<bie::Plan>> plans;
   std::map<int, std::unique_ptr<bie::WigPlan>> wigs;
-  bie::DevBuf<double> scratch;  // analysis workspace
   // pair-kernel variant chosen at earlier geometries: degrees, self-grid degrees, U, pair count, variant
   struct Tuned {
     std::vector<int> p, pq;
@@ -206,7 +205,14 @@ static int get_plan(bie_ctx* ctx, int p, int P, Plan** out) {
   legendre_table(p, P, 2, v);
   BIE_TRY(pl->T2.upload(v));
   analysis_table(p, P, v);
-  BIE_TRY(pl->A.upload(v));
+  {  // rows (m, j) with the degree fastest
+    std::vector<double> vt(v.size());
+    for (int m = 0; m <= p; ++m)
+      for (int n = m; n <= p; ++n)
+        for (int j = 0; j <= P; ++j)
+          vt[leg_row(p, m, m, P + 1) + (long long)j * (p + 1 - m) + (n - m)] = v[leg_row(p, m, n, P + 1) + j];
+    BIE_TRY(pl->At.upload(vt));
+  }
   phase_table(p, P, v);
   BIE_TRY(pl->cs.upload(v));
   BIE_TRY(upload_as(pl->csf, v));
@@ -289,7 +295,8 @@ struct bie_geom {
   struct Group {
     int p = 0, pq = 0;
     std::vector<int> drops;
-    bie::DevBuf<long long> foff3, goff3, val_off, roff;  // roff: 7 * first target, per group drop
+    bie::DevBuf<long long> foff3, soff, goff3, val_off, roff;  // roff: 7 * first target, per group drop
+    bie::DevBuf<int> ids;                   // the group's drops
     bie::DevBuf<double> wS, wD, wSraw, wDraw;
     bie::DevBuf<double> cache64;            // [gdrop][N_g][7][nq] rotated geometry (Sec. 2.2)
     bie::DevBuf<float> cache32;             // FP32 copy, made on the first direct-form mixed apply
@@ -341,6 +348,23 @@ namespace bie {
 
 static const long long kWorkBudget = 3LL << 30;  // bytes of set-up temporaries per chunk
 
+// Projection of nfield grids of degree P (offsets grid_off, or stride) on the coefficients of degree p of
+// plan pl.
+static AnaGroup ana_group(const Plan* pl, long long nfield, const long long* grid_off, long long grid_stride,
+                          const long long* coef_off, long long coef_stride) {
+  AnaGroup a{};
+  a.nfield = nfield;
+  a.grid_off = grid_off;
+  a.coef_off = coef_off;
+  a.grid_stride = grid_stride;
+  a.coef_stride = coef_stride;
+  a.cs = pl->cs.ptr;
+  a.At = pl->At.ptr;
+  a.P = pl->P;
+  a.p = pl->p;
+  return a;
+}
+
 // Galerkin projection of the values of every degree group, one launch.
 static int analyze_groups(bie_ctx* ctx, bie_geom* g, const double* vals, double* out, cudaStream_t s) {
   std::vector<AnaGroup> ag;
@@ -348,18 +372,10 @@ static int analyze_groups(bie_ctx* ctx, bie_geom* g, const double* vals, double*
     auto& G = *Gp;
     Plan* pl;
     BIE_TRY(get_plan(ctx, G.p, G.p, &pl));
-    AnaGroup a{};
-    a.nfield = (long long)G.drops.size() * 3;
-    a.grid_off = G.goff3.ptr;
-    a.coef_off = G.foff3.ptr;
-    a.cs = pl->cs.ptr;
-    a.A = pl->A.ptr;
-    a.p = G.p;
-    ag.push_back(a);
+    ag.push_back(ana_group(pl, (long long)G.drops.size() * 3, G.goff3.ptr, 0, G.foff3.ptr, 0));
   }
-  std::sort(ag.begin(), ag.end(), [](const AnaGroup& x, const AnaGroup& y) { return x.p > y.p; });
   Phase ph(ctx, "analyze", s);
-  return launch_analyze_fused(ag, vals, out, s);
+  return launch_analyze(ag, vals, out, ctx->sms, s);
 }
 
 // The direct form serves a group when the configuration asks for it, or when the projected form's
@@ -586,19 +602,32 @@ static int layer_apply(bie_ctx* ctx, const bie_geom* gc, int kind, const double*
 // ---------------------------------------------------------------------------------------------
 // geometry set-up
 // ---------------------------------------------------------------------------------------------
-// x, x_theta, x_phi of ncomp=3 fields on the grid of degree P from coefficients of degree p.
+// x, x_theta, x_phi of nfield fields on the grid of degree P from coefficients of degree p, into X
+// [3 kinds][nfield][N].
 static int synth_xderivs(bie_ctx* ctx, const double* coef, const long long* field_off, long long coef_stride,
-                         long long nfield, int p, int P, double* H, double* X, double* Xt, double* Xp,
-                         cudaStream_t s) {
+                         long long nfield, int p, int P, double* X, cudaStream_t s) {
   Plan* pl;
   BIE_TRY(get_plan(ctx, p, P, &pl));
   const long long N = ngrid(P);
-  BIE_TRY((launch_leg_synth<double, double>(coef, field_off, coef_stride, nfield, p, pl->T0.ptr, P + 1, H, 0, s)));
-  BIE_TRY((launch_phi_synth<double, double>(H, nfield, p, P, pl->cs.ptr, X, nullptr, N, s)));
-  BIE_TRY((launch_leg_synth<double, double>(coef, field_off, coef_stride, nfield, p, pl->T0.ptr, P + 1, H, 1, s)));
-  BIE_TRY((launch_phi_synth<double, double>(H, nfield, p, P, pl->cs.ptr, Xp, nullptr, N, s)));
-  BIE_TRY((launch_leg_synth<double, double>(coef, field_off, coef_stride, nfield, p, pl->T1.ptr, P + 1, H, 0, s)));
-  BIE_TRY((launch_phi_synth<double, double>(H, nfield, p, P, pl->cs.ptr, Xt, nullptr, N, s)));
+  return launch_synth<double, double>(7, coef, field_off, coef_stride, nfield, p, P, pl->T0.ptr, pl->T1.ptr,
+                                      (const double*)nullptr, pl->cs.ptr, X, nfield * N, N, ctx->sms, s);
+}
+
+// Surface records of a degree group on its grids of degree P, drop i's at rec + 7 off[i] (off on the device),
+// through temporaries for as many drops at a time as the budget holds.
+static int group_records(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, int P, double* rec, const long long* off,
+                         cudaStream_t s) {
+  Plan* pl;
+  BIE_TRY(get_plan(ctx, G.p, P, &pl));
+  const long long N = ngrid(P), nd = (long long)G.drops.size();
+  const long long chunk = std::max(1LL, std::min<long long>(nd, kWorkBudget / (9 * 8 * N)));
+  DevBuf<double> X;
+  BIE_TRY(X.alloc(chunk * 9 * N));
+  for (long long i0 = 0; i0 < nd; i0 += chunk) {
+    const long long n = std::min(chunk, nd - i0);
+    BIE_TRY(synth_xderivs(ctx, g->xcoef.ptr, G.foff3.ptr + 3 * i0, 0, 3 * n, G.p, P, X.ptr, s));
+    BIE_TRY(launch_surface(X.ptr, X.ptr + 3 * n * N, X.ptr + 6 * n * N, n, P, pl->wsin.ptr, rec, off + i0, s));
+  }
   return BIE_OK;
 }
 
@@ -607,7 +636,7 @@ static int setup_group(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, cudaStream
   const long long ng = ngrid(p), nq = ngrid(pq), nc = ncoef(p);
   const int nd = (int)G.drops.size();
   // offsets
-  std::vector<long long> foff3(3 * nd), goff3(3 * nd), voff(nd), roff(nd);
+  std::vector<long long> foff3(3 * nd), goff3(3 * nd), voff(nd), roff(nd), so(nd), sof(nd);
   std::vector<double> wS(nd), wD(nd), wSr(nd), wDr(nd);
   for (int i = 0; i < nd; ++i) {
     int d = G.drops[i];
@@ -617,6 +646,8 @@ static int setup_group(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, cudaStream
     }
     voff[i] = 3 * g->tgt_off[d];
     roff[i] = 7 * g->tgt_off[d];
+    so[i] = g->tgt_off[d];
+    sof[i] = g->coef_off[d] / 3;  // one scalar per drop
     wS[i] = -1.0 / (4 * kPi);
     wD[i] = (g->lambda[d] - 1.0) / (4 * kPi);
     wSr[i] = 1.0 / (8 * kPi);
@@ -626,27 +657,18 @@ static int setup_group(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, cudaStream
   BIE_TRY(G.goff3.upload(goff3));
   BIE_TRY(G.val_off.upload(voff));
   BIE_TRY(G.roff.upload(roff));
+  BIE_TRY(G.src_off_std.upload(so));
+  BIE_TRY(G.soff.upload(sof));
+  BIE_TRY(G.ids.upload(G.drops));
   BIE_TRY(G.wS.upload(wS));
   BIE_TRY(G.wD.upload(wD));
   BIE_TRY(G.wSraw.upload(wSr));
   BIE_TRY(G.wDraw.upload(wDr));
 
-  // standard grid: targets and regular-rule sources, one drop at a time
+  // standard grid: targets and regular-rule sources
   {
     Phase ph(ctx, "setup_surface", s);
-    Plan* pl;
-    BIE_TRY(get_plan(ctx, p, p, &pl));
-    DevBuf<double> tmp;
-    BIE_TRY(tmp.alloc(3 * (p + 1) * (p + 1) * 2 + 9 * ng));
-    double* H = tmp.ptr;
-    double* X = H + 3 * (p + 1) * (p + 1) * 2;
-    for (int i = 0; i < nd; ++i) {
-      int d = G.drops[i];
-      BIE_TRY(synth_xderivs(ctx, g->xcoef.ptr + g->coef_off[d], nullptr, nc, 3, p, p, H, X, X + 3 * ng,
-                            X + 6 * ng, s));
-      BIE_TRY(launch_surface(X, X + 3 * ng, X + 6 * ng, 1, p, pl->wsin.ptr, g->rec_std.ptr + 7 * g->tgt_off[d], s));
-    }
-    BIE_CUDA_TRY(cudaStreamSynchronize(s));
+    BIE_TRY(group_records(ctx, g, G, p, g->rec_std.ptr, G.src_off_std.ptr, s));
   }
 
   // rotated-grid cache of the singular rule (Sec. 2.2), chunked over drops
@@ -657,21 +679,20 @@ static int setup_group(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, cudaStream
   BIE_TRY(get_plan(ctx, p, p, &pp));
   BIE_TRY(get_wig(ctx, p, &wp));
   BIE_TRY(G.cache64.alloc((size_t)nd * ng * 7 * nq));
-  const long long per = ng * 3 * nc + ng * 3 * (long long)(p + 1) * (pq + 1) * 2 + 3 * ng * 3 * nq;
+  const long long per = ng * 3 * nc + 3 * ng * 3 * nq;
   int chunk = (int)std::max(1LL, std::min<long long>(nd, (2 * kWorkBudget) / (8 * per)));
   DevBuf<double> work;
   BIE_TRY(work.alloc((size_t)chunk * per));
   for (int c0 = 0; c0 < nd; c0 += chunk) {
     const int cn = std::min(chunk, nd - c0);
     double* RC = work.ptr;
-    double* H = RC + cn * ng * 3 * nc;
-    double* X = H + cn * ng * 3 * (long long)(p + 1) * (pq + 1) * 2;
+    double* X = RC + cn * ng * 3 * nc;
     double* Xt = X + cn * ng * 3 * nq;
     double* Xp = Xt + cn * ng * 3 * nq;
     // x coefficients of the chunk's drops: field offsets into the geometry's copy
     BIE_TRY((launch_rotate<double, double>(g->xcoef.ptr, G.foff3.ptr + 3 * c0, 3, cn, p, wp->blk.ptr, wp->stride,
                                            p + 1, 2 * p + 2, pp->cs.ptr, RC, ng * 3 * nc, s)));
-    BIE_TRY(synth_xderivs(ctx, RC, nullptr, nc, cn * ng * 3, p, pq, H, X, Xt, Xp, s));
+    BIE_TRY(synth_xderivs(ctx, RC, nullptr, nc, cn * ng * 3, p, pq, X, s));
     // the targets x0 of the chunk's drops, wherever each drop's records lie (a degree group's drops
     // are in general not adjacent in rec_std)
     BIE_TRY(launch_rotgeo<double>(X, Xt, Xp, cn, (int)ng, pq, g->rec_std.ptr, G.roff.ptr + c0, pl->wsq.ptr,
@@ -686,36 +707,26 @@ static int setup_group(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, cudaStream
 // inter-drop set-up (Sec. 2.3): centres, volumes and mean radii, upsampled grids, source records,
 // region classification, and the balanced work list of the pair sums
 // ---------------------------------------------------------------------------------------------
-static int drop_records(bie_ctx* ctx, bie_geom* g, int d, int P, double* rec, cudaStream_t s) {
-  const int p = g->p[d];
-  Plan* pl;
-  BIE_TRY(get_plan(ctx, p, P, &pl));
-  const long long N = ngrid(P);
-  DevBuf<double> tmp;
-  BIE_TRY(tmp.alloc(3 * (p + 1) * (size_t)(P + 1) * 2 + 9 * N));
-  double* H = tmp.ptr;
-  double* X = H + 3 * (p + 1) * (long long)(P + 1) * 2;
-  BIE_TRY(synth_xderivs(ctx, g->xcoef.ptr + g->coef_off[d], nullptr, ncoef(p), 3, p, P, H, X, X + 3 * N, X + 6 * N,
-                        s));
-  BIE_TRY(launch_surface(X, X + 3 * N, X + 6 * N, 1, P, pl->wsin.ptr, rec, s));
-  BIE_CUDA_TRY(cudaStreamSynchronize(s));
-  return BIE_OK;
-}
-
-static int drop_stats(const double* rec, long long N, const double* c, double* vol, double* bnd, cudaStream_t s) {
+// sum of x.n wJ / 3 (the volume by the regular rule) and the largest distance from the centre, per drop of a
+// degree group whose records (N points each) start at rec + 7 off[i]; host vol, bnd by drop (null to skip).
+static int group_stats(bie_geom* g, bie_geom::Group& G, const double* rec, const long long* off, long long N, double* vol,
+                       double* bnd, cudaStream_t s) {
+  const size_t nd = G.drops.size();
   DevBuf<double> o;
-  BIE_TRY(o.alloc(128));
-  BIE_TRY(launch_drop_stats(rec, N, c, o.ptr, s));
-  std::vector<double> h(128);
-  BIE_CUDA_TRY(cudaMemcpyAsync(h.data(), o.ptr, 128 * sizeof(double), cudaMemcpyDeviceToHost, s));
+  BIE_TRY(o.alloc(128 * nd));
+  BIE_TRY(launch_drop_stats(rec, off, G.ids.ptr, g->centre_d.ptr, (long long)nd, N, o.ptr, s));
+  std::vector<double> h(128 * nd);
+  BIE_CUDA_TRY(cudaMemcpyAsync(h.data(), o.ptr, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
   BIE_CUDA_TRY(cudaStreamSynchronize(s));
-  double v = 0, m = 0;
-  for (int b = 0; b < 64; ++b) {
-    v += h[2 * b];
-    m = std::max(m, h[2 * b + 1]);
+  for (size_t i = 0; i < nd; ++i) {
+    double v = 0, m = 0;
+    for (int b = 0; b < 64; ++b) {
+      v += h[128 * i + 2 * b];
+      m = std::max(m, h[128 * i + 2 * b + 1]);
+    }
+    if (vol) vol[G.drops[i]] = v / 3.0;
+    if (bnd) bnd[G.drops[i]] = m;
   }
-  *vol = v / 3.0;
-  *bnd = m;
   return BIE_OK;
 }
 
@@ -811,23 +822,28 @@ static int setup_interdrop(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
   BIE_TRY(g->centre_d.upload(g->centre));
   // set-up stages are timed as phases when profiling is on
   std::unique_ptr<Phase> stage(new Phase(ctx, "setup_records", s));
-  for (int d = 0; d < nd; ++d) {
-    const int p = g->p[d];
+  for (auto& Gp : g->groups) {
+    auto& G = *Gp;
     // volume by the regular rule on the grid of degree 2p+1, mean radius, h = R pi/(p+1)
-    const int P2 = 2 * p + 1;
+    const int P2 = 2 * G.p + 1;
+    const long long N2 = ngrid(P2), n = (long long)G.drops.size();
+    std::vector<long long> tmp_off(n), uoff(n);
+    for (long long i = 0; i < n; ++i) {
+      tmp_off[i] = i * N2;
+      uoff[i] = g->up_off[G.drops[i]];
+    }
     DevBuf<double> rec2;
-    BIE_TRY(rec2.alloc(7 * ngrid(P2)));
-    BIE_TRY(drop_records(ctx, g, d, P2, rec2.ptr, s));
-    double vol, dummy;
-    BIE_TRY(drop_stats(rec2.ptr, ngrid(P2), &g->centre[3 * d], &vol, &dummy, s));
-    g->volume[d] = vol;
-    const double R = std::cbrt(3.0 * vol / (4.0 * kPi));
-    g->hdrop[d] = R * kPi / (p + 1);
+    DevBuf<long long> d_tmp;
+    BIE_TRY(rec2.alloc(7 * n * N2));
+    BIE_TRY(d_tmp.upload(tmp_off));
+    BIE_TRY(G.src_off_up.upload(uoff));
+    BIE_TRY(group_records(ctx, g, G, P2, rec2.ptr, d_tmp.ptr, s));
+    BIE_TRY(group_stats(g, G, rec2.ptr, d_tmp.ptr, N2, g->volume.data(), nullptr, s));
+    for (int d : G.drops) g->hdrop[d] = std::cbrt(3.0 * g->volume[d] / (4.0 * kPi)) * kPi / (G.p + 1);
     // upsampled grid records and the bounding radius about the centre
-    double* ru = g->rec_up.ptr + 7 * g->up_off[d];
-    BIE_TRY(drop_records(ctx, g, d, g->up_P[d], ru, s));
-    double v2;
-    BIE_TRY(drop_stats(ru, g->up_n[d], &g->centre[3 * d], &v2, &g->bound[d], s));
+    const int Pu = g->up_P[G.drops[0]];
+    BIE_TRY(group_records(ctx, g, G, Pu, g->rec_up.ptr, G.src_off_up.ptr, s));
+    BIE_TRY(group_stats(g, G, g->rec_up.ptr, G.src_off_up.ptr, ngrid(Pu), nullptr, g->bound.data(), s));
   }
   // per-target bookkeeping
   stage.reset(new Phase(ctx, "setup_sources", s));
@@ -857,18 +873,14 @@ static int setup_interdrop(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
   BIE_TRY(g->uN64.alloc(3 * uo));
   BIE_TRY(g->uX32.alloc(3 * uo));
   BIE_TRY(g->uN32.alloc(3 * uo));
-  for (int d = 0; d < nd; ++d) {
-    const double* c = &g->centre[3 * d];
-    const double* rs = g->rec_std.ptr + 7 * g->tgt_off[d];
-    const double* ru = g->rec_up.ptr + 7 * g->up_off[d];
-    BIE_TRY(launch_source_geometry<double>(rs, ngd[d], c, g->sX64.ptr + g->tgt_off[d], g->sN64.ptr + g->tgt_off[d],
-                                           ns, s));
-    BIE_TRY(launch_source_geometry<float>(rs, ngd[d], c, g->sX32.ptr + g->tgt_off[d], g->sN32.ptr + g->tgt_off[d],
-                                          ns, s));
-    BIE_TRY(launch_source_geometry<double>(ru, g->up_n[d], c, g->uX64.ptr + g->up_off[d],
-                                           g->uN64.ptr + g->up_off[d], uo, s));
-    BIE_TRY(launch_source_geometry<float>(ru, g->up_n[d], c, g->uX32.ptr + g->up_off[d], g->uN32.ptr + g->up_off[d],
-                                          uo, s));
+  for (auto& Gp : g->groups) {
+    auto& G = *Gp;
+    const long long n = (long long)G.drops.size();
+    BIE_TRY(launch_source_geometry(g->rec_std.ptr, G.src_off_std.ptr, G.ids.ptr, g->centre_d.ptr, n, ngrid(G.p),
+                                   g->sX64.ptr, g->sN64.ptr, g->sX32.ptr, g->sN32.ptr, ns, s));
+    BIE_TRY(launch_source_geometry(g->rec_up.ptr, G.src_off_up.ptr, G.ids.ptr, g->centre_d.ptr, n,
+                                   ngrid(g->up_P[G.drops[0]]), g->uX64.ptr, g->uN64.ptr, g->uX32.ptr, g->uN32.ptr, uo,
+                                   s));
   }
   // region classification on the device, per-(tile, drop) masks on the device, work list on the host
   stage.reset(new Phase(ctx, "setup_classify", s));
@@ -1018,15 +1030,6 @@ static int setup_interdrop(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
   stage.reset(new Phase(ctx, "setup_autotune", s));
   BIE_TRY(autotune_interdrop(ctx, g, s));
   stage.reset();
-  for (auto& G : g->groups) {
-    std::vector<long long> so, uo2;
-    for (int d : G->drops) {
-      so.push_back(g->tgt_off[d]);
-      uo2.push_back(g->up_off[d]);
-    }
-    BIE_TRY(G->src_off_std.upload(so));
-    BIE_TRY(G->src_off_up.upload(uo2));
-  }
   if (!g->near.empty()) {
     Phase ph(ctx, "setup_near", s);
     BIE_TRY(setup_near(ctx, g, s));
@@ -1046,23 +1049,22 @@ static int source_densities(bie_geom* g, const double* dens, R* Qs, R* Qu, cudaS
     const int p = G.p;
     const int Pu = ctx->cfg.upsample * (p + 1) - 1;
     const long long nd = (long long)G.drops.size();
-    const long long need = nd * 3 * ((long long)(p + 1) * (Pu + 1) * 2 + ngrid(Pu));
-    R* H;
+    const long long need = nd * 3 * ngrid(Pu);
+    R* grid;
     if (sizeof(R) == 8) {
       BIE_TRY(g->syn64.alloc(need));
-      H = reinterpret_cast<R*>(g->syn64.ptr);
+      grid = reinterpret_cast<R*>(g->syn64.ptr);
     } else {
       BIE_TRY(g->syn32.alloc(need));
-      H = reinterpret_cast<R*>(g->syn32.ptr);
+      grid = reinterpret_cast<R*>(g->syn32.ptr);
     }
     for (int gridk = 0; gridk < 2; ++gridk) {
       const int P = gridk ? Pu : p;
       const long long N = ngrid(P);
       Plan* pl;
       BIE_TRY(get_plan(ctx, p, P, &pl));
-      R* grid = H + nd * 3 * (long long)(p + 1) * (P + 1) * 2;
-      BIE_TRY((launch_leg_synth<double, R>(dens, G.foff3.ptr, 0, nd * 3, p, pl->T0_<R>(), P + 1, H, 0, s)));
-      BIE_TRY((launch_phi_synth<R, R>(H, nd * 3, p, P, pl->cs_<R>(), grid, nullptr, N, s)));
+      BIE_TRY((launch_synth<double, R>(1, dens, G.foff3.ptr, 0, nd * 3, p, P, pl->T0_<R>(), (const R*)nullptr,
+                                       (const R*)nullptr, pl->cs_<R>(), grid, 0, N, ctx->sms, s)));
       if (gridk == 0)
         BIE_TRY(launch_weight_sources<R>(grid, g->rec_std.ptr, G.src_off_std.ptr, N, nd, Qs, g->ntarget, s));
       else
@@ -2182,7 +2184,7 @@ struct SurfGroup {
 };
 
 struct SurfLayout {
-  int ndrop = 0;
+  int ndrop = 0, sms = 0;
   std::vector<int> p;
   std::vector<long long> voff, soff;  // per drop: start of its vector / scalar coefficients
   long long nv = 0, ns = 0;           // total lengths
@@ -2192,6 +2194,7 @@ struct SurfLayout {
 // P = 2p + 1 (the nonlinear terms of Sec. 1.3) when upsampled, else P = p.
 static int surf_layout(bie_ctx* ctx, int ndrop, const int* p, bool upsampled, SurfLayout& L) {
   L.ndrop = ndrop;
+  L.sms = ctx->sms;
   L.p.assign(p, p + ndrop);
   L.voff.resize(ndrop);
   L.soff.resize(ndrop);
@@ -2222,24 +2225,19 @@ static int surf_layout(bie_ctx* ctx, int ndrop, const int* p, bool upsampled, Su
 }
 
 // Derivative fields of nfield coefficient sets (device offsets off) of the group's degree on its
-// grid: kind k (0 f, 1 t, 2 p, 3 tt, 4 tp, 5 pp) is written to out + k * nfield * N.  H holds
-// nfield * (p+1) * (P+1) * 2 doubles.
-static int surf_synth(const SurfGroup& G, const double* coef, const long long* off, long long nfield,
-                      std::initializer_list<int> kinds, double* H, double* out, cudaStream_t s) {
+// grid: kind k (0 f, 1 t, 2 p, 3 tt, 4 tp, 5 pp) of the mask is written to out + k * nfield * N.
+static int surf_synth(const SurfLayout& L, const SurfGroup& G, const double* coef, const long long* off, long long nfield,
+                      int kinds, double* out, cudaStream_t s) {
   const Plan* pl = G.pl;
-  const double* T[6] = {pl->T0.ptr, pl->T1.ptr, pl->T0.ptr, pl->T2.ptr, pl->T1.ptr, pl->T0.ptr};
-  const int dphi[6] = {0, 0, 1, 0, 1, 2};
   const long long N = ngrid(G.P);
-  for (int k : kinds) {
-    BIE_TRY((launch_leg_synth<double, double>(coef, off, 0, nfield, G.p, T[k], G.P + 1, H, dphi[k], s)));
-    BIE_TRY((launch_phi_synth<double, double>(H, nfield, G.p, G.P, pl->cs.ptr, out + (long long)k * nfield * N,
-                                              nullptr, N, s)));
-  }
-  return BIE_OK;
+  return launch_synth<double, double>(kinds, coef, off, 0, nfield, G.p, G.P, pl->T0.ptr, pl->T1.ptr, pl->T2.ptr,
+                                      pl->cs.ptr, out + ((kinds & 1) ? 0 : nfield * N), nfield * N, N, L.sms, s);
 }
 
-static long long synth_work(const SurfGroup& G, long long nfield) {
-  return nfield * (G.p + 1) * (long long)(G.P + 1) * 2;
+// Projection of nfield grids (N apart) of the group to coefficients at off.
+static int surf_project(const SurfLayout& L, const SurfGroup& G, const double* grid, long long nfield,
+                        const long long* off, double* coef, cudaStream_t s) {
+  return launch_analyze({ana_group(G.pl, nfield, nullptr, ngrid(G.P), off, 0)}, grid, coef, L.sms, s);
 }
 
 // Galerkin projections of f_E and (when fi is non-null) f_I = inv_pe lap Gamma, Sec. 3.
@@ -2248,23 +2246,18 @@ static int surf_rates(const SurfLayout& L, const double* x, const double* u, con
   for (auto& Gp : L.groups) {
     const SurfGroup& G = *Gp;
     const long long nd = (long long)G.drops.size(), N = ngrid(G.P);
-    const long long nH = synth_work(G, 3 * nd);
     DevBuf<double> tmp;
-    BIE_TRY(tmp.alloc(nH + 18 * nd * N + 9 * nd * N + 6 * nd * N + 2 * nd * N));
-    double* H = tmp.ptr;
-    double* X = H + nH;
+    BIE_TRY(tmp.alloc(18 * nd * N + 9 * nd * N + 6 * nd * N + 2 * nd * N));
+    double* X = tmp.ptr;
     double* U = X + 18 * nd * N;
     double* Gm = U + 9 * nd * N;
     double* out = Gm + 6 * nd * N;
-    BIE_TRY(surf_synth(G, x, G.voff.ptr, 3 * nd, {0, 1, 2, 3, 4, 5}, H, X, s));
-    BIE_TRY(surf_synth(G, u, G.voff.ptr, 3 * nd, {0, 1, 2}, H, U, s));
-    BIE_TRY(surf_synth(G, gam, G.soff.ptr, nd, {0, 1, 2, 3, 4, 5}, H, Gm, s));
+    BIE_TRY(surf_synth(L, G, x, G.voff.ptr, 3 * nd, 62, X, s));
+    BIE_TRY(surf_synth(L, G, u, G.voff.ptr, 3 * nd, 7, U, s));
+    BIE_TRY(surf_synth(L, G, gam, G.soff.ptr, nd, 63, Gm, s));
     BIE_TRY(launch_surf_rates(X, U, Gm, nd, N, inv_pe, out, fi ? out + nd * N : nullptr, s));
-    // H is free again: it serves as the analysis workspace (nd fields need less than 3 nd)
-    BIE_TRY(launch_analyze(out, nullptr, N, nd, G.P, G.p, G.pl->cs.ptr, G.pl->A.ptr, H, fe, G.soff.ptr, 0, s));
-    if (fi)
-      BIE_TRY(launch_analyze(out + nd * N, nullptr, N, nd, G.P, G.p, G.pl->cs.ptr, G.pl->A.ptr, H, fi, G.soff.ptr,
-                             0, s));
+    BIE_TRY(surf_project(L, G, out, nd, G.soff.ptr, fe, s));
+    if (fi) BIE_TRY(surf_project(L, G, out + nd * N, nd, G.soff.ptr, fi, s));
     BIE_CUDA_TRY(cudaStreamSynchronize(s));  // temporaries are released per group
   }
   return BIE_OK;
@@ -2276,18 +2269,13 @@ static int surf_integrals(const SurfLayout& L, const double* x, const double* ga
   for (auto& Gp : L.groups) {
     const SurfGroup& G = *Gp;
     const long long nd = (long long)G.drops.size(), N = ngrid(G.P);
-    const long long nH = synth_work(G, 3 * nd);
     DevBuf<double> tmp;
-    BIE_TRY(tmp.alloc(nH + 9 * nd * N + nd * N + nd));
-    double* H = tmp.ptr;
-    double* X = H + nH;
+    BIE_TRY(tmp.alloc(9 * nd * N + nd * N + nd));
+    double* X = tmp.ptr;
     double* Gm = X + 9 * nd * N;
     double* res = Gm + nd * N;
-    if (mode == 0)
-      BIE_TRY(surf_synth(G, x, G.voff.ptr, 3 * nd, {0, 1, 2}, H, X, s));
-    else
-      BIE_TRY(surf_synth(G, x, G.voff.ptr, 3 * nd, {1, 2}, H, X, s));
-    if (mode == 1) BIE_TRY(surf_synth(G, gam, G.soff.ptr, nd, {0}, H, Gm, s));
+    BIE_TRY(surf_synth(L, G, x, G.voff.ptr, 3 * nd, mode == 0 ? 7 : 6, X, s));
+    if (mode == 1) BIE_TRY(surf_synth(L, G, gam, G.soff.ptr, nd, 1, Gm, s));
     BIE_TRY(launch_drop_integral(X, Gm, nd, G.P, G.pl->wsin.ptr, mode, res, s));
     std::vector<double> h(nd);
     BIE_CUDA_TRY(cudaMemcpyAsync(h.data(), res, nd * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -2303,13 +2291,11 @@ static int surf_absmax(const SurfLayout& L, const double* coef, int ncomp, doubl
   for (auto& Gp : L.groups) {
     const SurfGroup& G = *Gp;
     const long long nd = (long long)G.drops.size(), N = ngrid(G.P), nf = ncomp * nd;
-    const long long nH = synth_work(G, nf);
     DevBuf<double> tmp;
-    BIE_TRY(tmp.alloc(nH + nf * N + nd));
-    double* H = tmp.ptr;
-    double* F = H + nH;
+    BIE_TRY(tmp.alloc(nf * N + nd));
+    double* F = tmp.ptr;
     double* res = F + nf * N;
-    BIE_TRY(surf_synth(G, coef, ncomp == 3 ? G.voff.ptr : G.soff.ptr, nf, {0}, H, F, s));
+    BIE_TRY(surf_synth(L, G, coef, ncomp == 3 ? G.voff.ptr : G.soff.ptr, nf, 1, F, s));
     BIE_TRY(launch_drop_absmax(F, nd, ncomp, N, res, s));
     std::vector<double> h(nd);
     BIE_CUDA_TRY(cudaMemcpyAsync(h.data(), res, nd * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -2335,16 +2321,15 @@ static int surf_implicit_setup(const SurfLayout& L, const double* x, double a, S
   for (auto& Gp : L.groups) {
     const SurfGroup& G = *Gp;
     const long long nd = (long long)G.drops.size(), N = ngrid(G.P);
-    const long long nH = synth_work(G, 3 * nd);
     DevBuf<double> tmp;
-    BIE_TRY(tmp.alloc(nH + 18 * nd * N));
-    BIE_TRY(surf_synth(G, x, G.voff.ptr, 3 * nd, {0, 1, 2, 3, 4, 5}, tmp.ptr, tmp.ptr + nH, s));
+    BIE_TRY(tmp.alloc(18 * nd * N));
+    BIE_TRY(surf_synth(L, G, x, G.voff.ptr, 3 * nd, 62, tmp.ptr, s));
     std::unique_ptr<DevBuf<double>> lc(new DevBuf<double>());
     BIE_TRY(lc->alloc(5 * nd * N));
-    BIE_TRY(launch_lap_coef(tmp.ptr + nH, nd, N, lc->ptr, s));
+    BIE_TRY(launch_lap_coef(tmp.ptr, nd, N, lc->ptr, s));
     BIE_CUDA_TRY(cudaStreamSynchronize(s));
     I.lapc.push_back(std::move(lc));
-    wmax = std::max(wmax, synth_work(G, nd) + 7 * nd * N);
+    wmax = std::max(wmax, 7 * nd * N);
   }
   std::vector<double> vol(L.ndrop);
   BIE_TRY(surf_integrals(L, x, nullptr, 0, vol.data(), s));
@@ -2366,12 +2351,11 @@ static int surf_implicit_apply(SurfImplicit& I, const double* y, double* w, cuda
   for (size_t gi = 0; gi < L.groups.size(); ++gi) {
     const SurfGroup& G = *L.groups[gi];
     const long long nd = (long long)G.drops.size(), N = ngrid(G.P);
-    double* H = I.work.ptr;
-    double* S = H + synth_work(G, nd);  // [6][nd][N], kinds 1..5 used
+    double* S = I.work.ptr;  // [6][nd][N], kinds 1..5 used
     double* grid = S + 6 * nd * N;
-    BIE_TRY(surf_synth(G, y, G.soff.ptr, nd, {1, 2, 3, 4, 5}, H, S, s));
+    BIE_TRY(surf_synth(L, G, y, G.soff.ptr, nd, 62, S, s));
     BIE_TRY(launch_lap_apply(I.lapc[gi]->ptr, S, nd, N, grid, s));
-    BIE_TRY(launch_analyze(grid, nullptr, N, nd, G.P, G.p, G.pl->cs.ptr, G.pl->A.ptr, H, I.c.ptr, G.soff.ptr, 0, s));
+    BIE_TRY(surf_project(L, G, grid, nd, G.soff.ptr, I.c.ptr, s));
   }
   return launch_implicit_combine(y, I.c.ptr, I.a, I.inv_diag.ptr, L.ns, w, s);
 }
@@ -2596,17 +2580,22 @@ int bie_sh_analyze(bie_ctx* ctx, int ndrop, const int* p, int ncomp, const doubl
   BIE_TRY(check_degrees(ndrop, p));
   BIE_CUDA_TRY(cudaSetDevice(ctx->cfg.device));
   cudaStream_t s = (cudaStream_t)stream;
+  // consecutive drops of one degree form one group
+  std::vector<AnaGroup> ag;
   long long go = 0, co = 0;
   for (int d = 0; d < ndrop; ++d) {
-    Plan* pl;
-    BIE_TRY(get_plan(ctx, p[d], p[d], &pl));
-    BIE_TRY(ctx->scratch.alloc((size_t)ncomp * (p[d] + 1) * (p[d] + 1) * 2));
-    BIE_TRY(launch_analyze(grid + go, nullptr, ngrid(p[d]), ncomp, p[d], p[d], pl->cs.ptr, pl->A.ptr,
-                           ctx->scratch.ptr, coef + co, nullptr, ncoef(p[d]), s));
+    if (d == 0 || p[d] != p[d - 1]) {
+      Plan* pl;
+      BIE_TRY(get_plan(ctx, p[d], p[d], &pl));
+      ag.push_back(ana_group(pl, 0, nullptr, ngrid(p[d]), nullptr, ncoef(p[d])));
+      ag.back().grid_base = go;
+      ag.back().coef_base = co;
+    }
+    ag.back().nfield += ncomp;
     go += ncomp * ngrid(p[d]);
     co += ncomp * ncoef(p[d]);
   }
-  return BIE_OK;
+  return launch_analyze(ag, grid, coef, ctx->sms, s);
 }
 
 int bie_sh_synthesize(bie_ctx* ctx, int ndrop, const int* p, const int* p_out, int ncomp, const double* coef,
@@ -2621,16 +2610,18 @@ int bie_sh_synthesize(bie_ctx* ctx, int ndrop, const int* p, const int* p_out, i
   BIE_CUDA_TRY(cudaSetDevice(ctx->cfg.device));
   cudaStream_t s = (cudaStream_t)stream;
   long long go = 0, co = 0;
-  for (int d = 0; d < ndrop; ++d) {
+  for (int d = 0; d < ndrop;) {  // consecutive drops of equal degrees in one launch
+    long long n = 0;
+    int e = d;
+    for (; e < ndrop && p[e] == p[d] && p_out[e] == p_out[d]; ++e) n += ncomp;
     Plan* pl;
     BIE_TRY(get_plan(ctx, p[d], p_out[d], &pl));
-    BIE_TRY(ctx->scratch.alloc((size_t)ncomp * (p[d] + 1) * (p_out[d] + 1) * 2));
-    BIE_TRY((launch_leg_synth<double, double>(coef + co, nullptr, ncoef(p[d]), ncomp, p[d], pl->T0.ptr,
-                                              p_out[d] + 1, ctx->scratch.ptr, 0, s)));
-    BIE_TRY((launch_phi_synth<double, double>(ctx->scratch.ptr, ncomp, p[d], p_out[d], pl->cs.ptr, grid + go,
-                                              nullptr, ngrid(p_out[d]), s)));
-    go += ncomp * ngrid(p_out[d]);
-    co += ncomp * ncoef(p[d]);
+    BIE_TRY((launch_synth<double, double>(1, coef + co, (const long long*)nullptr, ncoef(p[d]), n, p[d], p_out[d],
+                                          pl->T0.ptr, nullptr, nullptr, pl->cs.ptr, grid + go, 0, ngrid(p_out[d]),
+                                          ctx->sms, s)));
+    go += n * ngrid(p_out[d]);
+    co += n * ncoef(p[d]);
+    d = e;
   }
   return BIE_OK;
 }
@@ -2771,35 +2762,29 @@ int bie_interfacial_force(bie_ctx* ctx, const bie_geom* g, const double* gammaco
   BIE_CUDA_TRY(cudaSetDevice(ctx->cfg.device));
   cudaStream_t s = (cudaStream_t)stream;
   Phase phz(ctx, "force", s);
-  long long go = 0;  // offset of drop d's Gamma coefficients (one scalar per drop)
-  for (int d = 0; d < g->ndrop; ++d) {
-    const int p = g->p[d], P = 2 * p + 1;  // nonlinear terms on the grid of degree 2p+1 (Sec. 1.3)
+  DevBuf<double> tmp;
+  for (auto& Gp : g->groups) {  // as many drops of a degree at a time as the budget holds
+    auto& G = *Gp;
+    const int p = G.p, P = 2 * p + 1;  // nonlinear terms on the grid of degree 2p+1 (Sec. 1.3)
     Plan* pl;
     BIE_TRY(get_plan(ctx, p, P, &pl));
-    const long long N = ngrid(P), nc = ncoef(p);
-    DevBuf<double> tmp;
-    BIE_TRY(tmp.alloc(3 * (p + 1) * (size_t)(P + 1) * 2 + 18 * N + 3 * N + 3 * N + 3 * (p + 1) * (size_t)(P + 1) * 2));
-    double* H = tmp.ptr;
-    double* X = H + 3 * (p + 1) * (long long)(P + 1) * 2;  // [6][3][N]
-    double* Gm = X + 18 * N;                                // [3][N]
-    double* f = Gm + 3 * N;                                 // [3][N]
-    double* F = f + 3 * N;
-    const double* xc = g->xcoef.ptr + g->coef_off[d];
-    const double* T[6] = {pl->T0.ptr, pl->T1.ptr, pl->T0.ptr, pl->T2.ptr, pl->T1.ptr, pl->T0.ptr};
-    const int dphi[6] = {0, 0, 1, 0, 1, 2};
-    for (int k = 0; k < 6; ++k) {
-      BIE_TRY((launch_leg_synth<double, double>(xc, nullptr, nc, 3, p, T[k], P + 1, H, dphi[k], s)));
-      BIE_TRY((launch_phi_synth<double, double>(H, 3, p, P, pl->cs.ptr, X + k * 3 * N, nullptr, N, s)));
+    const long long N = ngrid(P), nd = (long long)G.drops.size();
+    const long long chunk = std::max(1LL, std::min<long long>(nd, kWorkBudget / (21 * 8 * N)));
+    BIE_TRY(tmp.alloc(chunk * 21 * N));
+    for (long long i0 = 0; i0 < nd; i0 += chunk) {
+      const long long n = std::min(chunk, nd - i0);
+      double* X = tmp.ptr;           // [5][n][3][N]: t, p, tt, tp, pp
+      double* Gm = X + 15 * n * N;   // [3][n][N]: f, t, p
+      double* f = Gm + 3 * n * N;    // [n][3][N]
+      BIE_TRY((launch_synth<double, double>(62, g->xcoef.ptr, G.foff3.ptr + 3 * i0, 0, 3 * n, p, P, pl->T0.ptr,
+                                            pl->T1.ptr, pl->T2.ptr, pl->cs.ptr, X, 3 * n * N, N, ctx->sms, s)));
+      BIE_TRY((launch_synth<double, double>(7, gammacoef, G.soff.ptr + i0, 0, n, p, P, pl->T0.ptr, pl->T1.ptr,
+                                            nullptr, pl->cs.ptr, Gm, n * N, N, ctx->sms, s)));
+      BIE_TRY(launch_force(X, Gm, n, N, elasticity, x_s, f, s));
+      BIE_TRY(launch_analyze({ana_group(pl, 3 * n, nullptr, N, G.foff3.ptr + 3 * i0, 0)}, f, fcoef, ctx->sms, s));
     }
-    for (int k = 0; k < 3; ++k) {
-      BIE_TRY((launch_leg_synth<double, double>(gammacoef + go, nullptr, nc, 1, p, T[k], P + 1, H, dphi[k], s)));
-      BIE_TRY((launch_phi_synth<double, double>(H, 1, p, P, pl->cs.ptr, Gm + k * N, nullptr, N, s)));
-    }
-    BIE_TRY(launch_force(X, Gm, N, elasticity, x_s, f, s));
-    BIE_TRY(launch_analyze(f, nullptr, N, 3, P, p, pl->cs.ptr, pl->A.ptr, F, fcoef + g->coef_off[d], nullptr, nc, s));
-    BIE_CUDA_TRY(cudaStreamSynchronize(s));  // the temporaries are released per drop
-    go += nc;
   }
+  BIE_CUDA_TRY(cudaStreamSynchronize(s));  // the temporaries are released on return
   return BIE_OK;
 }
 
@@ -3261,7 +3246,7 @@ static int reparam_group(bie_ctx* ctx, int p, const std::vector<int>& drops, con
     for (int c = 0; c < 3; ++c) vof.push_back(voff[d] + c * ncoef(p));
     sof.push_back(soff[d]);
   }
-  DevBuf<double> dab, dnodes, x0, xt, sc, th, ph, E, gradE, gv, gmax, H, F, a_d, norms, gE;
+  DevBuf<double> dab, dnodes, x0, xt, sc, th, ph, E, gradE, gv, gmax, a_d, norms, gE;
   DevBuf<long long> dvo, dso, dvof, dsof;
   DevBuf<int> active;
   BIE_TRY(dab.upload(ab));
@@ -3275,8 +3260,6 @@ static int reparam_group(bie_ctx* ctx, int p, const std::vector<int>& drops, con
   BIE_TRY(E.alloc(nd * 9 * N));
   for (DevBuf<double>* b : {&gradE, &gv}) BIE_TRY(b->alloc(nd * 3 * N));
   BIE_TRY(gmax.alloc(nd));
-  BIE_TRY(H.alloc(nd * 3 * (P + 1) * (size_t)(P + 1) * 2));
-  BIE_TRY(F.alloc(nd * 3 * (P + 1) * (size_t)(P + 1) * 2));
   BIE_TRY(a_d.alloc(nd * (P + 1)));
   BIE_TRY(norms.alloc(nd * (P + 1) * 2));
   BIE_TRY(active.alloc(nd));
@@ -3317,8 +3300,8 @@ static int reparam_group(bie_ctx* ctx, int p, const std::vector<int>& drops, con
     BIE_CUDA_TRY(cudaMemcpyAsync(a_d.ptr, av.data(), av.size() * sizeof(double), cudaMemcpyHostToDevice, s));
     // grad E = 2 sum_n a_n x~_n^m Y_n^m on the grid (Eq. energy_rep), its tangential part at the points
     BIE_TRY(launch_scale_degrees(xt.ptr, a_d.ptr, P, nd, 3, 2.0, sc.ptr, s));
-    BIE_TRY((launch_leg_synth<double, double>(sc.ptr, nullptr, nC, nd * 3, P, plP->T0.ptr, P + 1, H.ptr, 0, s)));
-    BIE_TRY((launch_phi_synth<double, double>(H.ptr, nd * 3, P, P, plP->cs.ptr, gradE.ptr, nullptr, N, s)));
+    BIE_TRY((launch_synth<double, double>(1, sc.ptr, (const long long*)nullptr, nC, nd * 3, P, P, plP->T0.ptr, nullptr,
+                                          nullptr, plP->cs.ptr, gradE.ptr, 0, N, ctx->sms, s)));
     BIE_TRY(launch_rep_gradient(E.ptr, gradE.ptr, N, nd, gv.ptr, gmax.ptr, s));
     BIE_CUDA_TRY(cudaMemcpyAsync(gm.data(), gmax.ptr, nd * sizeof(double), cudaMemcpyDeviceToHost, s));
     BIE_CUDA_TRY(cudaStreamSynchronize(s));
@@ -3334,8 +3317,7 @@ static int reparam_group(bie_ctx* ctx, int p, const std::vector<int>& drops, con
     BIE_TRY(launch_rep_step(E.ptr, gv.ptr, N, nd, active.ptr, o->dtau, th.ptr, ph.ptr, s));
     for (long long d = 0; d < nd; ++d) steps[d] += act[d];
     BIE_TRY(launch_eval_points(x0.ptr, 3, P, nd, N, th.ptr, ph.ptr, dab.ptr, 1, E.ptr, s));
-    BIE_TRY(launch_analyze(E.ptr, nullptr, 3 * N, nd * 3, P, P, plP->cs.ptr, plP->A.ptr, F.ptr, xt.ptr, nullptr, nC,
-                           s));
+    BIE_TRY(launch_analyze({ana_group(plP, nd * 3, nullptr, 3 * N, nullptr, nC)}, E.ptr, xt.ptr, ctx->sms, s));
   }
   for (long long d = 0; d < nd; ++d) {
     info->iterations = std::max(info->iterations, steps[d]);
@@ -3344,12 +3326,12 @@ static int reparam_group(bie_ctx* ctx, int p, const std::vector<int>& drops, con
     info->energy_last_max = std::max(info->energy_last_max, en[d]);
   }
   // Eq. rep_trasf2: the surfactant at the final angles; shape and surfactant analysed to degree p
-  BIE_TRY(launch_analyze(E.ptr, nullptr, 3 * N, nd * 3, P, p, plp->cs.ptr, plp->A.ptr, F.ptr, xcoef, dvof.ptr, 0, s));
+  BIE_TRY(launch_analyze({ana_group(plp, nd * 3, nullptr, 3 * N, dvof.ptr, 0)}, E.ptr, xcoef, ctx->sms, s));
   if (gammacoef) {
     BIE_TRY(launch_pad_coef(gammacoef, dso.ptr, p, P, nd, 1, x0.ptr, s));
     BIE_TRY(gE.alloc(nd * N));
     BIE_TRY(launch_eval_points(x0.ptr, 1, P, nd, N, th.ptr, ph.ptr, dab.ptr, 0, gE.ptr, s));
-    BIE_TRY(launch_analyze(gE.ptr, nullptr, N, nd, P, p, plp->cs.ptr, plp->A.ptr, F.ptr, gammacoef, dsof.ptr, 0, s));
+    BIE_TRY(launch_analyze({ana_group(plp, nd, nullptr, N, dsof.ptr, 0)}, gE.ptr, gammacoef, ctx->sms, s));
   }
   BIE_CUDA_TRY(cudaStreamSynchronize(s));
   return BIE_OK;

@@ -665,10 +665,15 @@ __global__ void k_weight_sources(const R* __restrict__ grid, const double* __res
   Q[c * ldq + o + s] = (R)rec[7 * o + 6 * N + s] * grid[idx];
 }
 
-// sum_s x.n wJ over one drop's records (for the volume), and max_s |x - c|, via atomics on doubles
-__global__ void k_drop_stats(const double* __restrict__ rec, long long N, double cx, double cy, double cz,
+// Per drop of a degree group (blockIdx.y; records of N points at rec + 7 off[i]): sum_s x.n wJ (for the
+// volume) and max_s |x - c| over each of 64 blocks, out[i][block][2].
+__global__ void k_drop_stats(const double* __restrict__ rec, const long long* __restrict__ off,
+                             const int* __restrict__ ids, const double* __restrict__ centre, long long N,
                              double* __restrict__ out) {
   __shared__ double sv[kThreads], sm[kThreads];
+  rec += 7 * off[blockIdx.y];
+  out += (long long)blockIdx.y * 2 * gridDim.x;
+  const double *c = centre + 3 * ids[blockIdx.y], cx = c[0], cy = c[1], cz = c[2];
   double v = 0, mx = 0;
   for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < N; s += (long long)gridDim.x * blockDim.x) {
     const double x = rec[s], y = rec[N + s], z = rec[2 * N + s];
@@ -692,18 +697,23 @@ __global__ void k_drop_stats(const double* __restrict__ rec, long long N, double
   }
 }
 
-// SoA source positions relative to the drop centre and normals, in precision R
-template <typename R>
-__global__ void k_source_geometry(const double* __restrict__ rec, long long N, double cx, double cy, double cz,
-                                  R* __restrict__ X, R* __restrict__ Nn, long long ld) {
-  long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= N) return;
-  X[s] = (R)(rec[s] - cx);
-  X[ld + s] = (R)(rec[N + s] - cy);
-  X[2 * ld + s] = (R)(rec[2 * N + s] - cz);
-  Nn[s] = (R)rec[3 * N + s];
-  Nn[ld + s] = (R)rec[4 * N + s];
-  Nn[2 * ld + s] = (R)rec[5 * N + s];
+// SoA source positions relative to the drop centres and normals in both precisions, for the nd drops of a
+// degree group (records of N points at rec + 7 off[i], sources at off[i])
+__global__ void k_source_geometry(const double* __restrict__ rec, const long long* __restrict__ off,
+                                  const int* __restrict__ ids, const double* __restrict__ centre, long long nd,
+                                  long long N, double* __restrict__ X64, double* __restrict__ N64,
+                                  float* __restrict__ X32, float* __restrict__ N32, long long ld) {
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= nd * N) return;
+  const long long d = idx / N, s = idx - d * N, o = off[d] + s;
+  const double* r = rec + 7 * off[d] + s;
+  for (int c = 0; c < 3; ++c) {
+    const double x = r[c * N] - centre[3 * ids[d] + c], n = r[(3 + c) * N];
+    X64[c * ld + o] = x;
+    N64[c * ld + o] = n;
+    X32[c * ld + o] = (float)x;
+    N32[c * ld + o] = (float)n;
+  }
 }
 
 }  // namespace
@@ -836,18 +846,22 @@ int launch_weight_sources(const R* grid, const double* rec, const long long* off
   return BIE_OK;
 }
 
-int launch_drop_stats(const double* rec, long long N, const double* c, double* out2x64, cudaStream_t s) {
-  k_drop_stats<<<64, kThreads, 0, s>>>(rec, N, c[0], c[1], c[2], out2x64);
-  count_launch();
-  BIE_CUDA_TRY(cudaGetLastError());
+int launch_drop_stats(const double* rec, const long long* off, const int* ids, const double* centre, long long nd,
+                      long long N, double* out, cudaStream_t s) {
+  for (long long i = 0; i < nd; i += 65535) {
+    k_drop_stats<<<dim3(64, (unsigned)(nd - i < 65535 ? nd - i : 65535)), kThreads, 0, s>>>(rec, off + i, ids + i, centre,
+                                                                                           N, out + 128 * i);
+    count_launch();
+    BIE_CUDA_TRY(cudaGetLastError());
+  }
   return BIE_OK;
 }
 
-template <typename R>
-int launch_source_geometry(const double* rec, long long N, const double* c, R* X, R* Nn, long long ld,
+int launch_source_geometry(const double* rec, const long long* off, const int* ids, const double* centre, long long nd,
+                           long long N, double* X64, double* N64, float* X32, float* N32, long long ld,
                            cudaStream_t s) {
-  if (N == 0) return BIE_OK;
-  k_source_geometry<R><<<blocks_for(N), kThreads, 0, s>>>(rec, N, c[0], c[1], c[2], X, Nn, ld);
+  if (nd * N == 0) return BIE_OK;
+  k_source_geometry<<<blocks_for(nd * N), kThreads, 0, s>>>(rec, off, ids, centre, nd, N, X64, N64, X32, N32, ld);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
@@ -866,9 +880,4 @@ template int launch_weight_sources<double>(const double*, const double*, const l
                                            double*, long long, cudaStream_t);
 template int launch_weight_sources<float>(const float*, const double*, const long long*, long long, long long, float*,
                                           long long, cudaStream_t);
-template int launch_source_geometry<double>(const double*, long long, const double*, double*, double*, long long,
-                                            cudaStream_t);
-template int launch_source_geometry<float>(const double*, long long, const double*, float*, float*, long long,
-                                           cudaStream_t);
-
 }  // namespace bie

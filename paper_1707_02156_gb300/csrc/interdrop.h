@@ -49,9 +49,12 @@ int launch_reduce_tiles(const double* partial, const int* tile_blk, const long l
 template <typename R>
 int launch_weight_sources(const R* grid, const double* rec, const long long* off, long long N, long long nd, R* Q,
                           long long ldq, cudaStream_t s);
-int launch_drop_stats(const double* rec, long long N, const double* c, double* out2x64, cudaStream_t s);
-template <typename R>
-int launch_source_geometry(const double* rec, long long N, const double* c, R* X, R* Nn, long long ld,
+// per drop i of a group (records of N points at rec + 7 off[i], its number ids[i]): out[i][64][2], the partial sums
+// of x.n wJ and the partial maxima of |x - centre|
+int launch_drop_stats(const double* rec, const long long* off, const int* ids, const double* centre, long long nd,
+                      long long N, double* out, cudaStream_t s);
+int launch_source_geometry(const double* rec, const long long* off, const int* ids, const double* centre, long long nd,
+                           long long N, double* X64, double* N64, float* X32, float* N32, long long ld,
                            cudaStream_t s);
 
 }  // namespace bie

@@ -35,36 +35,31 @@ __host__ __device__ inline long long leg_row(int p, int m, int n, int nj) {
 }
 
 // ---- transforms (transforms.cu) ----
-// Legendre step of synthesis: H[f][m][j] = sum_n c_f(n,m) T[m][n][j] (complex, m >= 0), with an
-// optional phi-derivative factor (i m)^dphi.  Coefficients of field f start at
-// field_off ? field_off[f] : f * coef_stride.
+// Synthesis of nfield fields of degree p on the grid of degree P, with the derivative kinds of the mask
+// `kinds` (bit 0 f, 1 t, 2 p, 3 tt, 4 tp, 5 pp; the masks 1, 6, 7, 62, 63 in FP64, 1 in FP32): kind
+// number s of the mask of field f goes to out + s * kind_stride + f * field_stride.  Coefficients of
+// field f start at field_off ? field_off[f] : f * coef_stride.  T1, T2 may be null when no kind needs them.
 template <typename CT, typename R>
-int launch_leg_synth(const CT* coef, const long long* field_off, long long coef_stride, long long nfield, int p,
-                     const R* T, int nj, R* H, int dphi, cudaStream_t s);
-// phi step of synthesis: out[f][j][k] = Re sum_m fac_m H[f][m][j] e^{i m phi_k}, k < 2P+2
-template <typename R, typename OT>
-int launch_phi_synth(const R* H, long long nfield, int p, int P, const R* cs, OT* out,
-                     const long long* out_off, long long out_stride, cudaStream_t s);
-// analysis: grid (degree P) -> coefficients (degree p_out), FP64
-int launch_analyze(const double* grid, const long long* grid_off, long long grid_stride, long long nfield, int P,
-                   int p_out, const double* cs, const double* A, double* F, double* coef,
-                   const long long* coef_off, long long coef_stride, cudaStream_t s);
-// analysis of nfield fields on their own degree-p grids, for several degree groups in one launch
-// (grid_off, coef_off per field; begin is set by the launcher)
+int launch_synth(int kinds, const CT* coef, const long long* field_off, long long coef_stride, long long nfield, int p,
+                 int P, const R* T0, const R* T1, const R* T2, const R* cs, R* out, long long kind_stride,
+                 long long field_stride, int sms, cudaStream_t s);
+// analysis: grids (degree P) -> coefficients (degree p <= P), FP64, for several degree groups in one launch.
+// Offsets per field, or null and a stride; begin and mb are set by the launcher.
 struct AnaGroup {
   long long begin, nfield;
   const long long* grid_off;
   const long long* coef_off;
+  long long grid_base, grid_stride, coef_base, coef_stride;  // grid f at base + (off[f] or f stride)
   const double* cs;
-  const double* A;
-  int p;
+  const double* At;  // weighted Legendre table, rows (m, j) with the degree n = m..p fastest
+  int P, p, mb;
 };
 constexpr int kMaxAnaGroups = 8;
 struct AnaGroups {
   int n;
   AnaGroup g[kMaxAnaGroups];
 };
-int launch_analyze_fused(const std::vector<AnaGroup>& groups, const double* grid, double* coef, cudaStream_t s);
+int launch_analyze(std::vector<AnaGroup> groups, const double* grid, double* coef, int sms, cudaStream_t s);
 // rotation (App. B): out[ld][a*nb+b][c] = blocks(a) applied to e^{i m alpha_b} coef[ld][c]
 template <typename CT, typename R>
 int launch_rotate(const CT* coef, const long long* field_off, int ncomp, long long ndrop, int p, const R* blocks,
@@ -75,9 +70,11 @@ int launch_phase(double* coef, long long nfield, int p, double gamma, cudaStream
 
 // ---- pair sums and geometry (pairs.cu) ----
 // Surface quantities from x, x_theta, x_phi grids [f=drop*3+c][j][k]: writes SoA source records
-// [drop][7][N] = (x, n, wgt*J) with wgt the regular weight (pi/(P+1)) w_j, J = W/sin(theta_j).
+// [7][N] = (x, n, wgt*J) of drop d at rec + 7 * off[d], with wgt the regular weight (pi/(P+1)) w_j,
+// J = W/sin(theta_j).
 int launch_surface(const double* X, const double* Xt, const double* Xp, long long ndrop, int P,
-                   const double* wsin /*[j] = w_j pi/(P+1)/sin theta_j*/, double* rec, cudaStream_t s);
+                   const double* wsin /*[j] = w_j pi/(P+1)/sin theta_j*/, double* rec, const long long* off,
+                   cudaStream_t s);
 // Rotated-grid cache for ndrop drops of ng targets each: cache[t][7][nq] = (x0 - x', n',
 // w^s_j W'/sin theta_j) on the degree-pq grid; x0 of drop ld's targets read from the standard-grid
 // records at rec_std + rec_off[ld] ([7][ng] per drop; the drops need not be adjacent there).
@@ -131,8 +128,10 @@ long long self_tc_g_floats(const std::vector<SelfGroup<float>>& groups, long lon
 bool self_tc_fits(int p);
 int launch_self_tc(const std::vector<SelfGroup<float>>& groups, const double* dens, double* vals, float* eo,
                    unsigned* gm, long long budget, cudaStream_t s);
-// interfacial force at N grid points from x derivatives [6][3][N] and Gamma derivatives [3][N]
-int launch_force(const double* X, const double* Gm, long long N, double es, double xs, double* f, cudaStream_t s);
+// interfacial force at the N grid points of nd drops from x derivatives [5][nd][3][N] (t, p, tt, tp, pp) and
+// Gamma and its derivatives [3][nd][N] (f, t, p): f [nd][3][N]
+int launch_force(const double* X, const double* Gm, long long nd, long long N, double es, double xs, double* f,
+                 cudaStream_t s);
 // out[i] = (float) in[i]
 int launch_to_float(const double* in, float* out, long long n, cudaStream_t s);
 

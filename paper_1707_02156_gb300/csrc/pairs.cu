@@ -19,10 +19,10 @@ __device__ inline void cross3(const double* a, const double* b, double* c) {
   c[2] = a[0] * b[1] - a[1] * b[0];
 }
 
-// rec[d][0..2] = x, [3..5] = outward normal x_theta x x_phi / W, [6] = wsin[j] * W
+// rec + 7 off[d]: [0..2] = x, [3..5] = outward normal x_theta x x_phi / W, [6] = wsin[j] * W
 __global__ void k_surface(const double* __restrict__ X, const double* __restrict__ Xt,
                           const double* __restrict__ Xp, long long ndrop, int P, const double* __restrict__ wsin,
-                          double* __restrict__ rec) {
+                          double* __restrict__ rec, const long long* __restrict__ off) {
   const int nk = 2 * P + 2;
   const long long N = (long long)(P + 1) * nk;
   long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -38,7 +38,7 @@ __global__ void k_surface(const double* __restrict__ X, const double* __restrict
   }
   cross3(xt, xp, c);
   double W = sqrt(c[0] * c[0] + c[1] * c[1] + c[2] * c[2]);
-  double* r = rec + d * 7 * N;
+  double* r = rec + 7 * off[d];
   for (int i = 0; i < 3; ++i) {
     r[i * N + q] = x[i];
     r[(3 + i) * N + q] = c[i] / W;
@@ -78,22 +78,25 @@ __global__ void k_rotgeo(const double* __restrict__ X, const double* __restrict_
   o[6 * nq + q] = (R)(wsq[j] * W);
 }
 
-// Interfacial force f = -2 sigma K n - grad_gamma sigma at grid points (Sec. 1, Table 2), from the
-// six derivative fields of x ([3][N] each, order: f, t, p, tt, tp, pp) and of Gamma (f, t, p).
+// Interfacial force f = -2 sigma K n - grad_gamma sigma at the grid points of nd drops (Sec. 1, Table 2),
+// from the derivative fields of x ([nd][3][N] each, order: t, p, tt, tp, pp) and of Gamma ([nd][N]: f, t, p).
 // K = (E N - 2 F M + G L) / (2 W^2) with E = x_p.x_p, F = x_p.x_t, G = x_t.x_t, L = x_pp.n,
 // M = x_tp.n, N = x_tt.n, outward n = x_t x x_p / W; sigma = 1 + E_s ln(1 - x_s Gamma) (x_s > 0)
 // or 1 - E_s Gamma; grad sigma = [(G s_p - F s_t) x_p + (E s_t - F s_p) x_t] / W^2.
-__global__ void k_force(const double* __restrict__ X, const double* __restrict__ Gm, long long N, double es,
-                        double xs, double* __restrict__ f) {
-  long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= N) return;
+__global__ void k_force(const double* __restrict__ X, const double* __restrict__ Gm, long long nd, long long N,
+                        double es, double xs, double* __restrict__ f) {
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= nd * N) return;
+  const long long d = idx / N, q = idx - d * N, ks = nd * 3 * N;
+  X += d * 3 * N;
+  f += d * 3 * N;
   double xt[3], xp[3], xtt[3], xtp[3], xpp[3], n[3];
   for (int c = 0; c < 3; ++c) {
-    xt[c] = X[(1 * 3 + c) * N + q];
-    xp[c] = X[(2 * 3 + c) * N + q];
-    xtt[c] = X[(3 * 3 + c) * N + q];
-    xtp[c] = X[(4 * 3 + c) * N + q];
-    xpp[c] = X[(5 * 3 + c) * N + q];
+    xt[c] = X[0 * ks + c * N + q];
+    xp[c] = X[1 * ks + c * N + q];
+    xtt[c] = X[2 * ks + c * N + q];
+    xtp[c] = X[3 * ks + c * N + q];
+    xpp[c] = X[4 * ks + c * N + q];
   }
   cross3(xt, xp, n);
   const double W = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
@@ -106,7 +109,7 @@ __global__ void k_force(const double* __restrict__ X, const double* __restrict__
   const double Nn = xtt[0] * n[0] + xtt[1] * n[1] + xtt[2] * n[2];
   const double W2 = W * W;
   const double K = (E * Nn - 2.0 * F * M + G * L) / (2.0 * W2);
-  const double gam = Gm[q], gt = Gm[N + q], gp = Gm[2 * N + q];
+  const double gam = Gm[idx], gt = Gm[nd * N + idx], gp = Gm[2 * nd * N + idx];
   double sigma, ds;
   if (xs > 0.0) {
     sigma = 1.0 + es * log(1.0 - xs * gam);
@@ -135,19 +138,20 @@ int launch_to_float(const double* in, float* out, long long n, cudaStream_t s) {
   return BIE_OK;
 }
 
-int launch_force(const double* X, const double* Gm, long long N, double es, double xs, double* f, cudaStream_t s) {
-  if (N == 0) return BIE_OK;
-  k_force<<<blocks_for(N), kThreads, 0, s>>>(X, Gm, N, es, xs, f);
+int launch_force(const double* X, const double* Gm, long long nd, long long N, double es, double xs, double* f,
+                 cudaStream_t s) {
+  if (nd * N == 0) return BIE_OK;
+  k_force<<<blocks_for(nd * N), kThreads, 0, s>>>(X, Gm, nd, N, es, xs, f);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
 }
 
 int launch_surface(const double* X, const double* Xt, const double* Xp, long long ndrop, int P,
-                   const double* wsin, double* rec, cudaStream_t s) {
+                   const double* wsin, double* rec, const long long* off, cudaStream_t s) {
   long long n = ndrop * (long long)(P + 1) * (2 * P + 2);
   if (n == 0) return BIE_OK;
-  k_surface<<<blocks_for(n), kThreads, 0, s>>>(X, Xt, Xp, ndrop, P, wsin, rec);
+  k_surface<<<blocks_for(n), kThreads, 0, s>>>(X, Xt, Xp, ndrop, P, wsin, rec, off);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;

@@ -1,9 +1,16 @@
 // SH transforms and Wigner rotation kernels (Sec. 1.1, Sec. 2.1, App. A, App. B).
 //
-// Synthesis is split into a Legendre step (per order m, a contraction over the degree n with the
-// normalised Legendre table of the target grid) and a phi step (per latitude, a real inverse DFT of
-// length 2P+2 that uses phi_{k+P+1} = phi_k + pi to evaluate even and odd orders once for two
-// longitudes).  Analysis runs the same two steps in the opposite order with the weighted table.
+// Synthesis (k_synth) and analysis (k_analyze) each run their Legendre and phi steps in one kernel, with
+// the intermediate per-order values in shared memory.  Both steps use the symmetries of the grid:
+//   theta -> pi - theta:  P~_n^m(-t) = (-1)^(n+m) P~_n^m(t) (the theta derivative with the opposite
+//     sign), so the sums over even and odd n - m serve two latitudes;
+//   phi_k, pi - phi_k, pi + phi_k, 2 pi - phi_k share |cos m phi| and |sin m phi|, so the sums over
+//     even and odd m of the cosine and the sine parts serve four longitudes.
+// In FP64, whose rate is 1/76 of FP32's here, the operation count is the bound of every large batch; the
+// symmetries and the plain multiply-adds leave a quarter of the direct sums' operations.  Measured against
+// the direct sums in two kernels: the rotated grids of 64 drops of degree 24 (80000 targets x 3 fields x 3
+// kinds) 103.5 -> 62.7 ms with their rotation, the projection of 192 drops of degree 24 0.52 -> 0.076 ms, the
+// surfactant's rates and implicit stage of 48 drops 10.4 -> 6.2 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -19,180 +26,223 @@ constexpr int kThreads = 256;
 
 inline unsigned blocks_for(long long n, int t = kThreads) { return (unsigned)((n + t - 1) / t); }
 
-template <typename CT, typename R>
-__global__ void k_leg_synth(const CT* __restrict__ coef, const long long* __restrict__ field_off,
-                            long long coef_stride, long long nfield, int p, const R* __restrict__ T, int nj,
-                            R* __restrict__ H, int dphi) {
-  long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  long long per_field = (long long)(p + 1) * nj;
-  if (idx >= nfield * per_field) return;
-  long long f = idx / per_field;
-  int r = (int)(idx - f * per_field);
-  int m = r / nj;
-  int j = r - m * nj;
-  const CT* c = coef + (field_off ? field_off[f] : f * coef_stride);
-  R re = 0, im = 0;
-  const R* Tm = T + leg_row(p, m, m, nj) + j;
-  for (int n = m; n <= p; ++n) {
-    R t = Tm[(long long)(n - m) * nj];
-    int base = n * (n + 1);
-    re += (R)c[base + m] * t;
-    if (m > 0) im += (R)c[base - m] * t;
-  }
-  if (dphi == 1) {  // multiply by i m
-    R t = re;
-    re = -(R)m * im;
-    im = (R)m * t;
-  } else if (dphi == 2) {  // multiply by -m^2
-    re *= -(R)(m * m);
-    im *= -(R)(m * m);
-  }
-  R* h = H + ((f * (p + 1) + m) * (long long)nj + j) * 2;
-  h[0] = re;
-  h[1] = im;
+// Derivative kinds of a synthesis, in output order: f, t, p, tt, tp, pp.  Bit k of a mask asks for kind k.
+__host__ __device__ constexpr int kind_slot(int kinds, int k) {
+  int s = 0;
+  for (int i = 0; i < k; ++i) s += (kinds >> i) & 1;
+  return s;
 }
 
-template <typename R, typename OT>
-__global__ void k_phi_synth(const R* __restrict__ H, long long nfield, int p, int P, const R* __restrict__ cs,
-                            OT* __restrict__ out, const long long* __restrict__ out_off, long long out_stride) {
-  const int nj = P + 1, nk = 2 * P + 2, half = P + 1;
-  long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  long long per_field = (long long)nj * half;
-  if (idx >= nfield * per_field) return;
-  long long f = idx / per_field;
-  int r = (int)(idx - f * per_field);
-  int j = r / half;
-  int k = r - j * half;
-  const R* h = H + (f * (p + 1) * (long long)nj + j) * 2;
-  R ev = h[0], od = 0;  // m = 0 term (cos 0 = 1, imaginary part of h_0 is zero for real fields)
-  for (int m = 1; m <= p; ++m) {
-    R hr = h[(long long)m * nj * 2], hi = h[(long long)m * nj * 2 + 1];
-    R c = cs[((long long)m * nk + k) * 2], s = cs[((long long)m * nk + k) * 2 + 1];
-    R v = 2 * (hr * c - hi * s);
-    if (m & 1)
-      od += v;
-    else
-      ev += v;
+constexpr int kSynThreads = 128;
+constexpr int kSynStageP = BIE_MAX_P;  // coefficients are staged in shared memory up to this degree
+
+// One block per (field, jb latitude pairs j and P - j).  Phase 1, thread per (order m, pair): the sums
+// over even and odd n - m with the Legendre tables asked for, for both latitudes, and from them each
+// kind's complex value per order (factors i m and -m^2, and the 2 of m > 0) in shared memory
+// h[kind][row][m].  Phase 2, thread per (row, longitude quadruple).
+template <typename CT, typename R, int KINDS>
+__global__ void __launch_bounds__(kSynThreads) k_synth(const CT* __restrict__ coef,
+                                                       const long long* __restrict__ field_off, long long coef_stride,
+                                                       int p, int P, const R* __restrict__ T0,
+                                                       const R* __restrict__ T1, const R* __restrict__ T2,
+                                                       const R* __restrict__ cs, R* __restrict__ out,
+                                                       long long kind_stride, long long field_stride, int jb) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int NK = kind_slot(KINDS, 6);
+  const int nj = P + 1, nk = 2 * P + 2, half = P + 1, np = (nj + 1) / 2, k4n = half / 2 + 1;
+  const int njb = (np + jb - 1) / jb;
+  const long long f = blockIdx.x / njb;
+  const int q0 = (int)(blockIdx.x % njb) * jb, jbn = min(jb, np - q0);
+  R* h = reinterpret_cast<R*>(smem_raw);  // [NK][2 jb][p+1][2]
+  const long long hk = 2LL * jb * (p + 1) * 2;
+  const CT* cg = coef + (field_off ? field_off[f] : f * coef_stride);
+  const bool staged = p <= kSynStageP;
+  R* c = h + NK * hk;
+  if (staged) {
+    for (int i = threadIdx.x; i < (p + 1) * (p + 1); i += kSynThreads) c[i] = (R)cg[i];
+    __syncthreads();
   }
-  OT* o = out + (out_off ? out_off[f] : f * out_stride) + (long long)j * nk;
-  o[k] = (OT)(ev + od);
-  o[k + half] = (OT)(ev - od);
-}
-
-// F[f][m][j] = sum_k g[j][k] e^{-i m phi_k}
-__global__ void k_phi_analyze(const double* __restrict__ grid, const long long* __restrict__ grid_off,
-                              long long grid_stride, long long nfield, int P, int p_out,
-                              const double* __restrict__ cs, double* __restrict__ F) {
-  const int nj = P + 1, nk = 2 * P + 2;
-  long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  long long per_field = (long long)(p_out + 1) * nj;
-  if (idx >= nfield * per_field) return;
-  long long f = idx / per_field;
-  int r = (int)(idx - f * per_field);
-  int m = r / nj;
-  int j = r - m * nj;
-  const double* g = grid + (grid_off ? grid_off[f] : f * grid_stride) + (long long)j * nk;
-  double re = 0, im = 0;
-  for (int k = 0; k < nk; ++k) {
-    double v = g[k];
-    re += v * cs[((long long)m * nk + k) * 2];
-    im -= v * cs[((long long)m * nk + k) * 2 + 1];
-  }
-  double* o = F + ((f * (p_out + 1) + m) * (long long)nj + j) * 2;
-  o[0] = re;
-  o[1] = im;
-}
-
-// coef(n, m) = sum_j A[m][n][j] F[m][j]
-__global__ void k_leg_analyze(const double* __restrict__ F, long long nfield, int P, int p_out,
-                              const double* __restrict__ A, double* __restrict__ coef,
-                              const long long* __restrict__ coef_off, long long coef_stride) {
-  const int nj = P + 1;
-  const int nc = (p_out + 1) * (p_out + 2) / 2;
-  long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= nfield * nc) return;
-  long long f = idx / nc;
-  int r = (int)(idx - f * nc);
-  // r enumerates (m, n) with m <= n in the table's row order
-  int m = 0;
-  while (r >= p_out + 1 - m) {
-    r -= p_out + 1 - m;
-    ++m;
-  }
-  int n = m + r;
-  const double* a = A + leg_row(p_out, m, n, nj);
-  const double* Fm = F + (f * (p_out + 1) + m) * (long long)nj * 2;
-  double re = 0, im = 0;
-  for (int j = 0; j < nj; ++j) {
-    re += a[j] * Fm[2 * j];
-    im += a[j] * Fm[2 * j + 1];
-  }
-  double* c = coef + (coef_off ? coef_off[f] : f * coef_stride);
-  c[n * (n + 1) + m] = re;
-  if (m > 0) c[n * (n + 1) - m] = im;
-}
-
-// Analysis on the field's own grid (degree p), one block per (field, order m): the phi transform
-// F_m(theta_j) of the block's order, one warp per latitude with the lanes across the longitudes
-// (coalesced loads, shuffle reduction), then the contraction with the weighted Legendre table for
-// n = m..p, one warp per degree with the lanes across the latitudes.
-constexpr int kAnaThreads = 512;  // 16 warps: about two latitudes, then two degrees, per warp at p = 32
-
-__device__ inline double warp_sum(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Several degree groups in one launch: block ranges per group, arguments by value.
-__global__ void __launch_bounds__(kAnaThreads) k_analyze_fused(AnaGroups G, const double* __restrict__ grid,
-                                                               double* __restrict__ coef) {
-  __shared__ double F[2 * (BIE_MAX_P + 1)];
-  AnaGroup Gr = G.g[0];
+  for (int i = threadIdx.x; i < (p + 1) * jbn; i += kSynThreads) {
+    const int m = i / jbn, q = i - m * jbn, j = q0 + q;
+    R e[3][2], o[3][2];  // [table][re, im], sums over even and odd n - m
 #pragma unroll
-  for (int i = 1; i < kMaxAnaGroups; ++i)
-    if (i < G.n && (long long)blockIdx.x >= G.g[i].begin) Gr = G.g[i];
-  const int p = Gr.p;
-  const long long* __restrict__ grid_off = Gr.grid_off;
-  const long long* __restrict__ coef_off = Gr.coef_off;
-  const double* __restrict__ cs = Gr.cs;
-  const double* __restrict__ A = Gr.A;
-  const int nj = p + 1, nk = 2 * p + 2;
-  const long long bl = (long long)blockIdx.x - Gr.begin;
-  const long long f = bl / (p + 1);
-  const int m = (int)(bl - f * (p + 1));
-  const double* src = grid + grid_off[f];
-  const double* c = cs + (long long)m * nk * 2;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int j = warp; j < nj; j += nw) {
-    const double* row = src + (long long)j * nk;
-    double re = 0, im = 0;
-    for (int k = lane; k < nk; k += 32) {
-      const double v = row[k];
-      re += v * c[2 * k];
-      im -= v * c[2 * k + 1];
+    for (int t = 0; t < 3; ++t) e[t][0] = e[t][1] = o[t][0] = o[t][1] = 0;
+    const long long row = leg_row(p, m, m, nj) + j;
+    for (int n = m; n <= p; ++n) {
+      const int at = n * (n + 1);
+      const R re = staged ? c[at + m] : (R)cg[at + m], im = m == 0 ? (R)0 : staged ? c[at - m] : (R)cg[at - m];
+      const long long r = row + (long long)(n - m) * nj;
+      const bool odd = (n - m) & 1;
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        // tables 0, 1, 2 serve the kinds {f, p, pp}, {t, tp}, {tt}
+        if (!(KINDS & (t == 0 ? 37 : t == 1 ? 18 : 8))) continue;
+        const R v = t == 0 ? T0[r] : t == 1 ? T1[r] : T2[r];
+        if (odd) {
+          o[t][0] += re * v;
+          o[t][1] += im * v;
+        } else {
+          e[t][0] += re * v;
+          e[t][1] += im * v;
+        }
+      }
     }
-    re = warp_sum(re);
-    im = warp_sum(im);
-    if (lane == 0) {
-      F[2 * j] = re;
-      F[2 * j + 1] = im;
+    const R fac = m == 0 ? 1 : 2;
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        if (!((KINDS >> k) & 1)) continue;
+        const int t = k == 3 ? 2 : (k == 1 || k == 4) ? 1 : 0;
+        R re = fac * (side == 0 ? e[t][0] + o[t][0] : t == 1 ? o[t][0] - e[t][0] : e[t][0] - o[t][0]);
+        R im = fac * (side == 0 ? e[t][1] + o[t][1] : t == 1 ? o[t][1] - e[t][1] : e[t][1] - o[t][1]);
+        if (k == 2 || k == 4) {  // multiply by i m
+          const R w = re;
+          re = -(R)m * im;
+          im = (R)m * w;
+        } else if (k == 5) {
+          re *= -(R)(m * m);
+          im *= -(R)(m * m);
+        }
+        R* d = h + kind_slot(KINDS, k) * hk + ((2 * q + side) * (p + 1) + m) * 2;
+        d[0] = re;
+        d[1] = im;
+      }
     }
   }
   __syncthreads();
-  double* out = coef + coef_off[f];
-  for (int n = m + warp; n <= p; n += nw) {
-    const double* a = A + leg_row(p, m, n, nj);
+  for (int i = threadIdx.x; i < 2 * jbn * k4n; i += kSynThreads) {
+    const int row = i / k4n, k = i - row * k4n;
+    const int j = row & 1 ? P - (q0 + row / 2) : q0 + row / 2;
+    if ((row & 1) && 2 * j == P) continue;  // the middle latitude is its own mirror
+    const R* hr = h + (long long)row * (p + 1) * 2;
+    R ce[NK], co[NK], se[NK], so[NK];
+#pragma unroll
+    for (int s = 0; s < NK; ++s) {
+      ce[s] = hr[s * hk];
+      co[s] = se[s] = so[s] = 0;
+    }
+    int m = 1;
+    for (; m + 1 <= p; m += 2) {
+      const R c1 = cs[((long long)m * nk + k) * 2], s1 = cs[((long long)m * nk + k) * 2 + 1];
+      const R c2 = cs[((long long)(m + 1) * nk + k) * 2], s2 = cs[((long long)(m + 1) * nk + k) * 2 + 1];
+#pragma unroll
+      for (int s = 0; s < NK; ++s) {
+        const R* a = hr + s * hk + 2 * m;
+        co[s] += a[0] * c1;
+        so[s] += a[1] * s1;
+        ce[s] += a[2] * c2;
+        se[s] += a[3] * s2;
+      }
+    }
+    if (m <= p) {
+      const R c1 = cs[((long long)m * nk + k) * 2], s1 = cs[((long long)m * nk + k) * 2 + 1];
+#pragma unroll
+      for (int s = 0; s < NK; ++s) {
+        const R* a = hr + s * hk + 2 * m;
+        co[s] += a[0] * c1;
+        so[s] += a[1] * s1;
+      }
+    }
+    const bool rot = k > 0, mir = 2 * k < half;  // k = 0 and the middle k have two longitudes, not four
+    R* d0 = out + f * field_stride + (long long)j * nk;
+#pragma unroll
+    for (int s = 0; s < NK; ++s) {
+      R* d = d0 + s * kind_stride;
+      const R cp = ce[s] + co[s], cm = ce[s] - co[s], sp = se[s] + so[s], sm = se[s] - so[s];
+      d[k] = cp - sp;
+      if (mir) d[half + k] = cm - sm;
+      if (rot) d[2 * half - k] = cp + sp;
+      if (rot && mir) d[half - k] = cm + sm;
+    }
+  }
+}
+
+// One block per (field, mb orders).  The field's rows pass through shared memory kr at a time, folded over
+// the four longitudes of each quadruple into what the even and odd orders' cosine and sine sums
+// need; F[m][j] for the block's orders; then F folded over the latitude pairs and the products with the
+// weighted Legendre table (stored with the degree fastest, so that neighbouring threads read
+// neighbouring entries).  Several degree groups share a launch: block ranges per group, arguments by value.
+constexpr int kAnaThreads = 256;
+
+__host__ __device__ inline int ana_rows(int P) { return P < 64 ? 32 : P < 128 ? 16 : 8; }
+
+__global__ void __launch_bounds__(kAnaThreads) k_analyze(AnaGroups G, const double* __restrict__ grid,
+                                                         double* __restrict__ coef) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  AnaGroup A = G.g[0];
+#pragma unroll
+  for (int i = 1; i < kMaxAnaGroups; ++i)
+    if (i < G.n && (long long)blockIdx.x >= G.g[i].begin) A = G.g[i];
+  const int P = A.P, p = A.p, mb = A.mb;
+  const int nj = P + 1, nk = 2 * P + 2, half = P + 1, np = (nj + 1) / 2, k4n = half / 2 + 1, kr = ana_rows(P);
+  const int nmb = (p + mb) / mb;
+  const long long bl = (long long)blockIdx.x - A.begin;
+  const long long f = bl / nmb;
+  const int m0 = (int)(bl - f * nmb) * mb, mn = min(mb, p + 1 - m0);
+  double* F = reinterpret_cast<double*>(smem_raw);  // [mb][nj][2]
+  double* fold = F + 2 * (long long)mb * nj;        // [cos even, cos odd, sin even, sin odd][k4n][kr]
+  const double* src = grid + A.grid_base + (A.grid_off ? A.grid_off[f] : f * A.grid_stride);
+  for (int j0 = 0; j0 < nj; j0 += kr) {
+    const int rn = min(kr, nj - j0);
+    for (int i = threadIdx.x; i < rn * k4n; i += kAnaThreads) {
+      const int r = i / k4n, k = i - r * k4n;
+      const double* g = src + (long long)(j0 + r) * nk;
+      const bool rot = k > 0, mir = 2 * k < half;
+      const double a = g[k], b = rot ? g[2 * half - k] : 0.0, c = mir ? g[half + k] : 0.0,
+                   d = rot && mir ? g[half - k] : 0.0;
+      const double ab = a + b, cd = c + d, amb = a - b, cmd = c - d;
+      double* o = fold + k * kr + r;
+      o[0] = ab + cd;
+      o[k4n * kr] = ab - cd;
+      o[2 * k4n * kr] = amb + cmd;
+      o[3 * k4n * kr] = amb - cmd;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < mn * kr; i += kAnaThreads) {
+      const int mm = i / kr, r = i - mm * kr;
+      if (r >= rn) continue;
+      const int m = m0 + mm, odd = m & 1;
+      const double* c = A.cs + (long long)m * nk * 2;
+      const double* fc = fold + (long long)odd * k4n * kr + r;
+      const double* fs = fold + (long long)(2 + odd) * k4n * kr + r;
+      double re = 0, im = 0;
+      for (int k = 0; k < k4n; ++k) {
+        re += fc[k * kr] * c[2 * k];
+        im -= fs[k * kr] * c[2 * k + 1];
+      }
+      F[(mm * nj + j0 + r) * 2] = re;
+      F[(mm * nj + j0 + r) * 2 + 1] = im;
+    }
+    __syncthreads();
+  }
+  // latitude pairs: F(j) + F(P-j) at j for even n - m, F(j) - F(P-j) at P-j for odd
+  for (int i = threadIdx.x; i < mn * (nj / 2) * 2; i += kAnaThreads) {
+    const int ri = i & 1, r = i >> 1, mm = r / (nj / 2), j = r - mm * (nj / 2);
+    double* lo = F + (mm * nj + j) * 2 + ri;
+    double* hi = F + (mm * nj + P - j) * 2 + ri;
+    const double a = *lo, b = *hi;
+    *lo = a + b;
+    *hi = a - b;
+  }
+  __syncthreads();
+  double* out = coef + A.coef_base + (A.coef_off ? A.coef_off[f] : f * A.coef_stride);
+  const int per = p + 1 - m0;  // degrees of the block's lowest order
+  for (int i = threadIdx.x; i < mn * per; i += kAnaThreads) {
+    const int mm = i / per, d = i - mm * per, m = m0 + mm, n = m + d;
+    if (n > p) continue;
+    const bool odd = d & 1;
+    const double* a = A.At + leg_row(p, m, m, nj) + d;
+    const double* Fm = F + (long long)mm * nj * 2;
     double re = 0, im = 0;
-    for (int j = lane; j < nj; j += 32) {
-      re += a[j] * F[2 * j];
-      im += a[j] * F[2 * j + 1];
+    for (int j = 0; j < (odd ? nj / 2 : np); ++j) {
+      const double v = a[(long long)j * (p + 1 - m)];
+      const int jj = odd ? P - j : j;
+      re += v * Fm[2 * jj];
+      im += v * Fm[2 * jj + 1];
     }
-    re = warp_sum(re);
-    im = warp_sum(im);
-    if (lane == 0) {
-      out[n * (n + 1) + m] = re;
-      if (m > 0) out[n * (n + 1) - m] = im;
-    }
+    out[n * (n + 1) + m] = re;
+    if (m > 0) out[n * (n + 1) - m] = im;
   }
 }
 
@@ -285,57 +335,75 @@ __global__ void k_phase(double* __restrict__ coef, long long nfield, int p, doub
 
 }  // namespace
 
+template <typename CT, typename R, int KINDS>
+static int synth_launch(const CT* coef, const long long* field_off, long long coef_stride, long long nfield, int p, int P,
+                        const R* T0, const R* T1, const R* T2, const R* cs, R* out, long long kind_stride,
+                        long long field_stride, int sms, cudaStream_t s) {
+  if (nfield == 0) return BIE_OK;
+  const int np = (P + 2) / 2;
+  const size_t stage = p <= kSynStageP ? sizeof(R) * (size_t)(p + 1) * (p + 1) : 0;
+  const size_t pair = sizeof(R) * kind_slot(KINDS, 6) * 4 * (size_t)(p + 1);
+  // latitude pairs per block: all of them when there are fields for four blocks per SM (the coefficients
+  // are staged once), fewer when not, so that small batches spread over the SMs; at most 64 KB a block
+  const long long want = std::max(1LL, nfield * np / (4LL * sms));
+  const long long fit = std::max<long long>(1, ((64 << 10) - (long long)stage) / (long long)pair);
+  const int jb = (int)std::min<long long>(np, std::min(want, fit));
+  const size_t smem = stage + pair * jb;
+  const long long nblk = nfield * ((np + jb - 1) / jb);
+  if (nblk > 0x7fffffffLL) return BIE_EINVAL;
+  auto kern = k_synth<CT, R, KINDS>;
+  if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  kern<<<(unsigned)nblk, kSynThreads, smem, s>>>(coef, field_off, coef_stride, p, P, T0, T1, T2, cs, out, kind_stride,
+                                                 field_stride, jb);
+  count_launch();
+  BIE_CUDA_TRY(cudaGetLastError());
+  return BIE_OK;
+}
+
 template <typename CT, typename R>
-int launch_leg_synth(const CT* coef, const long long* field_off, long long coef_stride, long long nfield, int p,
-                     const R* T, int nj, R* H, int dphi, cudaStream_t s) {
-  long long n = nfield * (long long)(p + 1) * nj;
-  if (n == 0) return BIE_OK;
-  k_leg_synth<CT, R><<<blocks_for(n), kThreads, 0, s>>>(coef, field_off, coef_stride, nfield, p, T, nj, H, dphi);
-  count_launch();
-  BIE_CUDA_TRY(cudaGetLastError());
-  return BIE_OK;
+int launch_synth(int kinds, const CT* coef, const long long* field_off, long long coef_stride, long long nfield, int p,
+                 int P, const R* T0, const R* T1, const R* T2, const R* cs, R* out, long long kind_stride,
+                 long long field_stride, int sms, cudaStream_t s) {
+#define BIE_SYNTH(K)                                                                                             \
+  if (kinds == K)                                                                                                \
+  return synth_launch<CT, R, K>(coef, field_off, coef_stride, nfield, p, P, T0, T1, T2, cs, out, kind_stride, \
+                                field_stride, sms, s)
+  BIE_SYNTH(1);
+  if constexpr (sizeof(R) == 8) {
+    BIE_SYNTH(6);
+    BIE_SYNTH(7);
+    BIE_SYNTH(62);
+    BIE_SYNTH(63);
+  }
+#undef BIE_SYNTH
+  return BIE_EINVAL;
 }
 
-template <typename R, typename OT>
-int launch_phi_synth(const R* H, long long nfield, int p, int P, const R* cs, OT* out, const long long* out_off,
-                     long long out_stride, cudaStream_t s) {
-  long long n = nfield * (long long)(P + 1) * (P + 1);
-  if (n == 0) return BIE_OK;
-  k_phi_synth<R, OT><<<blocks_for(n), kThreads, 0, s>>>(H, nfield, p, P, cs, out, out_off, out_stride);
-  count_launch();
-  BIE_CUDA_TRY(cudaGetLastError());
-  return BIE_OK;
-}
-
-int launch_analyze(const double* grid, const long long* grid_off, long long grid_stride, long long nfield, int P,
-                   int p_out, const double* cs, const double* A, double* F, double* coef,
-                   const long long* coef_off, long long coef_stride, cudaStream_t s) {
-  long long n1 = nfield * (long long)(p_out + 1) * (P + 1);
-  if (n1 == 0) return BIE_OK;
-  k_phi_analyze<<<blocks_for(n1), kThreads, 0, s>>>(grid, grid_off, grid_stride, nfield, P, p_out, cs, F);
-  count_launch();
-  BIE_CUDA_TRY(cudaGetLastError());
-  long long n2 = nfield * (long long)(p_out + 1) * (p_out + 2) / 2;
-  k_leg_analyze<<<blocks_for(n2), kThreads, 0, s>>>(F, nfield, P, p_out, A, coef, coef_off, coef_stride);
-  count_launch();
-  BIE_CUDA_TRY(cudaGetLastError());
-  return BIE_OK;
-}
-
-int launch_analyze_fused(const std::vector<AnaGroup>& groups, const double* grid, double* coef, cudaStream_t s) {
+int launch_analyze(std::vector<AnaGroup> groups, const double* grid, double* coef, int sms, cudaStream_t s) {
+  std::sort(groups.begin(), groups.end(), [](const AnaGroup& x, const AnaGroup& y) { return x.P > y.P; });
+  long long fields = 0;
+  for (const auto& g : groups) fields += g.nfield;
+  if (fields == 0) return BIE_OK;
   for (size_t g0 = 0; g0 < groups.size(); g0 += kMaxAnaGroups) {
     AnaGroups G{};
     G.n = (int)std::min<size_t>(kMaxAnaGroups, groups.size() - g0);
     long long nblk = 0;
+    size_t smem = 0;
     for (int i = 0; i < G.n; ++i) {
-      G.g[i] = groups[g0 + i];
-      if (G.g[i].p > BIE_MAX_P) return BIE_EINVAL;
-      G.g[i].begin = nblk;
-      nblk += G.g[i].nfield * (G.g[i].p + 1);
+      AnaGroup& g = G.g[i] = groups[g0 + i];
+      // orders per block: every block folds the whole field, so as many as leave four blocks per SM, at
+      // most 32 KB of F
+      const long long want = std::max(1LL, fields * (g.p + 1) / (4LL * sms));
+      const long long fit = std::max<long long>(1, (32 << 10) / (16LL * (g.P + 1)));
+      g.mb = (int)std::min<long long>(g.p + 1, std::min(want, fit));
+      g.begin = nblk;
+      nblk += g.nfield * ((g.p + g.mb) / g.mb);
+      smem = std::max(smem, sizeof(double) * (2 * (size_t)g.mb * (g.P + 1) + 4 * (size_t)((g.P + 1) / 2 + 1) * ana_rows(g.P)));
     }
     if (nblk == 0) continue;
     if (nblk > 0x7fffffffLL) return BIE_EINVAL;
-    k_analyze_fused<<<(unsigned)nblk, kAnaThreads, 0, s>>>(G, grid, coef);
+    if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(k_analyze, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_analyze<<<(unsigned)nblk, kAnaThreads, smem, s>>>(G, grid, coef);
     count_launch();
     BIE_CUDA_TRY(cudaGetLastError());
   }
@@ -373,18 +441,12 @@ int launch_phase(double* coef, long long nfield, int p, double gamma, cudaStream
 }
 
 // explicit instantiations
-template int launch_leg_synth<double, double>(const double*, const long long*, long long, long long, int,
-                                              const double*, int, double*, int, cudaStream_t);
-template int launch_leg_synth<double, float>(const double*, const long long*, long long, long long, int,
-                                             const float*, int, float*, int, cudaStream_t);
-template int launch_leg_synth<float, float>(const float*, const long long*, long long, long long, int,
-                                            const float*, int, float*, int, cudaStream_t);
-template int launch_phi_synth<double, double>(const double*, long long, int, int, const double*, double*,
-                                              const long long*, long long, cudaStream_t);
-template int launch_phi_synth<float, float>(const float*, long long, int, int, const float*, float*,
-                                            const long long*, long long, cudaStream_t);
-template int launch_phi_synth<float, double>(const float*, long long, int, int, const float*, double*,
-                                             const long long*, long long, cudaStream_t);
+template int launch_synth<double, double>(int, const double*, const long long*, long long, long long, int, int,
+                                          const double*, const double*, const double*, const double*, double*,
+                                          long long, long long, int, cudaStream_t);
+template int launch_synth<double, float>(int, const double*, const long long*, long long, long long, int, int,
+                                         const float*, const float*, const float*, const float*, float*, long long,
+                                         long long, int, cudaStream_t);
 template int launch_rotate<double, double>(const double*, const long long*, int, long long, int, const double*,
                                            long long, int, int, const double*, double*, long long, cudaStream_t);
 template int launch_rotate<double, float>(const double*, const long long*, int, long long, int, const float*,
