@@ -81,7 +81,7 @@ def parse(argv=None):
     ap.add_argument("--fp64-solve", action="store_true",
                     help="also time the plain FP64 GMRES solve of the headline workload (minutes on c5)")
     ap.add_argument("--tensor-rotation", action="store_true",
-                    help="rotate the projected self form on the tensor cores (bie_config.tensor_rotation)")
+                    help="set bie_config.tensor_rotation (accepted, without effect)")
     ap.add_argument("--coupled", default=None, choices=["c4", "c5"],
                     help="print only the timing of coupled drop/surfactant steps (Alg. 1) on this workload")
     return ap.parse_args(argv)
@@ -239,17 +239,11 @@ def profiled_traffic(kernel, workload):
 
 
 def self_work_per_target(name: str, p: int, pq: int):
-    """(flops, bytes) per target of the projected-form self kernel `name` (self_proj_*): the rotation
-    of four targets (theta, phi_b), (theta, phi_b + pi), (pi - theta, phi_b), (pi - theta, phi_b + pi)
-    in one pass over latitude theta's Wigner blocks (even/odd orders), then the contraction of each
-    rotated coefficient (n, m >= 0; Re, Im x 3 components) with the target's projected factors,
-    which are read once per apply (FMA = 2 flops)."""
+    """(flops, bytes) per target of the dense-form self kernel `name` (self_proj_*): the density's
+    3 (p+1)^2 coefficients against six symmetric 3x3 entries each, read once per apply (FMA = 2 flops)."""
     esize = 8 if name.endswith("f64") or name.endswith("df") else 4
-    wig = sum((n + 1) ** 2 + n * n for n in range(p + 1))
-    ng = (p + 1) * (2 * p + 2)
-    rot = 2.0 * 3 * wig * ((p + 2) // 2) * (p + 1) / ng
-    ntri = (p + 1) * (p + 2) // 2
-    return rot + 36.0 * ntri, 12.0 * ntri * esize
+    nc = (p + 1) ** 2
+    return 18.0 * nc, 6.0 * ((nc + 3) // 4 * 4) * esize
 
 
 def roofline(phases, info, peaks, workload, p_of=None):
@@ -314,7 +308,7 @@ class Case:
         torch.cuda.synchronize()
         self.setup = {"geometry": 1e3 * (time.perf_counter() - t0),
                       "stages": {k: v[0] for k, v in self.ctx.profile_read().items()},
-                      "note": "geometry set-up includes the projected kernel factors of both layers"}
+                      "note": "geometry set-up includes the self kernel factors of both layers"}
         self.ctx.profile(False)
         self.info = dict(self.geo.info)
         self.pairs = sum(self.info[k] for k in ("self_pairs", "far_pairs", "up_pairs", "near_pairs"))
@@ -940,7 +934,7 @@ def run_ours(args):
                    "pairs_per_apply": head.get("pairs_per_apply"),
                    "parallelism": "replicas" if world > 1 else "single",
                    "l2": "L2 flushed (512 MB write) before every timed step; within a step the applies re-read the "
-                         "projected kernel factors and sources"},
+                         "self kernel factors and sources"},
         "e2e": head.get("e2e"),
         "gpu_launches": head.get("gpu_launches"),
         "roofline": head.get("roofline"),

@@ -53,7 +53,7 @@ enum bie_status {
 /* precision flags (the low byte), OR-able with BIE_RAW */
 #define BIE_FP64 0   /* every step in double precision */
 #define BIE_MIXED 1  /* rotation, synthesis and pair sums in FP32; geometry, analysis in FP64 */
-#define BIE_DF 2     /* the rotation and contraction of the singular self term (projected form) and the
+#define BIE_DF 2     /* the contraction of the singular self term (dense form) and the
                         inter-drop pair sums (Omega_0, Omega_1) in double-float arithmetic (pairs of
                         FP32 numbers, about 44 significant bits) on the FP32 pipes; geometry, the
                         near-singular step and the analysis in FP64: FP64-grade results (relative
@@ -70,23 +70,20 @@ typedef struct bie_config {
   int upsample;      /* U: the intermediate region uses the grid of degree U(p+1)-1 (Sec. 2.3), >= 1 */
   double a_tilde;    /* A: Omega_0 / Omega_1 boundary at distance A*h (Sec. 2.3; the paper uses 5) */
   int n_interp;      /* L: check points of the near-singular interpolation (Sec. 2.3; 8) */
-  int self_direct;   /* 0: singular self term in projected form (the kernel weights of each target's
-                        rotated grid, phi-transformed and projected onto the associated Legendre
-                        functions once per geometry; an apply rotates the density and contracts it
-                        with them; the default); 1: direct form (synthesis on the rotated grid and
-                        kernel evaluation at every quadrature point on every apply) */
+  int self_direct;   /* 0: singular self term in dense form (the kernel weights of each target's rotated
+                        grid, projected onto the spherical harmonics of the density and rotated back to
+                        its frame once per geometry; an apply contracts the density with them; the
+                        default); 1: direct form (rotation, synthesis on the rotated grid and kernel
+                        evaluation at every quadrature point on every apply) */
   int use_graphs;    /* 1: an apply (kind, flags) is captured into a CUDA graph at its second call and
                         replayed afterwards (input and output pass through fixed internal buffers);
                         0: every apply launches its kernels one by one */
-  int tensor_rotation; /* 1: in BIE_MIXED applies the Wigner rotation of the projected self form
-                          (App. B) of degrees up to 58 runs on the tensor cores (TF32 with a 3-pass
-                          split, FP32 accumulation, about FP32 accuracy); 0 (default): on the CUDA cores
-                          in FP32, which measured 1.4-1.7 times faster on GB300.  FP64 and BIE_DF
-                          applies always rotate on the CUDA cores */
+  int tensor_rotation; /* 0 or 1, accepted and without effect: the dense self form holds the rotation (App. B)
+                          in its factors, so an apply has none left to run on the tensor cores */
 } bie_config;
 
-/* Fill a config with the paper's defaults: device 0, U = 4, A = 5, L = 8, projected self form, graphs
- * on, CUDA-core rotation. */
+/* Fill a config with the paper's defaults: device 0, U = 4, A = 5, L = 8, dense self form, graphs
+ * on. */
 void bie_config_default(bie_config* cfg);
 
 /* Create a context on cfg->device.  Plan tables are built lazily per degree and cached. */
@@ -145,8 +142,8 @@ int bie_rotate_noalloc(bie_ctx* ctx, int ndrop, const int* p, int ncomp, const d
  *          p <= pq <= 2p+1 (pq = 2p+1 is the "upsampled 2x for quadrature" rule);
  *   xcoef  [drop][3][(p+1)^2] device coefficients of x(theta, phi);
  *   lambda host [ndrop] viscosity ratios.
- * Synchronous: returns when the geometry is ready.  With the projected self form (the default) this
- * includes the projected kernel factors of both layers, after which the rotated-grid cache is
+ * Synchronous: returns when the geometry is ready.  With the dense self form (the default) this
+ * includes the kernel factors of both layers, after which the rotated-grid cache is
  * released; with bie_config.self_direct the cache is kept for the per-apply evaluation.
  * BIE_EOVERLAP if a grid point of one drop lies inside another.  The geometry owns its device
  * memory until bie_geometry_destroy. */
@@ -262,9 +259,9 @@ int bie_solve(bie_ctx* ctx, const bie_geom* geom, const double* rhs, double* u, 
  * bie_profile_read synchronises on the recorded events, returns per-phase totals (milliseconds and
  * number of timed calls, at most cap entries, *count = number of phases) and clears the record.
  * While profiling is on, applies launch their kernels one by one (no graph replay), so every phase
- * is timed.  Phases: "self_proj_f64/f32" (rotation + contraction with the projected kernel factors) and
+ * is timed.  Phases: "self_proj_f64/f32/df" (contraction with the dense kernel factors) and
  * "self_direct_f64/f32" (rotation + synthesis + the singular pair sum of Thm 1), "kernel_proj"
- * (projected kernel factors, once per geometry and kind), "analyze" (Galerkin
+ * (dense kernel factors, once per geometry and kind), "analyze" (Galerkin
  * projection), "interdrop" (regular and upsampled pair sums), "near" (near-singular step),
  * "source_synth" (source densities on the standard/upsampled grids), "gmres_vec",
  * "surfactant_rates" and "surfactant_implicit" (bie_surfactant_rates, bie_surfactant_implicit). */

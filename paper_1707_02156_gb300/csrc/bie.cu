@@ -82,7 +82,6 @@ struct Plan {
   int p = 0, P = 0;
   DevBuf<double> T0, T1, T2, At, cs, wsin, wsq;
   DevBuf<float> T0f, csf;
-  DevBuf<dff> csdf;
   template <typename R>
   const R* T0_() const;
   template <typename R>
@@ -104,17 +103,12 @@ template <>
 const float* Plan::cs_<float>() const {
   return csf.ptr;
 }
-template <>
-const dff* Plan::cs_<dff>() const {
-  return csdf.ptr;
-}
 
 struct WigPlan {  // rotation blocks for the p+1 latitudes of the degree-p grid
   int p = 0;
   long long stride = 0;
   DevBuf<double> blk;
   DevBuf<float> blkf;
-  DevBuf<dff> blkdf;
   template <typename R>
   const R* blk_() const;
 };
@@ -125,10 +119,6 @@ const double* WigPlan::blk_<double>() const {
 template <>
 const float* WigPlan::blk_<float>() const {
   return blkf.ptr;
-}
-template <>
-const dff* WigPlan::blk_<dff>() const {
-  return blkdf.ptr;
 }
 
 }  // namespace bie
@@ -216,7 +206,6 @@ static int get_plan(bie_ctx* ctx, int p, int P, Plan** out) {
   phase_table(p, P, v);
   BIE_TRY(pl->cs.upload(v));
   BIE_TRY(upload_as(pl->csf, v));
-  BIE_TRY(upload_as(pl->csdf, v));
   std::vector<double> t, w, ws;
   gauss_legendre(P + 1, t, w);
   singular_weights(P, ws);
@@ -249,7 +238,6 @@ static int get_wig(bie_ctx* ctx, int p, WigPlan** out) {
   for (int a = 0; a <= p; ++a) wigner_blocks(p, std::acos(t[a]), blk.data() + (size_t)a * wp->stride);
   BIE_TRY(wp->blk.upload(blk));
   BIE_TRY(upload_as(wp->blkf, blk));
-  BIE_TRY(upload_as(wp->blkdf, blk));
   *out = wp.get();
   ctx->wigs[p] = std::move(wp);
   return BIE_OK;
@@ -301,7 +289,7 @@ struct bie_geom {
     bie::DevBuf<double> cache64;            // [gdrop][N_g][7][nq] rotated geometry (Sec. 2.2)
     bie::DevBuf<float> cache32;             // FP32 copy, made on the first direct-form mixed apply
     bie::DevBuf<long long> src_off_std, src_off_up;  // first source of each drop on the two grids
-    bie::DevBuf<double> qk64[2];            // projected kernel factors of every target, S and D
+    bie::DevBuf<double> qk64[2];            // dense self factors of every target, S and D
     bie::DevBuf<float> qk32[2];
     bie::DevBuf<bie::dff> qkdf[2];          // double-float copy, made on the first BIE_DF apply
   };
@@ -333,8 +321,6 @@ struct bie_geom {
   int nblk = 0, ntile = 0;
   bool interdrop_ready = false;  // inter-drop data built: at set-up when ndrop > 1, else at the first off-surface evaluation
   int tpt32 = 2, tpt64 = 2;                         // targets per thread of the pair kernel (autotuned FP32)
-  bie::DevBuf<float> eo32;                          // tensor-core self path: rotated sums
-  bie::DevBuf<unsigned> g32;                        // and the split phase-shifted coefficients
   std::vector<std::pair<long long, int>> near;      // (target, source drop) pairs in Omega_2
   // near-singular step (Omega_2), Sec. 2.3
   int nnear_tgt = 0;
@@ -378,27 +364,40 @@ static int analyze_groups(bie_ctx* ctx, bie_geom* g, const double* vals, double*
   return launch_analyze(ag, vals, out, ctx->sms, s);
 }
 
-// The direct form serves a group when the configuration asks for it, or when the projected form's
+// The direct form serves a group when the configuration asks for it, or when the dense form's
 // per-target factors would not fit in shared memory while they are built.
 static bool group_uses_direct(const bie_ctx* ctx, const bie_geom::Group& G) {
   return ctx->cfg.self_direct != 0 || kernel_proj_smem(G.p, G.pq) > 227 * 1024;
 }
 
-// Projected-form kernel factors of one group, built from the FP64 rotated-grid cache.
-static int ensure_qk(bie_ctx* ctx, bie_geom::Group& G, int kind, cudaStream_t s) {
+// Dense-form factors of one group, built from the FP64 rotated-grid cache: the projected factors of a
+// chunk of latitude rows into temporaries, then the transposed rotation to their final place.
+static int ensure_qk(bie_ctx* ctx, bie_geom::Group& G, int kind, DevBuf<double>& work, cudaStream_t s) {
   if (G.qk64[kind].ptr) return BIE_OK;
-  Plan* pl;
+  Plan *pl, *pp;
+  WigPlan* wp;
   BIE_TRY(get_plan(ctx, G.p, G.pq, &pl));
-  const long long nt = (long long)G.drops.size() * ngrid(G.p);
-  const long long n = nt * 6 * (long long)(G.p + 1) * (G.p + 2);
+  BIE_TRY(get_plan(ctx, G.p, G.p, &pp));
+  BIE_TRY(get_wig(ctx, G.p, &wp));
+  const long long nb = 2 * G.p + 2, rows = (long long)G.drops.size() * (G.p + 1);
+  const long long per_row = nb * 6 * (long long)(G.p + 1) * (G.p + 2), nq = ngrid(G.pq);
+  const long long n = rows * nb * 6 * self_row(G.p);
+  const long long chunk = std::max(1LL, std::min<long long>(rows, kWorkBudget / (4 * 8 * per_row)));
   BIE_TRY(G.qk64[kind].alloc(n));
   BIE_TRY(G.qk32[kind].alloc(n));
+  BIE_TRY(work.alloc(chunk * per_row));
   Phase ph(ctx, "kernel_proj", s);
-  return launch_kernel_proj(kind, G.cache64.ptr, nt, G.p, G.pq, pl->cs.ptr, pl->T0.ptr, G.qk64[kind].ptr,
-                            G.qk32[kind].ptr, s);
+  for (long long r0 = 0; r0 < rows; r0 += chunk) {
+    const long long rn = std::min(chunk, rows - r0);
+    BIE_TRY(launch_kernel_proj(kind, G.cache64.ptr + r0 * nb * 7 * nq, rn * nb, G.p, G.pq, pl->cs.ptr, pl->T0.ptr,
+                               work.ptr, s));
+    BIE_TRY(launch_unrotate(work.ptr, r0, rn, G.p, wp->blk.ptr, wp->stride, pp->cs.ptr, G.qk64[kind].ptr,
+                            G.qk32[kind].ptr, s));
+  }
+  return BIE_OK;
 }
 
-// Projected factors of one group in the arithmetic type R (the double-float copy is split from the
+// Dense factors of one group in the arithmetic type R (the double-float copy is split from the
 // FP64 factors on first use).
 template <typename R>
 static int qk_of(bie_geom::Group& G, int kind, cudaStream_t s, const R** out);
@@ -426,28 +425,24 @@ static const char* self_phase_name() {
   return std::is_same<R, float>::value ? "self_proj_f32" : std::is_same<R, dff>::value ? "self_proj_df" : "self_proj_f64";
 }
 
-// Singular self part of every drop (Sec. 2.2): one launch for every projected-form degree group
+// Singular self part of every drop (Sec. 2.2): one launch for every dense-form degree group
 // (direct-form groups one launch each; in double-float arithmetic those run in FP64).
 template <typename R>
 static int self_apply(bie_geom* g, int kind, bool raw, const double* dens, cudaStream_t s) {
   using RD = typename std::conditional<std::is_same<R, dff>::value, double, R>::type;
   bie_ctx* ctx = g->ctx;
-  // the projected form keeps its per-target factors in shared memory while they are built; groups
-  // whose factors do not fit there use the direct form
-  auto use_direct = [&](const bie_geom::Group& G) { return group_uses_direct(ctx, G); };
-  std::vector<SelfGroup<R>> proj;
+  std::vector<SelfGroup<R>> dense;
   for (auto& Gp : g->groups) {
     auto& G = *Gp;
     const int p = G.p, pq = G.pq;
-    const bool direct = use_direct(G);
-    Plan *pl, *pp;
-    WigPlan* wp;
-    BIE_TRY(get_plan(ctx, p, pq, &pl));
-    BIE_TRY(get_plan(ctx, p, p, &pp));
-    BIE_TRY(get_wig(ctx, p, &wp));
     const double* wts = kind == 0 ? (raw ? G.wSraw.ptr : G.wS.ptr) : (raw ? G.wDraw.ptr : G.wD.ptr);
     const long long nd = (long long)G.drops.size();
-    if (direct) {
+    if (group_uses_direct(ctx, G)) {
+      Plan *pl, *pp;
+      WigPlan* wp;
+      BIE_TRY(get_plan(ctx, p, pq, &pl));
+      BIE_TRY(get_plan(ctx, p, p, &pp));
+      BIE_TRY(get_wig(ctx, p, &wp));
       if (sizeof(RD) == 4 && !G.cache32.ptr) {
         BIE_TRY(G.cache32.alloc(G.cache64.n));
         BIE_TRY(launch_to_float(G.cache64.ptr, G.cache32.ptr, (long long)G.cache64.n, s));
@@ -459,42 +454,19 @@ static int self_apply(bie_geom* g, int kind, bool raw, const double* dens, cudaS
                                      pp->cs_<RD>(), pl->T0_<RD>(), pl->cs_<RD>(), cache, wts, G.val_off.ptr,
                                      g->vals.ptr, sizeof(RD) == 8 ? 96 * 1024 : 40 * 1024, s));
     } else {
-      BIE_TRY(ensure_qk(ctx, G, kind, s));
       SelfGroup<R> sg{};
       sg.ndrop = nd;
       sg.foff3 = G.foff3.ptr;
-      sg.wblk = wp->blk_<R>();
-      sg.wstride = wp->stride;
-      sg.ph = pp->cs_<R>();
-      BIE_TRY(qk_of<R>(G, kind, s, &sg.Q));
+      BIE_TRY(qk_of<R>(G, kind, s, &sg.S));
       sg.wts = wts;
       sg.val_off = G.val_off.ptr;
       sg.p = p;
-      proj.push_back(sg);
+      dense.push_back(sg);
     }
   }
-  if (!proj.empty()) {  // every projected-form group in one launch; it reads the FP64 density directly
-    Phase ph(ctx, self_phase_name<R>(), s);
-    if constexpr (std::is_same<R, float>::value) {
-      if (ctx->cfg.tensor_rotation) {
-        // degrees whose rotation block fits one SM's shared memory go to the tensor cores, the rest
-        // (above 58) to the CUDA-core kernel
-        std::vector<SelfGroup<R>> tc, cc;
-        for (const auto& sg : proj) (self_tc_fits(sg.p) ? tc : cc).push_back(sg);
-        if (!tc.empty()) {
-          // E/O sums of a chunk of drops kept within 32 MB, so that they stay in L2 between the kernels
-          const long long budget = 8LL << 20;
-          BIE_TRY(g->eo32.alloc((size_t)self_tc_eo_floats(tc, budget)));
-          BIE_TRY(g->g32.alloc((size_t)self_tc_g_floats(tc, budget)));
-          BIE_TRY(launch_self_tc(tc, dens, g->vals.ptr, g->eo32.ptr, g->g32.ptr, budget, s));
-        }
-        if (!cc.empty()) BIE_TRY((launch_self_proj<R, double>(cc, dens, g->vals.ptr, s)));
-        return BIE_OK;
-      }
-    }
-    BIE_TRY((launch_self_proj<R, double>(proj, dens, g->vals.ptr, s)));
-  }
-  return BIE_OK;
+  if (dense.empty()) return BIE_OK;
+  Phase ph(ctx, self_phase_name<R>(), s);
+  return launch_self_dense<R, double>(dense, dens, g->vals.ptr, ctx->sms, s);
 }
 
 template <typename R>
@@ -2715,11 +2687,12 @@ int bie_geometry_setup(bie_ctx* ctx, int ndrop, const int* p, const int* pq, con
     self_pairs += (long long)G->drops.size() * ngrid(G->p) * ngrid(G->pq);
   }
   if (ndrop > 1) BIE_TRY(setup_interdrop(ctx, g.get(), s));
-  // projected-form groups: both kinds' factors now, then the rotated-grid cache is no longer needed
+  // dense-form groups: both kinds' factors now, then the rotated-grid cache is no longer needed
+  DevBuf<double> qwork;
   for (auto& G : g->groups) {
     if (group_uses_direct(ctx, *G)) continue;
-    BIE_TRY(ensure_qk(ctx, *G, 0, s));
-    BIE_TRY(ensure_qk(ctx, *G, 1, s));
+    BIE_TRY(ensure_qk(ctx, *G, 0, qwork, s));
+    BIE_TRY(ensure_qk(ctx, *G, 1, qwork, s));
     BIE_CUDA_TRY(cudaStreamSynchronize(s));
     G->cache64.release();
   }

@@ -82,7 +82,7 @@ template <typename R>
 int launch_rotgeo(const double* X, const double* Xt, const double* Xp, long long ndrop, int ng, int pq,
                   const double* rec_std, const long long* rec_off, const double* wsq, R* cache, cudaStream_t s);
 // Singular self interaction (Thm 1, Sec. 2.2), one block per target of ndrop drops of degree p:
-// direct form against the rotated-geometry cache, or projected form against Q (see self.cu).
+// direct form against the rotated-geometry cache.
 template <typename R>
 int launch_self_direct(int kind, const double* dens, const long long* foff3, long long ndrop, int p, int pq,
                        const R* wblk, long long wstride, const R* ph, const R* T0, const R* cs, const R* cache,
@@ -92,17 +92,20 @@ int launch_self_direct(int kind, const double* dens, const long long* foff3, lon
 // rotated-geometry cache and the degree-pq grid's Legendre table T0 (degrees <= p, all nodes).
 size_t kernel_proj_smem(int p, int pq);
 int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, int pq, const double* cs,
-                       const double* T0, double* Q64, float* Q32, cudaStream_t s);
-// One degree group of the projected-form apply (device pointers; begin is set by the launcher).
+                       const double* T0, double* Q64, cudaStream_t s);
+// Entries per plane of the dense self form: (p+1)^2 rounded up to whole 16-byte loads in every precision.
+__host__ __device__ inline int self_row(int p) { return ((p + 1) * (p + 1) + 3) & ~3; }
+// Dense factors S[target][6][self_row(p)] of the latitude rows row0 .. row0 + nrow - 1 (row = drop * (p+1) + a)
+// from their projected factors Q (Q64 starts at row0), written at the rows' places in S64 and S32.
+int launch_unrotate(const double* Q64, long long row0, long long nrow, int p, const double* wblk, long long wstride,
+                    const double* ph, double* S64, float* S32, cudaStream_t s);
+// One degree group of the dense-form apply (device pointers; begin is set by the launcher).
 template <typename R>
 struct SelfGroup {
   long long begin;          // first block of the group
   long long ndrop;          // drops of the group
   const long long* foff3;   // [drop][3] offsets of the density coefficients
-  const R* wblk;            // Wigner blocks of the group's latitudes, wstride apart
-  long long wstride;
-  const R* ph;              // cos, sin (m phi_b) of the degree-p grid
-  const R* Q;               // projected kernel factors
+  const R* S;               // dense factors
   const double* wts;        // per-drop weight
   const long long* val_off; // per-drop offset into vals
   int p;
@@ -116,18 +119,9 @@ struct SelfGroups {
 // out[i] = double-float split of in[i] (dff: dfloat.cuh)
 struct dff;
 int launch_split_dff(const double* in, dff* out, long long n, cudaStream_t s);
-// All projected-form groups in one launch (eight groups per launch at most).
+// All dense-form groups in one launch (eight groups per launch at most).
 template <typename R, typename CT>
-int launch_self_proj(std::vector<SelfGroup<R>> groups, const CT* dens, double* vals, cudaStream_t s);
-// The FP32 projected form with the Wigner rotation on the tensor cores (self_tc.cu): per chunk of
-// drops of one degree, the rotation products into eo (at most `budget` floats per chunk, at least one
-// drop's worth), then the contraction with the factors.  self_tc_eo_floats = the buffer it needs.
-long long self_tc_eo_floats(const std::vector<SelfGroup<float>>& groups, long long budget);
-long long self_tc_g_floats(const std::vector<SelfGroup<float>>& groups, long long budget);
-// whether k_rot_tc's shared memory at degree p fits one block (degrees up to 58)
-bool self_tc_fits(int p);
-int launch_self_tc(const std::vector<SelfGroup<float>>& groups, const double* dens, double* vals, float* eo,
-                   unsigned* gm, long long budget, cudaStream_t s);
+int launch_self_dense(std::vector<SelfGroup<R>> groups, const CT* dens, double* vals, int sms, cudaStream_t s);
 // interfacial force at the N grid points of nd drops from x derivatives [5][nd][3][N] (t, p, tt, tp, pp) and
 // Gamma and its derivatives [3][nd][N] (f, t, p): f [nd][3][N]
 int launch_force(const double* X, const double* Gm, long long nd, long long N, double es, double xs, double* f,

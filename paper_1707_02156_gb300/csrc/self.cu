@@ -7,13 +7,15 @@
 //    h_m(theta_j) = sum_n rho'_n^m P~_n^m(cos theta_j), runs in shared memory; the phi step rho'(theta_j, phi_k) = h_0 + 2 Re sum_m h_m e^{i m phi_k} is evaluated
 //    for the longitude pair (k, k + pq + 1) from the even and odd orders, and the Stokeslet or
 //    stresslet pair sum of Thm 1 is accumulated against the cached rotated geometry;
-//  * projected form: the same double sum reassociated exactly,
+//  * dense form (the default): the same double sum reassociated exactly,
 //        sum_{j,k} M_jk rho'_jk = sum_j sum_m c_m Re[ Mhat_jm h_m(theta_j) ]
 //                               = sum_{n, m >= 0} Re[ Q_nm rho'_n^m ],   Q_nm = c_m sum_j Mhat_jm P~_n^m(cos theta_j),
 //    with c_0 = 1, c_m = 2, M_jk the 3x3 kernel weight of the quadrature point
 //    (w^s_j K(x0 - x') W'/sin theta_j, geometry only) and Mhat_jm = sum_k M_jk e^{i m phi_k} its phi
-//    transform.  Q (6 complex entries per (n, m) and target) is built once per geometry; an apply
-//    then rotates the density and contracts it with Q, without the Legendre step.
+//    transform; and since rho' = R rho with the target's rotation R (App. B), the sum is
+//    sum_r (R^T Q)_r rho_r: the rotation is applied to the factors once per geometry, not to the
+//    density on every apply.  S = R^T Q (six symmetric 3x3 entries per coefficient and target) is what
+//    an apply reads, once.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -207,7 +209,7 @@ __global__ void __launch_bounds__(256) k_self_direct(
   write_target<R>(s0, s1, s2, wts, val_off, vals, ld, tl, ng);
 }
 
-// ---- projected form: set-up of Q (FP64, optional FP32 copy) ----
+// ---- dense form: set-up of the projected factors Q (FP64) ----
 // For each target, Q[t][e][ri][tri(n,m)] = c_m sum_j Mhat_{e,jm} P~_n^m(cos theta_j), with
 // Mhat_{e,jm} = sum_k M_{e,jk} e^{i m phi_k} the phi transform of entry e of the 3x3 kernel weight
 // over (xx, yy, zz, xy, xz, yz), ri = real / imaginary part, c_0 = 1 and c_m = 2.  Latitudes are
@@ -225,7 +227,7 @@ __device__ inline int tri_index_degree(int it) {
 template <int KIND>
 __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ cache, int pq, int p,
                                                      const double* __restrict__ cs, const double* __restrict__ T0,
-                                                     double* __restrict__ Q64, float* __restrict__ Q32) {
+                                                     double* __restrict__ Q64) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const long long t = blockIdx.x;
   const int nq_j = pq + 1, nk = 2 * pq + 2, half = pq + 1;
@@ -301,45 +303,98 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
     }
     __syncthreads();
   }
-  // The apply adds every product with a plus sign: the imaginary planes of targets on latitudes
-  // a <= p/2 are stored negated (imaginary parts enter as -Q_im), and targets on latitudes a > p/2,
-  // which the apply reaches as the mirror pi - theta of a lower latitude, carry (-1)^(n+m).
   double* o64 = Q64 + t * 12 * ntri;
-  float* o32 = Q32 ? Q32 + t * 12 * ntri : nullptr;
-  const int nbl = 2 * p + 2;
-  const int lat = (int)((t % ((long long)(p + 1) * nbl)) / nbl);
-  const bool mirror = 2 * lat > p;
   for (int i = threadIdx.x; i < 12 * ntri; i += blockDim.x) {
-    const int it = i % ntri, plane = i / ntri;
-    const int n = tri_index_degree(it);
-    const int m = it - n * (n + 1) / 2;
-    double v = (m == 0 ? 1.0 : 2.0) * sq[i];  // c_m
-    if (mirror) {
-      if ((n + m) & 1) v = -v;
-    } else if (plane & 1) {
-      v = -v;
-    }
-    o64[i] = v;
-    if (o32) o32[i] = (float)v;
+    const int m = i % ntri;
+    const int n = tri_index_degree(m);
+    o64[i] = (m == n * (n + 1) / 2 ? 1.0 : 2.0) * sq[i];  // c_m
   }
 }
 
-// ---- projected form: apply ----
-// One block per target quadruple: the latitudes theta_a and pi - theta_a (Gauss nodes t and -t) at the
-// longitudes phi_b and phi_b + pi.  One pass over latitude a's real Wigner blocks (C for the real
-// parts, S for the imaginary parts, column m the input order) gives the even-m and odd-m partial sums
-// E and O of every rotated coefficient (n, m'), and the four targets follow exactly:
-//   phi_b + pi:     e^{i m (phi + pi)} = (-1)^m e^{i m phi}                    -> E - O
-//   pi - theta_a:   d^n_{m m'}(pi - beta) = (-1)^(n + m') d^n_{-m m'}(beta), so
-//                   C' = (-1)^(n + m' + m) C and S' = -(-1)^(n + m' + m) S      -> +-(-1)^(n + m') (E -+ O)
-// Each rotated coefficient is contracted at once with the targets' projected kernel factors Q
-// (real parts with the real planes, imaginary parts with minus the imaginary planes), so rotated
-// coefficients never leave registers.  The middle latitude of an odd node count (t = 0) pairs with
-// itself and its block has two targets.  Shared memory: g4 [(p+1)^2][4], the phase-shifted input
-// coefficients e^{i m phi_b} rho_n^m with the three components interleaved.
+// ---- dense form: set-up, S = R^T Q ----
+// One block per (latitude row, degree n, chunk of kUnB longitudes).  With q_m = Q_re(n, m) for the real
+// and -Q_im(n, m) for the imaginary parts of rho'_n^m, and rho' = (C Re g, S Im g), g = e^{i m phi_b} rho,
+// the transposed rotation is s_re = C^T q_re, s_im = S^T q_im and the transposed phase
+// (s_re cos + s_im sin, s_im cos - s_re sin).  FP64-pipe-bound like the factors' own kernels (2n+1
+// multiply-adds per entry and coefficient); the leading dimensions of the staged blocks are odd, so
+// that the strided reads of the transposed products hit every bank.  64 drops of p = 24, both kinds: 20 ms, of
+// which an apply saves 1.5 ms in double-float and 0.45 ms in FP32.
+constexpr int kUnB = 8;
+
+__global__ void __launch_bounds__(128) k_unrotate(const double* __restrict__ Q64, long long row0, int p,
+                                                  const double* __restrict__ wblk, long long wstride,
+                                                  const double* __restrict__ ph, int ncp, double* __restrict__ S64,
+                                                  float* __restrict__ S32) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int nb = 2 * p + 2, nbch = (nb + kUnB - 1) / kUnB;
+  const int b0 = (int)(blockIdx.x % nbch) * kUnB;
+  const long long row = row0 + blockIdx.x / nbch;  // latitude row of the group: drop * (p+1) + a
+  const int a = (int)(row % (p + 1));
+  const int n = p - (int)blockIdx.y;  // the longest blocks first
+  const int nbh = min(kUnB, nb - b0);
+  const int ntri = (p + 1) * (p + 2) / 2, t0 = n * (n + 1) / 2;
+  const int ldC = (n + 1) | 1, ldS = n | 1;
+  double* sC = reinterpret_cast<double*>(smem_raw);  // [m][m']
+  double* sS = sC + (n + 1) * ldC;
+  double* sq = sS + n * ldS;                          // [bb][e][re 0..n, im 1..n]
+  const double* blk = wblk + (long long)a * wstride + (long long)n * (n + 1) * (2 * n + 1) / 6 +
+                      (long long)(n - 1) * n * (2 * n - 1) / 6;
+  for (int i = threadIdx.x; i < (n + 1) * (n + 1); i += blockDim.x) sC[(i / (n + 1)) * ldC + i % (n + 1)] = blk[i];
+  for (int i = threadIdx.x; i < n * n; i += blockDim.x) sS[(i / n) * ldS + i % n] = blk[(n + 1) * (n + 1) + i];
+  const int w = 2 * n + 1;
+  const double* Qr = Q64 + (row - row0) * nb * 12 * ntri;
+  for (int i = threadIdx.x; i < nbh * 12 * (n + 1); i += blockDim.x) {
+    const int m = i % (n + 1), g = i / (n + 1);
+    const int plane = g % 12, bb = g / 12;
+    const double v = Qr[((long long)(b0 + bb) * 12 + plane) * ntri + t0 + m];
+    double* q = sq + (bb * 6 + plane / 2) * w;
+    if (!(plane & 1))
+      q[m] = v;
+    else if (m > 0)
+      q[n + m] = -v;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nbh * 6 * (n + 1); i += blockDim.x) {
+    const int m = i % (n + 1), g = i / (n + 1);
+    const int bb = g / 6, e = g - bb * 6;
+    const double* q = sq + g * w;
+    const double* c = sC + m * ldC;
+    double re = 0, im = 0;
+    for (int k = 0; k <= n; ++k) re += c[k] * q[k];
+    if (m > 0) {
+      const double* sn = sS + (m - 1) * ldS;
+      for (int k = 1; k <= n; ++k) im += sn[k - 1] * q[n + k];
+    }
+    const double co = ph[((long long)m * nb + b0 + bb) * 2], si = ph[((long long)m * nb + b0 + bb) * 2 + 1];
+    const long long o = ((row * nb + b0 + bb) * 6 + e) * ncp + n * (n + 1);
+    const double vr = m > 0 ? re * co + im * si : re;
+    S64[o + m] = vr;
+    S32[o + m] = (float)vr;
+    if (m > 0) {
+      const double vi = im * co - re * si;
+      S64[o - m] = vi;
+      S32[o - m] = (float)vi;
+    } else if (n == p) {  // the padding of the row
+      for (int r = p + 1; r < ncp - p * (p + 1); ++r) {
+        S64[o + r] = 0.0;
+        S32[o + r] = 0.0f;
+      }
+    }
+  }
+}
+
+// ---- dense form: apply ----
+// vals[t] = sum_r S[t][r] rho[r] (symmetric 3x3 times 3-vector), one warp per target, the density of the
+// drop in shared memory.  Every factor is read once, with 128-bit loads: bound by memory in FP32 and
+// double-float (9 multiply-adds per 6 words), by the FP64 pipe in FP64.  Eight targets per block and
+// warp for large batches (the density is staged once per block), one when the batch is small, so that
+// every SM gets work.  Measured against rotating the density in every apply (36k flops per target, bound by
+// the latency of the Wigner loads): FP32, p = 32 41 -> 17 us with the launch (57 MB), 192 drops of p = 24
+// 1.93 -> 0.56 ms (6.5 TB/s); FP64, p = 16 41 -> 18 us, 16 drops of p = 16 and 24 0.67 -> 0.16 ms;
+// double-float, 80 drops of p = 24 2.42 -> 0.59 ms.
 constexpr int kSelfThreads = 256;
 
-// acc += S v for the symmetric 3x3 matrix S with entries (xx, yy, zz, xy, xz, yz) at planes q[0..5]
+// acc += S v for the symmetric 3x3 matrix S with entries (xx, yy, zz, xy, xz, yz) in q
 template <typename R>
 __device__ inline void sym_mul_add(const R* q, const R* v, R* acc) {
   acc[0] = fmad(q[4], v[2], fmad(q[3], v[1], fmad(q[0], v[0], acc[0])));
@@ -347,158 +402,87 @@ __device__ inline void sym_mul_add(const R* q, const R* v, R* acc) {
   acc[2] = fmad(q[2], v[2], fmad(q[5], v[1], fmad(q[4], v[0], acc[2])));
 }
 
-// One launch covers every degree group (a persistent batch over drops of uneven degree): the groups'
-// arguments travel by value, block ranges in descending degree so that the longest blocks start first.
+// value v of 16 loaded bytes
+template <typename R>
+__device__ __forceinline__ R lane_of(const uint4& u, int v);
+template <>
+__device__ __forceinline__ float lane_of<float>(const uint4& u, int v) {
+  return __uint_as_float(v == 0 ? u.x : v == 1 ? u.y : v == 2 ? u.z : u.w);
+}
+template <>
+__device__ __forceinline__ double lane_of<double>(const uint4& u, int v) {
+  return v == 0 ? __hiloint2double((int)u.y, (int)u.x) : __hiloint2double((int)u.w, (int)u.z);
+}
+template <>
+__device__ __forceinline__ dff lane_of<dff>(const uint4& u, int v) {
+  return v == 0 ? dff(__uint_as_float(u.x), __uint_as_float(u.y)) : dff(__uint_as_float(u.z), __uint_as_float(u.w));
+}
+
+// 16 bytes of a factor plane, read once: no L1 allocation
+__device__ __forceinline__ uint4 load_factor(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+
+// One launch covers every degree group (a batch over drops of uneven degree): the groups' arguments
+// travel by value.
 template <typename R, typename CT>
-__global__ void __launch_bounds__(kSelfThreads, sizeof(R) == 4 ? 4 : 2) k_self_proj(
-    SelfGroups<R> G, const CT* __restrict__ dens, double* __restrict__ vals) {
+__global__ void __launch_bounds__(kSelfThreads, 2) k_self_dense(SelfGroups<R> G, int per_warp,
+                                                                const CT* __restrict__ dens,
+                                                                double* __restrict__ vals) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ R red[kSelfThreads / 32][12];
+  constexpr int V = 16 / sizeof(R);
   SelfGroup<R> A = G.g[0];
 #pragma unroll
   for (int i = 1; i < kMaxSelfGroups; ++i)
     if (i < G.n && (long long)blockIdx.x >= G.g[i].begin) A = G.g[i];
   const int p = A.p;
-  const long long* __restrict__ foff3 = A.foff3;
-  const R* __restrict__ wblk = A.wblk;
-  const long long wstride = A.wstride;
-  const R* __restrict__ ph = A.ph;
-  const R* __restrict__ Q = A.Q;
-  const double* __restrict__ wts = A.wts;
-  const long long* __restrict__ val_off = A.val_off;
-  const int ntri = (p + 1) * (p + 2) / 2;
-  const int nc = (p + 1) * (p + 1);
-  const int ng = (p + 1) * (2 * p + 2);
-  R* g4 = reinterpret_cast<R*>(smem_raw);  // [(p+1)^2][4]
-  const int hb = p + 1, nb = 2 * p + 2, na2 = (p + 2) / 2;
+  const int nc = (p + 1) * (p + 1), ncp = self_row(p), ng = 2 * nc;
+  R* rho = reinterpret_cast<R*>(smem_raw);  // [3][ncp]
+  const int tb = per_warp * (kSelfThreads / 32), tiles = (ng + tb - 1) / tb;
   const long long bid = (long long)blockIdx.x - A.begin;
-  const long long ld = bid / ((long long)na2 * hb);
-  const int r = (int)(bid - ld * na2 * hb);
-  const int a = r / hb, b = r - a * hb;
-  const int a2 = p - a;
-  const bool quad = a2 != a;
-  const int tlA = a * nb + b, tlC = a2 * nb + b;  // targets A, B = A + hb, C, D = C + hb
-  // stage 0: g = e^{i m phi_b} rho_n^m
-  for (int i = threadIdx.x; i < 3 * nc; i += blockDim.x) {
-    const int c = i / nc, rr = i - c * nc;
-    const int n = degree_of(rr);
-    const int m = rr - n * (n + 1);
-    if (m < 0) continue;
-    const CT* f = dens + foff3[ld * 3 + c];
-    const R fr = (R)f[n * (n + 1) + m];
-    const R fi = m > 0 ? (R)f[n * (n + 1) - m] : (R)0;
-    const R co = ph[((long long)m * nb + b) * 2], si = ph[((long long)m * nb + b) * 2 + 1];
-    g4[(n * (n + 1) + m) * 4 + c] = fr * co - fi * si;
-    if (m > 0) g4[(n * (n + 1) - m) * 4 + c] = fr * si + fi * co;
+  const long long ld = bid / tiles;
+  const int t0 = (int)(bid - ld * tiles) * tb;
+  for (int i = threadIdx.x; i < 3 * ncp; i += kSelfThreads) {
+    const int c = i / ncp, r = i - c * ncp;
+    rho[i] = r < nc ? R(dens[A.foff3[ld * 3 + c] + r]) : R(0);
   }
   __syncthreads();
-  // stages 1-2: rotation (even / odd input orders) and contraction, per rotated coefficient
-  const R* blk = wblk + (long long)a * wstride;
-  const long long qstride = 12 * (long long)ntri;
-  const R* QA = Q + (ld * ng + tlA) * qstride;
-  const R* QC = Q + (ld * ng + tlC) * qstride;
-  const R* Qk_[4] = {QA, QA + hb * qstride, QC, QC + hb * qstride};
-  R acc[4][3];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) acc[k][0] = acc[k][1] = acc[k][2] = 0;
-  for (int i = threadIdx.x; i < nc; i += blockDim.x) {
-    const int n = degree_of(i);
-    const int o = i - n * n;
-    const long long boff = (long long)n * (n + 1) * (2 * n + 1) / 6 + (long long)(n - 1) * n * (2 * n - 1) / 6;
-    const R* g = g4 + n * (n + 1) * 4;
-    const bool re = o <= n;
-    const int mo = re ? o : o - n;  // output order m'
-    const int t = n * (n + 1) / 2 + mo;
-    const int ri = re ? 0 : 1;      // real or imaginary planes of Q
-    R q[4][6];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (k < 2 || quad) {
-        const R* Qk = Qk_[k] + t;
-#pragma unroll
-        for (int e = 0; e < 6; ++e) q[k][e] = Qk[(2 * e + ri) * (long long)ntri];
-      }
-    }
-    R E[3] = {0, 0, 0}, O[3] = {0, 0, 0};
-    if (re) {
-      const R* Cc = blk + boff + o;
-      int m = 0;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nv = ncp / V;
+  for (int k = 0; k < per_warp; ++k) {
+    const int t = t0 + k * (kSelfThreads / 32) + warp;
+    if (t >= ng) break;
+    const uint4* S = reinterpret_cast<const uint4*>(A.S + (ld * ng + t) * 6 * (long long)ncp);
+    R acc[3] = {R(0), R(0), R(0)};
 #pragma unroll 2
-      for (; m + 1 <= n; m += 2) {
-        const R cv = Cc[(long long)m * (n + 1)], cw = Cc[(long long)(m + 1) * (n + 1)];
-        const R* gm = g + 4 * m;
-        E[0] += cv * gm[0];
-        E[1] += cv * gm[1];
-        E[2] += cv * gm[2];
-        O[0] += cw * gm[4];
-        O[1] += cw * gm[5];
-        O[2] += cw * gm[6];
-      }
-      if (m <= n) {
-        const R cv = Cc[(long long)m * (n + 1)];
-        const R* gm = g + 4 * m;
-        E[0] += cv * gm[0];
-        E[1] += cv * gm[1];
-        E[2] += cv * gm[2];
-      }
-    } else {
-      const R* Sc = blk + boff + (long long)(n + 1) * (n + 1) + (mo - 1);
-      int m = 1;
-#pragma unroll 2
-      for (; m + 1 <= n; m += 2) {
-        const R sv = Sc[(long long)(m - 1) * n], sw = Sc[(long long)m * n];
-        const R* gm = g - 4 * m;
-        O[0] += sv * gm[0];
-        O[1] += sv * gm[1];
-        O[2] += sv * gm[2];
-        E[0] += sw * gm[-4];
-        E[1] += sw * gm[-3];
-        E[2] += sw * gm[-2];
-      }
-      if (m <= n) {
-        const R sv = Sc[(long long)(m - 1) * n];
-        const R* gm = g - 4 * m;
-        O[0] += sv * gm[0];
-        O[1] += sv * gm[1];
-        O[2] += sv * gm[2];
-      }
-    }
-    R vp[3], vm[3];
+    for (int i = lane; i < nv; i += 32) {
+      uint4 s[6], f[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      vp[c] = E[c] + O[c];
-      vm[c] = E[c] - O[c];
-    }
-    // Real parts enter with +Q_re, imaginary parts with -Q_im; latitude pi - theta_a carries
-    // (-1)^(n + m') on the real and -(-1)^(n + m') on the imaginary parts.  Both signs are stored in
-    // the factors (see k_kernel_proj), so every product is added.
-    sym_mul_add<R>(q[0], vp, acc[0]);
-    sym_mul_add<R>(q[1], vm, acc[1]);
-    if (quad) {
-      sym_mul_add<R>(q[2], vm, acc[2]);
-      sym_mul_add<R>(q[3], vp, acc[3]);
-    }
-  }
-  // block reduction of the 12 sums
+      for (int e = 0; e < 6; ++e) s[e] = load_factor(S + e * nv + i);
 #pragma unroll
-  for (int k = 0; k < 4; ++k)
+      for (int c = 0; c < 3; ++c) f[c] = reinterpret_cast<const uint4*>(rho + c * ncp)[i];
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        R q[6], x[3];
+#pragma unroll
+        for (int e = 0; e < 6; ++e) q[e] = lane_of<R>(s[e], v);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) x[c] = lane_of<R>(f[c], v);
+        sym_mul_add<R>(q, x, acc);
+      }
+    }
 #pragma unroll
     for (int c = 0; c < 3; ++c)
-      for (int off = 16; off > 0; off >>= 1) acc[k][c] += shfl_down(acc[k][c], off);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0)
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) red[w][k * 3 + c] = acc[k][c];
-  __syncthreads();
-  const int nt = quad ? 4 : 2;
-  if (threadIdx.x < 3 * nt) {
-    R v = 0;
-    for (int ww = 0; ww < (int)(blockDim.x >> 5); ++ww) v += red[ww][threadIdx.x];
-    const int k = threadIdx.x / 3, c = threadIdx.x - 3 * k;
-    const int tl = (k < 2 ? tlA : tlC) + (k & 1) * hb;
-    vals[val_off[ld] + (long long)c * ng + tl] = wts[ld] * (double)v;
+      for (int off = 16; off > 0; off >>= 1) acc[c] += shfl_down(acc[c], off);
+    if (lane == 0) {
+      double* v = vals + A.val_off[ld] + t;
+      v[0] = A.wts[ld] * (double)acc[0];
+      v[ng] = A.wts[ld] * (double)acc[1];
+      v[2 * ng] = A.wts[ld] * (double)acc[2];
+    }
   }
 }
 
@@ -554,25 +538,45 @@ size_t kernel_proj_smem(int p, int pq) {
 }
 
 int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, int pq, const double* cs,
-                       const double* T0, double* Q64, float* Q32, cudaStream_t s) {
+                       const double* T0, double* Q64, cudaStream_t s) {
   if (ntarget == 0) return BIE_OK;
   if (ntarget > 0x7fffffffLL) return BIE_EINVAL;
   const size_t smem = kernel_proj_smem(p, pq);
   if (smem > 227 * 1024) {
-    set_error("degree too large for the projected self form (shared memory)");
+    set_error("degree too large for the dense self form (shared memory)");
     return BIE_ENOTSUP;
   }
   auto kern = kind == 0 ? k_kernel_proj<0> : k_kernel_proj<1>;
   if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<(unsigned)ntarget, 256, smem, s>>>(cache, pq, p, cs, T0, Q64, Q32);
+  kern<<<(unsigned)ntarget, 256, smem, s>>>(cache, pq, p, cs, T0, Q64);
+  count_launch();
+  BIE_CUDA_TRY(cudaGetLastError());
+  return BIE_OK;
+}
+
+int launch_unrotate(const double* Q64, long long row0, long long nrow, int p, const double* wblk, long long wstride,
+                    const double* ph, double* S64, float* S32, cudaStream_t s) {
+  if (nrow == 0) return BIE_OK;
+  const int nbch = (2 * p + 2 + kUnB - 1) / kUnB;
+  if (nrow * nbch > 0x7fffffffLL) return BIE_EINVAL;
+  const size_t smem = sizeof(double) * ((size_t)(p + 1) * (p + 2) + (size_t)p * (p + 1) + (size_t)kUnB * 6 * (2 * p + 1));
+  if (smem > 48 * 1024)
+    BIE_CUDA_TRY(cudaFuncSetAttribute(k_unrotate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_unrotate<<<dim3((unsigned)(nrow * nbch), p + 1), 128, smem, s>>>(Q64, row0, p, wblk, wstride, ph, self_row(p), S64,
+                                                                     S32);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
 }
 
 template <typename R, typename CT>
-int launch_self_proj(std::vector<SelfGroup<R>> groups, const CT* dens, double* vals, cudaStream_t s) {
+int launch_self_dense(std::vector<SelfGroup<R>> groups, const CT* dens, double* vals, int sms, cudaStream_t s) {
   std::sort(groups.begin(), groups.end(), [](const SelfGroup<R>& x, const SelfGroup<R>& y) { return x.p > y.p; });
+  long long targets = 0;
+  for (const auto& g : groups) targets += g.ndrop * 2 * (long long)(g.p + 1) * (g.p + 1);
+  // one target per warp until every SM has about eight blocks, then up to eight
+  const int nw = kSelfThreads / 32;
+  const int per_warp = (int)std::max(1LL, std::min<long long>(8, targets / (8LL * nw * sms)));
   for (size_t g0 = 0; g0 < groups.size(); g0 += kMaxSelfGroups) {
     SelfGroups<R> G{};
     G.n = (int)std::min<size_t>(kMaxSelfGroups, groups.size() - g0);
@@ -580,17 +584,17 @@ int launch_self_proj(std::vector<SelfGroup<R>> groups, const CT* dens, double* v
     size_t smem = 0;
     for (int i = 0; i < G.n; ++i) {
       G.g[i] = groups[g0 + i];
-      const int p = G.g[i].p;
+      const int p = G.g[i].p, ng = 2 * (p + 1) * (p + 1);
       G.g[i].begin = nblk;
-      nblk += G.g[i].ndrop * ((p + 2) / 2) * (p + 1);
-      smem = std::max(smem, sizeof(R) * 4 * (size_t)(p + 1) * (p + 1));
-      if (G.g[i].ndrop * (long long)(p + 1) * (2 * p + 2) > 0x7fffffffLL) return BIE_EINVAL;
+      nblk += G.g[i].ndrop * ((ng + per_warp * nw - 1) / (per_warp * nw));
+      smem = std::max(smem, sizeof(R) * 3 * (size_t)self_row(p));
+      if (G.g[i].ndrop * (long long)ng > 0x7fffffffLL) return BIE_EINVAL;
     }
     if (nblk == 0) continue;
     if (nblk > 0x7fffffffLL) return BIE_EINVAL;
-    auto kern = k_self_proj<R, CT>;
+    auto kern = k_self_dense<R, CT>;
     if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kern<<<(unsigned)nblk, kSelfThreads, smem, s>>>(G, dens, vals);
+    kern<<<(unsigned)nblk, kSelfThreads, smem, s>>>(G, per_warp, dens, vals);
     count_launch();
     BIE_CUDA_TRY(cudaGetLastError());
   }
@@ -603,8 +607,8 @@ template int launch_self_direct<double>(int, const double*, const long long*, lo
 template int launch_self_direct<float>(int, const double*, const long long*, long long, int, int, const float*,
                                        long long, const float*, const float*, const float*, const float*,
                                        const double*, const long long*, double*, size_t, cudaStream_t);
-template int launch_self_proj<double, double>(std::vector<SelfGroup<double>>, const double*, double*, cudaStream_t);
-template int launch_self_proj<float, double>(std::vector<SelfGroup<float>>, const double*, double*, cudaStream_t);
-template int launch_self_proj<dff, double>(std::vector<SelfGroup<dff>>, const double*, double*, cudaStream_t);
+template int launch_self_dense<double, double>(std::vector<SelfGroup<double>>, const double*, double*, int, cudaStream_t);
+template int launch_self_dense<float, double>(std::vector<SelfGroup<float>>, const double*, double*, int, cudaStream_t);
+template int launch_self_dense<dff, double>(std::vector<SelfGroup<dff>>, const double*, double*, int, cudaStream_t);
 
 }  // namespace bie
