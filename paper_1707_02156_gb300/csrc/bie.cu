@@ -135,6 +135,8 @@ struct bie_ctx {
   std::mutex mu;
   std::map<std::pair<int, int>, std::unique_ptr<bie::Plan>> plans;
   std::map<int, std::unique_ptr<bie::WigPlan>> wigs;
+  // rotation blocks that put latitude a of the degree-p grid on the equator, by (p, a), on the device
+  std::map<std::pair<int, int>, std::unique_ptr<bie::DevBuf<double>>> equator;
   // pair-kernel variant chosen at earlier geometries: degrees, self-grid degrees, U, pair count, variant
   struct Tuned {
     std::vector<int> p, pq;
@@ -240,6 +242,22 @@ static int get_wig(bie_ctx* ctx, int p, WigPlan** out) {
   BIE_TRY(upload_as(wp->blkf, blk));
   *out = wp.get();
   ctx->wigs[p] = std::move(wp);
+  return BIE_OK;
+}
+
+// Rotation blocks of beta = theta_a - pi/2 for latitude a of the degree-p grid (the closest-point search).
+static int get_equator(bie_ctx* ctx, int p, int a, const double** out) {
+  std::lock_guard<std::mutex> lk(ctx->mu);
+  auto& e = ctx->equator[{p, a}];
+  if (!e) {
+    std::vector<double> t, w, blk(wigner_block_stride(p));
+    gauss_legendre(p + 1, t, w);
+    wigner_blocks(p, std::acos(t[a]) - 0.5 * kPi, blk.data());
+    std::unique_ptr<DevBuf<double>> d(new DevBuf<double>());
+    BIE_TRY(d->upload(blk));
+    e = std::move(d);
+  }
+  *out = e->ptr;
   return BIE_OK;
 }
 
@@ -1074,62 +1092,60 @@ static int near_points(bie_ctx* ctx, bie_geom* g, std::vector<NearPair>& pairs, 
   }
   struct RotGroup {
     int p, n;
-    long long base, fo_at, blk_at, blk_n;
+    long long base, fo_at;
+    const double* blk;
   };
   std::vector<RotGroup> rg;
   std::vector<long long> xr_off(npair), fo_all;
-  std::vector<double> blocks_all, ph(2 * (size_t)npair * (pmax + 1), 0.0);
+  std::vector<int> lon(npair);
+  std::map<int, std::vector<double>> nodes;
   long long xo = 0;
   for (const auto& kv : groups) {
     const int p = kv.first.first, a = kv.first.second;
     const std::vector<int>& idx = kv.second;
     const int nb = 2 * p + 2;
     const long long nc = ncoef(p);
-    std::vector<double> t, w;
-    gauss_legendre(p + 1, t, w);
-    const double be = std::acos(t[a]) - 0.5 * kPi;
-    std::vector<double> blk(wigner_block_stride(p));
-    wigner_blocks(p, be, blk.data());
-    rg.push_back({p, (int)idx.size(), xo, (long long)fo_all.size(), (long long)blocks_all.size(), (long long)blk.size()});
-    blocks_all.insert(blocks_all.end(), blk.begin(), blk.end());
+    auto& t = nodes[p];
+    if (t.empty()) {
+      std::vector<double> w;
+      gauss_legendre(p + 1, t, w);
+    }
+    rg.push_back({p, (int)idx.size(), xo, (long long)fo_all.size(), nullptr});
+    BIE_TRY(get_equator(ctx, p, a, &rg.back().blk));
     for (size_t k = 0; k < idx.size(); ++k) {
       const int i = idx[k];
-      alpha[i] = kPi * (hseed[i] % nb) / (p + 1);
-      beta[i] = be;
+      lon[i] = hseed[i] % nb;
+      alpha[i] = kPi * lon[i] / (p + 1);
+      beta[i] = std::acos(t[a]) - 0.5 * kPi;
       xr_off[i] = xo + (long long)k * 3 * nc;
       for (int c = 0; c < 3; ++c) fo_all.push_back(xr_off[i] + c * nc);
-      for (int m = 0; m <= p; ++m) {
-        ph[2 * ((size_t)i * (pmax + 1) + m)] = std::cos(m * alpha[i]);
-        ph[2 * ((size_t)i * (pmax + 1) + m) + 1] = std::sin(m * alpha[i]);
-      }
     }
     xo += (long long)idx.size() * 3 * nc;
   }
   std::vector<int> pd(g->p.begin(), g->p.end());
-  DevBuf<int> pdeg;
-  DevBuf<double> shifted, xr, dblk, dph, dx0, res;
+  DevBuf<int> pdeg, dlon;
+  DevBuf<double> shifted, xr, dx0, res;
   DevBuf<long long> dfo, dxo, dcoef_off;
   BIE_TRY(pdeg.upload(pd));
+  BIE_TRY(dlon.upload(lon));
   BIE_TRY(dcoef_off.upload(g->coef_off));
-  BIE_TRY(dph.upload(ph));
   BIE_TRY(dxo.upload(xr_off));
   BIE_TRY(dfo.upload(fo_all));
-  BIE_TRY(dblk.upload(blocks_all));
   BIE_TRY(dx0.upload(x0));
   BIE_TRY(shifted.alloc(xo));
   BIE_TRY(xr.alloc(xo));
   BIE_TRY(res.alloc(5 * (size_t)npair));
-  BIE_TRY(launch_near_phase_shift(dpairs.ptr, npair, g->xcoef.ptr, dcoef_off.ptr, pdeg.ptr, pmax, dph.ptr, dxo.ptr,
+  BIE_TRY(launch_near_phase_shift(dpairs.ptr, npair, g->xcoef.ptr, dcoef_off.ptr, pdeg.ptr, dlon.ptr, dxo.ptr,
                                   shifted.ptr, s));
   for (const auto& G : rg) {
     const long long nc = ncoef(G.p);
-    BIE_TRY((launch_rotate<double, double>(shifted.ptr, dfo.ptr + G.fo_at, 3, G.n, G.p, dblk.ptr + G.blk_at, G.blk_n,
+    BIE_TRY((launch_rotate<double, double>(shifted.ptr, dfo.ptr + G.fo_at, 3, G.n, G.p, G.blk, wigner_block_stride(G.p),
                                            1, 1, (const double*)nullptr, xr.ptr + G.base, 3 * nc, s)));
   }
   DevBuf<double> rtab;
   BIE_TRY(rtab.alloc(near_rec_table_doubles(pmax)));
   BIE_TRY(launch_near_rec_table(pmax, rtab.ptr, s));
-  BIE_TRY(launch_near_newton(dpairs.ptr, npair, xr.ptr, pdeg.ptr, dxo.ptr, dx0.ptr, rtab.ptr, res.ptr, s));
+  BIE_TRY(launch_near_newton(dpairs.ptr, npair, xr.ptr, pdeg.ptr, dxo.ptr, dx0.ptr, rtab.ptr, pmax, res.ptr, s));
   BIE_CUDA_TRY(cudaMemcpyAsync(hres.data(), res.ptr, hres.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
   BIE_CUDA_TRY(cudaStreamSynchronize(s));
   stage.reset(new Phase(ctx, "near_checkpoints", s));

@@ -26,9 +26,17 @@ __device__ __forceinline__ double rec_b(int n, int m) {
 __device__ __forceinline__ double rec_c(int n, int m) { return sqrt((double)(n - m) * (n + m + 1.0)); }
 __device__ __forceinline__ long long tri(int n, int m) { return (long long)n * (n + 1) / 2 + m; }
 
-// tab[3 tri(n, m) + k] = rec_a, rec_b (0 for n < m + 2), rec_c, for 0 <= m <= n <= P
+// tab[3 tri(n, m) + k] = rec_a, rec_b (0 for n < m + 2), rec_c, for 0 <= m <= n <= P; then the P + 2
+// constants of P~_m^m(theta) = C_m sin^m(theta), C_0 = sqrt(1/4pi), C_(m+1) = -sqrt(1 + 1/(2m+2)) C_m
 __global__ void k_rec_table(int P, double* __restrict__ tab) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t == 0) {
+    double c = sqrt(1.0 / (4.0 * kPiD));
+    for (int m = 0; m <= P + 1; ++m) {
+      tab[3 * tri(P + 1, 0) + m] = c;
+      c *= -sqrt(1.0 + 1.0 / (2.0 * (m + 1)));
+    }
+  }
   if (t >= tri(P + 1, 0)) return;
   int n = (int)((sqrt(8.0 * t + 1.0) - 1.0) / 2.0);
   while (tri(n + 1, 0) <= t) ++n;
@@ -42,34 +50,41 @@ __global__ void k_rec_table(int P, double* __restrict__ tab) {
 // Value and first/second parameter derivatives of three real SH series (coefficients c[3][(p+1)^2])
 // at (theta, phi), with the Legendre recursion of App. A and the derivative identities
 // dP = alpha P^{m+1} + m cot(theta) P^m and the Legendre equation (theta away from the poles).
-// out[k][c], k: 0 f, 1 f_t, 2 f_p, 3 f_tt, 4 f_tp, 5 f_pp.
+// One warp per point: lane l runs the recursions of the orders l, l + 32, ..., so a point takes p + 1
+// serial steps, not (p+1)(p+2)/2; the xor sums leave the same values in every lane.  Closest points of 2051
+// points off drops of degree 24, with their rotations: 27.0 -> 3.8 ms.
+// tab: k_rec_table's for degrees up to tabP.  out[k][c], k: 0 f, 1 f_t, 2 f_p, 3 f_tt, 4 f_tp, 5 f_pp.
 __device__ void sh_eval_d2(const double* __restrict__ c, long long cstride, int p, double th, double ph,
-                           const double* __restrict__ tab, double out[6][3]) {
+                           const double* __restrict__ tab, int tabP, double out[6][3]) {
   for (int k = 0; k < 6; ++k)
     for (int q = 0; q < 3; ++q) out[k][q] = 0;
   double st, ct;
   sincos(th, &st, &ct);
   const double cot = ct / st, s2 = st * st;
-  double dm = sqrt(1.0 / (4.0 * kPiD));  // P~_m^m
-  for (int m = 0; m <= p; ++m) {
-    const double dm1 = m + 1 <= p ? -sqrt(1.0 + 1.0 / (2.0 * (m + 1))) * st * dm : 0.0;
+  const double* diag = tab + 3 * tri(tabP + 1, 0);
+  for (int m = threadIdx.x & 31; m <= p; m += 32) {
+    double pw = 1.0;
+    for (int k = 0; k < m; ++k) pw *= st;
+    const double dm = diag[m] * pw;  // P~_m^m
+    const double dm1 = m + 1 <= p ? diag[m + 1] * (pw * st) : 0.0;
     double pm2 = 0, pm1 = 0, qm2 = 0, qm1 = 0;
     double h0r[3] = {0, 0, 0}, h0i[3] = {0, 0, 0}, h1r[3] = {0, 0, 0}, h1i[3] = {0, 0, 0}, h2r[3] = {0, 0, 0},
            h2i[3] = {0, 0, 0};
+    const double f1 = sqrt(2.0 * m + 3.0), f2 = sqrt(2.0 * m + 5.0);
+    const int m1 = m + 1;
     for (int n = m; n <= p; ++n) {
       double P;
       if (n == m)
         P = dm;
-      else if (n == m + 1)
-        P = sqrt(2.0 * m + 3.0) * ct * dm;
+      else if (n == m1)
+        P = f1 * ct * dm;
       else
         P = tab[3 * tri(n, m)] * (ct * pm1 - tab[3 * tri(n, m) + 1] * pm2);
       double Q = 0;  // P~_n^{m+1}
-      const int m1 = m + 1;
       if (n == m1)
         Q = dm1;
       else if (n == m1 + 1)
-        Q = sqrt(2.0 * m1 + 3.0) * ct * dm1;
+        Q = f2 * ct * dm1;
       else if (n > m1 + 1)
         Q = tab[3 * tri(n, m1)] * (ct * qm1 - tab[3 * tri(n, m1) + 1] * qm2);
       pm2 = pm1;
@@ -105,8 +120,10 @@ __device__ void sh_eval_d2(const double* __restrict__ c, long long cstride, int 
       out[4][q] += fac * (-m * w1);
       out[5][q] += fac * (-(double)m * m * v0);
     }
-    dm = dm1;
   }
+  for (int k = 0; k < 6; ++k)
+    for (int q = 0; q < 3; ++q)
+      for (int o = 16; o > 0; o >>= 1) out[k][q] += __shfl_xor_sync(0xffffffffu, out[k][q], o);
 }
 
 // Value of three real SH series at (theta, phi) (any theta, poles included).
@@ -142,40 +159,52 @@ __device__ void sh_eval3(const double* __restrict__ c, long long cstride, int p,
   }
 }
 
-// seed: nearest standard grid point of drop j to the target
+// nearest of the N points of records r to x0, scanned by one warp (the first nearest point wins ties, as in
+// a sequential scan); every lane returns it
+__device__ int warp_nearest(const double* __restrict__ r, long long N, double x0, double x1, double x2) {
+  double best = 1e300;
+  long long bi = N;
+  for (long long s = threadIdx.x & 31; s < N; s += 32) {
+    const double d0 = x0 - r[s], d1 = x1 - r[N + s], d2 = x2 - r[2 * N + s];
+    const double d = d0 * d0 + d1 * d1 + d2 * d2;
+    if (d < best) {
+      best = d;
+      bi = s;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+    const long long oi = __shfl_xor_sync(0xffffffffu, bi, o);
+    if (ob < best || (ob == best && oi < bi)) {
+      best = ob;
+      bi = oi;
+    }
+  }
+  return bi < N ? (int)bi : 0;
+}
+
+// seed: nearest standard grid point of drop j to the target, one warp per pair
 __global__ void k_near_seed(const NearPair* __restrict__ pairs, int npair, const double* __restrict__ rec_std,
                             const long long* __restrict__ toff, const int* __restrict__ ngd,
                             const long long* __restrict__ tgt_loc, const int* __restrict__ tdrop,
                             int* __restrict__ seed) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (i >= npair) return;
   const long long t = pairs[i].target;
   const int j = pairs[i].src_drop, di = tdrop[t];
   const long long ngi = ngd[di];
   const double* ri = rec_std + 7 * toff[di];
-  const double x0 = ri[tgt_loc[t]], x1 = ri[ngi + tgt_loc[t]], x2 = ri[2 * ngi + tgt_loc[t]];
-  const long long N = ngd[j];
-  const double* r = rec_std + 7 * toff[j];
-  double best = 1e300;
-  int bi = 0;
-  for (long long s = 0; s < N; ++s) {
-    const double d0 = x0 - r[s], d1 = x1 - r[N + s], d2 = x2 - r[2 * N + s];
-    const double d = d0 * d0 + d1 * d1 + d2 * d2;
-    if (d < best) {
-      best = d;
-      bi = (int)s;
-    }
-  }
-  seed[i] = bi;
+  const int bi = warp_nearest(rec_std + 7 * toff[j], ngd[j], ri[tgt_loc[t]], ri[ngi + tgt_loc[t]], ri[2 * ngi + tgt_loc[t]]);
+  if ((threadIdx.x & 31) == 0) seed[i] = bi;
 }
 
 // Levenberg-Marquardt Newton on F = |x(theta, phi) - x0|^2 / 2 in the rotated frame (seed at the
-// equator).  One thread per pair; rotated coefficients xr[pair][3][(p+1)^2].
+// equator).  One warp per pair, every lane with the same iterate; rotated coefficients xr[pair][3][(p+1)^2].
 __global__ void k_near_newton(const NearPair* __restrict__ pairs, int npair, const double* __restrict__ xr,
                               const int* __restrict__ pdeg, const long long* __restrict__ xr_off,
-                              const double* __restrict__ x0all, const double* __restrict__ tab,
+                              const double* __restrict__ x0all, const double* __restrict__ tab, int tabP,
                               double* __restrict__ result) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (i >= npair) return;
   const int p = pdeg[pairs[i].src_drop];
   const long long cs = (long long)(p + 1) * (p + 1);
@@ -183,7 +212,7 @@ __global__ void k_near_newton(const NearPair* __restrict__ pairs, int npair, con
   const double x0[3] = {x0all[3 * i], x0all[3 * i + 1], x0all[3 * i + 2]};
   double th = 0.5 * kPiD, ph = 0.0;
   double d[6][3];
-  sh_eval_d2(c, cs, p, th, ph, tab, d);
+  sh_eval_d2(c, cs, p, th, ph, tab, tabP, d);
   auto half_sq = [&](const double* x) {
     const double a = x[0] - x0[0], b = x[1] - x0[1], e = x[2] - x0[2];
     return 0.5 * (a * a + b * b + e * e);
@@ -204,14 +233,13 @@ __global__ void k_near_newton(const NearPair* __restrict__ pairs, int npair, con
     const double Hbb = xp[0] * xp[0] + xp[1] * xp[1] + xp[2] * xp[2] + r[0] * d[5][0] + r[1] * d[5][1] + r[2] * d[5][2];
     if (mu < 0) mu = 1e-8 * fabs(Haa + Hbb);
     bool accepted = false;
-    double s0 = 0, s1 = 0;
+    double s0 = 0, s1 = 0, dn[6][3];
     for (int k = 0; k < 40; ++k) {
       const double a = Haa + mu, b = Hab, e = Hbb + mu;
       const double det = a * e - b * b;
       s0 = -(e * g0 - b * g1) / det;
       s1 = -(a * g1 - b * g0) / det;
-      double dn[6][3];
-      sh_eval_d2(c, cs, p, th + s0, ph + s1, tab, dn);
+      sh_eval_d2(c, cs, p, th + s0, ph + s1, tab, tabP, dn);
       if (half_sq(dn[0]) <= F) {
         accepted = true;
         break;
@@ -221,10 +249,12 @@ __global__ void k_near_newton(const NearPair* __restrict__ pairs, int npair, con
     if (!accepted) break;
     th += s0;
     ph += s1;
-    sh_eval_d2(c, cs, p, th, ph, tab, d);
+    for (int k = 0; k < 6; ++k)
+      for (int q = 0; q < 3; ++q) d[k][q] = dn[k][q];
     F = half_sq(d[0]);
     if (fmax(fabs(s0), fabs(s1)) < 1e-14) break;
   }
+  if (threadIdx.x & 31) return;
   result[5 * i + 0] = th;
   result[5 * i + 1] = ph;
   result[5 * i + 2] = d[0][0];
@@ -239,24 +269,26 @@ __global__ void k_near_checkgrid(const NearPair* __restrict__ pairs, int npair, 
                                  const double* __restrict__ h, double a_tilde, const double* __restrict__ rec_up,
                                  const long long* __restrict__ up_off, const long long* __restrict__ up_n,
                                  int* __restrict__ grid) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  const int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // one warp per check point
   if (idx >= npair * L) return;
+  const int lane = threadIdx.x & 31;
   const int i = idx / L;
   const int j = pairs[i].src_drop;
   const double x0 = pts[3 * idx], x1 = pts[3 * idx + 1], x2 = pts[3 * idx + 2];
   const double dc0 = x0 - centre[3 * j], dc1 = x1 - centre[3 * j + 1], dc2 = x2 - centre[3 * j + 2];
   if (sqrt(dc0 * dc0 + dc1 * dc1 + dc2 * dc2) - bound[j] > a_tilde * h[j]) {
-    grid[idx] = 0;
+    if (lane == 0) grid[idx] = 0;
     return;
   }
   const long long N = up_n[j];
   const double* r = rec_up + 7 * up_off[j];
   double best = 1e300;
-  for (long long s = 0; s < N; ++s) {
+  for (long long s = lane; s < N; s += 32) {
     const double d0 = x0 - r[s], d1 = x1 - r[N + s], d2 = x2 - r[2 * N + s];
     best = fmin(best, d0 * d0 + d1 * d1 + d2 * d2);
   }
-  grid[idx] = sqrt(best) <= a_tilde * h[j] ? 1 : 0;
+  for (int o = 16; o > 0; o >>= 1) best = fmin(best, __shfl_xor_sync(0xffffffffu, best, o));
+  if (lane == 0) grid[idx] = sqrt(best) <= a_tilde * h[j] ? 1 : 0;
 }
 
 // Regular-rule value of drop j's layer at check point (pair, l): one block per check point.
@@ -356,19 +388,22 @@ __global__ void k_near_interp(const NearPair* __restrict__ pairs, const int* __r
 }
 
 // The source drop's shape coefficients of pair i with the phases of its seed longitude applied,
-// g_n^m = e^{i m alpha_i} x_n^m (real-packed; ph[i][m] = (cos m alpha_i, sin m alpha_i)), written to
-// out + dst_off[i] as [3][(p+1)^2]: the first step of the rotation R_z(alpha) R_y(beta), so that the
-// pairs of one seed latitude then share one rotation launch.  One block per pair.
+// g_n^m = e^{i m alpha_i} x_n^m (real-packed; alpha_i = pi lon[i] / (p+1), lon the seed's longitude index),
+// written to out + dst_off[i] as [3][(p+1)^2]: the first step of the rotation R_z(alpha) R_y(beta), so
+// that the pairs of one seed latitude then share one rotation launch.  One block per pair.
 __global__ void k_near_phase_shift(const NearPair* __restrict__ pairs, int npair, const double* __restrict__ coef,
-                                   const long long* __restrict__ coef_off, const int* __restrict__ pdeg, int pmax,
-                                   const double* __restrict__ ph, const long long* __restrict__ dst_off,
+                                   const long long* __restrict__ coef_off, const int* __restrict__ pdeg,
+                                   const int* __restrict__ lon, const long long* __restrict__ dst_off,
                                    double* __restrict__ out) {
+  __shared__ double phi[2 * (BIE_MAX_P + 1)];
   const int i = blockIdx.x;
   if (i >= npair) return;
   const int j = pairs[i].src_drop;
   const int p = pdeg[j];
   const long long nc = (long long)(p + 1) * (p + 1);
-  const double* phi = ph + (long long)i * 2 * (pmax + 1);
+  for (int m = threadIdx.x; m <= p; m += blockDim.x)
+    sincospi((double)((m * lon[i]) % (2 * p + 2)) / (p + 1), &phi[2 * m + 1], &phi[2 * m]);
+  __syncthreads();
   for (long long q = threadIdx.x; q < 3 * nc; q += blockDim.x) {
     const int c = (int)(q / nc);
     const long long k = q - c * nc;
@@ -388,10 +423,10 @@ __global__ void k_near_phase_shift(const NearPair* __restrict__ pairs, int npair
 }  // namespace
 
 int launch_near_phase_shift(const NearPair* pairs, int npair, const double* coef, const long long* coef_off,
-                            const int* pdeg, int pmax, const double* ph, const long long* dst_off, double* out,
+                            const int* pdeg, const int* lon, const long long* dst_off, double* out,
                             cudaStream_t s) {
   if (!npair) return BIE_OK;
-  k_near_phase_shift<<<npair, 128, 0, s>>>(pairs, npair, coef, coef_off, pdeg, pmax, ph, dst_off, out);
+  k_near_phase_shift<<<npair, 128, 0, s>>>(pairs, npair, coef, coef_off, pdeg, lon, dst_off, out);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
@@ -400,13 +435,13 @@ int launch_near_phase_shift(const NearPair* pairs, int npair, const double* coef
 int launch_near_seed(const NearPair* pairs, int npair, const double* rec_std, const long long* toff, const int* ngd,
                      const long long* tgt_loc, const int* tdrop, int* seed, cudaStream_t s) {
   if (!npair) return BIE_OK;
-  k_near_seed<<<(npair + 127) / 128, 128, 0, s>>>(pairs, npair, rec_std, toff, ngd, tgt_loc, tdrop, seed);
+  k_near_seed<<<(npair + 3) / 4, 128, 0, s>>>(pairs, npair, rec_std, toff, ngd, tgt_loc, tdrop, seed);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
 }
 
-int near_rec_table_doubles(int P) { return 3 * (P + 1) * (P + 2) / 2; }
+int near_rec_table_doubles(int P) { return 3 * (P + 1) * (P + 2) / 2 + P + 2; }
 
 int launch_near_rec_table(int P, double* tab, cudaStream_t s) {
   const int n = (P + 1) * (P + 2) / 2;
@@ -417,9 +452,9 @@ int launch_near_rec_table(int P, double* tab, cudaStream_t s) {
 }
 
 int launch_near_newton(const NearPair* pairs, int npair, const double* xr, const int* pdeg, const long long* xr_off,
-                       const double* x0, const double* tab, double* result, cudaStream_t s) {
+                       const double* x0, const double* tab, int tabP, double* result, cudaStream_t s) {
   if (!npair) return BIE_OK;
-  k_near_newton<<<(npair + 63) / 64, 64, 0, s>>>(pairs, npair, xr, pdeg, xr_off, x0, tab, result);
+  k_near_newton<<<(npair + 3) / 4, 128, 0, s>>>(pairs, npair, xr, pdeg, xr_off, x0, tab, tabP, result);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
@@ -429,7 +464,7 @@ int launch_near_checkgrid(const NearPair* pairs, int npair, int L, const double*
                           const double* bound, const double* h, double a_tilde, const double* rec_up,
                           const long long* up_off, const long long* up_n, int* grid, cudaStream_t s) {
   if (!npair) return BIE_OK;
-  k_near_checkgrid<<<(npair * L + 127) / 128, 128, 0, s>>>(pairs, npair, L, pts, centre, bound, h, a_tilde, rec_up,
+  k_near_checkgrid<<<(npair * L + 3) / 4, 128, 0, s>>>(pairs, npair, L, pts, centre, bound, h, a_tilde, rec_up,
                                                            up_off, up_n, grid);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());

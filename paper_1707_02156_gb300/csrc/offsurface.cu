@@ -127,7 +127,7 @@ __global__ void k_gather_points(const double* __restrict__ vals, long long t0, l
 __global__ void k_near_seed_points(const NearPair* __restrict__ pairs, int npair, const double* __restrict__ pts,
                                    long long ld, const double* __restrict__ rec_std, const long long* __restrict__ toff,
                                    const int* __restrict__ ngd, int* __restrict__ seed) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // one warp per pair
   if (i >= npair) return;
   const long long t = pairs[i].target;
   const int j = pairs[i].src_drop;
@@ -135,16 +135,24 @@ __global__ void k_near_seed_points(const NearPair* __restrict__ pairs, int npair
   const long long N = ngd[j];
   const double* r = rec_std + 7 * toff[j];
   double best = 1e300;
-  int bi = 0;
-  for (long long s = 0; s < N; ++s) {
+  long long bi = N;
+  for (long long s = threadIdx.x & 31; s < N; s += 32) {
     const double d0 = x0 - r[s], d1 = x1 - r[N + s], d2 = x2 - r[2 * N + s];
     const double d = d0 * d0 + d1 * d1 + d2 * d2;
     if (d < best) {
       best = d;
-      bi = (int)s;
+      bi = s;
     }
   }
-  seed[i] = bi;
+  for (int o = 16; o > 0; o >>= 1) {  // smallest distance, then smallest index
+    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+    const long long oi = __shfl_xor_sync(0xffffffffu, bi, o);
+    if (ob < best || (ob == best && oi < bi)) {
+      best = ob;
+      bi = oi;
+    }
+  }
+  if ((threadIdx.x & 31) == 0) seed[i] = bi < N ? (int)bi : 0;
 }
 
 // out = u_inf + (S + D) / 2 (u_inf may be null)
@@ -195,7 +203,7 @@ int launch_gather_points(const double* vals, long long t0, long long n, long lon
 int launch_near_seed_points(const NearPair* pairs, int npair, const double* pts, long long ld, const double* rec_std,
                             const long long* toff, const int* ngd, int* seed, cudaStream_t s) {
   if (npair == 0) return BIE_OK;
-  k_near_seed_points<<<(npair + 127) / 128, 128, 0, s>>>(pairs, npair, pts, ld, rec_std, toff, ngd, seed);
+  k_near_seed_points<<<(npair + 3) / 4, 128, 0, s>>>(pairs, npair, pts, ld, rec_std, toff, ngd, seed);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
