@@ -344,7 +344,10 @@ struct bie_geom {
   int nnear_tgt = 0;
   bie::DevBuf<bie::NearPair> npairs;
   bie::DevBuf<int> ntbeg, ngrid_l, pdeg_d;
-  bie::DevBuf<double> npts, ncv, selfvals, selfcoef, hdrop_d;
+  bie::DevBuf<double> npts, ncv, selfcoef, hdrop_d;
+  bie::DevBuf<double> nrows[2];                     // the rule as rows of the operator, S and D (first apply of a kind)
+  bie::DevBuf<long long> nrow_off;
+  long long nrow_total = 0;                         // doubles per kind; 0: the rows are not used
   bie::DevBuf<long long> coef_off_d, up_off_d, up_n_d;
 };
 
@@ -1190,7 +1193,6 @@ static int near_points(bie_ctx* ctx, bie_geom* g, std::vector<NearPair>& pairs, 
 // buffers of the on-surface expansions, made once per geometry.
 static int near_tables(bie_geom* g) {
   if (g->pdeg_d.ptr) return BIE_OK;
-  BIE_TRY(g->selfvals.alloc(3 * g->ntarget));
   BIE_TRY(g->selfcoef.alloc(g->ncoef_total));
   BIE_TRY(g->hdrop_d.upload(g->hdrop));
   BIE_TRY(g->coef_off_d.upload(g->coef_off));
@@ -1237,6 +1239,21 @@ static int setup_near(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
   BIE_TRY(g->npairs.upload(pairs));
   BIE_TRY(g->ncv.alloc(3 * (size_t)npair * L));
   BIE_TRY(near_tables(g));
+  // The rule becomes rows of the operator unless they would take more than 4 GB per kind, or a block's
+  // sums do not fit in shared memory (degrees above 56): a row costs about 1.3 evaluations of its
+  // check-point sums to build, once, and makes every further apply of the kind read 7 (p+1)^2 doubles
+  // per pair instead.
+  std::vector<long long> ro(npair);
+  long long rtot = 0;
+  bool fit = true;
+  for (int i = 0; i < npair; ++i) {
+    const int p = g->p[pairs[i].src_drop];
+    ro[i] = rtot;
+    rtot += 7LL * self_row(p);
+    fit = fit && near_rows_smem(p, std::max(p, ctx->cfg.upsample * (p + 1) - 1)) <= 220 * 1024;
+  }
+  g->nrow_total = fit && rtot * 8 <= (4LL << 30) ? rtot : 0;
+  if (g->nrow_total) BIE_TRY(g->nrow_off.upload(ro));
   long long npairs_eval = 0;
   std::vector<int> hgrid((size_t)npair * L);
   BIE_CUDA_TRY(cudaMemcpy(hgrid.data(), g->ngrid_l.ptr, hgrid.size() * sizeof(int), cudaMemcpyDeviceToHost));
@@ -1249,12 +1266,40 @@ static int setup_near(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
   return BIE_OK;
 }
 
-// Self-interaction values of every drop as SH coefficients (weighted units): the on-surface
-// values of the near-singular interpolation come from these expansions.
+// Self-interaction values of every drop as SH coefficients (weighted units), taken while vals holds only
+// those: the on-surface values of the near-singular interpolation come from these expansions.
 static int near_snapshot(bie_geom* g, cudaStream_t s) {
-  BIE_CUDA_TRY(cudaMemcpyAsync(g->selfvals.ptr, g->vals.ptr, 3 * g->ntarget * sizeof(double),
-                               cudaMemcpyDeviceToDevice, s));
-  BIE_TRY(analyze_groups(g->ctx, g, g->selfvals.ptr, g->selfcoef.ptr, s));
+  return analyze_groups(g->ctx, g, g->vals.ptr, g->selfcoef.ptr, s);
+}
+
+// The rows of one kind, built at its first apply on the geometry (see near.cu).
+static int ensure_near_rows(bie_geom* g, int kind, cudaStream_t s) {
+  if (g->nrows[kind].ptr) return BIE_OK;
+  bie_ctx* ctx = g->ctx;
+  Phase ph(ctx, "near_rows", s);
+  std::map<int, std::vector<int>> byp;
+  for (size_t i = 0; i < g->near.size(); ++i) byp[g->p[g->near[i].second]].push_back((int)i);
+  std::vector<int> all;
+  for (const auto& kv : byp) all.insert(all.end(), kv.second.begin(), kv.second.end());
+  DevBuf<int> list;
+  DevBuf<double> rows;
+  BIE_TRY(list.upload(all));
+  BIE_TRY(rows.alloc(g->nrow_total));
+  size_t at = 0;
+  for (const auto& kv : byp) {
+    const int p = kv.first, Pu = ctx->cfg.upsample * (p + 1) - 1, n = (int)kv.second.size();
+    Plan *ps, *pu;
+    BIE_TRY(get_plan(ctx, p, p, &ps));
+    BIE_TRY(get_plan(ctx, p, Pu, &pu));
+    const NearRowsSrc std_{p, ps->T0.ptr, ps->cs.ptr, g->sX64.ptr, g->sN64.ptr, g->ntarget, g->rec_std.ptr, g->toff.ptr};
+    const NearRowsSrc up{Pu, pu->T0.ptr, pu->cs.ptr, g->uX64.ptr, g->uN64.ptr, g->nup_total, g->rec_up.ptr, g->up_off_d.ptr};
+    BIE_TRY(launch_near_rows(kind, g->npairs.ptr, list.ptr + at, n, p, ctx->cfg.n_interp, g->npts.ptr, g->ngrid_l.ptr,
+                             g->centre_d.ptr, g->hdrop_d.ptr, std_, up, g->nrow_off.ptr, rows.ptr, s));
+    at += n;
+  }
+  BIE_CUDA_TRY(cudaStreamSynchronize(s));  // the list is released on return
+  std::swap(g->nrows[kind].ptr, rows.ptr);
+  std::swap(g->nrows[kind].n, rows.n);
   return BIE_OK;
 }
 
@@ -1263,6 +1308,13 @@ static int near_apply(bie_geom* g, int kind, bool raw, int prec, const double* d
   bie_ctx* ctx = g->ctx;
   const int npair = (int)g->near.size(), L = ctx->cfg.n_interp;
   const double* wts = kind == 0 ? (raw ? g->wSr_all.ptr : g->wS_all.ptr) : (raw ? g->wDr_all.ptr : g->wD_all.ptr);
+  if (g->nrow_total) {
+    BIE_TRY(ensure_near_rows(g, kind, s));
+    Phase ph(ctx, "near", s);
+    return launch_near_rows_apply(g->npairs.ptr, g->ntbeg.ptr, g->nnear_tgt, g->nrows[kind].ptr, g->nrow_off.ptr,
+                                  g->selfcoef.ptr, dens, g->coef_off_d.ptr, g->pdeg_d.ptr, wts, g->tdrop.ptr,
+                                  g->tgt_loc.ptr, g->val_off_all.ptr, g->ngd.ptr, g->vals.ptr, s);
+  }
   // The check-point values are always summed in FP64: the interpolation through (0, h sqrt(l)),
   // l = 1..8, amplifies their errors by its Lebesgue constant (about 1.9e3 on [0, h]).
   if (prec != BIE_FP64) {

@@ -387,6 +387,250 @@ __global__ void k_near_interp(const NearPair* __restrict__ pairs, const int* __r
   v[2 * ng] += acc[2];
 }
 
+// ---- the near-singular rule as rows of the operator ----
+// The interpolated value of a pair is linear in the source drop's density: with the Lagrange weights b_l
+// at the target's distance, x_l the check points and rho = sum_r c_r Y_r on the grids,
+//     sum_l b_l sum_s K(x_l - x_s) wJ_s rho_s = sum_r [ sum_s (sum_l b_l K(x_l - x_s)) wJ_s Y_r(s) ] c_r,
+// so the sum over the check points is taken once per geometry and kind, and projected on Y_r by the
+// transposed synthesis (phi sums over longitude quadruples, then P~_n^m over latitude pairs).  A row has
+// six symmetric 3x3 planes; for the double layer the jump -4 pi b_0 u(x*) of the exterior limit is part
+// of them.  A seventh plane holds b_0 Y_r(x*), which meets the drop's own on-surface expansion.  Building
+// a row costs about 1.3 evaluations of its check-point sums (31 FP64 operations per check point and source,
+// the projection a quarter of that) and every apply after that reads 7 (p+1)^2 doubles instead.  Two drops of
+// degree 32 at gap 0.05 (U = 4): the near step of an apply 6.1 -> 0.05 ms, a solve with its 15 applies 100 ->
+// 7.2 ms, its first one on a new geometry 27 ms.
+constexpr int kNearThreads = 256;
+
+template <int KIND>
+__global__ void __launch_bounds__(kNearThreads) k_near_rows(const NearPair* __restrict__ pairs,
+                                                            const int* __restrict__ list, int p, int L,
+                                                            const double* __restrict__ pts,
+                                                            const int* __restrict__ grid,
+                                                            const double* __restrict__ centre,
+                                                            const double* __restrict__ hdrop, NearRowsSrc g0,
+                                                            NearRowsSrc g1, const long long* __restrict__ row_off,
+                                                            double* __restrict__ rows) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double bas[17], cx[16][3];
+  __shared__ int any[2], onup[16];
+  const int i = list[blockIdx.x];
+  const NearPair pr = pairs[i];
+  const int j = pr.src_drop, ntri = (p + 1) * (p + 2) / 2, nc = (p + 1) * (p + 1), ncp = self_row(p);
+  const int nkmax = 2 * (g0.P > g1.P ? g0.P : g1.P) + 2;
+  double* sq = reinterpret_cast<double*>(smem_raw);  // [12][ntri]
+  double* sk = sq + 12 * ntri;                       // [2 rows][6][nkmax]
+  double* sd = sk + 12 * nkmax;                      // [even, odd][12][p+1]
+  double* sy = sd + 24 * (p + 1);                    // [ncp] b_0 Y_r(x*)
+  for (int k = threadIdx.x; k < 12 * ntri; k += kNearThreads) sq[k] = 0.0;
+  if (threadIdx.x < 2) any[threadIdx.x] = 0;
+  __syncthreads();
+  if (threadIdx.x <= L) {
+    const int l = threadIdx.x;
+    const double h = hdrop[j], xl = l == 0 ? 0.0 : h * sqrt((double)l);
+    double b = 1.0;
+    for (int k = 0; k <= L; ++k) {
+      if (k == l) continue;
+      const double xk = k == 0 ? 0.0 : h * sqrt((double)k);
+      b *= (pr.d0 - xk) / (xl - xk);
+    }
+    bas[l] = b;
+    if (l > 0) {
+      for (int c = 0; c < 3; ++c) cx[l - 1][c] = pts[3 * ((long long)i * L + l - 1) + c] - centre[3 * j + c];
+      onup[l - 1] = grid[(long long)i * L + l - 1] != 0;
+      any[onup[l - 1]] = 1;
+    }
+  }
+  __syncthreads();
+  for (int gk = 0; gk < 2; ++gk) {
+    if (!any[gk]) continue;
+    const NearRowsSrc& G = gk ? g1 : g0;
+    const int P = G.P, nj = P + 1, nk = 2 * P + 2, half = P + 1, np = (nj + 1) / 2, k4n = half / 2 + 1;
+    const long long s0 = G.off[j], ng = (long long)nj * nk;
+    const double* wJ = G.rec + 7 * s0 + 6 * ng;
+    for (int q = 0; q < np; ++q) {
+      const int nrow = 2 * q == P ? 1 : 2;
+      // combined kernel weights of the rows q and P - q
+      for (int t = threadIdx.x; t < nrow * nk; t += kNearThreads) {
+        const int r = t / nk, k = t - r * nk;
+        const long long o = (long long)(r ? P - q : q) * nk + k, s = s0 + o;
+        const double w = wJ[o], x0 = G.X[s], x1 = G.X[G.ld + s], x2 = G.X[2 * G.ld + s];
+        double n0 = 0, n1 = 0, n2 = 0;
+        if (KIND) {
+          n0 = w * G.N[s];
+          n1 = w * G.N[G.ld + s];
+          n2 = w * G.N[2 * G.ld + s];
+        }
+        double m[6] = {0, 0, 0, 0, 0, 0}, dsum = 0;
+        for (int l = 0; l < L; ++l) {
+          if (onup[l] != gk) continue;
+          const double dx = cx[l][0] - x0, dy = cx[l][1] - x1, dz = cx[l][2] - x2;
+          const double ri = rsqrt_<double>(dx * dx + dy * dy + dz * dz), ri2 = ri * ri;
+          double c;
+          if (KIND == 0) {
+            const double a = bas[l + 1] * w * ri;
+            dsum += a;
+            c = a * ri2;
+          } else {
+            c = (bas[l + 1] * (dx * n0 + dy * n1 + dz * n2)) * (ri2 * ri2 * ri);
+          }
+          const double ax = c * dx, ay = c * dy;
+          m[0] += ax * dx;
+          m[1] += ay * dy;
+          m[2] += (c * dz) * dz;
+          m[3] += ax * dy;
+          m[4] += ax * dz;
+          m[5] += ay * dz;
+        }
+        const double f = KIND ? -6.0 : 1.0;
+#pragma unroll
+        for (int e = 0; e < 6; ++e) sk[(r * 6 + e) * nkmax + k] = f * m[e] + (e < 3 ? dsum : 0.0);
+      }
+      __syncthreads();
+      // fold the longitude quadruples in place: even and odd orders' cosine sums at k and half + k, sine
+      // sums at 2 half - k and half - k (the middle k has two longitudes: one cosine and one sine sum)
+      for (int t = threadIdx.x; t < nrow * 6 * k4n; t += kNearThreads) {
+        const int k = t % k4n;
+        double* v = sk + (t / k4n) * nkmax;
+        const double a = v[k], c = v[half + k];
+        if (k == 0) {
+          v[0] = a + c;
+          v[half] = a - c;
+        } else if (2 * k == half) {
+          v[k] = a + c;
+          v[half + k] = a - c;
+        } else {
+          const double b = v[2 * half - k], d = v[half - k];
+          v[k] = (a + b) + (c + d);
+          v[half + k] = (a + b) - (c + d);
+          v[2 * half - k] = (a - b) + (c - d);
+          v[half - k] = (a - b) - (c - d);
+        }
+      }
+      __syncthreads();
+      // phi transform of both rows, then their sum and difference (even and odd n - m)
+      for (int t = threadIdx.x; t < 6 * (p + 1); t += kNearThreads) {
+        const int m = t % (p + 1), e = t / (p + 1);
+        const double* cm = G.cs + (long long)m * nk * 2;
+        double re[2] = {0, 0}, im[2] = {0, 0};
+        const int mid = half % 2 == 0 ? half / 2 : -1;
+        for (int r = 0; r < nrow; ++r) {
+          const double* v = sk + (r * 6 + e) * nkmax;
+          const double* vc = (m & 1) ? v + half : v;
+          const double* vs = (m & 1) ? v + half : v + 2 * half;
+          double a = vc[0], b = 0;
+          for (int k = 1; 2 * k < half; ++k) {
+            a += vc[k] * cm[2 * k];
+            b += vs[-k] * cm[2 * k + 1];
+          }
+          if (mid > 0) {
+            if (m & 1)
+              b += v[half + mid] * cm[2 * mid + 1];
+            else
+              a += v[mid] * cm[2 * mid];
+          }
+          re[r] = a;
+          im[r] = b;
+        }
+        sd[(2 * e) * (p + 1) + m] = re[0] + re[1];
+        sd[(2 * e + 1) * (p + 1) + m] = im[0] + im[1];
+        sd[(12 + 2 * e) * (p + 1) + m] = re[0] - re[1];
+        sd[(12 + 2 * e + 1) * (p + 1) + m] = im[0] - im[1];
+      }
+      __syncthreads();
+      for (int t = threadIdx.x; t < ntri; t += kNearThreads) {
+        int n = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
+        while ((n + 1) * (n + 2) / 2 <= t) ++n;
+        while (n * (n + 1) / 2 > t) --n;
+        const int m = t - n * (n + 1) / 2;
+        const double Pv = G.T0[leg_row(p, m, n, nj) + q];
+        const double* d = sd + (((n - m) & 1) ? 12 : 0) * (p + 1) + m;
+#pragma unroll
+        for (int e = 0; e < 12; ++e) sq[e * ntri + t] += d[e * (p + 1)] * Pv;
+      }
+      __syncthreads();
+    }
+  }
+  // b_0 Y_r(x*), one thread per order
+  {
+    double st, ct;
+    sincos(pr.theta_v, &st, &ct);
+    for (int m = threadIdx.x; m <= p; m += kNearThreads) {
+      double dm = sqrt(1.0 / (4.0 * kPiD));
+      for (int k = 0; k < m; ++k) dm *= -sqrt(1.0 + 1.0 / (2.0 * (k + 1))) * st;
+      double sm, cm, pm1 = 0, pm2 = 0;
+      sincos(m * pr.phi_v, &sm, &cm);
+      const double fac = (m == 0 ? 1.0 : 2.0) * bas[0];
+      for (int n = m; n <= p; ++n) {
+        const double v = n == m ? dm : n == m + 1 ? sqrt(2.0 * m + 3.0) * ct * dm : rec_a(n, m) * (ct * pm1 - rec_b(n, m) * pm2);
+        pm2 = pm1;
+        pm1 = v;
+        sy[n * (n + 1) + m] = fac * v * cm;
+        if (m > 0) sy[n * (n + 1) - m] = -fac * v * sm;
+      }
+    }
+    for (int r = nc + threadIdx.x; r < ncp; r += kNearThreads) sy[r] = 0.0;
+  }
+  __syncthreads();
+  double* out = rows + row_off[i];
+  for (int t = threadIdx.x; t < 7 * ncp; t += kNearThreads) {
+    const int e = t / ncp, r = t - e * ncp;
+    double v = e == 6 ? sy[r] : 0.0;
+    if (e < 6 && r < nc) {
+      const int n = degree_of(r), m = r - n * (n + 1), it = n * (n + 1) / 2 + (m < 0 ? -m : m);
+      v = m == 0 ? sq[2 * e * ntri + it] : m > 0 ? 2.0 * sq[2 * e * ntri + it] : -2.0 * sq[(2 * e + 1) * ntri + it];
+      if (KIND && e < 3) v -= 4.0 * kPiD * sy[r];
+    }
+    out[t] = v;
+  }
+}
+
+// vals += the near values of one target from its pairs' rows: one warp per target, its pairs in order.
+__global__ void __launch_bounds__(128) k_near_rows_apply(const NearPair* __restrict__ pairs,
+                                                         const int* __restrict__ tbeg, int ntgt,
+                                                         const double* __restrict__ rows,
+                                                         const long long* __restrict__ row_off,
+                                                         const double* __restrict__ selfcoef,
+                                                         const double* __restrict__ dens,
+                                                         const long long* __restrict__ coef_off,
+                                                         const int* __restrict__ pdeg, const double* __restrict__ wts,
+                                                         const int* __restrict__ tdrop,
+                                                         const long long* __restrict__ tgt_loc,
+                                                         const long long* __restrict__ val_off,
+                                                         const int* __restrict__ ngd, double* __restrict__ vals) {
+  const int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (u >= ntgt) return;
+  double acc[3] = {0, 0, 0};
+  for (int i = tbeg[u]; i < tbeg[u + 1]; ++i) {
+    const int j = pairs[i].src_drop, p = pdeg[j], nc = (p + 1) * (p + 1), ncp = self_row(p);
+    const double* M = rows + row_off[i];
+    const double *d = dens + coef_off[j], *sc = selfcoef + coef_off[j];
+    double a[3] = {0, 0, 0};
+#pragma unroll 2
+    for (int r = lane; r < nc; r += 32) {
+      const double x = d[r], y = d[nc + r], z = d[2 * nc + r], Y = M[6 * ncp + r];
+      const double m0 = M[r], m1 = M[ncp + r], m2 = M[2 * ncp + r], m3 = M[3 * ncp + r], m4 = M[4 * ncp + r],
+                   m5 = M[5 * ncp + r];
+      a[0] += m0 * x + m3 * y + m4 * z;
+      a[1] += m3 * x + m1 * y + m5 * z;
+      a[2] += m4 * x + m5 * y + m2 * z;
+      acc[0] += Y * sc[r];
+      acc[1] += Y * sc[nc + r];
+      acc[2] += Y * sc[2 * nc + r];
+    }
+    for (int c = 0; c < 3; ++c) acc[c] += wts[j] * a[c];
+  }
+  for (int c = 0; c < 3; ++c)
+    for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_down_sync(0xffffffffu, acc[c], o);
+  if (lane) return;
+  const long long t = pairs[tbeg[u]].target;
+  const int d = tdrop[t];
+  const long long ng = ngd[d];
+  double* v = vals + val_off[d] + tgt_loc[t];
+  v[0] += acc[0];
+  v[ng] += acc[1];
+  v[2 * ng] += acc[2];
+}
+
 // The source drop's shape coefficients of pair i with the phases of its seed longitude applied,
 // g_n^m = e^{i m alpha_i} x_n^m (real-packed; alpha_i = pi lon[i] / (p+1), lon the seed's longitude index),
 // written to out + dst_off[i] as [3][(p+1)^2]: the first step of the rotation R_z(alpha) R_y(beta), so
@@ -427,6 +671,35 @@ int launch_near_phase_shift(const NearPair* pairs, int npair, const double* coef
                             cudaStream_t s) {
   if (!npair) return BIE_OK;
   k_near_phase_shift<<<npair, 128, 0, s>>>(pairs, npair, coef, coef_off, pdeg, lon, dst_off, out);
+  count_launch();
+  BIE_CUDA_TRY(cudaGetLastError());
+  return BIE_OK;
+}
+
+size_t near_rows_smem(int p, int P) {
+  return sizeof(double) * (6 * (size_t)(p + 1) * (p + 2) + 12 * (size_t)(2 * P + 2) + 24 * (size_t)(p + 1) + self_row(p));
+}
+
+int launch_near_rows(int kind, const NearPair* pairs, const int* list, int n, int p, int L, const double* pts,
+                     const int* grid, const double* centre, const double* hdrop, const NearRowsSrc& std_,
+                     const NearRowsSrc& up, const long long* row_off, double* rows, cudaStream_t s) {
+  if (!n) return BIE_OK;
+  const size_t smem = near_rows_smem(p, std_.P > up.P ? std_.P : up.P);
+  auto kern = kind == 0 ? k_near_rows<0> : k_near_rows<1>;
+  if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  kern<<<n, kNearThreads, smem, s>>>(pairs, list, p, L, pts, grid, centre, hdrop, std_, up, row_off, rows);
+  count_launch();
+  BIE_CUDA_TRY(cudaGetLastError());
+  return BIE_OK;
+}
+
+int launch_near_rows_apply(const NearPair* pairs, const int* tbeg, int ntgt, const double* rows, const long long* row_off,
+                           const double* selfcoef, const double* dens, const long long* coef_off, const int* pdeg,
+                           const double* wts, const int* tdrop, const long long* tgt_loc, const long long* val_off,
+                           const int* ngd, double* vals, cudaStream_t s) {
+  if (!ntgt) return BIE_OK;
+  k_near_rows_apply<<<(ntgt + 3) / 4, 128, 0, s>>>(pairs, tbeg, ntgt, rows, row_off, selfcoef, dens, coef_off, pdeg, wts,
+                                                   tdrop, tgt_loc, val_off, ngd, vals);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;

@@ -40,4 +40,28 @@ int launch_near_interp(const NearPair* pairs, const int* tbeg, int ntgt, int L, 
                        const double* wts, const double* cv, const int* tdrop, const long long* tgt_loc,
                        const long long* val_off, const int* ngd, double* vals, cudaStream_t s);
 
+// One grid (standard or upsampled) of the drops of one degree p, as the rows read it.
+struct NearRowsSrc {
+  int P;
+  const double* T0;  // Legendre table of (p, P)
+  const double* cs;  // its phases
+  const double* X;   // sources relative to their drop's centre, normals: [3][ld]
+  const double* N;
+  long long ld;
+  const double* rec;     // records, weights in row 6
+  const long long* off;  // first source, by drop
+};
+// The near-singular rule of the n pairs list[] (source drops of degree p) as rows of the operator (near.cu):
+// 7 planes of self_row(p) doubles at rows + row_off[pair].  near_rows_smem: the block's shared memory, with P
+// the larger of the two grids' degrees.
+size_t near_rows_smem(int p, int P);
+int launch_near_rows(int kind, const NearPair* pairs, const int* list, int n, int p, int L, const double* pts,
+                     const int* grid, const double* centre, const double* hdrop, const NearRowsSrc& std_,
+                     const NearRowsSrc& up, const long long* row_off, double* rows, cudaStream_t s);
+// vals += the near values of the ntgt targets from their pairs' rows
+int launch_near_rows_apply(const NearPair* pairs, const int* tbeg, int ntgt, const double* rows, const long long* row_off,
+                           const double* selfcoef, const double* dens, const long long* coef_off, const int* pdeg,
+                           const double* wts, const int* tdrop, const long long* tgt_loc, const long long* val_off,
+                           const int* ngd, double* vals, cudaStream_t s);
+
 }  // namespace bie
