@@ -46,7 +46,8 @@ __global__ void k_surface(const double* __restrict__ X, const double* __restrict
   r[6 * N + q] = wsin[j] * W;
 }
 
-// cache[t][0..2] = x0 - x', [3..5] = n', [6] = w^s_j W'/sin(theta_j), on the degree-pq grid.
+// cache[t][0..2] = x0 - x', [3..5] = w n', [6] = w = w^s_j W'/sin(theta_j), on the degree-pq grid (the layer
+// kernels need the normal only with its weight, so it is never divided by W').
 template <typename R>
 __global__ void k_rotgeo(const double* __restrict__ X, const double* __restrict__ Xt, const double* __restrict__ Xp,
                          long long ndrop, int ng, int pq, const double* __restrict__ rec_std,
@@ -68,14 +69,14 @@ __global__ void k_rotgeo(const double* __restrict__ X, const double* __restrict_
     xp[i] = Xp[(t * 3 + i) * nq + q];
   }
   cross3(xt, xp, c);
-  double W = sqrt(c[0] * c[0] + c[1] * c[1] + c[2] * c[2]);
+  const double W2 = c[0] * c[0] + c[1] * c[1] + c[2] * c[2], ws = wsq[j];
   R* o = cache + t * 7 * nq;
   for (int i = 0; i < 3; ++i) {
     double x0 = rec_std[rec_off[ld] + (long long)i * ng + tl];
     o[i * nq + q] = (R)(x0 - x[i]);
-    o[(3 + i) * nq + q] = (R)(c[i] / W);
+    o[(3 + i) * nq + q] = (R)(ws * c[i]);
   }
-  o[6 * nq + q] = (R)(wsq[j] * W);
+  o[6 * nq + q] = (R)(ws * (W2 * rsqrt_<double>(W2)));
 }
 
 // Interfacial force f = -2 sigma K n - grad_gamma sigma at the grid points of nd drops (Sec. 1, Table 2),

@@ -185,19 +185,18 @@ __global__ void __launch_bounds__(256) k_self_direct(
         const R r1 = side ? e1 - o1 : e1 + o1;
         const R r2 = side ? e2 - o2 : e2 + o2;
         const R x0 = geo[q], x1 = geo[nq + q], x2 = geo[2 * nq + q];
-        const R w = geo[6 * nq + q];
         const R ri = rsqrt_<R>(x0 * x0 + x1 * x1 + x2 * x2);
         const R xr = x0 * r0 + x1 * r1 + x2 * r2;
         if (KIND == 0) {
-          const R wi = w * ri;
+          const R wi = geo[6 * nq + q] * ri;
           const R c = wi * xr * ri * ri;
           s0 += wi * r0 + c * x0;
           s1 += wi * r1 + c * x1;
           s2 += wi * r2 + c * x2;
         } else {
-          const R xn = x0 * geo[3 * nq + q] + x1 * geo[4 * nq + q] + x2 * geo[5 * nq + q];
+          const R xn = x0 * geo[3 * nq + q] + x1 * geo[4 * nq + q] + x2 * geo[5 * nq + q];  // with the weight
           const R ri2 = ri * ri;
-          const R c = (R)(-6) * w * xr * xn * ri2 * ri2 * ri;
+          const R c = (R)(-6) * xr * xn * ri2 * ri2 * ri;
           s0 += c * x0;
           s1 += c * x1;
           s2 += c * x2;
@@ -213,12 +212,15 @@ __global__ void __launch_bounds__(256) k_self_direct(
 // For each target, Q[t][e][ri][tri(n,m)] = c_m sum_j Mhat_{e,jm} P~_n^m(cos theta_j), with
 // Mhat_{e,jm} = sum_k M_{e,jk} e^{i m phi_k} the phi transform of entry e of the 3x3 kernel weight
 // over (xx, yy, zz, xy, xz, yz), ri = real / imaginary part, c_0 = 1 and c_m = 2.  Latitudes are
-// processed kDftJ at a time: kernel weights, their phi transform, then the Legendre projection,
-// accumulated in shared memory.
-constexpr int kDftJ = 3;
+// processed kProjPairs pairs (q, pq - q) at a time: kernel weights; their sums over the longitude
+// quadruples that share |cos m phi| and |sin m phi|, in place; the phi transform of both rows, whose sum
+// and difference serve even and odd n - m; and the Legendre projection, accumulated in shared memory.
+// Bound by the FP64 pipe: at p = pq = 24 about 0.21M operations per target and kind against 0.36M
+// without the symmetries and with the IEEE quotient and root for 1/r: 64 drops, both kinds 127 -> 64 ms.
+constexpr int kProjPairs = 2;
 
 __device__ inline int tri_index_degree(int it) {
-  int n = (int)((sqrt(8.0 * it + 1.0) - 1.0) * 0.5);
+  int n = (int)((sqrtf(8.0f * it + 1.0f) - 1.0f) * 0.5f);
   while ((n + 1) * (n + 2) / 2 <= it) ++n;
   while (n * (n + 1) / 2 > it) --n;
   return n;
@@ -230,73 +232,108 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
                                                      double* __restrict__ Q64) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const long long t = blockIdx.x;
-  const int nq_j = pq + 1, nk = 2 * pq + 2, half = pq + 1;
+  const int nq_j = pq + 1, nk = 2 * pq + 2, half = pq + 1, np = (nq_j + 1) / 2, k4n = half / 2 + 1;
   const int ntri = (p + 1) * (p + 2) / 2;
-  double* sg = reinterpret_cast<double*>(smem_raw);  // [jj][e][even/odd][k < half]
-  double* sm = sg + kDftJ * 12 * half;               // [jj][12][m]
-  double* sq = sm + kDftJ * 12 * (p + 1);            // [12][tri]
+  const int mid = half % 2 == 0 ? half / 2 : -1;
+  double* sk = reinterpret_cast<double*>(smem_raw);  // [pair][row][6][nk]
+  double* sd = sk + kProjPairs * 12 * nk;            // [pair][even, odd][12][p+1]
+  double* sq = sd + kProjPairs * 24 * (p + 1);       // [12][ntri]
   const long long nq = (long long)nq_j * nk;
   const double* geo = cache + t * 7 * nq;
   for (int i = threadIdx.x; i < 12 * ntri; i += blockDim.x) sq[i] = 0.0;
-  for (int j0 = 0; j0 < nq_j; j0 += kDftJ) {
-    const int jn = min(kDftJ, nq_j - j0);
-    for (int i = threadIdx.x; i < jn * half; i += blockDim.x) {
-      const int jj = i / half, k = i - jj * half;
-      double Mv[2][6];
+  for (int q0 = 0; q0 < np; q0 += kProjPairs) {
+    const int qn = min(kProjPairs, np - q0);
+    for (int i = threadIdx.x; i < qn * 2 * nk; i += blockDim.x) {
+      const int row = i / nk, k = i - row * nk;
+      const int q = q0 + row / 2, j = row & 1 ? pq - q : q;
+      double* v = sk + row * 6 * nk + k;
+      if ((row & 1) && 2 * q == pq) {  // the middle latitude has no mirror
 #pragma unroll
-      for (int side = 0; side < 2; ++side) {
-        const long long q = (long long)(j0 + jj) * nk + k + side * half;
-        const double x0 = geo[q], x1 = geo[nq + q], x2 = geo[2 * nq + q], w = geo[6 * nq + q];
-        const double ri = 1.0 / sqrt(x0 * x0 + x1 * x1 + x2 * x2);
-        double d, c;
-        if (KIND == 0) {
-          d = w * ri;
-          c = w * ri * ri * ri;
-        } else {
-          const double xn = x0 * geo[3 * nq + q] + x1 * geo[4 * nq + q] + x2 * geo[5 * nq + q];
-          const double ri2 = ri * ri;
-          d = 0.0;
-          c = -6.0 * w * xn * ri2 * ri2 * ri;
-        }
-        Mv[side][0] = d + c * x0 * x0;
-        Mv[side][1] = d + c * x1 * x1;
-        Mv[side][2] = d + c * x2 * x2;
-        Mv[side][3] = c * x0 * x1;
-        Mv[side][4] = c * x0 * x2;
-        Mv[side][5] = c * x1 * x2;
+        for (int e = 0; e < 6; ++e) v[e * nk] = 0.0;
+        continue;
       }
-#pragma unroll
-      for (int e = 0; e < 6; ++e) {
-        sg[((jj * 6 + e) * 2 + 0) * half + k] = Mv[0][e] + Mv[1][e];  // even orders
-        sg[((jj * 6 + e) * 2 + 1) * half + k] = Mv[0][e] - Mv[1][e];  // odd orders
+      const long long o = (long long)j * nk + k;
+      const double x0 = geo[o], x1 = geo[nq + o], x2 = geo[2 * nq + o];
+      const double ri = rsqrt_<double>(x0 * x0 + x1 * x1 + x2 * x2), ri2 = ri * ri;
+      double d = 0.0, c;
+      if (KIND == 0) {
+        d = geo[6 * nq + o] * ri;
+        c = d * ri2;
+      } else {
+        c = (-6.0 * (x0 * geo[3 * nq + o] + x1 * geo[4 * nq + o] + x2 * geo[5 * nq + o])) * (ri2 * ri2 * ri);
+      }
+      const double a0 = c * x0, a1 = c * x1;
+      v[0] = d + a0 * x0;
+      v[nk] = d + a1 * x1;
+      v[2 * nk] = d + (c * x2) * x2;
+      v[3 * nk] = a0 * x1;
+      v[4 * nk] = a0 * x2;
+      v[5 * nk] = a1 * x2;
+    }
+    __syncthreads();
+    // cosine sums of the even and odd orders at k and half + k, sine sums at 2 half - k and half - k (a middle
+    // k has two longitudes: one cosine sum at k, one sine sum at half + k)
+    for (int i = threadIdx.x; i < qn * 12 * k4n; i += blockDim.x) {
+      const int k = i % k4n;
+      double* v = sk + (i / k4n) * nk;
+      const double a = v[k], c = v[half + k];
+      if (k == 0 || k == mid) {
+        v[k] = a + c;
+        v[half + k] = a - c;
+      } else {
+        const double b = v[2 * half - k], d = v[half - k];
+        const double ab = a + b, cd = c + d, amb = a - b, cmd = c - d;
+        v[k] = ab + cd;
+        v[half + k] = ab - cd;
+        v[2 * half - k] = amb + cmd;
+        v[half - k] = amb - cmd;
       }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < jn * 6 * (p + 1); i += blockDim.x) {
+    for (int i = threadIdx.x; i < qn * 6 * (p + 1); i += blockDim.x) {
       const int m = i % (p + 1);
       const int r = i / (p + 1);
-      const int e = r % 6, jj = r / 6;
-      const double* src = sg + ((jj * 6 + e) * 2 + (m & 1)) * half;
-      double re = 0, im = 0;
-      for (int k = 0; k < half; ++k) {
-        re += src[k] * cs[((long long)m * nk + k) * 2];
-        im += src[k] * cs[((long long)m * nk + k) * 2 + 1];
+      const int e = r % 6, pair = r / 6;
+      const double* cm = cs + (long long)m * nk * 2;
+      const double* v0 = sk + (pair * 12 + e) * nk;  // row q; row pq - q is 6 nk further
+      const double* vc = v0 + ((m & 1) ? half : 0);
+      const double* vs = v0 + ((m & 1) ? half : 2 * half);
+      double re0 = vc[0], re1 = vc[6 * nk], im0 = 0, im1 = 0;
+      for (int k = 1; 2 * k < half; ++k) {
+        const double co = cm[2 * k], si = cm[2 * k + 1];
+        re0 += vc[k] * co;
+        re1 += vc[6 * nk + k] * co;
+        im0 += vs[-k] * si;
+        im1 += vs[6 * nk - k] * si;
       }
-      sm[(jj * 12 + 2 * e) * (p + 1) + m] = re;
-      sm[(jj * 12 + 2 * e + 1) * (p + 1) + m] = im;
+      if (mid > 0) {
+        if (m & 1) {
+          im0 += v0[half + mid] * cm[2 * mid + 1];
+          im1 += v0[6 * nk + half + mid] * cm[2 * mid + 1];
+        } else {
+          re0 += v0[mid] * cm[2 * mid];
+          re1 += v0[6 * nk + mid] * cm[2 * mid];
+        }
+      }
+      double* d = sd + (pair * 24 + 2 * e) * (p + 1) + m;
+      d[0] = re0 + re1;
+      d[p + 1] = im0 + im1;
+      d[12 * (p + 1)] = re0 - re1;
+      d[13 * (p + 1)] = im0 - im1;
     }
     __syncthreads();
     for (int it = threadIdx.x; it < ntri; it += blockDim.x) {
       const int n = tri_index_degree(it);
       const int m = it - n * (n + 1) / 2;
-      const double* Tn = T0 + leg_row(p, m, n, nq_j) + j0;
+      const double* Tn = T0 + leg_row(p, m, n, nq_j) + q0;
       double acc[12];
 #pragma unroll
       for (int e = 0; e < 12; ++e) acc[e] = sq[e * ntri + it];
-      for (int jj = 0; jj < jn; ++jj) {
-        const double P = Tn[jj];
+      for (int pair = 0; pair < qn; ++pair) {
+        const double P = Tn[pair];
+        const double* d = sd + (pair * 24 + (((n - m) & 1) ? 12 : 0)) * (p + 1) + m;
 #pragma unroll
-        for (int e = 0; e < 12; ++e) acc[e] += sm[(jj * 12 + e) * (p + 1) + m] * P;
+        for (int e = 0; e < 12; ++e) acc[e] += d[e * (p + 1)] * P;
       }
 #pragma unroll
       for (int e = 0; e < 12; ++e) sq[e * ntri + it] = acc[e];
@@ -305,9 +342,9 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
   }
   double* o64 = Q64 + t * 12 * ntri;
   for (int i = threadIdx.x; i < 12 * ntri; i += blockDim.x) {
-    const int m = i % ntri;
-    const int n = tri_index_degree(m);
-    o64[i] = (m == n * (n + 1) / 2 ? 1.0 : 2.0) * sq[i];  // c_m
+    const int it = i % ntri;
+    const int n = tri_index_degree(it);
+    o64[i] = (it == n * (n + 1) / 2 ? 1.0 : 2.0) * sq[i];  // c_m
   }
 }
 
@@ -534,7 +571,7 @@ int launch_self_direct(int kind, const double* dens, const long long* foff3, lon
 }
 
 size_t kernel_proj_smem(int p, int pq) {
-  return sizeof(double) * ((size_t)kDftJ * 12 * (pq + 1) + (size_t)kDftJ * 12 * (p + 1) + 6 * (size_t)(p + 1) * (p + 2));
+  return sizeof(double) * ((size_t)kProjPairs * 24 * (pq + 1) + (size_t)kProjPairs * 24 * (p + 1) + 6 * (size_t)(p + 1) * (p + 2));
 }
 
 int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, int pq, const double* cs,
