@@ -429,176 +429,184 @@ __global__ void __launch_bounds__(kTile / TPT) k_interdrop_x2(
 }
 
 // ---- double-float pair sums ----
-// A double-float value is an unevaluated sum hi + lo of two FP32 numbers (about 44 significant
-// bits).  Sums use Knuth's TwoSum and products the FMA-based TwoProduct (both error-free
-// transformations).  Results are left unnormalised (|lo| may exceed ulp(hi)/2 by a few units, which
-// costs no accuracy in the short chains of one pair); the per-target accumulators are renormalised
-// by Dekker's Fast2Sum after every staged chunk of sources.  1/sqrt starts from the FP32 estimate and
-// takes one Newton step in double-float.  Every operation runs on the FP32 pipes.
+// A double-float value is an unevaluated sum h + l of two FP32 numbers (about 44 significant bits).
+// Every operation runs on the FP32 pipe, packed for two targets at a time (fma/mul/add/sub.rn.f32x2): the
+// kernel is bound by that pipe's operations, and the packed form leaves half of the issue slots for the
+// shared-memory loads and the rest.  Sums use Knuth's TwoSum, products the FMA-based TwoProduct; results are
+// left unnormalised (l may exceed ulp(h)/2 by a few units, which costs no accuracy in the short chains of
+// one pair) and the per-target sums are renormalised after every staged chunk.  1/r^3 and 1/r^5 come from
+// the estimate y of 1/r directly: with e = 1 - r^2 y^2 (about 2^-22),
+// r^-k = y^k (1 - e)^(-k/2) = y^k (1 + (k/2) e + (k/2)(k/2 + 1)/2 e^2 + O(e^3)).
+// About 170 operations per pair; scalar, the kernel reached 67% of the pipe at 75% of the issue slots.  80
+// drops of degree 24 (1.0e10 pairs): 90.4 -> 68.7 ms.  Rounding the high parts of positions to a common grid,
+// so that their difference is exact in one operation, saved another tenth but lost accuracy where the
+// points of a tile lie at very different distances (4e-11 of the field instead of 1e-11), and was left out.
+struct d2 {
+  fx2 h, l;
+};
 struct df2 {
   float h, l;
 };
 
+__device__ __forceinline__ fx2 x2_add(fx2 a, fx2 b) {
+  fx2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ fx2 x2_neg(fx2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ fx2 x2_both(float v) { return x2_pack(v, v); }
 __device__ inline df2 df_from(double x) {
   const float h = (float)x;
   return {h, (float)(x - (double)h)};
 }
-__device__ inline df2 fast2sum(float a, float b) {  // |a| >= |b|
-  const float s = a + b;
-  return {s, b - (s - a)};
+__device__ __forceinline__ d2 d2_add(d2 a, d2 b) {
+  const fx2 s = x2_add(a.h, b.h), v = x2_sub(s, a.h);
+  return {s, x2_add(x2_add(x2_add(x2_sub(a.h, x2_sub(s, v)), x2_sub(b.h, v)), a.l), b.l)};
 }
-__device__ inline df2 df_add(df2 a, df2 b) {
-  const float s = a.h + b.h;
-  const float v = s - a.h;
-  return {s, (a.h - (s - v)) + (b.h - v) + a.l + b.l};
+__device__ __forceinline__ d2 d2_sub(d2 a, d2 b) {
+  const fx2 s = x2_sub(a.h, b.h), v = x2_sub(s, a.h);
+  return {s, x2_sub(x2_add(x2_sub(x2_sub(a.h, x2_sub(s, v)), x2_add(b.h, v)), a.l), b.l)};
 }
-__device__ inline df2 df_renorm(df2 a) {  // TwoSum of the two parts
-  const float s = a.h + a.l;
-  const float v = s - a.h;
-  return {s, (a.h - (s - v)) + (a.l - v)};
+__device__ __forceinline__ d2 d2_renorm(d2 a) {
+  const fx2 s = x2_add(a.h, a.l), v = x2_sub(s, a.h);
+  return {s, x2_add(x2_sub(a.h, x2_sub(s, v)), x2_sub(a.l, v))};
 }
-__device__ inline df2 df_neg(df2 a) { return {-a.h, -a.l}; }
-__device__ inline df2 df_mul(df2 a, df2 b) {
-  const float p = a.h * b.h;
-  float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, e);
-  e = fmaf(a.l, b.h, e);
-  return {p, e};
+__device__ __forceinline__ d2 d2_mul(d2 a, d2 b) {
+  const fx2 p = x2_mul(a.h, b.h);
+  return {p, x2_fma(a.l, b.h, x2_fma(a.h, b.l, x2_fma(a.h, b.h, x2_neg(p))))};
 }
-__device__ inline df2 df_sqr(df2 a) {
-  const float p = a.h * a.h;
-  float e = fmaf(a.h, a.h, -p);
-  e = fmaf(2.0f * a.h, a.l, e);
-  return {p, e};
+__device__ __forceinline__ d2 d2_sqr(d2 a) {
+  const fx2 p = x2_mul(a.h, a.h);
+  return {p, x2_fma(x2_add(a.h, a.h), a.l, x2_fma(a.h, a.h, x2_neg(p)))};
 }
-__device__ inline df2 df_rsqrt(df2 a) {
-  const float y = rsqrtf(a.h);
-  const float y2 = y * y;
-  const df2 ay2 = df_mul(a, {y2, fmaf(y, y, -y2)});
-  const float e = (1.0f - ay2.h) - ay2.l;  // 1 - a y^2, of the order of the estimate's error
-  return fast2sum(y, 0.5f * y * e);
+// a b for b without a low part
+__device__ __forceinline__ d2 d2_mul1(d2 a, fx2 b) {
+  const fx2 p = x2_mul(a.h, b);
+  return {p, x2_fma(a.l, b, x2_fma(a.h, b, x2_neg(p)))};
 }
 
-// Same work list and layout as k_interdrop; sources are read in FP64 and split into double-float
-// pairs as they are staged through shared memory, targets are split once per item.
-template <int KIND, int TPT>
-__global__ void __launch_bounds__(kTile / TPT) k_interdrop_df(
+// Same work list and result as k_interdrop; the sources are read in FP64 and split as they are staged, each
+// part duplicated in both lanes; the thread's targets tid and tid + 64 share the lanes.
+template <int KIND>
+__global__ void __launch_bounds__(kTile / 2) k_interdrop_df(
     const PairItem* __restrict__ items, const int* __restrict__ blk_item, const long long* __restrict__ tile_t0,
     const int* __restrict__ tile_n, const int* __restrict__ tile_drop, const long long* __restrict__ tgt_loc,
     const long long* __restrict__ toff_std, const int* __restrict__ ngd, const double* __restrict__ rec_std,
     const double* __restrict__ centre, const double* __restrict__ Xs, const double* __restrict__ Ns,
     const double* __restrict__ Qs, long long nstd, const double* __restrict__ Xu, const double* __restrict__ Nu,
     const double* __restrict__ Qu, long long nup, const double* __restrict__ wts, double* __restrict__ partial) {
-  constexpr int NT = kTile / TPT;
+  constexpr int NT = kTile / 2;
   constexpr int NV = KIND ? 9 : 6;  // staged values per source: x, q (and n)
-  __shared__ df2 sv[NV][kChunk];
+  __shared__ __align__(16) d2 sv[NV][kChunk];
   const int b = blockIdx.x;
   const int it0 = blk_item[b], it1 = blk_item[b + 1];
   const int tile = items[it0].tile;
   const int tid = threadIdx.x;
   const int nt = tile_n[tile];
   const int di = tile_drop[tile];
-  double tx[TPT], ty[TPT], tz[TPT], acc[TPT][3];
+  double tx[2][3], acc[2][3];
 #pragma unroll
-  for (int u = 0; u < TPT; ++u) {
+  for (int u = 0; u < 2; ++u) {
     const int k = tid + u * NT;
-    tx[u] = ty[u] = tz[u] = 0;
-    acc[u][0] = acc[u][1] = acc[u][2] = 0;
-    if (k < nt) {
-      const long long t = tile_t0[tile] + k;
-      const long long ng = ngd[di];
-      const double* ri = rec_std + 7 * toff_std[di];
-      const long long l = tgt_loc[t];
-      tx[u] = ri[l];
-      ty[u] = ri[ng + l];
-      tz[u] = ri[2 * ng + l];
+    const long long ng = ngd[di];
+    const double* ri = rec_std + 7 * toff_std[di] + tgt_loc[tile_t0[tile] + (k < nt ? k : 0)];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      tx[u][c] = ri[c * ng];
+      acc[u][c] = 0;
     }
   }
   for (int it = it0; it < it1; ++it) {
     const PairItem item = items[it];
     const int j = item.src_drop;
-    bool act[TPT], any = false;
-    df2 px[TPT], py[TPT], pz[TPT];
+    bool act[2];
 #pragma unroll
-    for (int u = 0; u < TPT; ++u) {
+    for (int u = 0; u < 2; ++u) {
       const int k = tid + u * NT;
       act[u] = k < nt && ((item.mask[k >> 5] >> (k & 31)) & 1u);
-      any = any || act[u];
-      px[u] = df_from(tx[u] - centre[3 * j]);
-      py[u] = df_from(ty[u] - centre[3 * j + 1]);
-      pz[u] = df_from(tz[u] - centre[3 * j + 2]);
+    }
+    d2 px[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const df2 a = df_from(tx[0][c] - centre[3 * j + c]), e = df_from(tx[1][c] - centre[3 * j + c]);
+      px[c] = {x2_pack(a.h, e.h), x2_pack(a.l, e.l)};
     }
     const double* X = item.grid ? Xu : Xs;
     const double* N = item.grid ? Nu : Ns;
     const double* Q = item.grid ? Qu : Qs;
     const long long ld = item.grid ? nup : nstd;
-    df2 s[TPT][3];
+    d2 s[3];
 #pragma unroll
-    for (int u = 0; u < TPT; ++u) s[u][0] = s[u][1] = s[u][2] = {0.0f, 0.0f};
+    for (int c = 0; c < 3; ++c) s[c] = {0ull, 0ull};
     for (long long c0 = item.s0; c0 < item.s1; c0 += kChunk) {
       const int cn = (int)min((long long)kChunk, item.s1 - c0);
       for (int k = tid; k < cn; k += NT) {
         const long long sidx = c0 + k;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          sv[c][k] = df_from(X[c * ld + sidx]);
-          sv[3 + c][k] = df_from(Q[c * ld + sidx]);
-          if (KIND) sv[6 + c][k] = df_from(N[c * ld + sidx]);
+          const df2 x = df_from(X[c * ld + sidx]), q = df_from(Q[c * ld + sidx]);
+          sv[c][k] = {x2_both(x.h), x2_both(x.l)};
+          sv[3 + c][k] = {x2_both(q.h), x2_both(q.l)};
+          if (KIND) {
+            const df2 n = df_from(N[c * ld + sidx]);
+            sv[6 + c][k] = {x2_both(n.h), x2_both(n.l)};
+          }
         }
       }
       __syncthreads();
-      if (any) {
+      if (act[0] || act[1]) {
         for (int k = 0; k < cn; ++k) {
-          const df2 xs_ = sv[0][k], ys_ = sv[1][k], zs_ = sv[2][k];
-          const df2 q0 = sv[3][k], q1 = sv[4][k], q2 = sv[5][k];
+          d2 dx[3];
 #pragma unroll
-          for (int u = 0; u < TPT; ++u) {
-            const df2 dx = df_add(px[u], df_neg(xs_)), dy = df_add(py[u], df_neg(ys_)),
-                      dz = df_add(pz[u], df_neg(zs_));
-            const df2 r2 = df_add(df_add(df_sqr(dx), df_sqr(dy)), df_sqr(dz));
-            const df2 ri = df_rsqrt(r2);
-            const df2 xq = df_add(df_add(df_mul(dx, q0), df_mul(dy, q1)), df_mul(dz, q2));
-            if (KIND == 0) {  // Stokeslet
-              const df2 ri3 = df_mul(df_sqr(ri), ri);
-              const df2 c = df_mul(xq, ri3);
-              s[u][0] = df_add(s[u][0], df_add(df_mul(q0, ri), df_mul(c, dx)));
-              s[u][1] = df_add(s[u][1], df_add(df_mul(q1, ri), df_mul(c, dy)));
-              s[u][2] = df_add(s[u][2], df_add(df_mul(q2, ri), df_mul(c, dz)));
-            } else {  // stresslet
-              const df2 n0 = sv[6][k], n1 = sv[7][k], n2 = sv[8][k];
-              const df2 xn = df_add(df_add(df_mul(dx, n0), df_mul(dy, n1)), df_mul(dz, n2));
-              const df2 ri2 = df_sqr(ri);
-              const df2 ri5 = df_mul(df_sqr(ri2), ri);
-              const df2 c = df_mul(df_mul(xq, xn), ri5);  // the factor -6 goes with the weight
-              s[u][0] = df_add(s[u][0], df_mul(c, dx));
-              s[u][1] = df_add(s[u][1], df_mul(c, dy));
-              s[u][2] = df_add(s[u][2], df_mul(c, dz));
-            }
+          for (int c = 0; c < 3; ++c) dx[c] = d2_sub(px[c], sv[c][k]);
+          const d2 r2 = d2_add(d2_add(d2_sqr(dx[0]), d2_sqr(dx[1])), d2_sqr(dx[2]));
+          const fx2 y = x2_rsqrt(r2.h);
+          const fx2 yy = x2_mul(y, y);
+          const d2 y2 = {yy, x2_fma(y, y, x2_neg(yy))};
+          const d2 ay2 = d2_mul(r2, y2);
+          const fx2 e = x2_sub(x2_sub(x2_both(1.0f), ay2.h), ay2.l);
+          const d2 q0 = sv[3][k], q1 = sv[4][k], q2 = sv[5][k];
+          const d2 xq = d2_add(d2_add(d2_mul(dx[0], q0), d2_mul(dx[1], q1)), d2_mul(dx[2], q2));
+          if (KIND == 0) {  // Stokeslet: q/r + (xh.q) xh/r^3
+            const fx2 t1 = x2_mul(e, x2_fma(x2_both(0.375f), e, x2_both(0.5f)));
+            const fx2 t3 = x2_mul(e, x2_fma(x2_both(1.875f), e, x2_both(1.5f)));
+            const d2 ri = {y, x2_mul(y, t1)};
+            d2 c3 = d2_mul1(y2, y);
+            c3.l = x2_fma(c3.h, t3, c3.l);
+            const d2 c = d2_mul(xq, c3);
+            s[0] = d2_add(s[0], d2_add(d2_mul(q0, ri), d2_mul(c, dx[0])));
+            s[1] = d2_add(s[1], d2_add(d2_mul(q1, ri), d2_mul(c, dx[1])));
+            s[2] = d2_add(s[2], d2_add(d2_mul(q2, ri), d2_mul(c, dx[2])));
+          } else {  // stresslet without its factor -6: (xh.q)(xh.n) xh/r^5
+            const fx2 t5 = x2_mul(e, x2_fma(x2_both(4.375f), e, x2_both(2.5f)));
+            d2 c5 = d2_mul1(d2_sqr(y2), y);
+            c5.l = x2_fma(c5.h, t5, c5.l);
+            const d2 xn = d2_add(d2_add(d2_mul(dx[0], sv[6][k]), d2_mul(dx[1], sv[7][k])), d2_mul(dx[2], sv[8][k]));
+            const d2 c = d2_mul(d2_mul(xq, xn), c5);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) s[a] = d2_add(s[a], d2_mul(c, dx[a]));
           }
         }
       }
       __syncthreads();
 #pragma unroll
-      for (int u = 0; u < TPT; ++u)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) s[u][c] = df_renorm(s[u][c]);
+      for (int c = 0; c < 3; ++c) s[c] = d2_renorm(s[c]);
     }
     const double wj = KIND ? -6.0 * wts[j] : wts[j];
 #pragma unroll
-    for (int u = 0; u < TPT; ++u) {
-      const double w = act[u] ? wj : 0.0;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) acc[u][c] += w * ((double)s[u][c].h + (double)s[u][c].l);
+    for (int c = 0; c < 3; ++c) {
+      float h0, h1, l0, l1;
+      x2_unpack(s[c].h, h0, h1);
+      x2_unpack(s[c].l, l0, l1);
+      if (act[0]) acc[0][c] += wj * ((double)h0 + (double)l0);
+      if (act[1]) acc[1][c] += wj * ((double)h1 + (double)l1);
     }
   }
   double* pp = partial + (long long)b * 3 * kTile;
 #pragma unroll
-  for (int u = 0; u < TPT; ++u) {
-    const int k = tid + u * NT;
-    pp[k] = acc[u][0];
-    pp[kTile + k] = acc[u][1];
-    pp[2 * kTile + k] = acc[u][2];
-  }
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) pp[c * kTile + tid + u * NT] = acc[u][c];
 }
 
 // Per (tile, source drop j): the tile's targets in Omega_0, Omega_1 and Omega_2 of drop j as 128-bit
@@ -805,9 +813,8 @@ int launch_interdrop_df(int kind, int nblk, const PairItem* items, const int* bl
                         const double* Ns, const double* Qs, long long nstd, const double* Xu, const double* Nu,
                         const double* Qu, long long nup, const double* wts, double* partial, cudaStream_t s) {
   if (nblk == 0) return BIE_OK;
-  constexpr int TPT = 2;
-  auto kern = kind == 0 ? k_interdrop_df<0, TPT> : k_interdrop_df<1, TPT>;
-  kern<<<nblk, kTile / TPT, 0, s>>>(items, blk_item, tile_t0, tile_n, tile_drop, tgt_loc, toff_std, ngd, rec_std,
+  auto kern = kind == 0 ? k_interdrop_df<0> : k_interdrop_df<1>;
+  kern<<<nblk, kTile / 2, 0, s>>>(items, blk_item, tile_t0, tile_n, tile_drop, tgt_loc, toff_std, ngd, rec_std,
                                     centre, Xs, Ns, Qs, nstd, Xu, Nu, Qu, nup, wts, partial);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
