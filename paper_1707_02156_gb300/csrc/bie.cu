@@ -789,6 +789,17 @@ static int autotune_interdrop(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
   return BIE_OK;
 }
 
+// Sources per block of the pair sums' work list, given the sources of all tiles: about 32 blocks per SM in all,
+// at least 128 (two staged chunks), so that a few drops still fill the SMs, and at most 4096, so that the
+// last wave of a large list stays short; a tile takes at most kTileBlocks blocks (their partial sums are
+// added in order).  Before, 2048 to 65536: the FP32 pair sums of 8 drops of degree 16 (160 one-warp blocks) 205
+// -> 37 us an apply, of 192 drops of degree 24 46.8 -> 42 ms, the double-float ones of 80 drops 68.7 -> 54 ms.
+// Half as many blocks per SM cost 10% on 20 drops of degree 16 to 48, 16384 sources 7% on the 80 drops.
+constexpr long long kTileBlocks = 64;
+static long long block_sources(const bie_ctx* ctx, long long all_sources) {
+  return std::max<long long>(128, std::min<long long>(4096, all_sources / (32LL * ctx->sms)));
+}
+
 static int setup_interdrop(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
   const int nd = g->ndrop;
   const int U = ctx->cfg.upsample;
@@ -915,7 +926,7 @@ static int setup_interdrop(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
     for (int q = 0; q < 4; ++q) c += __builtin_popcount(m[q]);
     return c;
   };
-  // total sources over all tiles, to aim at >= 8 blocks per SM overall
+  // total sources over all tiles
   long long all_sources = 0;
   for (int ti = 0; ti < ntile; ++ti)
     for (int j = 0; j < nd; ++j) {
@@ -923,7 +934,7 @@ static int setup_interdrop(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
       const TileMask& tmj = tmask[(size_t)ti * nd + j];
       all_sources += (popc(tmj.m[0]) ? ngd[j] : 0) + (popc(tmj.m[1]) ? g->up_n[j] : 0);
     }
-  const long long cap_global = std::max<long long>(2048, std::min<long long>(65536, all_sources / (8LL * ctx->sms)));
+  const long long cap_global = block_sources(ctx, all_sources);
   std::vector<PairItem> items;
   std::vector<int> blk_item, tile_blk(ntile + 1, 0);
   long long far_pairs = 0, up_pairs = 0, slots = 0;
@@ -972,7 +983,7 @@ static int setup_interdrop(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
       }
     }
     // split the tile's items into blocks of at most `cap` sources
-    const long long cap = std::max(cap_global, (total + 15) / 16);  // at most 16 blocks per tile
+    const long long cap = std::max(cap_global, (total + kTileBlocks - 1) / kTileBlocks);
     tile_blk[ti] = (int)blk_item.size();
     long long used = cap;  // forces a new block at the first item
     for (auto it : mine) {
@@ -1467,7 +1478,6 @@ static int eval_layers(bie_ctx* ctx, bie_geom* g, long long npt, const double* p
   std::vector<std::pair<long long, int>> near;  // (point, drop) pairs in Omega_2
   long long all_sources = 0;
   for (int j = 0; j < nd; ++j) all_sources += ngrid(g->p[j]);
-  const long long cap_global = std::max<long long>(2048, std::min<long long>(65536, all_sources / (8LL * ctx->sms)));
   auto popc = [](const unsigned* m) {
     int c = 0;
     for (int q = 0; q < 4; ++q) c += __builtin_popcount(m[q]);
@@ -1517,7 +1527,7 @@ static int eval_layers(bie_ctx* ctx, bie_geom* g, long long npt, const double* p
             for (int k = 0; k < h_n[ti]; ++k)
               if ((m.m[2][k >> 5] >> (k & 31)) & 1u) near.emplace_back(t0 + (long long)ti * kTile + k, j);
         }
-        const long long cap = std::max(cap_global, (total + 15) / 16);  // at most 16 blocks per tile
+        const long long cap = std::max(block_sources(ctx, all_sources * ntile), (total + kTileBlocks - 1) / kTileBlocks);
         tile_blk[ti] = (int)blk_item.size();
         long long used = cap;
         for (auto it : mine) {
