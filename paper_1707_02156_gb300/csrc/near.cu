@@ -126,13 +126,15 @@ __device__ void sh_eval_d2(const double* __restrict__ c, long long cstride, int 
       for (int o = 16; o > 0; o >>= 1) out[k][q] += __shfl_xor_sync(0xffffffffu, out[k][q], o);
 }
 
-// Value of three real SH series at (theta, phi) (any theta, poles included).
+// Value of three real SH series at (theta, phi) (any theta, poles included), by one warp: lane l runs the
+// orders l, l + 32, ...; every lane returns the value.
 __device__ void sh_eval3(const double* __restrict__ c, long long cstride, int p, double th, double ph, double* out) {
   out[0] = out[1] = out[2] = 0;
   double st, ct;
   sincos(th, &st, &ct);
-  double dm = sqrt(1.0 / (4.0 * kPiD));
-  for (int m = 0; m <= p; ++m) {
+  for (int m = threadIdx.x & 31; m <= p; m += 32) {
+    double dm = sqrt(1.0 / (4.0 * kPiD));
+    for (int k = 0; k < m; ++k) dm *= -sqrt(1.0 + 1.0 / (2.0 * (k + 1))) * st;
     double pm2 = 0, pm1 = 0;
     double hr[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
     for (int n = m; n <= p; ++n) {
@@ -142,8 +144,7 @@ __device__ void sh_eval3(const double* __restrict__ c, long long cstride, int p,
       else if (n == m + 1)
         P = sqrt(2.0 * m + 3.0) * ct * dm;
       else
-        P = sqrt((4.0 * n * n - 1.0) / ((double)n * n - (double)m * m)) *
-            (ct * pm1 - sqrt(((n - 1.0) * (n - 1.0) - (double)m * m) / (4.0 * (n - 1.0) * (n - 1.0) - 1.0)) * pm2);
+        P = rec_a(n, m) * (ct * pm1 - rec_b(n, m) * pm2);
       pm2 = pm1;
       pm1 = P;
       for (int q = 0; q < 3; ++q) {
@@ -155,8 +156,9 @@ __device__ void sh_eval3(const double* __restrict__ c, long long cstride, int p,
     sincos(m * ph, &sm, &cm);
     const double fac = m == 0 ? 1.0 : 2.0;
     for (int q = 0; q < 3; ++q) out[q] += fac * (hr[q] * cm - hi[q] * sm);
-    dm = m + 1 <= p ? -sqrt(1.0 + 1.0 / (2.0 * (m + 1))) * st * dm : 0.0;
   }
+  for (int q = 0; q < 3; ++q)
+    for (int o = 16; o > 0; o >>= 1) out[q] += __shfl_xor_sync(0xffffffffu, out[q], o);
 }
 
 // nearest of the N points of records r to x0, scanned by one warp (the first nearest point wins ties, as in
@@ -342,7 +344,7 @@ __global__ void __launch_bounds__(256) k_near_checks(
   }
 }
 
-// One thread per target with near pairs: anchor from the source drop's (weighted) self expansion,
+// One warp per target with near pairs: anchor from the source drop's (weighted) self expansion,
 // minus 4 pi w_j u(x*) for the double layer, then Lagrange interpolation at the target's distance.
 __global__ void k_near_interp(const NearPair* __restrict__ pairs, const int* __restrict__ tbeg, int ntgt, int L,
                               int kind, const double* __restrict__ selfcoef, const double* __restrict__ dens,
@@ -351,7 +353,7 @@ __global__ void k_near_interp(const NearPair* __restrict__ pairs, const int* __r
                               const double* __restrict__ cv, const int* __restrict__ tdrop,
                               const long long* __restrict__ tgt_loc, const long long* __restrict__ val_off,
                               const int* __restrict__ ngd, double* __restrict__ vals) {
-  const int u = blockIdx.x * blockDim.x + threadIdx.x;
+  const int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (u >= ntgt) return;
   double acc[3] = {0, 0, 0};
   const long long t = pairs[tbeg[u]].target;
@@ -366,9 +368,10 @@ __global__ void k_near_interp(const NearPair* __restrict__ pairs, const int* __r
       sh_eval3(dens + coef_off[j], cs, p, P.theta_v, P.phi_v, us);
       for (int q = 0; q < 3; ++q) anchor[q] -= 4.0 * kPiD * wts[j] * us[q];
     }
-    // Lagrange through (0, anchor) and (h sqrt(l), cv_l), l = 1..L, at distance d0
+    // Lagrange through (0, anchor) and (h sqrt(l), cv_l), l = 1..L, at distance d0, lane l node l
     const double h = hdrop[j], x = P.d0;
-    for (int l = 0; l <= L; ++l) {
+    const int l = threadIdx.x & 31;
+    if (l <= L) {
       const double xl = l == 0 ? 0.0 : h * sqrt((double)l);
       double bas = 1.0;
       for (int k = 0; k <= L; ++k) {
@@ -379,6 +382,9 @@ __global__ void k_near_interp(const NearPair* __restrict__ pairs, const int* __r
       for (int q = 0; q < 3; ++q) acc[q] += bas * (l == 0 ? anchor[q] : cv[3 * ((long long)i * L + (l - 1)) + q]);
     }
   }
+  for (int q = 0; q < 3; ++q)
+    for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_down_sync(0xffffffffu, acc[q], o);
+  if (threadIdx.x & 31) return;
   const int d = tdrop[t];
   const long long ng = ngd[d];
   double* v = vals + val_off[d] + tgt_loc[t];
@@ -766,7 +772,7 @@ int launch_near_interp(const NearPair* pairs, const int* tbeg, int ntgt, int L, 
                        const double* wts, const double* cv, const int* tdrop, const long long* tgt_loc,
                        const long long* val_off, const int* ngd, double* vals, cudaStream_t s) {
   if (!ntgt) return BIE_OK;
-  k_near_interp<<<(ntgt + 63) / 64, 64, 0, s>>>(pairs, tbeg, ntgt, L, kind, selfcoef, dens, coef_off, pdeg, hdrop,
+  k_near_interp<<<(ntgt + 3) / 4, 128, 0, s>>>(pairs, tbeg, ntgt, L, kind, selfcoef, dens, coef_off, pdeg, hdrop,
                                                 wts, cv, tdrop, tgt_loc, val_off, ngd, vals);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
