@@ -265,7 +265,7 @@ __device__ __forceinline__ fx2 x2_fma(fx2 a, fx2 b, fx2 c) {
 __device__ __forceinline__ fx2 x2_rsqrt(fx2 v) {
   float lo, hi;
   x2_unpack(v, lo, hi);
-  return x2_pack(rsqrtf(lo), rsqrtf(hi));
+  return x2_pack(rsqrt_est(lo), rsqrt_est(hi));
 }
 
 constexpr int kChunkX2 = 64;  // sources staged per pass of the packed kernel
