@@ -15,23 +15,51 @@ __device__ __forceinline__ float rsqrt_est(float v) {
 
 template <typename R>
 __device__ inline R rsqrt_(R v);
-// 1/sqrt(v) in FP64 from the FP32 hardware estimate y and one third-order correction: with
-// e = 1 - v y^2 (about 2^-22), 1/sqrt(v) = y (1 - e)^(-1/2) = y (1 + e/2 + 3e^2/8 + O(e^3)), so the
-// truncated series leaves a relative error of order e^3 (2^-66), below FP64 rounding; e is formed
-// with one fused multiply-add from y^2, so its rounding error is 2^-53 absolute and enters the
-// result as 2^-54 relative.  Five FP64 operations against seven for two Newton steps.  Outside the
-// FP32 exponent range the estimate is unusable and the quotient of the IEEE square root is
-// returned instead.
+// FP64 powers of 1/sqrt(v) from the FP32 hardware estimate y of 1/sqrt(v): with e = 1 - v y^2 (about 2^-22,
+// formed by one fused multiply-add since y^2 is exact),
+//   v^(-k/2) = y^k (1 - e)^(-k/2) = y^k (1 + (k/2) e + (k/2)(k/2 + 1)/2 e^2 + O(e^3)),
+// so the truncated series leaves a relative error of order e^3 (2^-64), below FP64 rounding.  The FP64 pipe is
+// the bound of every kernel that calls these, and conversions and comparisons of doubles run on it too:
+// the estimate's argument and result pass through the integer pipe (rebased exponent, mantissa cut to
+// 23 bits), and the test for the FP32 exponent range looks at the high word.  Five FP64 operations for
+// 1/sqrt(v), seven for v^(-5/2).  Outside 2^-99 <= v < 2^99 (negative, infinite and NaN arguments
+// included) the estimate is unusable and est returns false.
+__device__ __forceinline__ bool rsqrt_est64(double v, double& y, double& e) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  if (hi - (924u << 20) >= (198u << 20)) return false;
+  const unsigned f = __float_as_uint(rsqrt_est(__uint_as_float(((hi - (896u << 20)) << 3) | (lo >> 29))));
+  y = __hiloint2double((int)((f >> 3) + (896u << 20)), (int)(f << 29));
+  e = fma(-v, y * y, 1.0);
+  return true;
+}
 template <>
 __device__ inline double rsqrt_<double>(double v) {
-  if (!(v > 1e-30 && v < 1e30)) return 1.0 / sqrt(v);
-  const double y = (double)rsqrt_est((float)v);
-  const double e = fma(-v, y * y, 1.0);
+  double y, e;
+  if (!rsqrt_est64(v, y, e)) return 1.0 / sqrt(v);
   return fma(y, e * fma(0.375, e, 0.5), y);
 }
 template <>
 __device__ inline float rsqrt_<float>(float v) {
   return rsqrt_est(v);
+}
+
+// v^(-5/2)
+template <typename R>
+__device__ inline R rsqrt5_(R v);
+template <>
+__device__ inline double rsqrt5_<double>(double v) {
+  double y, e;
+  if (!rsqrt_est64(v, y, e)) {
+    const double r = 1.0 / sqrt(v), r2 = r * r;
+    return r2 * r2 * r;
+  }
+  const double y2 = y * y, y5 = y2 * y2 * y;
+  return fma(y5, e * fma(4.375, e, 2.5), y5);
+}
+template <>
+__device__ inline float rsqrt5_<float>(float v) {
+  const float r = rsqrt_est(v), r2 = r * r;
+  return r2 * r2 * r;
 }
 
 // Block-wide sum of three values; the result is valid in thread 0.  sh holds 3 * 32 entries.

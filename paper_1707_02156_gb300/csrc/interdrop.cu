@@ -192,17 +192,17 @@ __global__ void __launch_bounds__(kTile / TPT) k_interdrop(
 #pragma unroll
           for (int u = 0; u < TPT; ++u) {
             const R dx = px[u] - xs_, dy = py[u] - ys_, dz = pz[u] - zs_;
-            const R ri = rsqrt_<R>(dx * dx + dy * dy + dz * dz);
+            const R r2 = dx * dx + dy * dy + dz * dz;
             const R xq = dx * q0 + dy * q1 + dz * q2;
             if (KIND == 0) {  // Stokeslet
+              const R ri = rsqrt_<R>(r2);
               const R c = xq * ri * ri * ri;
               s[u][0] += q0 * ri + c * dx;
               s[u][1] += q1 * ri + c * dy;
               s[u][2] += q2 * ri + c * dz;
             } else {  // stresslet, without its factor -6
               const R xn = dx * v[6] + dy * v[7] + dz * v[8];
-              const R ri2 = ri * ri;
-              const R c = xq * xn * ri2 * ri2 * ri;
+              const R c = xq * xn * rsqrt5_<R>(r2);
               s[u][0] += c * dx;
               s[u][1] += c * dy;
               s[u][2] += c * dz;

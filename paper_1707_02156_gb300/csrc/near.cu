@@ -318,18 +318,18 @@ __global__ void __launch_bounds__(256) k_near_checks(
   R a0 = 0, a1 = 0, a2 = 0;
   for (long long s = s0 + threadIdx.x; s < s1; s += blockDim.x) {
     const R dx = px - X[s], dy = py - X[ld + s], dz = pz - X[2 * ld + s];
-    const R ri = rsqrt_<R>(dx * dx + dy * dy + dz * dz);
+    const R r2 = dx * dx + dy * dy + dz * dz;
     const R q0 = Q[s], q1 = Q[ld + s], q2 = Q[2 * ld + s];
     const R xq = dx * q0 + dy * q1 + dz * q2;
     if (KIND == 0) {
+      const R ri = rsqrt_<R>(r2);
       const R c = xq * ri * ri * ri;
       a0 += q0 * ri + c * dx;
       a1 += q1 * ri + c * dy;
       a2 += q2 * ri + c * dz;
     } else {
       const R xn = dx * N[s] + dy * N[ld + s] + dz * N[2 * ld + s];
-      const R ri2 = ri * ri;
-      const R c = (R)(-6) * xq * xn * ri2 * ri2 * ri;
+      const R c = (R)(-6) * xq * xn * rsqrt5_<R>(r2);
       a0 += c * dx;
       a1 += c * dy;
       a2 += c * dz;
@@ -470,14 +470,14 @@ __global__ void __launch_bounds__(kNearThreads) k_near_rows(const NearPair* __re
         for (int l = 0; l < L; ++l) {
           if (onup[l] != gk) continue;
           const double dx = cx[l][0] - x0, dy = cx[l][1] - x1, dz = cx[l][2] - x2;
-          const double ri = rsqrt_<double>(dx * dx + dy * dy + dz * dz), ri2 = ri * ri;
+          const double r2 = dx * dx + dy * dy + dz * dz;
           double c;
           if (KIND == 0) {
-            const double a = bas[l + 1] * w * ri;
+            const double ri = rsqrt_<double>(r2), a = bas[l + 1] * w * ri;
             dsum += a;
-            c = a * ri2;
+            c = a * (ri * ri);
           } else {
-            c = (bas[l + 1] * (dx * n0 + dy * n1 + dz * n2)) * (ri2 * ri2 * ri);
+            c = (bas[l + 1] * (dx * n0 + dy * n1 + dz * n2)) * rsqrt5_<double>(r2);
           }
           const double ax = c * dx, ay = c * dy;
           m[0] += ax * dx;

@@ -254,13 +254,14 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
       }
       const long long o = (long long)j * nk + k;
       const double x0 = geo[o], x1 = geo[nq + o], x2 = geo[2 * nq + o];
-      const double ri = rsqrt_<double>(x0 * x0 + x1 * x1 + x2 * x2), ri2 = ri * ri;
+      const double r2 = x0 * x0 + x1 * x1 + x2 * x2;
       double d = 0.0, c;
       if (KIND == 0) {
+        const double ri = rsqrt_<double>(r2);
         d = geo[6 * nq + o] * ri;
-        c = d * ri2;
+        c = d * (ri * ri);
       } else {
-        c = (-6.0 * (x0 * geo[3 * nq + o] + x1 * geo[4 * nq + o] + x2 * geo[5 * nq + o])) * (ri2 * ri2 * ri);
+        c = (-6.0 * (x0 * geo[3 * nq + o] + x1 * geo[4 * nq + o] + x2 * geo[5 * nq + o])) * rsqrt5_<double>(r2);
       }
       const double a0 = c * x0, a1 = c * x1;
       v[0] = d + a0 * x0;
