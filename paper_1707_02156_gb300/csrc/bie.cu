@@ -1088,21 +1088,20 @@ static int source_densities(bie_geom* g, const double* dens, R* Qs, R* Qu, cudaS
 // (the source drop's standard-grid point nearest to x0) on the equator; then the check points
 // x_l = x* + h_j sqrt(l) e, e = (x0 - x*)/|x0 - x*|, l = 1..L, and the grid (standard or upsampled)
 // each is summed on.  x0: 3 per pair (host); seeds: standard-grid index per pair.  Fills d0 and the
-// parameters of x* in drop j's own frame into the pairs and returns the check points [pair][L][3]
-// and their grids [pair][L] on the device.
-static int near_points(bie_ctx* ctx, bie_geom* g, std::vector<NearPair>& pairs, const std::vector<double>& x0,
-                       const std::vector<int>& hseed, DevBuf<double>& pts_d, DevBuf<int>& grid_d, cudaStream_t s) {
+// parameters of x* in drop j's own frame into the pairs dpairs on the device and returns the check points
+// [pair][L][3] and their grids [pair][L] there.
+static int near_points(bie_ctx* ctx, bie_geom* g, const std::vector<NearPair>& pairs, NearPair* dpairs,
+                       const std::vector<double>& x0, const std::vector<int>& hseed, DevBuf<double>& pts_d,
+                       DevBuf<int>& grid_d, cudaStream_t s) {
   const int npair = (int)pairs.size();
   const int L = ctx->cfg.n_interp;
-  DevBuf<NearPair> dpairs;
-  BIE_TRY(dpairs.upload(pairs));
   // rotated shape coefficients: (alpha, beta) = (phi_b, theta_a - pi/2) puts the seed (latitude a,
   // longitude b) at the equator.  The phases e^{i m alpha} of every pair are applied in one launch;
   // then the pairs of one degree and one seed latitude share one rotation launch (the small-d blocks
   // of that beta), and one Newton launch serves every pair.  The rotated coefficients lie in group
   // order, [pair][3][(p+1)^2].
   std::unique_ptr<Phase> stage(new Phase(ctx, "near_newton", s));
-  std::vector<double> alpha(npair), beta(npair), hres(5 * (size_t)npair);
+  std::vector<double> beta(npair);
   std::map<std::pair<int, int>, std::vector<int>> groups;  // (degree, seed latitude) -> pairs
   int pmax = 0;
   for (int i = 0; i < npair; ++i) {
@@ -1135,7 +1134,6 @@ static int near_points(bie_ctx* ctx, bie_geom* g, std::vector<NearPair>& pairs, 
     for (size_t k = 0; k < idx.size(); ++k) {
       const int i = idx[k];
       lon[i] = hseed[i] % nb;
-      alpha[i] = kPi * lon[i] / (p + 1);
       beta[i] = std::acos(t[a]) - 0.5 * kPi;
       xr_off[i] = xo + (long long)k * 3 * nc;
       for (int c = 0; c < 3; ++c) fo_all.push_back(xr_off[i] + c * nc);
@@ -1144,7 +1142,7 @@ static int near_points(bie_ctx* ctx, bie_geom* g, std::vector<NearPair>& pairs, 
   }
   std::vector<int> pd(g->p.begin(), g->p.end());
   DevBuf<int> pdeg, dlon;
-  DevBuf<double> shifted, xr, dx0, res;
+  DevBuf<double> shifted, xr, dx0, dbeta, res;
   DevBuf<long long> dfo, dxo, dcoef_off;
   BIE_TRY(pdeg.upload(pd));
   BIE_TRY(dlon.upload(lon));
@@ -1152,10 +1150,11 @@ static int near_points(bie_ctx* ctx, bie_geom* g, std::vector<NearPair>& pairs, 
   BIE_TRY(dxo.upload(xr_off));
   BIE_TRY(dfo.upload(fo_all));
   BIE_TRY(dx0.upload(x0));
+  BIE_TRY(dbeta.upload(beta));
   BIE_TRY(shifted.alloc(xo));
   BIE_TRY(xr.alloc(xo));
   BIE_TRY(res.alloc(5 * (size_t)npair));
-  BIE_TRY(launch_near_phase_shift(dpairs.ptr, npair, g->xcoef.ptr, dcoef_off.ptr, pdeg.ptr, dlon.ptr, dxo.ptr,
+  BIE_TRY(launch_near_phase_shift(dpairs, npair, g->xcoef.ptr, dcoef_off.ptr, pdeg.ptr, dlon.ptr, dxo.ptr,
                                   shifted.ptr, s));
   for (const auto& G : rg) {
     const long long nc = ncoef(G.p);
@@ -1165,34 +1164,9 @@ static int near_points(bie_ctx* ctx, bie_geom* g, std::vector<NearPair>& pairs, 
   DevBuf<double> rtab;
   BIE_TRY(rtab.alloc(near_rec_table_doubles(pmax)));
   BIE_TRY(launch_near_rec_table(pmax, rtab.ptr, s));
-  BIE_TRY(launch_near_newton(dpairs.ptr, npair, xr.ptr, pdeg.ptr, dxo.ptr, dx0.ptr, rtab.ptr, pmax, res.ptr, s));
-  BIE_CUDA_TRY(cudaMemcpyAsync(hres.data(), res.ptr, hres.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
-  BIE_CUDA_TRY(cudaStreamSynchronize(s));
+  BIE_TRY(launch_near_newton(dpairs, npair, xr.ptr, pdeg.ptr, dxo.ptr, dx0.ptr, rtab.ptr, pmax, res.ptr, s));
   stage.reset(new Phase(ctx, "near_checkpoints", s));
-  std::vector<double> pts(3 * (size_t)npair * L);
-  for (int i = 0; i < npair; ++i) {
-    const int j = pairs[i].src_drop;
-    const double th = hres[5 * i], phv = hres[5 * i + 1];
-    const double xs[3] = {hres[5 * i + 2], hres[5 * i + 3], hres[5 * i + 4]};
-    double e[3], d0 = 0;
-    for (int c = 0; c < 3; ++c) {
-      e[c] = x0[3 * i + c] - xs[c];
-      d0 += e[c] * e[c];
-    }
-    d0 = std::sqrt(d0);
-    for (int c = 0; c < 3; ++c) e[c] /= d0;
-    pairs[i].d0 = d0;
-    // parameters of x* in drop j's own frame: v = R_z(alpha) R_y(beta) s(theta*, phi*)
-    const double sv[3] = {std::sin(th) * std::cos(phv), std::sin(th) * std::sin(phv), std::cos(th)};
-    const double cb = std::cos(beta[i]), sb = std::sin(beta[i]), ca = std::cos(alpha[i]), sa = std::sin(alpha[i]);
-    const double y0 = cb * sv[0] + sb * sv[2], y1 = sv[1], y2 = -sb * sv[0] + cb * sv[2];
-    const double v0 = ca * y0 - sa * y1, v1 = sa * y0 + ca * y1, v2 = y2;
-    pairs[i].theta_v = std::acos(std::max(-1.0, std::min(1.0, v2)));
-    pairs[i].phi_v = std::atan2(v1, v0);
-    for (int l = 1; l <= L; ++l)
-      for (int c = 0; c < 3; ++c) pts[3 * ((size_t)i * L + (l - 1)) + c] = xs[c] + g->hdrop[j] * std::sqrt((double)l) * e[c];
-  }
-  BIE_TRY(pts_d.upload(pts));
+  BIE_TRY(pts_d.alloc(3 * (size_t)npair * L));
   BIE_TRY(grid_d.alloc((size_t)npair * L));
   DevBuf<double> bnd, hh;
   DevBuf<long long> uoff, un;
@@ -1200,7 +1174,9 @@ static int near_points(bie_ctx* ctx, bie_geom* g, std::vector<NearPair>& pairs, 
   BIE_TRY(hh.upload(g->hdrop));
   BIE_TRY(uoff.upload(g->up_off));
   BIE_TRY(un.upload(g->up_n));
-  BIE_TRY(launch_near_checkgrid(dpairs.ptr, npair, L, pts_d.ptr, g->centre_d.ptr, bnd.ptr, hh.ptr, ctx->cfg.a_tilde,
+  BIE_TRY(launch_near_checkpoints(dpairs, npair, L, res.ptr, dx0.ptr, dlon.ptr, dbeta.ptr, pdeg.ptr, hh.ptr, pts_d.ptr,
+                                  s));
+  BIE_TRY(launch_near_checkgrid(dpairs, npair, L, pts_d.ptr, g->centre_d.ptr, bnd.ptr, hh.ptr, ctx->cfg.a_tilde,
                                 g->rec_up.ptr, uoff.ptr, un.ptr, grid_d.ptr, s));
   BIE_CUDA_TRY(cudaStreamSynchronize(s));
   return BIE_OK;
@@ -1252,8 +1228,7 @@ static int setup_near(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
     const long long ngi = ngrid(g->p[di]), l = tt - g->tgt_off[di];
     for (int c = 0; c < 3; ++c) x0[3 * i + c] = rec[7 * g->tgt_off[di] + c * ngi + l];
   }
-  BIE_TRY(near_points(ctx, g, pairs, x0, hseed, g->npts, g->ngrid_l, s));
-  BIE_TRY(g->npairs.upload(pairs));
+  BIE_TRY(near_points(ctx, g, pairs, g->npairs.ptr, x0, hseed, g->npts, g->ngrid_l, s));
   BIE_TRY(g->ncv.alloc(3 * (size_t)npair * L));
   BIE_TRY(near_tables(g));
   // The rule becomes rows of the operator unless they would take more than 4 GB per kind, or a block's
@@ -1625,8 +1600,7 @@ static int eval_layers(bie_ctx* ctx, bie_geom* g, long long npt, const double* p
   std::vector<double> x0(3 * (size_t)npair);
   for (int i = 0; i < npair; ++i)
     for (int c = 0; c < 3; ++c) x0[3 * i + c] = hp[c * npt + pairs[i].target];
-  BIE_TRY(near_points(ctx, g, pairs, x0, hseed, d_npts, d_grid, s));
-  BIE_TRY(d_pairs.upload(pairs));
+  BIE_TRY(near_points(ctx, g, pairs, d_pairs.ptr, x0, hseed, d_npts, d_grid, s));
   BIE_TRY(d_tbeg.upload(tbeg));
   BIE_TRY(near_tables(g));
   BIE_TRY(d_cv.alloc(3 * (size_t)npair * L));

@@ -264,6 +264,37 @@ __global__ void k_near_newton(const NearPair* __restrict__ pairs, int npair, con
   result[5 * i + 4] = d[0][2];
 }
 
+// From the Newton results (theta*, phi* in the rotated frame, x*): the pair's distance d0, the parameters of x*
+// in drop j's own frame (v = R_z(alpha) R_y(beta) s(theta*, phi*), alpha = pi lon / (p+1)) and the check
+// points x_l = x* + h_j sqrt(l) e, e = (x0 - x*)/|x0 - x*|, l = 1..L.
+__global__ void k_near_checkpoints(NearPair* __restrict__ pairs, int npair, int L, const double* __restrict__ res,
+                                   const double* __restrict__ x0all, const int* __restrict__ lon,
+                                   const double* __restrict__ beta, const int* __restrict__ pdeg,
+                                   const double* __restrict__ hdrop, double* __restrict__ pts) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= npair) return;
+  const int j = pairs[i].src_drop;
+  double e[3], d0 = 0;
+  for (int c = 0; c < 3; ++c) {
+    e[c] = x0all[3 * i + c] - res[5 * i + 2 + c];
+    d0 += e[c] * e[c];
+  }
+  d0 = sqrt(d0);
+  for (int c = 0; c < 3; ++c) e[c] /= d0;
+  double st, ct, sp, cp, sb, cb, sa, ca;
+  sincos(res[5 * i], &st, &ct);
+  sincos(res[5 * i + 1], &sp, &cp);
+  sincos(beta[i], &sb, &cb);
+  sincospi((double)lon[i] / (pdeg[j] + 1), &sa, &ca);
+  const double y0 = cb * (st * cp) + sb * ct, y1 = st * sp, y2 = -sb * (st * cp) + cb * ct;
+  pairs[i].d0 = d0;
+  pairs[i].theta_v = acos(fmax(-1.0, fmin(1.0, y2)));
+  pairs[i].phi_v = atan2(sa * y0 + ca * y1, ca * y0 - sa * y1);
+  for (int l = 1; l <= L; ++l)
+    for (int c = 0; c < 3; ++c)
+      pts[3 * ((long long)i * L + (l - 1)) + c] = res[5 * i + 2 + c] + hdrop[j] * sqrt((double)l) * e[c];
+}
+
 // grid of each check point: 0 standard (Omega_0), 1 upsampled otherwise (same distance rule as the
 // region split)
 __global__ void k_near_checkgrid(const NearPair* __restrict__ pairs, int npair, int L, const double* __restrict__ pts,
@@ -734,6 +765,15 @@ int launch_near_newton(const NearPair* pairs, int npair, const double* xr, const
                        const double* x0, const double* tab, int tabP, double* result, cudaStream_t s) {
   if (!npair) return BIE_OK;
   k_near_newton<<<(npair + 3) / 4, 128, 0, s>>>(pairs, npair, xr, pdeg, xr_off, x0, tab, tabP, result);
+  count_launch();
+  BIE_CUDA_TRY(cudaGetLastError());
+  return BIE_OK;
+}
+
+int launch_near_checkpoints(NearPair* pairs, int npair, int L, const double* res, const double* x0, const int* lon,
+                            const double* beta, const int* pdeg, const double* hdrop, double* pts, cudaStream_t s) {
+  if (!npair) return BIE_OK;
+  k_near_checkpoints<<<(npair + 63) / 64, 64, 0, s>>>(pairs, npair, L, res, x0, lon, beta, pdeg, hdrop, pts);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;

@@ -27,6 +27,9 @@ int near_rec_table_doubles(int P);
 int launch_near_rec_table(int P, double* tab, cudaStream_t s);
 int launch_near_newton(const NearPair* pairs, int npair, const double* xr, const int* pdeg, const long long* xr_off,
                        const double* x0, const double* tab, int tabP, double* result, cudaStream_t s);
+// d0 and the own-frame parameters of x* into the pairs, and the check points [pair][L][3], from the Newton results
+int launch_near_checkpoints(NearPair* pairs, int npair, int L, const double* res, const double* x0, const int* lon,
+                            const double* beta, const int* pdeg, const double* hdrop, double* pts, cudaStream_t s);
 int launch_near_checkgrid(const NearPair* pairs, int npair, int L, const double* pts, const double* centre,
                           const double* bound, const double* h, double a_tilde, const double* rec_up,
                           const long long* up_off, const long long* up_n, int* grid, cudaStream_t s);
