@@ -330,8 +330,6 @@ struct bie_geom {
   bie::DevBuf<double> rec_up;                       // [drop][7][N_up] upsampled-grid records
   bie::DevBuf<double> sX64, sN64, uX64, uN64, sQ64, uQ64;  // sources: positions rel. centre, normals, weighted density
   bie::DevBuf<float> sX32, sN32, uX32, uN32, sQ32, uQ32;
-  bie::DevBuf<double> syn64;                        // synthesis temporaries for the source densities
-  bie::DevBuf<float> syn32;
   bie::DevBuf<bie::PairItem> items;
   bie::DevBuf<int> blk_item, tile_n, tile_drop, tile_blk, tdrop, ngd;
   bie::DevBuf<long long> tile_t0, tgt_loc, toff, val_off_all;
@@ -1059,27 +1057,13 @@ static int source_densities(bie_geom* g, const double* dens, R* Qs, R* Qu, cudaS
     const int p = G.p;
     const int Pu = ctx->cfg.upsample * (p + 1) - 1;
     const long long nd = (long long)G.drops.size();
-    const long long need = nd * 3 * ngrid(Pu);
-    R* grid;
-    if (sizeof(R) == 8) {
-      BIE_TRY(g->syn64.alloc(need));
-      grid = reinterpret_cast<R*>(g->syn64.ptr);
-    } else {
-      BIE_TRY(g->syn32.alloc(need));
-      grid = reinterpret_cast<R*>(g->syn32.ptr);
-    }
-    for (int gridk = 0; gridk < 2; ++gridk) {
-      const int P = gridk ? Pu : p;
-      const long long N = ngrid(P);
-      Plan* pl;
-      BIE_TRY(get_plan(ctx, p, P, &pl));
-      BIE_TRY((launch_synth<double, R>(1, dens, G.foff3.ptr, 0, nd * 3, p, P, pl->T0_<R>(), (const R*)nullptr,
-                                       (const R*)nullptr, pl->cs_<R>(), grid, 0, N, ctx->sms, s)));
-      if (gridk == 0)
-        BIE_TRY(launch_weight_sources<R>(grid, g->rec_std.ptr, G.src_off_std.ptr, N, nd, Qs, g->ntarget, s));
-      else
-        BIE_TRY(launch_weight_sources<R>(grid, g->rec_up.ptr, G.src_off_up.ptr, N, nd, Qu, g->nup_total, s));
-    }
+    Plan *ps, *pu;
+    BIE_TRY(get_plan(ctx, p, p, &ps));
+    BIE_TRY(get_plan(ctx, p, Pu, &pu));
+    BIE_TRY(launch_synth_sources<R>(dens, G.foff3.ptr, nd, p, p, ps->T0_<R>(), ps->cs_<R>(),
+                                    {g->rec_std.ptr, G.src_off_std.ptr, g->ntarget}, Qs, ctx->sms, s));
+    BIE_TRY(launch_synth_sources<R>(dens, G.foff3.ptr, nd, p, Pu, pu->T0_<R>(), pu->cs_<R>(),
+                                    {g->rec_up.ptr, G.src_off_up.ptr, g->nup_total}, Qu, ctx->sms, s));
   }
   return BIE_OK;
 }

@@ -659,48 +659,23 @@ __global__ void k_tile_masks(const unsigned char* __restrict__ region, int nd, c
   out[idx] = m;
 }
 
-// vals += sum of the partials of the tile's blocks, in block order
+// vals += sum of the partials of the tile's blocks, in block order; one thread per (tile, component, target)
 __global__ void k_reduce_tiles(const double* __restrict__ partial, const int* __restrict__ tile_blk,
                                const long long* __restrict__ tile_t0, const int* __restrict__ tile_n,
                                const int* __restrict__ tile_drop, const long long* __restrict__ tgt_loc,
                                const long long* __restrict__ val_off, const int* __restrict__ ngd, int ntile,
                                double* __restrict__ vals) {
-  long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)ntile * kTile) return;
-  const int tile = (int)(idx / kTile), tid = (int)(idx - (long long)tile * kTile);
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= 3LL * ntile * kTile) return;
+  const int tile = (int)(idx / (3 * kTile)), r = (int)(idx - 3LL * tile * kTile), c = r / kTile, tid = r - c * kTile;
   if (tid >= tile_n[tile]) return;
   const int b0 = tile_blk[tile], b1 = tile_blk[tile + 1];
   if (b0 == b1) return;
-  double a0 = 0, a1 = 0, a2 = 0;
-  for (int b = b0; b < b1; ++b) {
-    const double* pp = partial + (long long)b * 3 * kTile;
-    a0 += pp[tid];
-    a1 += pp[kTile + tid];
-    a2 += pp[2 * kTile + tid];
-  }
+  double a = 0;
+#pragma unroll 8
+  for (int b = b0; b < b1; ++b) a += partial[3LL * kTile * b + r];
   const int d = tile_drop[tile];
-  const long long l = tgt_loc[tile_t0[tile] + tid];
-  const long long ng = ngd[d];
-  double* v = vals + val_off[d] + l;
-  v[0] += a0;
-  v[ng] += a1;
-  v[2 * ng] += a2;
-}
-
-// Q[c][off_d + s] = wJ[s] * grid[d][c][s] for the nd drops of one degree group, whose source records
-// rec [7][N] start at 7 * off_d (weight in row 6).
-template <typename R>
-__global__ void k_weight_sources(const R* __restrict__ grid, const double* __restrict__ rec,
-                                 const long long* __restrict__ off, long long N, long long nd, R* __restrict__ Q,
-                                 long long ldq) {
-  long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= nd * 3 * N) return;
-  const long long d = idx / (3 * N);
-  const long long r = idx - d * 3 * N;
-  const int c = (int)(r / N);
-  const long long s = r - c * N;
-  const long long o = off[d];
-  Q[c * ldq + o + s] = (R)rec[7 * o + 6 * N + s] * grid[idx];
+  vals[val_off[d] + (long long)c * ngd[d] + tgt_loc[tile_t0[tile] + tid]] += a;
 }
 
 // Per drop of a degree group (blockIdx.y; records of N points at rec + 7 off[i]): sum_s x.n wJ (for the
@@ -864,20 +839,10 @@ int launch_tile_masks(const unsigned char* region, int nd, const long long* tile
 int launch_reduce_tiles(const double* partial, const int* tile_blk, const long long* tile_t0, const int* tile_n,
                         const int* tile_drop, const long long* tgt_loc, const long long* val_off, const int* ngd,
                         int ntile, double* vals, cudaStream_t s) {
-  long long n = (long long)ntile * kTile;
+  long long n = 3LL * ntile * kTile;
   if (n == 0) return BIE_OK;
   k_reduce_tiles<<<blocks_for(n), kThreads, 0, s>>>(partial, tile_blk, tile_t0, tile_n, tile_drop, tgt_loc, val_off,
                                                      ngd, ntile, vals);
-  count_launch();
-  BIE_CUDA_TRY(cudaGetLastError());
-  return BIE_OK;
-}
-
-template <typename R>
-int launch_weight_sources(const R* grid, const double* rec, const long long* off, long long N, long long nd, R* Q,
-                          long long ldq, cudaStream_t s) {
-  if (N == 0 || nd == 0) return BIE_OK;
-  k_weight_sources<R><<<blocks_for(nd * 3 * N), kThreads, 0, s>>>(grid, rec, off, N, nd, Q, ldq);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
@@ -913,8 +878,4 @@ template int launch_interdrop<float>(int, int, int, const PairItem*, const int*,
                                      const long long*, const long long*, const int*, const double*, const double*,
                                      const float*, const float*, const float*, long long, const float*, const float*,
                                      const float*, long long, const double*, double*, cudaStream_t);
-template int launch_weight_sources<double>(const double*, const double*, const long long*, long long, long long,
-                                           double*, long long, cudaStream_t);
-template int launch_weight_sources<float>(const float*, const double*, const long long*, long long, long long, float*,
-                                          long long, cudaStream_t);
 }  // namespace bie

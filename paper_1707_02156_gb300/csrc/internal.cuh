@@ -36,13 +36,23 @@ __host__ __device__ inline long long leg_row(int p, int m, int n, int nj) {
 
 // ---- transforms (transforms.cu) ----
 // Synthesis of nfield fields of degree p on the grid of degree P, with the derivative kinds of the mask
-// `kinds` (bit 0 f, 1 t, 2 p, 3 tt, 4 tp, 5 pp; the masks 1, 6, 7, 62, 63 in FP64, 1 in FP32): kind
+// `kinds` (bit 0 f, 1 t, 2 p, 3 tt, 4 tp, 5 pp; the masks 1, 6, 7, 62, 63): kind
 // number s of the mask of field f goes to out + s * kind_stride + f * field_stride.  Coefficients of
 // field f start at field_off ? field_off[f] : f * coef_stride.  T1, T2 may be null when no kind needs them.
 template <typename CT, typename R>
 int launch_synth(int kinds, const CT* coef, const long long* field_off, long long coef_stride, long long nfield, int p,
                  int P, const R* T0, const R* T1, const R* T2, const R* cs, R* out, long long kind_stride,
                  long long field_stride, int sms, cudaStream_t s);
+// Weighted source densities of nd drops, fields [drop][3]: w_s f_c(s) on the degree-P grid to Q[c * ld + off[drop] + s],
+// the weights in row 6 of the records rec ([7][N] at 7 off[drop]).
+struct SynthSources {
+  const double* rec;
+  const long long* off;
+  long long ld;
+};
+template <typename R>
+int launch_synth_sources(const double* coef, const long long* field_off, long long nd, int p, int P, const R* T0,
+                         const R* cs, const SynthSources& src, R* Q, int sms, cudaStream_t s);
 // analysis: grids (degree P) -> coefficients (degree p <= P), FP64, for several degree groups in one launch.
 // Offsets per field, or null and a stride; begin and mb are set by the launcher.
 struct AnaGroup {

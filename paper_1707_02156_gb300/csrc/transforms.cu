@@ -39,14 +39,17 @@ constexpr int kSynStageP = BIE_MAX_P;  // coefficients are staged in shared memo
 // One block per (field, jb latitude pairs j and P - j).  Phase 1, thread per (order m, pair): the sums
 // over even and odd n - m with the Legendre tables asked for, for both latitudes, and from them each
 // kind's complex value per order (factors i m and -m^2, and the 2 of m > 0) in shared memory
-// h[kind][row][m].  Phase 2, thread per (row, longitude quadruple).
-template <typename CT, typename R, int KINDS>
+// h[kind][row][m].  Phase 2, thread per (row, longitude quadruple).  With SRC (values only) field 3 d + c is
+// component c of drop d's density, and the weighted source w_s f(s) goes to the sources' place instead of
+// the value to a grid.
+template <typename CT, typename R, int KINDS, bool SRC>
 __global__ void __launch_bounds__(kSynThreads) k_synth(const CT* __restrict__ coef,
                                                        const long long* __restrict__ field_off, long long coef_stride,
                                                        int p, int P, const R* __restrict__ T0,
                                                        const R* __restrict__ T1, const R* __restrict__ T2,
                                                        const R* __restrict__ cs, R* __restrict__ out,
-                                                       long long kind_stride, long long field_stride, int jb) {
+                                                       long long kind_stride, long long field_stride, int jb,
+                                                       SynthSources src) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int NK = kind_slot(KINDS, 6);
   const int nj = P + 1, nk = 2 * P + 2, half = P + 1, np = (nj + 1) / 2, k4n = half / 2 + 1;
@@ -145,15 +148,34 @@ __global__ void __launch_bounds__(kSynThreads) k_synth(const CT* __restrict__ co
       }
     }
     const bool rot = k > 0, mir = 2 * k < half;  // k = 0 and the middle k have two longitudes, not four
-    R* d0 = out + f * field_stride + (long long)j * nk;
+    R* d0;
+    R w[4] = {1, 1, 1, 1};  // the weights at k, half + k, 2 half - k, half - k
+    if constexpr (SRC) {
+      const long long o = src.off[f / 3], N = (long long)nj * nk;
+      const double* wj = src.rec + 7 * o + 6 * N + (long long)j * nk;
+      d0 = out + (f % 3) * src.ld + o + (long long)j * nk;
+      w[0] = (R)wj[k];
+      if (mir) w[1] = (R)wj[half + k];
+      if (rot) w[2] = (R)wj[2 * half - k];
+      if (rot && mir) w[3] = (R)wj[half - k];
+    } else {
+      d0 = out + f * field_stride + (long long)j * nk;
+    }
 #pragma unroll
     for (int s = 0; s < NK; ++s) {
       R* d = d0 + s * kind_stride;
       const R cp = ce[s] + co[s], cm = ce[s] - co[s], sp = se[s] + so[s], sm = se[s] - so[s];
-      d[k] = cp - sp;
-      if (mir) d[half + k] = cm - sm;
-      if (rot) d[2 * half - k] = cp + sp;
-      if (rot && mir) d[half - k] = cm + sm;
+      if (SRC) {
+        d[k] = w[0] * (cp - sp);
+        if (mir) d[half + k] = w[1] * (cm - sm);
+        if (rot) d[2 * half - k] = w[2] * (cp + sp);
+        if (rot && mir) d[half - k] = w[3] * (cm + sm);
+      } else {
+        d[k] = cp - sp;
+        if (mir) d[half + k] = cm - sm;
+        if (rot) d[2 * half - k] = cp + sp;
+        if (rot && mir) d[half - k] = cm + sm;
+      }
     }
   }
 }
@@ -335,10 +357,10 @@ __global__ void k_phase(double* __restrict__ coef, long long nfield, int p, doub
 
 }  // namespace
 
-template <typename CT, typename R, int KINDS>
+template <typename CT, typename R, int KINDS, bool SRC = false>
 static int synth_launch(const CT* coef, const long long* field_off, long long coef_stride, long long nfield, int p, int P,
                         const R* T0, const R* T1, const R* T2, const R* cs, R* out, long long kind_stride,
-                        long long field_stride, int sms, cudaStream_t s) {
+                        long long field_stride, int sms, cudaStream_t s, SynthSources src = {}) {
   if (nfield == 0) return BIE_OK;
   const int np = (P + 2) / 2;
   const size_t stage = p <= kSynStageP ? sizeof(R) * (size_t)(p + 1) * (p + 1) : 0;
@@ -351,10 +373,10 @@ static int synth_launch(const CT* coef, const long long* field_off, long long co
   const size_t smem = stage + pair * jb;
   const long long nblk = nfield * ((np + jb - 1) / jb);
   if (nblk > 0x7fffffffLL) return BIE_EINVAL;
-  auto kern = k_synth<CT, R, KINDS>;
+  auto kern = k_synth<CT, R, KINDS, SRC>;
   if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kern<<<(unsigned)nblk, kSynThreads, smem, s>>>(coef, field_off, coef_stride, p, P, T0, T1, T2, cs, out, kind_stride,
-                                                 field_stride, jb);
+                                                 field_stride, jb, src);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
@@ -369,14 +391,18 @@ int launch_synth(int kinds, const CT* coef, const long long* field_off, long lon
   return synth_launch<CT, R, K>(coef, field_off, coef_stride, nfield, p, P, T0, T1, T2, cs, out, kind_stride, \
                                 field_stride, sms, s)
   BIE_SYNTH(1);
-  if constexpr (sizeof(R) == 8) {
-    BIE_SYNTH(6);
-    BIE_SYNTH(7);
-    BIE_SYNTH(62);
-    BIE_SYNTH(63);
-  }
+  BIE_SYNTH(6);
+  BIE_SYNTH(7);
+  BIE_SYNTH(62);
+  BIE_SYNTH(63);
 #undef BIE_SYNTH
   return BIE_EINVAL;
+}
+
+template <typename R>
+int launch_synth_sources(const double* coef, const long long* field_off, long long nd, int p, int P, const R* T0,
+                         const R* cs, const SynthSources& src, R* Q, int sms, cudaStream_t s) {
+  return synth_launch<double, R, 1, true>(coef, field_off, 0, 3 * nd, p, P, T0, nullptr, nullptr, cs, Q, 0, 0, sms, s, src);
 }
 
 int launch_analyze(std::vector<AnaGroup> groups, const double* grid, double* coef, int sms, cudaStream_t s) {
@@ -444,9 +470,10 @@ int launch_phase(double* coef, long long nfield, int p, double gamma, cudaStream
 template int launch_synth<double, double>(int, const double*, const long long*, long long, long long, int, int,
                                           const double*, const double*, const double*, const double*, double*,
                                           long long, long long, int, cudaStream_t);
-template int launch_synth<double, float>(int, const double*, const long long*, long long, long long, int, int,
-                                         const float*, const float*, const float*, const float*, float*, long long,
-                                         long long, int, cudaStream_t);
+template int launch_synth_sources<double>(const double*, const long long*, long long, int, int, const double*,
+                                          const double*, const SynthSources&, double*, int, cudaStream_t);
+template int launch_synth_sources<float>(const double*, const long long*, long long, int, int, const float*, const float*,
+                                         const SynthSources&, float*, int, cudaStream_t);
 template int launch_rotate<double, double>(const double*, const long long*, int, long long, int, const double*,
                                            long long, int, int, const double*, double*, long long, cudaStream_t);
 template int launch_rotate<double, float>(const double*, const long long*, int, long long, int, const float*,
