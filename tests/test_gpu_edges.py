@@ -1,0 +1,101 @@
+"""GPU parity at the sizes where the kernels' folds, paddings and splits have their edges.
+
+The transforms fold latitude pairs (a middle latitude exists for an even degree P) and longitude
+quadruples (a middle longitude exists for an odd P), and a block takes more or fewer latitude pairs and
+orders with the number of fields; the dense self factors pad (p+1)^2 to whole 16-byte loads; the rows of
+the near-singular rule fold the standard and the upsampled grid.  Every parity and remainder is
+compared with the FP64 oracle at the bars of the other parity tests."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import layer, sh
+from paper_1707_02156_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+FP64_TOL, MIXED_TOL, DF_TOL = 1e-12, 2e-6, 1e-11
+
+
+@pytest.fixture(scope="module")
+def api():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1707_02156_gb300 import api, build
+    build.build()
+    return api
+
+
+def dev(a):
+    return torch.as_tensor(np.ascontiguousarray(a, dtype=np.float64)).cuda()
+
+
+def host(t):
+    torch.cuda.synchronize()
+    return t.cpu().numpy()
+
+
+def relerr(a, b):
+    a, b = np.asarray(a).ravel(), np.asarray(b).ravel()
+    return max(np.linalg.norm(a - b) / np.linalg.norm(b), np.max(np.abs(a - b)) / np.max(np.abs(b)))
+
+
+@pytest.mark.parametrize("p, P", [(1, 1), (1, 2), (2, 2), (2, 5), (3, 4), (6, 7), (16, 31), (48, 48), (49, 49), (64, 64), (5, 129)])
+@pytest.mark.parametrize("ndrop", [1, 40])
+def test_transforms_at_every_grid_parity(api, p, P, ndrop):
+    rng = np.random.default_rng(100 * p + P)
+    coefs = [inputs.random_bandlimited(rng, p, 3, decay_pow=0.5) for _ in range(2)]
+    ctx = api.Context(0)
+    c = dev(np.concatenate([coefs[d % 2].ravel() for d in range(ndrop)]))
+    g = torch.full((ndrop, 3, (P + 1) * (2 * P + 2)), float("nan"), dtype=torch.float64, device="cuda")
+    ctx.sh_synthesize([p] * ndrop, [P] * ndrop, 3, c, g)
+    gh = host(g)
+    for d in {0, ndrop - 1}:
+        for k in range(3):
+            assert relerr(gh[d, k], sh.synthesize(coefs[d % 2][k], p, P)) < FP64_TOL
+    if p == P:
+        back = torch.full_like(c, float("nan"))
+        ctx.sh_analyze([p] * ndrop, 3, g, back)
+        assert relerr(host(back), host(c)) < FP64_TOL
+    ctx.close()
+
+
+@pytest.mark.parametrize("p, double", [(1, False), (1, True), (2, False), (3, True), (4, False), (7, False), (10, True)])
+def test_dense_self_term_at_every_row_padding(api, p, double):
+    w = inputs.perturbed_drop(p=p, pq=None if double else p, lam=3.0, nmax=min(p, 6))
+    ctx = api.Context(0)
+    geo = ctx.geometry(w.p, w.pq, dev(w.xcoef), w.lam)
+    drops = layer.Drops([w.xcoef.reshape(3, -1)], w.p, w.pq, w.lam)
+    f = dev(w.density)
+    out = torch.zeros_like(f)
+    for fn, ref in ((geo.apply_single, drops.apply_single), (geo.apply_double, drops.apply_double)):
+        r = ref([w.density])[0]
+        for prec, tol in ((0, FP64_TOL), (1, MIXED_TOL), (2, DF_TOL)):
+            fn(f, out, precision=prec)
+            assert relerr(host(out), r) < tol, (prec,)
+    geo.close()
+    ctx.close()
+
+
+@pytest.mark.parametrize("p, up", [(6, 2), (7, 3), (8, 1), (9, 4)])
+def test_near_rows_at_every_grid_parity(api, p, up):
+    w = inputs.two_drops(p=p, gap=0.05, up=up, lam=0.5)
+    nc = 3 * (p + 1) ** 2
+    xs = [w.xcoef[:nc].reshape(3, -1), w.xcoef[nc:].reshape(3, -1)]
+    fs = [w.density[:nc].reshape(3, -1), w.density[nc:].reshape(3, -1)]
+    drops = layer.Drops(xs, w.p, w.pq, w.lam, up=up)
+    ctx = api.Context(0, upsample=up)
+    geo = ctx.geometry(w.p, w.pq, dev(w.xcoef), w.lam)
+    assert geo.info["near_targets"] == sum(int(np.sum(r == 2)) for r in drops.region.values()) > 0
+    f = dev(w.density)
+    out = torch.zeros_like(f)
+    for fn, ref in ((geo.apply_single, drops.apply_single), (geo.apply_double, drops.apply_double)):
+        r = np.concatenate([v.ravel() for v in ref(fs)])
+        for prec, tol in ((0, FP64_TOL), (1, 5e-6)):
+            for _ in range(3):  # the rows are built by the first apply, the third one is a graph replay
+                out.fill_(float("nan"))
+                fn(f, out, precision=prec)
+                assert relerr(host(out), r) < tol, (prec,)
+    geo.close()
+    ctx.close()
