@@ -389,33 +389,6 @@ static bool group_uses_direct(const bie_ctx* ctx, const bie_geom::Group& G) {
   return ctx->cfg.self_direct != 0 || kernel_proj_smem(G.p, G.pq) > 227 * 1024;
 }
 
-// Dense-form factors of one group, built from the FP64 rotated-grid cache: the projected factors of a
-// chunk of latitude rows into temporaries, then the transposed rotation to their final place.
-static int ensure_qk(bie_ctx* ctx, bie_geom::Group& G, int kind, DevBuf<double>& work, cudaStream_t s) {
-  if (G.qk64[kind].ptr) return BIE_OK;
-  Plan *pl, *pp;
-  WigPlan* wp;
-  BIE_TRY(get_plan(ctx, G.p, G.pq, &pl));
-  BIE_TRY(get_plan(ctx, G.p, G.p, &pp));
-  BIE_TRY(get_wig(ctx, G.p, &wp));
-  const long long nb = 2 * G.p + 2, rows = (long long)G.drops.size() * (G.p + 1);
-  const long long per_row = nb * 6 * (long long)(G.p + 1) * (G.p + 2), nq = ngrid(G.pq);
-  const long long n = rows * nb * 6 * self_row(G.p);
-  const long long chunk = std::max(1LL, std::min<long long>(rows, kWorkBudget / (4 * 8 * per_row)));
-  BIE_TRY(G.qk64[kind].alloc(n));
-  BIE_TRY(G.qk32[kind].alloc(n));
-  BIE_TRY(work.alloc(chunk * per_row));
-  Phase ph(ctx, "kernel_proj", s);
-  for (long long r0 = 0; r0 < rows; r0 += chunk) {
-    const long long rn = std::min(chunk, rows - r0);
-    BIE_TRY(launch_kernel_proj(kind, G.cache64.ptr + r0 * nb * 7 * nq, rn * nb, G.p, G.pq, pl->cs.ptr, pl->T0.ptr,
-                               work.ptr, s));
-    BIE_TRY(launch_unrotate(work.ptr, r0, rn, G.p, wp->blk.ptr, wp->stride, pp->cs.ptr, G.qk64[kind].ptr,
-                            G.qk32[kind].ptr, s));
-  }
-  return BIE_OK;
-}
-
 // Dense factors of one group in the arithmetic type R (the double-float copy is split from the
 // FP64 factors on first use).
 template <typename R>
@@ -629,8 +602,8 @@ static int group_records(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, int P, d
 }
 
 static int setup_group(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, cudaStream_t s) {
-  const int p = G.p, pq = G.pq;
-  const long long ng = ngrid(p), nq = ngrid(pq), nc = ncoef(p);
+  const int p = G.p;
+  const long long ng = ngrid(p), nc = ncoef(p);
   const int nd = (int)G.drops.size();
   // offsets
   std::vector<long long> foff3(3 * nd), goff3(3 * nd), voff(nd), roff(nd), so(nd), sof(nd);
@@ -668,37 +641,69 @@ static int setup_group(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, cudaStream
     BIE_TRY(group_records(ctx, g, G, p, g->rec_std.ptr, G.src_off_std.ptr, s));
   }
 
-  // rotated-grid cache of the singular rule (Sec. 2.2), chunked over drops
-  Phase ph(ctx, "setup_rotcache", s);
+  return BIE_OK;
+}
+
+// The self rule of one group (Sec. 2.2).  Direct form: the rotated-grid cache of every target, kept.  Dense
+// form: the cache of a chunk of targets, the projected kernel factors of both layers from it and their
+// transposed rotation to the final place, chunk by chunk through one workspace (whole drops, or some
+// latitudes of one drop when a drop alone is larger), so that set-up needs 2 GB beside the factors and not
+// the cache of all targets (45 GB for 512 drops of degree 24, whose allocation and release cost as much as
+// a tenth of the work: 64 drops, 5.7 GB of cache, 197 -> 190 ms with force and right-hand side).
+static int setup_self(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, DevBuf<double>& work, cudaStream_t s) {
+  const int p = G.p, pq = G.pq;
+  const long long ng = ngrid(p), nq = ngrid(pq), nc = ncoef(p), nb = 2 * p + 2;
+  const int nd = (int)G.drops.size();
+  const bool direct = group_uses_direct(ctx, G);
   Plan *pl, *pp;
   WigPlan* wp;
   BIE_TRY(get_plan(ctx, p, pq, &pl));
   BIE_TRY(get_plan(ctx, p, p, &pp));
   BIE_TRY(get_wig(ctx, p, &wp));
-  BIE_TRY(G.cache64.alloc((size_t)nd * ng * 7 * nq));
-  const long long per = ng * 3 * nc + 3 * ng * 3 * nq;
-  int chunk = (int)std::max(1LL, std::min<long long>(nd, (2 * kWorkBudget) / (8 * per)));
-  DevBuf<double> work;
-  BIE_TRY(work.alloc((size_t)chunk * per));
-  for (int c0 = 0; c0 < nd; c0 += chunk) {
-    const int cn = std::min(chunk, nd - c0);
-    double* RC = work.ptr;
-    double* X = RC + cn * ng * 3 * nc;
-    double* Xt = X + cn * ng * 3 * nq;
-    double* Xp = Xt + cn * ng * 3 * nq;
-    // x coefficients of the chunk's drops: field offsets into the geometry's copy
-    BIE_TRY((launch_rotate<double, double>(g->xcoef.ptr, G.foff3.ptr + 3 * c0, 3, cn, p, wp->blk.ptr, wp->stride,
-                                           p + 1, 2 * p + 2, pp->cs.ptr, RC, ng * 3 * nc, s)));
-    BIE_TRY(synth_xderivs(ctx, RC, nullptr, nc, cn * ng * 3, p, pq, X, s));
-    // the targets x0 of the chunk's drops, wherever each drop's records lie (a degree group's drops
-    // are in general not adjacent in rec_std)
-    BIE_TRY(launch_rotgeo<double>(X, Xt, Xp, cn, (int)ng, pq, g->rec_std.ptr, G.roff.ptr + c0, pl->wsq.ptr,
-                                  G.cache64.ptr + (long long)c0 * ng * 7 * nq, s));
-    BIE_CUDA_TRY(cudaStreamSynchronize(s));
+  // doubles per target: rotated coefficients, x and its derivatives, and in dense form the cache and the
+  // projected factors of one layer
+  const long long nQ = 6LL * (p + 1) * (p + 2);
+  const long long per = 3 * nc + 9 * nq + (direct ? 0 : 7 * nq + nQ);
+  const long long fit = std::max<long long>(nb, (2LL << 30) / 8 / per);  // targets at a time
+  const int dstep = (int)std::max<long long>(1, std::min<long long>(nd, fit / ng));
+  const int astep = (int)std::max<long long>(1, std::min<long long>(p + 1, fit / nb));
+  if (direct) {
+    BIE_TRY(G.cache64.alloc((size_t)nd * ng * 7 * nq));
+  } else {
+    for (int kind = 0; kind < 2; ++kind) {
+      BIE_TRY(G.qk64[kind].alloc(nd * ng * 6 * (long long)self_row(p)));
+      BIE_TRY(G.qk32[kind].alloc(G.qk64[kind].n));
+    }
+  }
+  BIE_TRY(work.alloc((size_t)(dstep > 1 ? dstep * ng : astep * nb) * per));
+  for (int d0 = 0; d0 < nd; d0 += dstep) {
+    const int dn = std::min(dstep, nd - d0);
+    for (int a0 = 0; a0 <= p; a0 += dn > 1 ? p + 1 : astep) {
+      const int an = dn > 1 ? p + 1 : std::min(astep, p + 1 - a0);
+      const long long nt = dn * an * nb, t0 = d0 * ng + a0 * nb;  // targets of the chunk, the group's first one
+      double* RC = work.ptr;
+      double* X = RC + nt * 3 * nc;
+      double* cache = direct ? G.cache64.ptr + t0 * 7 * nq : X + nt * 9 * nq;
+      double* Q = cache + nt * 7 * nq;
+      {
+        Phase ph(ctx, "setup_rotcache", s);
+        BIE_TRY((launch_rotate<double, double>(g->xcoef.ptr, G.foff3.ptr + 3 * d0, 3, dn, p, wp->blk.ptr + a0 * wp->stride,
+                                               wp->stride, an, (int)nb, pp->cs.ptr, RC, an * nb * 3 * nc, s)));
+        BIE_TRY(synth_xderivs(ctx, RC, nullptr, nc, nt * 3, p, pq, X, s));
+        BIE_TRY(launch_rotgeo<double>(X, X + nt * 3 * nq, X + nt * 6 * nq, dn, (int)(an * nb), (int)(a0 * nb), (int)ng, pq,
+                                      g->rec_std.ptr, G.roff.ptr + d0, pl->wsq.ptr, cache, s));
+      }
+      if (direct) continue;
+      Phase ph(ctx, "kernel_proj", s);
+      for (int kind = 0; kind < 2; ++kind) {
+        BIE_TRY(launch_kernel_proj(kind, cache, nt, p, pq, pl->cs.ptr, pl->T0.ptr, Q, s));
+        BIE_TRY(launch_unrotate(Q, t0 / nb, nt / nb, p, wp->blk.ptr, wp->stride, pp->cs.ptr, G.qk64[kind].ptr,
+                                G.qk32[kind].ptr, s));
+      }
+    }
   }
   return BIE_OK;
 }
-
 
 // ---------------------------------------------------------------------------------------------
 // inter-drop set-up (Sec. 2.3): centres, volumes and mean radii, upsampled grids, source records,
@@ -2729,14 +2734,10 @@ int bie_geometry_setup(bie_ctx* ctx, int ndrop, const int* p, const int* pq, con
     self_pairs += (long long)G->drops.size() * ngrid(G->p) * ngrid(G->pq);
   }
   if (ndrop > 1) BIE_TRY(setup_interdrop(ctx, g.get(), s));
-  // dense-form groups: both kinds' factors now, then the rotated-grid cache is no longer needed
-  DevBuf<double> qwork;
-  for (auto& G : g->groups) {
-    if (group_uses_direct(ctx, *G)) continue;
-    BIE_TRY(ensure_qk(ctx, *G, 0, qwork, s));
-    BIE_TRY(ensure_qk(ctx, *G, 1, qwork, s));
+  {
+    DevBuf<double> work;  // for all groups
+    for (auto& G : g->groups) BIE_TRY(setup_self(ctx, g.get(), *G, work, s));
     BIE_CUDA_TRY(cudaStreamSynchronize(s));
-    G->cache64.release();
   }
   BIE_CUDA_TRY(cudaStreamSynchronize(s));
   g->info.ndrop = ndrop;

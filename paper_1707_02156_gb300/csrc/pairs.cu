@@ -50,17 +50,17 @@ __global__ void k_surface(const double* __restrict__ X, const double* __restrict
 // kernels need the normal only with its weight, so it is never divided by W').
 template <typename R>
 __global__ void k_rotgeo(const double* __restrict__ X, const double* __restrict__ Xt, const double* __restrict__ Xp,
-                         long long ndrop, int ng, int pq, const double* __restrict__ rec_std,
+                         long long ndrop, int nt, int tl0, int ng, int pq, const double* __restrict__ rec_std,
                          const long long* __restrict__ rec_off, const double* __restrict__ wsq,
                          R* __restrict__ cache) {
   const int nk = 2 * pq + 2;
   const long long nq = (long long)(pq + 1) * nk;
   long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  long long total = ndrop * ng * nq;
+  long long total = ndrop * nt * nq;
   if (idx >= total) return;
   long long t = idx / nq;
   long long q = idx - t * nq;
-  long long ld = t / ng, tl = t - ld * ng;
+  long long ld = t / nt, tl = tl0 + t - ld * nt;
   int j = (int)(q / nk);
   double x[3], xt[3], xp[3], c[3];
   for (int i = 0; i < 3; ++i) {
@@ -159,19 +159,17 @@ int launch_surface(const double* X, const double* Xt, const double* Xp, long lon
 }
 
 template <typename R>
-int launch_rotgeo(const double* X, const double* Xt, const double* Xp, long long ndrop, int ng, int pq,
+int launch_rotgeo(const double* X, const double* Xt, const double* Xp, long long ndrop, int nt, int tl0, int ng, int pq,
                   const double* rec_std, const long long* rec_off, const double* wsq, R* cache, cudaStream_t s) {
-  long long n = ndrop * ng * (long long)(pq + 1) * (2 * pq + 2);
+  long long n = ndrop * nt * (long long)(pq + 1) * (2 * pq + 2);
   if (n == 0) return BIE_OK;
-  k_rotgeo<R><<<blocks_for(n), kThreads, 0, s>>>(X, Xt, Xp, ndrop, ng, pq, rec_std, rec_off, wsq, cache);
+  k_rotgeo<R><<<blocks_for(n), kThreads, 0, s>>>(X, Xt, Xp, ndrop, nt, tl0, ng, pq, rec_std, rec_off, wsq, cache);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
 }
 
-template int launch_rotgeo<double>(const double*, const double*, const double*, long long, int, int, const double*,
-                                   const long long*, const double*, double*, cudaStream_t);
-template int launch_rotgeo<float>(const double*, const double*, const double*, long long, int, int, const double*,
-                                  const long long*, const double*, float*, cudaStream_t);
+template int launch_rotgeo<double>(const double*, const double*, const double*, long long, int, int, int, int,
+                                   const double*, const long long*, const double*, double*, cudaStream_t);
 }  // namespace bie
 
