@@ -54,7 +54,7 @@ template <typename R>
 int launch_synth_sources(const double* coef, const long long* field_off, long long nd, int p, int P, const R* T0,
                          const R* cs, const SynthSources& src, R* Q, int sms, cudaStream_t s);
 // analysis: grids (degree P) -> coefficients (degree p <= P), FP64, for several degree groups in one launch.
-// Offsets per field, or null and a stride; begin and mb are set by the launcher.
+// Offsets per field, or null and a stride; begin is set by the launcher.
 struct AnaGroup {
   long long begin, nfield;
   const long long* grid_off;
@@ -62,11 +62,11 @@ struct AnaGroup {
   long long grid_base, grid_stride, coef_base, coef_stride;  // grid f at base + (off[f] or f stride)
   const double* cs;
   const double* At;  // weighted Legendre table, rows (m, j) with the degree n = m..p fastest
-  int P, p, mb;
+  int P, p;
 };
 constexpr int kMaxAnaGroups = 8;
 struct AnaGroups {
-  int n;
+  int n, cl, orders;  // groups; blocks per field, or (orders) one block per field and order
   AnaGroup g[kMaxAnaGroups];
 };
 int launch_analyze(std::vector<AnaGroup> groups, const double* grid, double* coef, int sms, cudaStream_t s);

@@ -11,6 +11,7 @@
 // the direct sums in two kernels: the rotated grids of 64 drops of degree 24 (80000 targets x 3 fields x 3
 // kinds) 103.5 -> 62.7 ms with their rotation, the projection of 192 drops of degree 24 0.52 -> 0.076 ms, the
 // surfactant's rates and implicit stage of 48 drops 10.4 -> 6.2 ms.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -21,6 +22,8 @@
 namespace bie {
 
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int kThreads = 256;
 
@@ -180,33 +183,48 @@ __global__ void __launch_bounds__(kSynThreads) k_synth(const CT* __restrict__ co
   }
 }
 
-// One block per (field, mb orders).  The field's rows pass through shared memory kr at a time, folded over
-// the four longitudes of each quadruple into what the even and odd orders' cosine and sine sums
-// need; F[m][j] for the block's orders; then F folded over the latitude pairs and the products with the
-// weighted Legendre table (stored with the degree fastest, so that neighbouring threads read
-// neighbouring entries).  Several degree groups share a launch: block ranges per group, arguments by value.
+// One cluster of cl blocks per field (cl = 1, 2, 4 or 8).  Block r of the cluster takes every cl-th part of the
+// field's rows: they pass through shared memory kr at a time, folded over the four longitudes of each
+// quadruple into what the even and odd orders' cosine and sine sums need, and F(m, row) of all orders stays
+// in the block's shared memory.  Then block r takes the orders m = r, r + cl, ...: it folds F(m, .) over the
+// latitude pairs (rows of the other blocks through distributed shared memory) and forms the products with
+// the weighted Legendre table (stored with the degree fastest, so that neighbouring threads read
+// neighbouring entries).  A large batch has one block per field; fewer fields spread over cl blocks each, so
+// that every row is folded once however many blocks share a field (blocks of some orders, each folding the
+// whole field, spend four fifths of their additions on that: 16 fields of degree 32 on the degree-65
+// grid 27 us, 22 by clusters).  Only when every order of every field can have a block of its own on the SMs
+// (one drop) do the blocks take one order each and fold the whole field: no block then waits for another
+// (one drop of degree 32: 12 us, 16 by clusters).  Several degree groups share a launch: block ranges per
+// group, arguments by value.
 constexpr int kAnaThreads = 256;
 
-__host__ __device__ inline int ana_rows(int P) { return P < 64 ? 32 : P < 128 ? 16 : 8; }
+__host__ __device__ inline int ana_rows(int P, int cl) {  // rows per pass: at most 40 KB folded
+  const int own = (P + cl) / cl, fit = (40 << 10) / (32 * ((P + 1) / 2 + 1));
+  return own < fit ? own : fit < 1 ? 1 : fit;
+}
 
 __global__ void __launch_bounds__(kAnaThreads) k_analyze(AnaGroups G, const double* __restrict__ grid,
                                                          double* __restrict__ coef) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  cg::cluster_group cluster = cg::this_cluster();
   AnaGroup A = G.g[0];
 #pragma unroll
   for (int i = 1; i < kMaxAnaGroups; ++i)
     if (i < G.n && (long long)blockIdx.x >= G.g[i].begin) A = G.g[i];
-  const int P = A.P, p = A.p, mb = A.mb;
-  const int nj = P + 1, nk = 2 * P + 2, half = P + 1, np = (nj + 1) / 2, k4n = half / 2 + 1, kr = ana_rows(P);
-  const int nmb = (p + mb) / mb;
-  const long long bl = (long long)blockIdx.x - A.begin;
-  const long long f = bl / nmb;
-  const int m0 = (int)(bl - f * nmb) * mb, mn = min(mb, p + 1 - m0);
-  double* F = reinterpret_cast<double*>(smem_raw);  // [mb][nj][2]
-  double* fold = F + 2 * (long long)mb * nj;        // [cos even, cos odd, sin even, sin odd][k4n][kr]
+  // one order per block (G.orders): the block's only row part is the whole field, its only order m_own
+  const int P = A.P, p = A.p, cl = G.cl, rank = (int)cluster.block_rank();
+  const int per_f = G.orders ? p + 1 : cl;
+  const int nj = P + 1, nk = 2 * P + 2, half = P + 1, np = (nj + 1) / 2, k4n = half / 2 + 1, kr = ana_rows(P, cl);
+  const long long f = ((long long)blockIdx.x - A.begin) / per_f;
+  const int m_own = G.orders ? (int)((long long)blockIdx.x - A.begin - f * per_f) : 0, nm = G.orders ? 1 : p + 1;
+  const int own = (nj + cl - 1) / cl;  // rows per block: rank * own ..
+  const int r0 = rank * own, r1 = min(nj, r0 + own);
+  double* F = reinterpret_cast<double*>(smem_raw);      // [own][nm][2]
+  double* fold = F + 2LL * own * nm;               // [cos even, cos odd, sin even, sin odd][k4n][kr]
+  double* E = fold;                                     // later: [nj][2] per order of a pass
   const double* src = grid + A.grid_base + (A.grid_off ? A.grid_off[f] : f * A.grid_stride);
-  for (int j0 = 0; j0 < nj; j0 += kr) {
-    const int rn = min(kr, nj - j0);
+  for (int j0 = r0; j0 < r1; j0 += kr) {
+    const int rn = min(kr, r1 - j0);
     for (int i = threadIdx.x; i < rn * k4n; i += kAnaThreads) {
       const int r = i / k4n, k = i - r * k4n;
       const double* g = src + (long long)(j0 + r) * nk;
@@ -221,51 +239,79 @@ __global__ void __launch_bounds__(kAnaThreads) k_analyze(AnaGroups G, const doub
       o[3 * k4n * kr] = amb - cmd;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < mn * kr; i += kAnaThreads) {
-      const int mm = i / kr, r = i - mm * kr;
-      if (r >= rn) continue;
-      const int m = m0 + mm, odd = m & 1;
+    for (int i = threadIdx.x; i < nm * rn; i += kAnaThreads) {
+      const int mi = i / rn, r = i - mi * rn, m = m_own + mi, odd = m & 1;
       const double* c = A.cs + (long long)m * nk * 2;
       const double* fc = fold + (long long)odd * k4n * kr + r;
       const double* fs = fold + (long long)(2 + odd) * k4n * kr + r;
       double re = 0, im = 0;
+#pragma unroll 4
       for (int k = 0; k < k4n; ++k) {
         re += fc[k * kr] * c[2 * k];
         im -= fs[k * kr] * c[2 * k + 1];
       }
-      F[(mm * nj + j0 + r) * 2] = re;
-      F[(mm * nj + j0 + r) * 2 + 1] = im;
+      double* o = F + 2 * ((long long)(j0 - r0 + r) * nm + mi);
+      o[0] = re;
+      o[1] = im;
     }
     __syncthreads();
   }
-  // latitude pairs: F(j) + F(P-j) at j for even n - m, F(j) - F(P-j) at P-j for odd
-  for (int i = threadIdx.x; i < mn * (nj / 2) * 2; i += kAnaThreads) {
-    const int ri = i & 1, r = i >> 1, mm = r / (nj / 2), j = r - mm * (nj / 2);
-    double* lo = F + (mm * nj + j) * 2 + ri;
-    double* hi = F + (mm * nj + P - j) * 2 + ri;
-    const double a = *lo, b = *hi;
-    *lo = a + b;
-    *hi = a - b;
-  }
-  __syncthreads();
+  cluster.sync();
   double* out = coef + A.coef_base + (A.coef_off ? A.coef_off[f] : f * A.coef_stride);
-  const int per = p + 1 - m0;  // degrees of the block's lowest order
-  for (int i = threadIdx.x; i < mn * per; i += kAnaThreads) {
-    const int mm = i / per, d = i - mm * per, m = m0 + mm, n = m + d;
-    if (n > p) continue;
-    const bool odd = d & 1;
-    const double* a = A.At + leg_row(p, m, m, nj) + d;
-    const double* Fm = F + (long long)mm * nj * 2;
-    double re = 0, im = 0;
-    for (int j = 0; j < (odd ? nj / 2 : np); ++j) {
-      const double v = a[(long long)j * (p + 1 - m)];
-      const int jj = odd ? P - j : j;
-      re += v * Fm[2 * jj];
-      im += v * Fm[2 * jj + 1];
+  const int mp = max(1, 2 * k4n * kr / nj);  // orders per pass: E in the space of the folded rows
+  for (int a0 = m_own + rank; a0 < m_own + nm; a0 += cl * mp) {
+    const int mn = min(mp, (m_own + nm - 1 - a0) / cl + 1);  // orders a0, a0 + cl, ...
+    // latitude pairs: F(j) + F(P-j) at j for even n - m, F(j) - F(P-j) at P-j for odd
+    for (int i = threadIdx.x; i < mn * np; i += kAnaThreads) {
+      const int mm = i / np, j = i - mm * np, m = a0 + mm * cl, jm = P - j;
+      const double* lo = cluster.map_shared_rank(F, j / own) + 2 * ((long long)(j % own) * nm + m - m_own);
+      const double* hi = cluster.map_shared_rank(F, jm / own) + 2 * ((long long)(jm % own) * nm + m - m_own);
+      const double ar = lo[0], ai = lo[1], br = hi[0], bi = hi[1];
+      double* e = E + 2 * (long long)mm * nj;
+      if (j == jm) {  // the middle latitude is its own mirror
+        e[2 * j] = ar;
+        e[2 * j + 1] = ai;
+      } else {
+        e[2 * j] = ar + br;
+        e[2 * j + 1] = ai + bi;
+        e[2 * jm] = ar - br;
+        e[2 * jm + 1] = ai - bi;
+      }
     }
-    out[n * (n + 1) + m] = re;
-    if (m > 0) out[n * (n + 1) - m] = im;
+    __syncthreads();
+    const int per = p + 1 - a0;  // degrees of the pass's lowest order
+    // a pass of few sums splits each over four neighbouring threads (a quarter of the serial loads), a pass of
+    // many does not (the partial sums would cost half as many additions again)
+    const int split = mn * per <= kAnaThreads / 4 ? 4 : 1;
+    for (int i0 = 0; i0 < mn * per * split; i0 += kAnaThreads) {
+      const int i = (i0 + (int)threadIdx.x) / split, part = threadIdx.x % split;
+      const int mm = i / per, d = i - mm * per, m = a0 + mm * cl, n = m + d;
+      const bool valid = i < mn * per && n <= p;
+      double re = 0, im = 0;
+      if (valid) {
+        const bool odd = d & 1;
+        const double* a = A.At + leg_row(p, m, m, nj) + d;
+        const double* Em = E + 2 * (long long)mm * nj;
+#pragma unroll 4
+        for (int j = part; j < (odd ? nj / 2 : np); j += split) {
+          const double v = a[(long long)j * (p + 1 - m)];
+          const int jj = odd ? P - j : j;
+          re += v * Em[2 * jj];
+          im += v * Em[2 * jj + 1];
+        }
+      }
+      if (split > 1)
+        for (int o = 2; o > 0; o >>= 1) {
+          re += __shfl_xor_sync(0xffffffffu, re, o);
+          im += __shfl_xor_sync(0xffffffffu, im, o);
+        }
+      if (!valid || part) continue;
+      out[n * (n + 1) + m] = re;
+      if (m > 0) out[n * (n + 1) - m] = im;
+    }
+    __syncthreads();
   }
+  cluster.sync();  // a block's F stays until the others have read it
 }
 
 constexpr int kRotB = 16;  // targets (longitudes) per rotation block
@@ -374,7 +420,7 @@ static int synth_launch(const CT* coef, const long long* field_off, long long co
   const long long nblk = nfield * ((np + jb - 1) / jb);
   if (nblk > 0x7fffffffLL) return BIE_EINVAL;
   auto kern = k_synth<CT, R, KINDS, SRC>;
-  if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   kern<<<(unsigned)nblk, kSynThreads, smem, s>>>(coef, field_off, coef_stride, p, P, T0, T1, T2, cs, out, kind_stride,
                                                  field_stride, jb, src);
   count_launch();
@@ -413,23 +459,44 @@ int launch_analyze(std::vector<AnaGroup> groups, const double* grid, double* coe
   for (size_t g0 = 0; g0 < groups.size(); g0 += kMaxAnaGroups) {
     AnaGroups G{};
     G.n = (int)std::min<size_t>(kMaxAnaGroups, groups.size() - g0);
+    for (int i = 0; i < G.n; ++i) G.g[i] = groups[g0 + i];
+    long long orders = 0;
+    for (int i = 0; i < G.n; ++i) orders += G.g[i].nfield * (G.g[i].p + 1);
+    G.orders = orders <= sms;
+    auto bytes = [&](int cl) {
+      size_t v = 0;
+      for (int i = 0; i < G.n; ++i) {
+        const int P = G.g[i].P;
+        v = std::max(v, sizeof(double) * (2 * (size_t)((P + cl) / cl) * (G.orders ? 1 : G.g[i].p + 1) +
+                                          std::max(4 * (size_t)((P + 1) / 2 + 1) * ana_rows(P, cl), 2 * (size_t)(P + 1))));
+      }
+      return v;
+    };
+    // blocks per field: as few as give two blocks per SM, and as many as the largest group's F needs
+    G.cl = 1;
+    while (!G.orders && G.cl < 8 && (fields * G.cl < 2LL * sms || bytes(G.cl) > 96 * 1024)) G.cl *= 2;
+    const size_t smem = bytes(G.cl);
+    if (smem > 227 * 1024) return BIE_EINVAL;
     long long nblk = 0;
-    size_t smem = 0;
     for (int i = 0; i < G.n; ++i) {
-      AnaGroup& g = G.g[i] = groups[g0 + i];
-      // orders per block: every block folds the whole field, so as many as leave four blocks per SM, at
-      // most 32 KB of F
-      const long long want = std::max(1LL, fields * (g.p + 1) / (4LL * sms));
-      const long long fit = std::max<long long>(1, (32 << 10) / (16LL * (g.P + 1)));
-      g.mb = (int)std::min<long long>(g.p + 1, std::min(want, fit));
-      g.begin = nblk;
-      nblk += g.nfield * ((g.p + g.mb) / g.mb);
-      smem = std::max(smem, sizeof(double) * (2 * (size_t)g.mb * (g.P + 1) + 4 * (size_t)((g.P + 1) / 2 + 1) * ana_rows(g.P)));
+      G.g[i].begin = nblk;
+      nblk += G.g[i].nfield * (G.orders ? G.g[i].p + 1 : G.cl);
     }
     if (nblk == 0) continue;
     if (nblk > 0x7fffffffLL) return BIE_EINVAL;
-    if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(k_analyze, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_analyze<<<(unsigned)nblk, kAnaThreads, smem, s>>>(G, grid, coef);
+    if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(k_analyze, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)G.cl;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)nblk);
+    cfg.blockDim = dim3(kAnaThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    BIE_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_analyze, G, grid, coef));
     count_launch();
     BIE_CUDA_TRY(cudaGetLastError());
   }
