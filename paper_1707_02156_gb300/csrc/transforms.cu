@@ -39,10 +39,15 @@ __host__ __device__ constexpr int kind_slot(int kinds, int k) {
 constexpr int kSynThreads = 128;
 constexpr int kSynStageP = BIE_MAX_P;  // coefficients are staged in shared memory up to this degree
 
-// One block per (field, jb latitude pairs j and P - j).  Phase 1, thread per (order m, pair): the sums
-// over even and odd n - m with the Legendre tables asked for, for both latitudes, and from them each
-// kind's complex value per order (factors i m and -m^2, and the 2 of m > 0) in shared memory
-// h[kind][row][m].  Phase 2, thread per (row, longitude quadruple).  With SRC (values only) field 3 d + c is
+// One block per (field, jb latitude pairs j and P - j).  Phase 1, thread per (Legendre table, orders m and p - m,
+// pair): the sums over even and odd n - m for both latitudes, and from them the complex value per order of
+// each kind that the table serves (factors i m and -m^2, and the 2 of m > 0) in shared memory
+// h[kind][row][m].  Phase 2, thread per (kind, row, longitude quadruple).  The two orders make every
+// thread's sums p + 2 long, and the tables and kinds go to threads of their own: a block of one latitude
+// pair (a few fields spread over the SMs) otherwise ran two warps, the second with one lane, each as long
+// as its lowest order: 16 fields of degree 32 with five kinds on the degree-65 grid 50 -> 42 us (cold cache),
+// the rotated grids of 64 drops of degree 24 56.8 -> 50.3 ms.  Where the block has a thread for every order
+// anyway, each takes one.  With SRC (values only) field 3 d + c is
 // component c of drop d's density, and the weighted source w_s f(s) goes to the sources' place instead of
 // the value to a grid.
 template <typename CT, typename R, int KINDS, bool SRC>
@@ -68,87 +73,78 @@ __global__ void __launch_bounds__(kSynThreads) k_synth(const CT* __restrict__ co
     for (int i = threadIdx.x; i < (p + 1) * (p + 1); i += kSynThreads) c[i] = (R)cg[i];
     __syncthreads();
   }
-  for (int i = threadIdx.x; i < (p + 1) * jbn; i += kSynThreads) {
-    const int m = i / jbn, q = i - m * jbn, j = q0 + q;
-    R e[3][2], o[3][2];  // [table][re, im], sums over even and odd n - m
-#pragma unroll
-    for (int t = 0; t < 3; ++t) e[t][0] = e[t][1] = o[t][0] = o[t][1] = 0;
-    const long long row = leg_row(p, m, m, nj) + j;
-    for (int n = m; n <= p; ++n) {
-      const int at = n * (n + 1);
-      const R re = staged ? c[at + m] : (R)cg[at + m], im = m == 0 ? (R)0 : staged ? c[at - m] : (R)cg[at - m];
-      const long long r = row + (long long)(n - m) * nj;
-      const bool odd = (n - m) & 1;
-#pragma unroll
-      for (int t = 0; t < 3; ++t) {
-        // tables 0, 1, 2 serve the kinds {f, p, pp}, {t, tp}, {tt}
-        if (!(KINDS & (t == 0 ? 37 : t == 1 ? 18 : 8))) continue;
-        const R v = t == 0 ? T0[r] : t == 1 ? T1[r] : T2[r];
-        if (odd) {
-          o[t][0] += re * v;
-          o[t][1] += im * v;
-        } else {
-          e[t][0] += re * v;
-          e[t][1] += im * v;
+  constexpr int TABS = ((KINDS & 37) != 0) | ((KINDS & 18) != 0) << 1 | ((KINDS & 8) != 0) << 2;  // {f, p, pp}, {t, tp}, {tt}
+  constexpr int NT = (TABS & 1) + (TABS >> 1 & 1) + (TABS >> 2);
+  const bool both = NT * (p + 1) * jbn > kSynThreads;
+  const int mh = both ? p / 2 + 1 : p + 1;  // orders a and p - a, or a alone
+  for (int i = threadIdx.x; i < NT * mh * jbn; i += kSynThreads) {
+    const int q = i % jbn, a = i / jbn % mh, j = q0 + q;
+    int t = i / (jbn * mh);  // the t-th table in use
+    if (!(TABS & 1)) ++t;
+    if (t > 0 && !(TABS & 2)) ++t;
+    const R* T = t == 0 ? T0 : t == 1 ? T1 : T2;
+    for (int half_m = 0; half_m < 2; ++half_m) {
+      const int m = half_m ? p - a : a;
+      if (half_m && (!both || m == a)) break;
+      R er = 0, ei = 0, odr = 0, odi = 0;  // sums over even and odd n - m
+      const R* Tm = T + leg_row(p, m, m, nj) + j;
+      int n = m;
+#pragma unroll 2
+      for (; n + 1 <= p; n += 2) {
+        const int at = n * (n + 1), bt = at + 2 * n + 2;
+        const R v = Tm[(long long)(n - m) * nj], w = Tm[(long long)(n + 1 - m) * nj];
+        const R r0 = staged ? c[at + m] : (R)cg[at + m], r1 = staged ? c[bt + m] : (R)cg[bt + m];
+        er += r0 * v;
+        odr += r1 * w;
+        if (m > 0) {
+          const R i0 = staged ? c[at - m] : (R)cg[at - m], i1 = staged ? c[bt - m] : (R)cg[bt - m];
+          ei += i0 * v;
+          odi += i1 * w;
         }
       }
-    }
-    const R fac = m == 0 ? 1 : 2;
+      if (n <= p) {
+        const int at = n * (n + 1);
+        const R v = Tm[(long long)(n - m) * nj];
+        er += (staged ? c[at + m] : (R)cg[at + m]) * v;
+        if (m > 0) ei += (staged ? c[at - m] : (R)cg[at - m]) * v;
+      }
+      const R fac = m == 0 ? 1 : 2;
 #pragma unroll
-    for (int side = 0; side < 2; ++side) {
+      for (int side = 0; side < 2; ++side) {
+        const R re = fac * (side == 0 ? er + odr : t == 1 ? odr - er : er - odr);
+        const R im = fac * (side == 0 ? ei + odi : t == 1 ? odi - ei : ei - odi);
+        R* d = h + ((2 * q + side) * (p + 1) + m) * 2;
 #pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        if (!((KINDS >> k) & 1)) continue;
-        const int t = k == 3 ? 2 : (k == 1 || k == 4) ? 1 : 0;
-        R re = fac * (side == 0 ? e[t][0] + o[t][0] : t == 1 ? o[t][0] - e[t][0] : e[t][0] - o[t][0]);
-        R im = fac * (side == 0 ? e[t][1] + o[t][1] : t == 1 ? o[t][1] - e[t][1] : e[t][1] - o[t][1]);
-        if (k == 2 || k == 4) {  // multiply by i m
-          const R w = re;
-          re = -(R)m * im;
-          im = (R)m * w;
-        } else if (k == 5) {
-          re *= -(R)(m * m);
-          im *= -(R)(m * m);
+        for (int k = 0; k < 6; ++k) {
+          if (!((KINDS >> k) & 1) || t != (k == 3 ? 2 : (k == 1 || k == 4) ? 1 : 0)) continue;
+          R* e = d + kind_slot(KINDS, k) * hk;
+          e[0] = k == 2 || k == 4 ? -(R)m * im : k == 5 ? -(R)(m * m) * re : re;  // times 1, i m or -m^2
+          e[1] = k == 2 || k == 4 ? (R)m * re : k == 5 ? -(R)(m * m) * im : im;
         }
-        R* d = h + kind_slot(KINDS, k) * hk + ((2 * q + side) * (p + 1) + m) * 2;
-        d[0] = re;
-        d[1] = im;
       }
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 2 * jbn * k4n; i += kSynThreads) {
-    const int row = i / k4n, k = i - row * k4n;
+  for (int i = threadIdx.x; i < NK * 2 * jbn * k4n; i += kSynThreads) {
+    const int s = i / (2 * jbn * k4n), rk = i - s * 2 * jbn * k4n, row = rk / k4n, k = rk - row * k4n;
     const int j = row & 1 ? P - (q0 + row / 2) : q0 + row / 2;
     if ((row & 1) && 2 * j == P) continue;  // the middle latitude is its own mirror
-    const R* hr = h + (long long)row * (p + 1) * 2;
-    R ce[NK], co[NK], se[NK], so[NK];
-#pragma unroll
-    for (int s = 0; s < NK; ++s) {
-      ce[s] = hr[s * hk];
-      co[s] = se[s] = so[s] = 0;
-    }
+    const R* hr = h + s * hk + (long long)row * (p + 1) * 2;
+    R ce = hr[0], co = 0, se = 0, so = 0;
     int m = 1;
+#pragma unroll 2
     for (; m + 1 <= p; m += 2) {
       const R c1 = cs[((long long)m * nk + k) * 2], s1 = cs[((long long)m * nk + k) * 2 + 1];
       const R c2 = cs[((long long)(m + 1) * nk + k) * 2], s2 = cs[((long long)(m + 1) * nk + k) * 2 + 1];
-#pragma unroll
-      for (int s = 0; s < NK; ++s) {
-        const R* a = hr + s * hk + 2 * m;
-        co[s] += a[0] * c1;
-        so[s] += a[1] * s1;
-        ce[s] += a[2] * c2;
-        se[s] += a[3] * s2;
-      }
+      const R* a = hr + 2 * m;
+      co += a[0] * c1;
+      so += a[1] * s1;
+      ce += a[2] * c2;
+      se += a[3] * s2;
     }
     if (m <= p) {
-      const R c1 = cs[((long long)m * nk + k) * 2], s1 = cs[((long long)m * nk + k) * 2 + 1];
-#pragma unroll
-      for (int s = 0; s < NK; ++s) {
-        const R* a = hr + s * hk + 2 * m;
-        co[s] += a[0] * c1;
-        so[s] += a[1] * s1;
-      }
+      co += hr[2 * m] * cs[((long long)m * nk + k) * 2];
+      so += hr[2 * m + 1] * cs[((long long)m * nk + k) * 2 + 1];
     }
     const bool rot = k > 0, mir = 2 * k < half;  // k = 0 and the middle k have two longitudes, not four
     R* d0;
@@ -164,22 +160,12 @@ __global__ void __launch_bounds__(kSynThreads) k_synth(const CT* __restrict__ co
     } else {
       d0 = out + f * field_stride + (long long)j * nk;
     }
-#pragma unroll
-    for (int s = 0; s < NK; ++s) {
-      R* d = d0 + s * kind_stride;
-      const R cp = ce[s] + co[s], cm = ce[s] - co[s], sp = se[s] + so[s], sm = se[s] - so[s];
-      if (SRC) {
-        d[k] = w[0] * (cp - sp);
-        if (mir) d[half + k] = w[1] * (cm - sm);
-        if (rot) d[2 * half - k] = w[2] * (cp + sp);
-        if (rot && mir) d[half - k] = w[3] * (cm + sm);
-      } else {
-        d[k] = cp - sp;
-        if (mir) d[half + k] = cm - sm;
-        if (rot) d[2 * half - k] = cp + sp;
-        if (rot && mir) d[half - k] = cm + sm;
-      }
-    }
+    R* d = d0 + s * kind_stride;
+    const R cp = ce + co, cm = ce - co, sp = se + so, sm = se - so;
+    d[k] = w[0] * (cp - sp);
+    if (mir) d[half + k] = w[1] * (cm - sm);
+    if (rot) d[2 * half - k] = w[2] * (cp + sp);
+    if (rot && mir) d[half - k] = w[3] * (cm + sm);
   }
 }
 
