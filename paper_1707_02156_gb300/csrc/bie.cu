@@ -1644,7 +1644,8 @@ namespace bie {
 namespace {
 
 constexpr int kRedThreads = 256;
-constexpr int kRedBlocks = 120;
+constexpr int kRedBlocks = 304;  // two per SM
+constexpr int BIE_MAX_RESTART = 64;  // bie_solve's limit
 
 // partial[i][b] = sum over block b's slice of V_i . w   (i < k)
 __global__ void k_multidot(const double* __restrict__ V, long long ldv, const double* __restrict__ w, long long n,
@@ -1721,11 +1722,25 @@ __device__ inline void kry_slice(long long n, long long* x0, long long* x1) {
   *x1 = min(n, *x0 + chunk);
 }
 
-// partial[i][block] = V_i . w over the block's slice for i < nv (V_nv = w itself when with_norm)
-__device__ void kry_block_dots(const double* __restrict__ V, long long ldv, const double* __restrict__ w, int nv,
-                               bool with_norm, long long x0, long long x1, double* __restrict__ partial) {
-  __shared__ double sh[kKryThreads / 32][kKryGroup];
+constexpr int kKrySlice = 64;  // entries of a block whose slice is kept in shared memory
+
+// partial[i][block] = V_i . w over the block's slice for i < nv (V_nv = w itself when with_norm).  A short
+// slice: one warp per vector, with w from shared memory; a long one: every thread of the block on four
+// vectors at a time.
+__device__ void kry_block_dots(const double* V, long long ldv, const double* w, const double* ws, int nv, bool with_norm,
+                               long long x0, long long x1, double* __restrict__ partial) {
   const int nt = nv + (with_norm ? 1 : 0);
+  if (x1 - x0 <= kKrySlice) {
+    const int len = (int)(x1 - x0), lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < nt; i += blockDim.x >> 5) {
+      double a = 0;
+      for (int x = lane; x < len; x += 32) a += (i < nv ? V[(long long)i * ldv + x0 + x] : ws[x]) * ws[x];
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+      if (lane == 0) partial[(long long)i * gridDim.x + blockIdx.x] = a;
+    }
+    return;
+  }
+  __shared__ double sh[kKryThreads / 32][kKryGroup];
   for (int i0 = 0; i0 < nt; i0 += kKryGroup) {
     double a[kKryGroup];
 #pragma unroll
@@ -1755,6 +1770,36 @@ __device__ void kry_block_dots(const double* __restrict__ V, long long ldv, cons
   }
 }
 
+// w -= V h (i <= k) on the block's slice, kept in ws when it is short.  A short slice shares the vectors of an
+// entry among four threads, whose sums are added in order.
+__device__ void kry_subtract(double* w, const double* V, long long n, int k, const double* h, long long x0, long long x1,
+                             double* ws) {
+  __shared__ double hs[BIE_MAX_RESTART + 1], ps[4][kKrySlice];
+  if (x1 - x0 <= kKrySlice) {
+    for (int i = threadIdx.x; i <= k; i += blockDim.x) hs[i] = h[i];
+    const int x = threadIdx.x % kKrySlice, part = threadIdx.x / kKrySlice, len = (int)(x1 - x0);
+    const double wx = x < len ? w[x0 + x] : 0.0;
+    __syncthreads();
+    double t = 0;
+    if (x < len)
+#pragma unroll 4
+      for (int i = part; i <= k; i += 4) t += hs[i] * V[(long long)i * n + x0 + x];
+    ps[part][x] = t;
+    __syncthreads();
+    if (part == 0 && x < len) {
+      ws[x] = wx - (((ps[0][x] + ps[1][x]) + ps[2][x]) + ps[3][x]);
+      w[x0 + x] = ws[x];
+    }
+  } else {
+    for (long long x = x0 + threadIdx.x; x < x1; x += blockDim.x) {
+      double t = w[x];
+      for (int i = 0; i <= k; ++i) t -= h[i] * V[(long long)i * n + x];
+      w[x] = t;
+    }
+  }
+  __syncthreads();
+}
+
 // true in the last block to finish; the counter is reset for the next launch
 __device__ inline bool kry_last_block(unsigned* counter) {
   __shared__ bool last;
@@ -1769,27 +1814,39 @@ __device__ inline bool kry_last_block(unsigned* counter) {
   return last;
 }
 
-// out[i] = sum over blocks of partial[i][b], b in order (i < nt), by the last block
+// out[i] = sum over blocks of partial[i][b] (i < nt), by the last block: one warp per entry, its lanes
+// over the blocks, so that the loads overlap (a fixed order of summation)
 __device__ inline void kry_finish(const double* partial, int nt, double* out) {
-  for (int i = threadIdx.x; i < nt; i += blockDim.x) {
+  for (int i = threadIdx.x >> 5; i < nt; i += blockDim.x >> 5) {
     double t = 0;
-    for (int b = 0; b < (int)gridDim.x; ++b) t += __ldcg(partial + (long long)i * gridDim.x + b);
-    out[i] = t;
+    for (int b = threadIdx.x & 31; b < (int)gridDim.x; b += 32) t += __ldcg(partial + (long long)i * gridDim.x + b);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) out[i] = t;
   }
 }
 
-// w = (lambda + 1) u - d (system operator of Eq. main_eq), then h = V_i . w for i <= k
-__global__ void __launch_bounds__(kKryThreads) k_kry_sysop_dots(const double* __restrict__ lam,
-                                                                const double* __restrict__ u,
+// Normalisation of u = V_k by the scale the previous step left (scale null: u is normalised already; d is
+// then the operator of the vector before that, scaled here as well), w = (lambda + 1) u - d (system operator
+// of Eq. main_eq; lambda null: w = d, d the operator itself), then h = V_i . w for i <= k
+__global__ void __launch_bounds__(kKryThreads) k_kry_sysop_dots(const double* __restrict__ lam, double* u,
                                                                 const double* __restrict__ d, double* __restrict__ w,
-                                                                const double* __restrict__ V, long long n, int k,
+                                                                const double* V, long long n, int k,
+                                                                const double* __restrict__ scale,
                                                                 double* __restrict__ partial, unsigned* counter,
                                                                 double* __restrict__ h) {
   long long x0, x1;
   kry_slice(n, &x0, &x1);
-  for (long long x = x0 + threadIdx.x; x < x1; x += blockDim.x) w[x] = (lam[x] + 1.0) * u[x] - d[x];
+  __shared__ double ws[kKrySlice];
+  const double sc = scale ? scale[0] : 1.0;
+  for (long long x = x0 + threadIdx.x; x < x1; x += blockDim.x) {
+    const double v = sc * u[x];
+    if (scale) u[x] = v;
+    const double t = lam ? (lam[x] + 1.0) * v - sc * d[x] : sc * d[x];
+    w[x] = t;
+    if (x - x0 < kKrySlice) ws[x - x0] = t;
+  }
   __syncthreads();
-  kry_block_dots(V, n, w, k + 1, false, x0, x1, partial);
+  kry_block_dots(V, n, w, ws, k + 1, false, x0, x1, partial);
   if (kry_last_block(counter)) kry_finish(partial, k + 1, h);
 }
 
@@ -1800,13 +1857,9 @@ __global__ void __launch_bounds__(kKryThreads) k_kry_sub_dots(double* __restrict
                                                               double* __restrict__ h) {
   long long x0, x1;
   kry_slice(n, &x0, &x1);
-  for (long long x = x0 + threadIdx.x; x < x1; x += blockDim.x) {
-    double t = w[x];
-    for (int i = 0; i <= k; ++i) t -= hprev[i] * V[(long long)i * n + x];
-    w[x] = t;
-  }
-  __syncthreads();
-  kry_block_dots(V, n, w, k + 1, true, x0, x1, partial);
+  __shared__ double ws[kKrySlice];
+  kry_subtract(w, V, n, k, hprev, x0, x1, ws);
+  kry_block_dots(V, n, w, ws, k + 1, true, x0, x1, partial);
   if (kry_last_block(counter)) kry_finish(partial, k + 2, h);
 }
 
@@ -1824,41 +1877,48 @@ __global__ void __launch_bounds__(kKryThreads) k_kry_sub_tail(double* __restrict
                                                               double* __restrict__ scale, double* __restrict__ res) {
   long long x0, x1;
   kry_slice(n, &x0, &x1);
-  for (long long x = x0 + threadIdx.x; x < x1; x += blockDim.x) {
-    double t = w[x];
-    for (int i = 0; i <= k; ++i) t -= h2[i] * V[(long long)i * n + x];
-    w[x] = t;
+  __shared__ double ws[kKrySlice];
+  kry_subtract(w, V, n, k, h2, x0, x1, ws);
+  kry_block_dots(V, n, w, ws, 0, true, x0, x1, partial);
+  if (!kry_last_block(counter)) return;
+  // the column, the rotations and |w|^2 come in with one round of loads; the recurrence runs in shared memory
+  __shared__ double col[BIE_MAX_RESTART + 2], rc[BIE_MAX_RESTART], rs[BIE_MAX_RESTART], wn2;
+  kry_finish(partial, 1, &wn2);
+  for (int i = threadIdx.x; i <= k; i += blockDim.x) {
+    col[i] = h1[i] + h2[i];
+    if (i < k) {
+      rc[i] = cs[i];
+      rs[i] = sn[i];
+    }
   }
   __syncthreads();
-  kry_block_dots(V, n, w, 0, true, x0, x1, partial);
-  if (!kry_last_block(counter)) return;
-  if (threadIdx.x != 0) return;
-  double wn2 = 0;
-  for (int b = 0; b < (int)gridDim.x; ++b) wn2 += __ldcg(partial + b);
-  const double hn = sqrt(wn2);
-  for (int i = 0; i <= k; ++i) H[(long long)i * m + k] = h1[i] + h2[i];
-  for (int i = 0; i < k; ++i) {
-    const double a = H[(long long)i * m + k], b = H[(long long)(i + 1) * m + k];
-    H[(long long)i * m + k] = cs[i] * a + sn[i] * b;
-    H[(long long)(i + 1) * m + k] = -sn[i] * a + cs[i] * b;
+  if (threadIdx.x == 0) {
+    const double hn = sqrt(wn2);
+    for (int i = 0; i < k; ++i) {
+      const double a = col[i], b = col[i + 1];
+      col[i] = rc[i] * a + rs[i] * b;
+      col[i + 1] = -rs[i] * a + rc[i] * b;
+    }
+    const double a = col[k];
+    const double den = hypot(a, hn);
+    const double c = den > 0 ? a / den : 1.0, sv = den > 0 ? hn / den : 0.0, g = gv[k];
+    cs[k] = c;
+    sn[k] = sv;
+    col[k] = den;
+    gv[k + 1] = -sv * g;
+    gv[k] = c * g;
+    scale[0] = hn > 0 ? 1.0 / hn : 0.0;
+    res[k] = fabs(-sv * g);
   }
-  const double a = H[(long long)k * m + k];
-  const double den = hypot(a, hn);
-  cs[k] = den > 0 ? a / den : 1.0;
-  sn[k] = den > 0 ? hn / den : 0.0;
-  H[(long long)k * m + k] = den;
-  gv[k + 1] = -sn[k] * gv[k];
-  gv[k] = cs[k] * gv[k];
-  scale[0] = hn > 0 ? 1.0 / hn : 0.0;
-  res[k] = fabs(gv[k + 1]);
+  __syncthreads();
+  for (int i = threadIdx.x; i <= k; i += blockDim.x) H[(long long)i * m + k] = col[i];
 }
 
-inline int kry_blocks(long long n) { return (int)std::max(1LL, std::min<long long>(120, (n + 255) / 256)); }
-
-// y = s * y with the scale read from the device
-__global__ void k_scale_dev(double* __restrict__ y, const double* __restrict__ scale, long long n) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) y[i] *= scale[0];
+// Blocks of the fused kernels: kKrySlice entries each while kRedBlocks of them cover the vector (19456 entries),
+// then longer slices.  With 256 entries a block and every vector's
+// products reduced by all warps, the three kernels of a step took 30 us on one drop of degree 32, now 24.
+inline int kry_blocks(long long n) {
+  return (int)std::max(1LL, std::min<long long>(kRedBlocks, (n + kKrySlice - 1) / kKrySlice));
 }
 
 // start of a cycle: gv = (beta, 0, ..., 0), V_0 = r / beta
@@ -1869,15 +1929,20 @@ __global__ void k_cycle_start(const double* __restrict__ r, double beta, double*
   if (i <= m) gv[i] = i == 0 ? beta : 0.0;
 }
 
-// back substitution y = H^-1 gv on the leading k x k triangle (one thread)
+// back substitution y = H^-1 gv on the leading k x k triangle (one warp)
 __global__ void k_backsub(const double* __restrict__ H, const double* __restrict__ gv, int k, int m,
                           double* __restrict__ y) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int i = k - 1; i >= 0; --i) {
-    double t = gv[i];
-    for (int q = i + 1; q < k; ++q) t -= H[(long long)i * m + q] * y[q];
-    y[i] = t / H[(long long)i * m + i];
+  __shared__ double sy[BIE_MAX_RESTART];
+  const int lane = threadIdx.x;
+  for (int i = k - 1; i >= 0; --i) {  // the lanes share the products of a row
+    double t = 0;
+    for (int q = i + 1 + lane; q < k; q += 32) t += H[(long long)i * m + q] * sy[q];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    const double v = (gv[i] - t) / H[(long long)i * m + i];
+    if (lane == 0) sy[i] = v;
+    __syncwarp();
   }
+  for (int i = lane; i < k; i += 32) y[i] = sy[i];
 }
 
 inline unsigned nblk(long long n) { return (unsigned)((n + 255) / 256); }
@@ -1900,6 +1965,38 @@ struct Krylov {
   };
   std::map<long long, StepGraph> steps;  // captured Arnoldi steps by (precision, restart, k)
   bool steps_failed = false;             // a capture failed: step eagerly from then on
+  // workspace of restart length mr for vectors of length n_
+  int init(long long n_, int mr) {
+    n = n_;
+    m = mr;
+    BIE_TRY(V.alloc((size_t)(mr + 1) * n));
+    BIE_TRY(tmp.alloc(3 * n));
+    BIE_TRY(partial.alloc((size_t)kRedBlocks * (mr + 2)));
+    BIE_TRY(hdev.alloc(2 * (mr + 2)));
+    BIE_TRY(Hd.alloc((size_t)(mr + 1) * mr));
+    BIE_TRY(csd.alloc(mr));
+    BIE_TRY(snd.alloc(mr));
+    BIE_TRY(gvd.alloc(mr + 1));
+    BIE_TRY(scale.alloc(1));
+    BIE_TRY(resd.alloc(mr));
+    BIE_TRY(yd.alloc(mr));
+    if (!counter.ptr) {
+      BIE_TRY(counter.alloc(1));
+      BIE_CUDA_TRY(cudaMemset(counter.ptr, 0, sizeof(unsigned)));
+    }
+    if (hpin_n < std::max(mr, 2)) {
+      if (hpin) cudaFreeHost(hpin);
+      hpin = nullptr;
+      BIE_CUDA_TRY(cudaMallocHost(&hpin, std::max(mr, 2) * sizeof(double)));
+      hpin_n = std::max(mr, 2);
+    }
+    while ((int)ev.size() < mr) {
+      cudaEvent_t e;
+      BIE_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+      ev.push_back(e);
+    }
+    return BIE_OK;
+  }
   ~Krylov() {
     if (hpin) cudaFreeHost(hpin);
     for (auto e : ev) cudaEventDestroy(e);
@@ -1970,40 +2067,45 @@ static int sys_matvec(bie_ctx* ctx, const bie_geom* g, const double* u, double* 
   return BIE_OK;
 }
 
-// Arnoldi step k on stream s: normalisation of V_k (deferred from step k - 1), the operator apply
-// into the temporary t2 (its kernels launched one by one when eager_apply), the three fused
-// Gram-Schmidt kernels and the copy of the residual estimate to the pinned host array.
+// The end of Arnoldi step k behind the operator t2 of V_k (not yet normalised for k > 0): the three fused
+// kernels and the copy of the residual estimate to the pinned host array.
+static int arnoldi_tail(Krylov& K, const double* lam, const double* t2, long long n, int k, int m, cudaStream_t s) {
+  double* V = K.V.ptr;
+  double* vk = V + (long long)k * n;
+  double* vk1 = V + (long long)(k + 1) * n;
+  double* h1 = K.hdev.ptr;
+  double* h2d = K.hdev.ptr + (m + 2);
+  const int nbk = kry_blocks(n);
+  k_kry_sysop_dots<<<nbk, kKryThreads, 0, s>>>(lam, vk, t2, vk1, V, n, k, k > 0 ? K.scale.ptr : nullptr, K.partial.ptr,
+                                       K.counter.ptr, h1);
+  count_launch();
+  BIE_CUDA_TRY(cudaGetLastError());
+  k_kry_sub_dots<<<nbk, kKryThreads, 0, s>>>(vk1, V, n, k, h1, K.partial.ptr, K.counter.ptr, h2d);
+  count_launch();
+  BIE_CUDA_TRY(cudaGetLastError());
+  k_kry_sub_tail<<<nbk, kKryThreads, 0, s>>>(vk1, V, n, k, m, h1, h2d, K.partial.ptr, K.counter.ptr, K.Hd.ptr, K.csd.ptr,
+                                     K.snd.ptr, K.gvd.ptr, K.scale.ptr, K.resd.ptr);
+  count_launch();
+  BIE_CUDA_TRY(cudaGetLastError());
+  BIE_CUDA_TRY(cudaMemcpyAsync(K.hpin + k, K.resd.ptr + k, sizeof(double), cudaMemcpyDeviceToHost, s));
+  return BIE_OK;
+}
+
+// Arnoldi step k on stream s: the operator apply into the temporary t2 (its kernels launched one by one when
+// eager_apply), the three fused Gram-Schmidt kernels (the first one also normalises V_k, deferred from
+// step k - 1) and the copy of the residual estimate to the pinned host array.
 static int arnoldi_step(bie_ctx* ctx, const bie_geom* g, Krylov& K, int prec, int k, int m, bool eager_apply,
                         cudaStream_t s) {
   const long long n = g->ncoef_total;
   double* V = K.V.ptr;
   double* t2 = K.tmp.ptr + n;
   double* vk = V + (long long)k * n;
-  double* vk1 = V + (long long)(k + 1) * n;
-  if (k > 0) {
-    k_scale_dev<<<nblk(n), 256, 0, s>>>(vk, K.scale.ptr, n);
-    count_launch();
-    BIE_CUDA_TRY(cudaGetLastError());
-  }
+  // V_k is normalised by k_kry_sysop_dots, behind the apply: the operator is linear
   if (eager_apply)
     BIE_TRY(layer_apply_eager(ctx, g, 1, vk, t2, prec, s));
   else
     BIE_TRY(layer_apply(ctx, g, 1, vk, t2, prec, s));
-  double* h1 = K.hdev.ptr;
-  double* h2d = K.hdev.ptr + (m + 2);
-  const int nbk = kry_blocks(n);
-  k_kry_sysop_dots<<<nbk, kKryThreads, 0, s>>>(g->lamc.ptr, vk, t2, vk1, V, n, k, K.partial.ptr, K.counter.ptr, h1);
-  count_launch();
-  BIE_CUDA_TRY(cudaGetLastError());
-  k_kry_sub_dots<<<nbk, kKryThreads, 0, s>>>(vk1, V, n, k, h1, K.partial.ptr, K.counter.ptr, h2d);
-  count_launch();
-  BIE_CUDA_TRY(cudaGetLastError());
-  k_kry_sub_tail<<<nbk, kKryThreads, 0, s>>>(vk1, V, n, k, m, h1, h2d, K.partial.ptr, K.counter.ptr, K.Hd.ptr,
-                                             K.csd.ptr, K.snd.ptr, K.gvd.ptr, K.scale.ptr, K.resd.ptr);
-  count_launch();
-  BIE_CUDA_TRY(cudaGetLastError());
-  BIE_CUDA_TRY(cudaMemcpyAsync(K.hpin + k, K.resd.ptr + k, sizeof(double), cudaMemcpyDeviceToHost, s));
-  return BIE_OK;
+  return arnoldi_tail(K, g->lamc.ptr, t2, n, k, m, s);
 }
 
 // Arnoldi step k as a CUDA graph: captured on the geometry's capture stream at its first use (once
@@ -2208,6 +2310,11 @@ struct SurfLayout {
   std::vector<long long> voff, soff;  // per drop: start of its vector / scalar coefficients
   long long nv = 0, ns = 0;           // total lengths
   std::vector<std::unique_ptr<SurfGroup>> groups;
+  long long group_points() const {    // grid points of the largest group
+    long long v = 0;
+    for (const auto& G : groups) v = std::max<long long>(v, (long long)G->drops.size() * ngrid(G->P));
+    return v;
+  }
 };
 
 // P = 2p + 1 (the nonlinear terms of Sec. 1.3) when upsampled, else P = p.
@@ -2262,11 +2369,11 @@ static int surf_project(const SurfLayout& L, const SurfGroup& G, const double* g
 // Galerkin projections of f_E and (when fi is non-null) f_I = inv_pe lap Gamma, Sec. 3.
 static int surf_rates(const SurfLayout& L, const double* x, const double* u, const double* gam, double inv_pe,
                       double* fe, double* fi, cudaStream_t s) {
+  DevBuf<double> tmp;  // for the largest group; the groups follow one another on the stream
+  BIE_TRY(tmp.alloc(35 * L.group_points()));
   for (auto& Gp : L.groups) {
     const SurfGroup& G = *Gp;
     const long long nd = (long long)G.drops.size(), N = ngrid(G.P);
-    DevBuf<double> tmp;
-    BIE_TRY(tmp.alloc(18 * nd * N + 9 * nd * N + 6 * nd * N + 2 * nd * N));
     double* X = tmp.ptr;
     double* U = X + 18 * nd * N;
     double* Gm = U + 9 * nd * N;
@@ -2277,30 +2384,34 @@ static int surf_rates(const SurfLayout& L, const double* x, const double* u, con
     BIE_TRY(launch_surf_rates(X, U, Gm, nd, N, inv_pe, out, fi ? out + nd * N : nullptr, s));
     BIE_TRY(surf_project(L, G, out, nd, G.soff.ptr, fe, s));
     if (fi) BIE_TRY(surf_project(L, G, out + nd * N, nd, G.soff.ptr, fi, s));
-    BIE_CUDA_TRY(cudaStreamSynchronize(s));  // temporaries are released per group
   }
+  BIE_CUDA_TRY(cudaStreamSynchronize(s));  // the temporaries are released on return
   return BIE_OK;
 }
 
 // Per-drop integrals on the grid of each group (mode 0: volume of x, mode 1: mass of Gamma), host out[d].
 static int surf_integrals(const SurfLayout& L, const double* x, const double* gam, int mode, double* out,
                           cudaStream_t s) {
+  DevBuf<double> tmp, res_all;
+  BIE_TRY(tmp.alloc(10 * L.group_points()));
+  BIE_TRY(res_all.alloc(L.ndrop));
+  double* res = res_all.ptr;
+  std::vector<double> h(L.ndrop);
   for (auto& Gp : L.groups) {
     const SurfGroup& G = *Gp;
     const long long nd = (long long)G.drops.size(), N = ngrid(G.P);
-    DevBuf<double> tmp;
-    BIE_TRY(tmp.alloc(9 * nd * N + nd * N + nd));
     double* X = tmp.ptr;
     double* Gm = X + 9 * nd * N;
-    double* res = Gm + nd * N;
     BIE_TRY(surf_synth(L, G, x, G.voff.ptr, 3 * nd, mode == 0 ? 7 : 6, X, s));
     if (mode == 1) BIE_TRY(surf_synth(L, G, gam, G.soff.ptr, nd, 1, Gm, s));
     BIE_TRY(launch_drop_integral(X, Gm, nd, G.P, G.pl->wsin.ptr, mode, res, s));
-    std::vector<double> h(nd);
-    BIE_CUDA_TRY(cudaMemcpyAsync(h.data(), res, nd * sizeof(double), cudaMemcpyDeviceToHost, s));
-    BIE_CUDA_TRY(cudaStreamSynchronize(s));
-    for (long long i = 0; i < nd; ++i) out[G.drops[i]] = h[i];
+    res += nd;
   }
+  BIE_CUDA_TRY(cudaMemcpyAsync(h.data(), res_all.ptr, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+  BIE_CUDA_TRY(cudaStreamSynchronize(s));
+  size_t at = 0;
+  for (auto& Gp : L.groups)
+    for (int d : Gp->drops) out[d] = h[at++];
   return BIE_OK;
 }
 
@@ -2329,26 +2440,25 @@ static int surf_absmax(const SurfLayout& L, const double* coef, int ncomp, doubl
 struct SurfImplicit {
   const SurfLayout* L = nullptr;
   double a = 0;
-  std::vector<std::unique_ptr<DevBuf<double>>> lapc;  // per group [5][nd][N]
+  DevBuf<double> lapc;  // per group [5][nd][N], one after another
   DevBuf<double> inv_diag, c, work;
 };
 
 static int surf_implicit_setup(const SurfLayout& L, const double* x, double a, SurfImplicit& I, cudaStream_t s) {
   I.L = &L;
   I.a = a;
-  long long wmax = 0;
+  long long total = 0, at = 0;
+  for (auto& Gp : L.groups) total += 5 * (long long)Gp->drops.size() * ngrid(Gp->P);
+  DevBuf<double> tmp;
+  BIE_TRY(tmp.alloc(18 * L.group_points()));
+  BIE_TRY(I.lapc.alloc(total));
+  BIE_TRY(I.work.alloc(7 * L.group_points()));
   for (auto& Gp : L.groups) {
     const SurfGroup& G = *Gp;
     const long long nd = (long long)G.drops.size(), N = ngrid(G.P);
-    DevBuf<double> tmp;
-    BIE_TRY(tmp.alloc(18 * nd * N));
     BIE_TRY(surf_synth(L, G, x, G.voff.ptr, 3 * nd, 62, tmp.ptr, s));
-    std::unique_ptr<DevBuf<double>> lc(new DevBuf<double>());
-    BIE_TRY(lc->alloc(5 * nd * N));
-    BIE_TRY(launch_lap_coef(tmp.ptr, nd, N, lc->ptr, s));
-    BIE_CUDA_TRY(cudaStreamSynchronize(s));
-    I.lapc.push_back(std::move(lc));
-    wmax = std::max(wmax, 7 * nd * N);
+    BIE_TRY(launch_lap_coef(tmp.ptr, nd, N, I.lapc.ptr + at, s));
+    at += 5 * nd * N;
   }
   std::vector<double> vol(L.ndrop);
   BIE_TRY(surf_integrals(L, x, nullptr, 0, vol.data(), s));
@@ -2361,151 +2471,81 @@ static int surf_implicit_setup(const SurfLayout& L, const double* x, double a, S
   }
   BIE_TRY(I.inv_diag.upload(inv));
   BIE_TRY(I.c.alloc(L.ns));
-  BIE_TRY(I.work.alloc(wmax));
   return BIE_OK;
 }
 
 static int surf_implicit_apply(SurfImplicit& I, const double* y, double* w, cudaStream_t s) {
   const SurfLayout& L = *I.L;
-  for (size_t gi = 0; gi < L.groups.size(); ++gi) {
-    const SurfGroup& G = *L.groups[gi];
+  long long at = 0;
+  for (auto& Gp : L.groups) {
+    const SurfGroup& G = *Gp;
     const long long nd = (long long)G.drops.size(), N = ngrid(G.P);
     double* S = I.work.ptr;  // [6][nd][N], kinds 1..5 used
     double* grid = S + 6 * nd * N;
     BIE_TRY(surf_synth(L, G, y, G.soff.ptr, nd, 62, S, s));
-    BIE_TRY(launch_lap_apply(I.lapc[gi]->ptr, S, nd, N, grid, s));
+    BIE_TRY(launch_lap_apply(I.lapc.ptr + at, S, nd, N, grid, s));
+    at += 5 * nd * N;
     BIE_TRY(surf_project(L, G, grid, nd, G.soff.ptr, I.c.ptr, s));
   }
   return launch_implicit_combine(y, I.c.ptr, I.a, I.inv_diag.ptr, L.ns, w, s);
 }
 
-// Restarted GMRES (classical Gram-Schmidt with one re-orthogonalisation, Givens rotations on the
-// host) for op x = b from x = 0; stops on ||b - op x|| <= tol ||b||.
-struct SurfKrylov {
-  long long n = 0;
-  int m = 0;
-  DevBuf<double> V, partial, hdev, ydev;
-  int init(long long n_, int m_) {
-    n = n_;
-    m = m_;
-    BIE_TRY(V.alloc((size_t)(m + 1) * n));
-    BIE_TRY(partial.alloc((size_t)kRedBlocks * (m + 1)));
-    BIE_TRY(hdev.alloc(m + 1));
-    BIE_TRY(ydev.alloc(m + 1));
-    return BIE_OK;
-  }
-};
-
-// out[i] = V_i . w for i < k (V_i n apart), on the host
-static int surf_dots(SurfKrylov& K, const double* V, int k, const double* w, double* out, cudaStream_t s) {
-  k_multidot<<<dim3(kRedBlocks, k), kRedThreads, 0, s>>>(V, K.n, w, K.n, k, K.partial.ptr);
-  count_launch();
-  BIE_CUDA_TRY(cudaGetLastError());
-  k_sum_partials<<<k, 128, 0, s>>>(K.partial.ptr, kRedBlocks, k, K.hdev.ptr);
-  count_launch();
-  BIE_CUDA_TRY(cudaGetLastError());
-  BIE_CUDA_TRY(cudaMemcpyAsync(out, K.hdev.ptr, k * sizeof(double), cudaMemcpyDeviceToHost, s));
-  BIE_CUDA_TRY(cudaStreamSynchronize(s));
-  return BIE_OK;
-}
-
-// x += sum_i c_i V_i (c on the host, k entries)
-static int surf_comb(SurfKrylov& K, double* x, const double* V, const double* c, int k, cudaStream_t s) {
-  BIE_CUDA_TRY(cudaMemcpyAsync(K.ydev.ptr, c, k * sizeof(double), cudaMemcpyHostToDevice, s));
-  k_add_comb<<<nblk(K.n), 256, 0, s>>>(x, V, K.n, K.ydev.ptr, k, K.n);
-  count_launch();
-  BIE_CUDA_TRY(cudaGetLastError());
-  BIE_CUDA_TRY(cudaStreamSynchronize(s));  // c may change on return
-  return BIE_OK;
-}
-
-static int surf_gmres(SurfKrylov& K, const std::function<int(const double*, double*)>& op, const double* b,
-                      double* x, double tol, int max_it, int* iters, double* relres, cudaStream_t s) {
+// Restarted GMRES for op x = b from x = 0 on the device kernels of the velocity solve (classical Gram-Schmidt
+// with one re-orthogonalisation, Givens rotations in k_kry_sub_tail); stops on ||b - op x|| <= tol ||b||.
+// The host reads the residual estimate of step k - 1 while step k runs, so an iteration has no
+// synchronisation of its own (five before, each with copies from and to pageable memory).
+static int surf_gmres(Krylov& K, const std::function<int(const double*, double*)>& op, const double* b, double* x,
+                      double tol, int max_it, int* iters, cudaStream_t s) {
   const long long n = K.n;
   const int m = K.m;
-  double* V = K.V.ptr;
-  BIE_CUDA_TRY(cudaMemsetAsync(x, 0, n * sizeof(double), s));
-  double bb;
-  BIE_TRY(surf_dots(K, b, 1, b, &bb, s));
-  const double bnorm = std::sqrt(bb);
+  double *V = K.V.ptr, *r = K.tmp.ptr, *t2 = K.tmp.ptr + n;
   *iters = 0;
-  *relres = 0;
+  BIE_CUDA_TRY(cudaMemsetAsync(x, 0, n * sizeof(double), s));
+  double bnorm, beta;
+  BIE_TRY(norm2(K, b, &bnorm, s));
   if (bnorm == 0.0) return BIE_OK;
-  std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), h(m + 1), h2(m + 1), y(m);
-  auto Hr = [&](int i, int k) -> double& { return H[(size_t)i * m + k]; };
   int it = 0;
-  bool xzero = true;
+  BIE_CUDA_TRY(cudaMemcpyAsync(r, b, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
+  beta = bnorm;
   while (true) {
-    double* r = V;
-    if (xzero) {
-      BIE_CUDA_TRY(cudaMemcpyAsync(r, b, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    } else {
-      BIE_TRY(op(x, r));
-      k_axpby<<<nblk(n), 256, 0, s>>>(1.0, b, -1.0, r, n);
-      count_launch();
-      BIE_CUDA_TRY(cudaGetLastError());
-    }
-    double rr;
-    BIE_TRY(surf_dots(K, r, 1, r, &rr, s));
-    const double beta = std::sqrt(rr);
-    *relres = beta / bnorm;
     *iters = it;
     if (beta / bnorm <= tol) return BIE_OK;
     if (it >= max_it) {
       set_error("surfactant implicit solve: GMRES did not converge");
       return BIE_ENOCONV;
     }
-    k_scale<<<nblk(n), 256, 0, s>>>(1.0 / beta, r, n);
+    k_cycle_start<<<nblk(std::max<long long>(n, m + 1)), 256, 0, s>>>(r, beta, V, n, K.gvd.ptr, m);
     count_launch();
     BIE_CUDA_TRY(cudaGetLastError());
-    std::fill(g.begin(), g.end(), 0.0);
-    g[0] = beta;
-    int used = 0;
-    for (int k = 0; k < m; ++k) {
-      double* w = V + (long long)(k + 1) * n;
-      BIE_TRY(op(V + (long long)k * n, w));
-      BIE_TRY(surf_dots(K, V, k + 1, w, h.data(), s));
-      for (int i = 0; i <= k; ++i) h2[i] = -h[i];
-      BIE_TRY(surf_comb(K, w, V, h2.data(), k + 1, s));
-      BIE_TRY(surf_dots(K, V, k + 1, w, h2.data(), s));
-      for (int i = 0; i <= k; ++i) {
-        h[i] += h2[i];
-        h2[i] = -h2[i];
+    const int kmax = std::min(m, max_it - it);
+    int used = -1;
+    for (int k = 0; k < kmax; ++k) {
+      BIE_TRY(op(V + (long long)k * n, t2));
+      BIE_TRY(arnoldi_tail(K, nullptr, t2, n, k, m, s));
+      BIE_CUDA_TRY(cudaEventRecord(K.ev[k], s));
+      if (k == 0) continue;
+      BIE_CUDA_TRY(cudaEventSynchronize(K.ev[k - 1]));
+      if (K.hpin[k - 1] / bnorm <= tol) {
+        used = k;
+        break;
       }
-      BIE_TRY(surf_comb(K, w, V, h2.data(), k + 1, s));
-      double ww;
-      BIE_TRY(surf_dots(K, w, 1, w, &ww, s));
-      const double hk1 = std::sqrt(ww);
-      if (hk1 > 0.0) {
-        k_scale<<<nblk(n), 256, 0, s>>>(1.0 / hk1, w, n);
-        count_launch();
-        BIE_CUDA_TRY(cudaGetLastError());
-      }
-      for (int i = 0; i <= k; ++i) Hr(i, k) = h[i];
-      Hr(k + 1, k) = hk1;
-      for (int i = 0; i < k; ++i) {
-        const double t = cs[i] * Hr(i, k) + sn[i] * Hr(i + 1, k);
-        Hr(i + 1, k) = -sn[i] * Hr(i, k) + cs[i] * Hr(i + 1, k);
-        Hr(i, k) = t;
-      }
-      const double den = std::hypot(Hr(k, k), Hr(k + 1, k));
-      cs[k] = Hr(k, k) / den;
-      sn[k] = Hr(k + 1, k) / den;
-      Hr(k, k) = den;
-      Hr(k + 1, k) = 0.0;
-      g[k + 1] = -sn[k] * g[k];
-      g[k] = cs[k] * g[k];
-      ++it;
-      used = k + 1;
-      if (std::fabs(g[k + 1]) / bnorm <= tol || it >= max_it || hk1 == 0.0) break;
     }
-    for (int i = used - 1; i >= 0; --i) {
-      double t = g[i];
-      for (int j = i + 1; j < used; ++j) t -= Hr(i, j) * y[j];
-      y[i] = t / Hr(i, i);
+    if (used < 0) {
+      BIE_CUDA_TRY(cudaEventSynchronize(K.ev[kmax - 1]));
+      used = kmax;
     }
-    BIE_TRY(surf_comb(K, x, V, y.data(), used, s));
-    xzero = false;
+    it += used;
+    k_backsub<<<1, 32, 0, s>>>(K.Hd.ptr, K.gvd.ptr, used, m, K.yd.ptr);
+    count_launch();
+    BIE_CUDA_TRY(cudaGetLastError());
+    k_add_comb<<<nblk(n), 256, 0, s>>>(x, V, n, K.yd.ptr, used, n);
+    count_launch();
+    BIE_CUDA_TRY(cudaGetLastError());
+    BIE_TRY(op(x, r));
+    k_axpby<<<nblk(n), 256, 0, s>>>(1.0, b, -1.0, r, n);
+    count_launch();
+    BIE_CUDA_TRY(cudaGetLastError());
+    BIE_TRY(norm2(K, r, &beta, s));
   }
 }
 
@@ -2522,11 +2562,10 @@ static int surf_implicit_solve(const SurfLayout& L, const double* x, const doubl
   DevBuf<double> bp;
   BIE_TRY(bp.alloc(L.ns));
   BIE_TRY(launch_mul(b, I.inv_diag.ptr, L.ns, bp.ptr, s));
-  SurfKrylov K;
+  Krylov K;
   BIE_TRY(K.init(L.ns, 60));
-  double rel;
   auto op = [&](const double* in, double* out) { return surf_implicit_apply(I, in, out, s); };
-  return surf_gmres(K, op, bp.ptr, y, tol, 600, iters, &rel, s);
+  return surf_gmres(K, op, bp.ptr, y, tol, 600, iters, s);
 }
 
 }  // namespace bie
@@ -2903,35 +2942,7 @@ int bie_solve(bie_ctx* ctx, const bie_geom* g, const double* rhs, double* u, con
     gm->kry = new bie::Krylov();
   }
   bie::Krylov& K = *gm->kry;
-  K.n = n;
-  K.m = opts->restart;
-  BIE_TRY(K.V.alloc((size_t)(opts->restart + 1) * n));
-  BIE_TRY(K.tmp.alloc(3 * n));
-  BIE_TRY(K.partial.alloc((size_t)kRedBlocks * (opts->restart + 2)));
-  BIE_TRY(K.hdev.alloc(2 * (opts->restart + 2)));
-  const int mr = opts->restart;
-  BIE_TRY(K.Hd.alloc((size_t)(mr + 1) * mr));
-  BIE_TRY(K.csd.alloc(mr));
-  BIE_TRY(K.snd.alloc(mr));
-  BIE_TRY(K.gvd.alloc(mr + 1));
-  BIE_TRY(K.scale.alloc(1));
-  BIE_TRY(K.resd.alloc(mr));
-  BIE_TRY(K.yd.alloc(mr));
-  if (!K.counter.ptr) {
-    BIE_TRY(K.counter.alloc(1));
-    BIE_CUDA_TRY(cudaMemset(K.counter.ptr, 0, sizeof(unsigned)));
-  }
-  if (K.hpin_n < std::max(mr, 2)) {
-    if (K.hpin) cudaFreeHost(K.hpin);
-    K.hpin = nullptr;
-    BIE_CUDA_TRY(cudaMallocHost(&K.hpin, std::max(mr, 2) * sizeof(double)));
-    K.hpin_n = std::max(mr, 2);
-  }
-  while ((int)K.ev.size() < mr) {
-    cudaEvent_t e;
-    BIE_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    K.ev.push_back(e);
-  }
+  BIE_TRY(K.init(n, opts->restart));
   double rel = 0;
   int st;
   if ((opts->precision & 0xff) == BIE_FP64) {
