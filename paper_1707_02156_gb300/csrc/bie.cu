@@ -82,6 +82,8 @@ struct Plan {
   int p = 0, P = 0;
   DevBuf<double> T0, T1, T2, At, cs, wsin, wsq;
   DevBuf<float> T0f, csf;
+  DevBuf<int4> CT;  // fixed-point tables of the kernel factors (p <= P <= 2p+1): see launch_kernel_proj
+  DevBuf<int2> PT;
   template <typename R>
   const R* T0_() const;
   template <typename R>
@@ -104,10 +106,18 @@ const float* Plan::cs_<float>() const {
   return csf.ptr;
 }
 
+// v 2^bits as the two parts of fixed.cuh
+static int2 fix_host(double v, int bits) {
+  const long long f = std::llround(std::ldexp(v, bits));
+  const int h = (int)((f + (1LL << 27)) >> 28);
+  return make_int2(h, (int)(f - ((long long)h << 28)));
+}
+
 struct WigPlan {  // rotation blocks for the p+1 latitudes of the degree-p grid
   int p = 0;
   long long stride = 0;
   DevBuf<double> blk;
+  DevBuf<int2> blkx;  // times 2^54 in fixed point (entries up to 2)
   DevBuf<float> blkf;
   template <typename R>
   const R* blk_() const;
@@ -192,6 +202,15 @@ static int get_plan(bie_ctx* ctx, int p, int P, Plan** out) {
   legendre_table(p, P, 0, v);
   BIE_TRY(pl->T0.upload(v));
   BIE_TRY(upload_as(pl->T0f, v));
+  if (P <= 2 * p + 1) {  // a self-rule grid
+    const int nh = P / 2 + 1;
+    std::vector<int2> x((size_t)nh * (p + 1) * (p + 2) / 2);
+    for (int n = 0; n <= p; ++n)
+      for (int m = 0; m <= n; ++m)
+        for (int j = 0; j < nh; ++j)
+          x[(size_t)j * (p + 1) * (p + 2) / 2 + n * (n + 1) / 2 + m] = fix_host(v[leg_row(p, m, n, P + 1) + j], 53);
+    BIE_TRY(pl->PT.upload(x));
+  }
   legendre_table(p, P, 1, v);
   BIE_TRY(pl->T1.upload(v));
   legendre_table(p, P, 2, v);
@@ -207,6 +226,16 @@ static int get_plan(bie_ctx* ctx, int p, int P, Plan** out) {
   }
   phase_table(p, P, v);
   BIE_TRY(pl->cs.upload(v));
+  if (P <= 2 * p + 1) {
+    const int kn = (P + 1) / 2 + 1, nk = 2 * P + 2;
+    std::vector<int4> x((size_t)kn * (p + 1));
+    for (int k = 0; k < kn; ++k)
+      for (int m = 0; m <= p; ++m) {
+        const int2 c = fix_host(v[((size_t)m * nk + k) * 2], 55), sn = fix_host(v[((size_t)m * nk + k) * 2 + 1], 55);
+        x[(size_t)k * (p + 1) + m] = make_int4(c.x, c.y, sn.x, sn.y);
+      }
+    BIE_TRY(pl->CT.upload(x));
+  }
   BIE_TRY(upload_as(pl->csf, v));
   std::vector<double> t, w, ws;
   gauss_legendre(P + 1, t, w);
@@ -239,6 +268,11 @@ static int get_wig(bie_ctx* ctx, int p, WigPlan** out) {
   std::vector<double> blk((size_t)(p + 1) * wp->stride);
   for (int a = 0; a <= p; ++a) wigner_blocks(p, std::acos(t[a]), blk.data() + (size_t)a * wp->stride);
   BIE_TRY(wp->blk.upload(blk));
+  {
+    std::vector<int2> x(blk.size());
+    for (size_t i = 0; i < blk.size(); ++i) x[i] = fix_host(blk[i], 54);
+    BIE_TRY(wp->blkx.upload(x));
+  }
   BIE_TRY(upload_as(wp->blkf, blk));
   *out = wp.get();
   ctx->wigs[p] = std::move(wp);
@@ -696,8 +730,8 @@ static int setup_self(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, DevBuf<doub
       if (direct) continue;
       Phase ph(ctx, "kernel_proj", s);
       for (int kind = 0; kind < 2; ++kind) {
-        BIE_TRY(launch_kernel_proj(kind, cache, nt, p, pq, pl->cs.ptr, pl->T0.ptr, Q, s));
-        BIE_TRY(launch_unrotate(Q, t0 / nb, nt / nb, p, wp->blk.ptr, wp->stride, pp->cs.ptr, G.qk64[kind].ptr,
+        BIE_TRY(launch_kernel_proj(kind, cache, nt, p, pq, pl->CT.ptr, pl->PT.ptr, Q, s));
+        BIE_TRY(launch_unrotate(Q, t0 / nb, nt / nb, p, wp->blkx.ptr, wp->stride, pp->cs.ptr, G.qk64[kind].ptr,
                                 G.qk32[kind].ptr, s));
       }
     }

@@ -99,15 +99,17 @@ int launch_self_direct(int kind, const double* dens, const long long* foff3, lon
                        const double* wts, const long long* val_off, double* vals, size_t smem_budget,
                        cudaStream_t s);
 // Projected kernel factors Q[t][12][tri(n,m)] of ntarget targets (see self.cu), from the FP64
-// rotated-geometry cache and the degree-pq grid's Legendre table T0 (degrees <= p, all nodes).
+// rotated-geometry cache, with fixed-point tables (fixed.cuh): CT[k][m] = cos, sin (m phi_k) 2^55 for the
+// longitudes k <= (pq+1)/2, PT[j][tri(n, m)] = P~_n^m(t_j) 2^53 for the latitudes j <= pq/2.
 size_t kernel_proj_smem(int p, int pq);
-int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, int pq, const double* cs,
-                       const double* T0, double* Q64, cudaStream_t s);
+int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, int pq, const int4* CT, const int2* PT,
+                       double* Q64, cudaStream_t s);
 // Entries per plane of the dense self form: (p+1)^2 rounded up to whole 16-byte loads in every precision.
 __host__ __device__ inline int self_row(int p) { return ((p + 1) * (p + 1) + 3) & ~3; }
 // Dense factors S[target][6][self_row(p)] of the latitude rows row0 .. row0 + nrow - 1 (row = drop * (p+1) + a)
-// from their projected factors Q (Q64 starts at row0), written at the rows' places in S64 and S32.
-int launch_unrotate(const double* Q64, long long row0, long long nrow, int p, const double* wblk, long long wstride,
+// from their projected factors Q (Q64 starts at row0), written at the rows' places in S64 and S32; wblk: the
+// Wigner blocks times 2^54 in fixed point.
+int launch_unrotate(const double* Q64, long long row0, long long nrow, int p, const int2* wblk, long long wstride,
                     const double* ph, double* S64, float* S32, cudaStream_t s);
 // One degree group of the dense-form apply (device pointers; begin is set by the launcher).
 template <typename R>

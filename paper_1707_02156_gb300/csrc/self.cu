@@ -23,6 +23,7 @@
 
 #include "dfloat.cuh"
 #include "device.cuh"
+#include "fixed.cuh"
 #include "internal.cuh"
 
 namespace bie {
@@ -215,8 +216,10 @@ __global__ void __launch_bounds__(256) k_self_direct(
 // processed kProjPairs pairs (q, pq - q) at a time: kernel weights; their sums over the longitude
 // quadruples that share |cos m phi| and |sin m phi|, in place; the phi transform of both rows, whose sum
 // and difference serve even and odd n - m; and the Legendre projection, accumulated in shared memory.
-// Bound by the FP64 pipe: at p = pq = 24 about 0.21M operations per target and kind against 0.36M
-// without the symmetries and with the IEEE quotient and root for 1/r: 64 drops, both kinds 127 -> 64 ms.
+// The phi transform and the projection (0.15M multiply-adds per target and kind at p = pq = 24) run in
+// fixed point on the integer pipe (fixed.cuh), on one scale per target from a first pass over the kernel
+// weights; the FP64 pipe, which bounded the kernel before, keeps the weights themselves (37k operations).
+// 64 drops of degree 24, both kinds: 127 ms by the direct sums, 62 by the symmetries in FP64, now 32.
 constexpr int kProjPairs = 2;
 
 __device__ inline int tri_index_degree(int it) {
@@ -226,22 +229,49 @@ __device__ inline int tri_index_degree(int it) {
   return n;
 }
 
+// a bound on the exponent of the six entries at a point: |entry| <= 2 w / r for the Stokeslet and
+// 6 |x.a| / r^3 for the stresslet
+template <int KIND>
+__device__ __forceinline__ int weight_exponent(double r2, double wx) {
+  const double ri = rsqrt_<double>(r2);
+  return fix_exponent(KIND == 0 ? 2.0001 * wx * ri : 6.0001 * wx * ri * (ri * ri));
+}
+
 template <int KIND>
 __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ cache, int pq, int p,
-                                                     const double* __restrict__ cs, const double* __restrict__ T0,
+                                                     const int4* __restrict__ CT, const int2* __restrict__ PT,
                                                      double* __restrict__ Q64) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int emax;
   const long long t = blockIdx.x;
   const int nq_j = pq + 1, nk = 2 * pq + 2, half = pq + 1, np = (nq_j + 1) / 2, k4n = half / 2 + 1;
   const int ntri = (p + 1) * (p + 2) / 2;
   const int mid = half % 2 == 0 ? half / 2 : -1;
-  double* sk = reinterpret_cast<double*>(smem_raw);  // [pair][row][6][nk]
-  double* sd = sk + kProjPairs * 12 * nk;            // [pair][even, odd][12][p+1]
-  double* sq = sd + kProjPairs * 24 * (p + 1);       // [12][ntri]
+  double* sk = reinterpret_cast<double*>(smem_raw);                                  // [pair][row][6][nk]
+  int2* si = reinterpret_cast<int2*>(sk);                                            // the folded sums, in place
+  int2* sd = reinterpret_cast<int2*>(sk + kProjPairs * 12 * nk);                     // [pair][even, odd][12][p+1]
+  long long* sq = reinterpret_cast<long long*>(sd + kProjPairs * 24 * (p + 1));      // [12][ntri]
   const long long nq = (long long)nq_j * nk;
   const double* geo = cache + t * 7 * nq;
-  for (int i = threadIdx.x; i < 12 * ntri; i += blockDim.x) sq[i] = 0.0;
-  for (int q0 = 0; q0 < np; q0 += kProjPairs) {
+  for (int i = threadIdx.x; i < 12 * ntri; i += blockDim.x) sq[i] = 0;
+  if (threadIdx.x == 0) emax = fix_none;
+  __syncthreads();
+  {
+    int e = fix_none;
+    for (int o = threadIdx.x; o < nq; o += blockDim.x) {
+      const double x0 = geo[o], x1 = geo[nq + o], x2 = geo[2 * nq + o];
+      const double wx = KIND == 0 ? geo[6 * nq + o] : x0 * geo[3 * nq + o] + x1 * geo[4 * nq + o] + x2 * geo[5 * nq + o];
+      e = max(e, weight_exponent<KIND>(x0 * x0 + x1 * x1 + x2 * x2, wx));
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((threadIdx.x & 31) == 0) atomicMax(&emax, e);
+  }
+  __syncthreads();
+  const int e = emax == fix_none ? 0 : emax;
+  // units: folded sums 2^(e-54), of four entries, below 2^56; their phi transforms (tables 2^-55) 2^(e-53), below
+  // 2^(56 + log2 k4n), cut by sh bits to below 2^55; the projections (tables 2^-53) 2^(e-50+sh), accumulated with xb more bits
+  const int sh = ceil_log2(k4n) + 1, xb = 8 - ceil_log2(np);
+  for (int q0 = 0; q0 < np && e < fix_bad; q0 += kProjPairs) {
     const int qn = min(kProjPairs, np - q0);
     for (int i = threadIdx.x; i < qn * 2 * nk; i += blockDim.x) {
       const int row = i / nk, k = i - row * nk;
@@ -249,7 +279,7 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
       double* v = sk + row * 6 * nk + k;
       if ((row & 1) && 2 * q == pq) {  // the middle latitude has no mirror
 #pragma unroll
-        for (int e = 0; e < 6; ++e) v[e * nk] = 0.0;
+        for (int c = 0; c < 6; ++c) v[c * nk] = 0.0;
         continue;
       }
       const long long o = (long long)j * nk + k;
@@ -277,67 +307,76 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
     for (int i = threadIdx.x; i < qn * 12 * k4n; i += blockDim.x) {
       const int k = i % k4n;
       double* v = sk + (i / k4n) * nk;
-      const double a = v[k], c = v[half + k];
+      int2* w = si + (i / k4n) * nk;
+      const long long a = fix_encode(v[k], e), c = fix_encode(v[half + k], e);
       if (k == 0 || k == mid) {
-        v[k] = a + c;
-        v[half + k] = a - c;
+        w[k] = fix_split(a + c);
+        w[half + k] = fix_split(a - c);
       } else {
-        const double b = v[2 * half - k], d = v[half - k];
-        const double ab = a + b, cd = c + d, amb = a - b, cmd = c - d;
-        v[k] = ab + cd;
-        v[half + k] = ab - cd;
-        v[2 * half - k] = amb + cmd;
-        v[half - k] = amb - cmd;
+        const long long b = fix_encode(v[2 * half - k], e), d = fix_encode(v[half - k], e);
+        w[k] = fix_split((a + b) + (c + d));
+        w[half + k] = fix_split((a + b) - (c + d));
+        w[2 * half - k] = fix_split((a - b) + (c - d));
+        w[half - k] = fix_split((a - b) - (c - d));
       }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < qn * 6 * (p + 1); i += blockDim.x) {
       const int m = i % (p + 1);
       const int r = i / (p + 1);
-      const int e = r % 6, pair = r / 6;
-      const double* cm = cs + (long long)m * nk * 2;
-      const double* v0 = sk + (pair * 12 + e) * nk;  // row q; row pq - q is 6 nk further
-      const double* vc = v0 + ((m & 1) ? half : 0);
-      const double* vs = v0 + ((m & 1) ? half : 2 * half);
-      double re0 = vc[0], re1 = vc[6 * nk], im0 = 0, im1 = 0;
+      const int c = r % 6, pair = r / 6;
+      const int2* v0 = si + (pair * 12 + c) * nk;  // row q; row pq - q is 6 nk further
+      const int2* vc = v0 + ((m & 1) ? half : 0);
+      const int2* vs = v0 + ((m & 1) ? half : 2 * half);
+      long long h[4] = {0, 0, 0, 0}, x[4] = {0, 0, 0, 0};  // cosine and sine sums of the two rows
+      const int4 c0 = CT[m];
+      fix_mad(h[0], x[0], vc[0], make_int2(c0.x, c0.y));
+      fix_mad(h[1], x[1], vc[6 * nk], make_int2(c0.x, c0.y));
+#pragma unroll 2
       for (int k = 1; 2 * k < half; ++k) {
-        const double co = cm[2 * k], si = cm[2 * k + 1];
-        re0 += vc[k] * co;
-        re1 += vc[6 * nk + k] * co;
-        im0 += vs[-k] * si;
-        im1 += vs[6 * nk - k] * si;
+        const int4 cs = CT[k * (p + 1) + m];
+        const int2 co = make_int2(cs.x, cs.y), sn = make_int2(cs.z, cs.w);
+        fix_mad(h[0], x[0], vc[k], co);
+        fix_mad(h[1], x[1], vc[6 * nk + k], co);
+        fix_mad(h[2], x[2], vs[-k], sn);
+        fix_mad(h[3], x[3], vs[6 * nk - k], sn);
       }
       if (mid > 0) {
+        const int4 cs = CT[mid * (p + 1) + m];
         if (m & 1) {
-          im0 += v0[half + mid] * cm[2 * mid + 1];
-          im1 += v0[6 * nk + half + mid] * cm[2 * mid + 1];
+          fix_mad(h[2], x[2], v0[half + mid], make_int2(cs.z, cs.w));
+          fix_mad(h[3], x[3], v0[6 * nk + half + mid], make_int2(cs.z, cs.w));
         } else {
-          re0 += v0[mid] * cm[2 * mid];
-          re1 += v0[6 * nk + mid] * cm[2 * mid];
+          fix_mad(h[0], x[0], v0[mid], make_int2(cs.x, cs.y));
+          fix_mad(h[1], x[1], v0[6 * nk + mid], make_int2(cs.x, cs.y));
         }
       }
-      double* d = sd + (pair * 24 + 2 * e) * (p + 1) + m;
-      d[0] = re0 + re1;
-      d[p + 1] = im0 + im1;
-      d[12 * (p + 1)] = re0 - re1;
-      d[13 * (p + 1)] = im0 - im1;
+      const long long re0 = fix_sum(h[0], x[0], 0), re1 = fix_sum(h[1], x[1], 0), im0 = fix_sum(h[2], x[2], 0),
+                      im1 = fix_sum(h[3], x[3], 0);
+      const long long rnd = 1LL << (sh - 1);
+      int2* d = sd + (pair * 24 + 2 * c) * (p + 1) + m;
+      d[0] = fix_split((re0 + re1 + rnd) >> sh);
+      d[p + 1] = fix_split((im0 + im1 + rnd) >> sh);
+      d[12 * (p + 1)] = fix_split((re0 - re1 + rnd) >> sh);
+      d[13 * (p + 1)] = fix_split((im0 - im1 + rnd) >> sh);
     }
     __syncthreads();
     for (int it = threadIdx.x; it < ntri; it += blockDim.x) {
       const int n = tri_index_degree(it);
       const int m = it - n * (n + 1) / 2;
-      const double* Tn = T0 + leg_row(p, m, n, nq_j) + q0;
-      double acc[12];
+      int2 P[kProjPairs];
 #pragma unroll
-      for (int e = 0; e < 12; ++e) acc[e] = sq[e * ntri + it];
-      for (int pair = 0; pair < qn; ++pair) {
-        const double P = Tn[pair];
-        const double* d = sd + (pair * 24 + (((n - m) & 1) ? 12 : 0)) * (p + 1) + m;
+      for (int pair = 0; pair < kProjPairs; ++pair)
+        P[pair] = pair < qn ? PT[(long long)(q0 + pair) * ntri + it] : make_int2(0, 0);
+      const int2* d = sd + (((n - m) & 1) ? 12 : 0) * (p + 1) + m;
 #pragma unroll
-        for (int e = 0; e < 12; ++e) acc[e] += d[e * (p + 1)] * P;
+      for (int c = 0; c < 12; ++c) {
+        long long h = 0, x = 0;
+#pragma unroll
+        for (int pair = 0; pair < kProjPairs; ++pair)
+          if (pair < qn) fix_mad(h, x, d[(pair * 24 + c) * (p + 1)], P[pair]);
+        sq[c * ntri + it] += fix_sum(h, x, xb);
       }
-#pragma unroll
-      for (int e = 0; e < 12; ++e) sq[e * ntri + it] = acc[e];
     }
     __syncthreads();
   }
@@ -345,7 +384,8 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
   for (int i = threadIdx.x; i < 12 * ntri; i += blockDim.x) {
     const int it = i % ntri;
     const int n = tri_index_degree(it);
-    o64[i] = (it == n * (n + 1) / 2 ? 1.0 : 2.0) * sq[i];  // c_m
+    const double v = e < fix_bad ? fix_decode(sq[i], e - 50 + sh - xb) : __longlong_as_double(0x7ff8000000000000LL);
+    o64[i] = (it == n * (n + 1) / 2 ? 1.0 : 2.0) * v;  // c_m
   }
 }
 
@@ -353,17 +393,18 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
 // One block per (latitude row, degree n, chunk of kUnB longitudes).  With q_m = Q_re(n, m) for the real
 // and -Q_im(n, m) for the imaginary parts of rho'_n^m, and rho' = (C Re g, S Im g), g = e^{i m phi_b} rho,
 // the transposed rotation is s_re = C^T q_re, s_im = S^T q_im and the transposed phase
-// (s_re cos + s_im sin, s_im cos - s_re sin).  FP64-pipe-bound like the factors' own kernels (2n+1
-// multiply-adds per entry and coefficient); the leading dimensions of the staged blocks are odd, so
-// that the strided reads of the transposed products hit every bank.  64 drops of p = 24, both kinds: 20 ms, of
-// which an apply saves 1.5 ms in double-float and 0.45 ms in FP32.
+// (s_re cos + s_im sin, s_im cos - s_re sin).  The 2n+1 products per entry and coefficient run in fixed point
+// on the integer pipe (fixed.cuh), on one scale per block; two entries at a time share the reads of the
+// Wigner block, and the leading dimensions of the staged blocks are odd, so that the strided reads of the
+// transposed products hit every bank.  64 drops of p = 24, both kinds: 20 ms in FP64, now 12.
 constexpr int kUnB = 8;
 
 __global__ void __launch_bounds__(128) k_unrotate(const double* __restrict__ Q64, long long row0, int p,
-                                                  const double* __restrict__ wblk, long long wstride,
+                                                  const int2* __restrict__ wblk, long long wstride,
                                                   const double* __restrict__ ph, int ncp, double* __restrict__ S64,
                                                   float* __restrict__ S32) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int emax;
   const int nb = 2 * p + 2, nbch = (nb + kUnB - 1) / kUnB;
   const int b0 = (int)(blockIdx.x % nbch) * kUnB;
   const long long row = row0 + blockIdx.x / nbch;  // latitude row of the group: drop * (p+1) + a
@@ -372,50 +413,80 @@ __global__ void __launch_bounds__(128) k_unrotate(const double* __restrict__ Q64
   const int nbh = min(kUnB, nb - b0);
   const int ntri = (p + 1) * (p + 2) / 2, t0 = n * (n + 1) / 2;
   const int ldC = (n + 1) | 1, ldS = n | 1;
-  double* sC = reinterpret_cast<double*>(smem_raw);  // [m][m']
-  double* sS = sC + (n + 1) * ldC;
-  double* sq = sS + n * ldS;                          // [bb][e][re 0..n, im 1..n]
-  const double* blk = wblk + (long long)a * wstride + (long long)n * (n + 1) * (2 * n + 1) / 6 +
-                      (long long)(n - 1) * n * (2 * n - 1) / 6;
+  int2* sC = reinterpret_cast<int2*>(smem_raw);  // [m][m']
+  int2* sS = sC + (n + 1) * ldC;
+  int2* sq = sS + n * ldS;                        // [bb][e][re 0..n, im 1..n]
+  const int2* blk = wblk + (long long)a * wstride + (long long)n * (n + 1) * (2 * n + 1) / 6 +
+                    (long long)(n - 1) * n * (2 * n - 1) / 6;
+  if (threadIdx.x == 0) emax = fix_none;
   for (int i = threadIdx.x; i < (n + 1) * (n + 1); i += blockDim.x) sC[(i / (n + 1)) * ldC + i % (n + 1)] = blk[i];
   for (int i = threadIdx.x; i < n * n; i += blockDim.x) sS[(i / n) * ldS + i % n] = blk[(n + 1) * (n + 1) + i];
-  const int w = 2 * n + 1;
-  const double* Qr = Q64 + (row - row0) * nb * 12 * ntri;
-  for (int i = threadIdx.x; i < nbh * 12 * (n + 1); i += blockDim.x) {
-    const int m = i % (n + 1), g = i / (n + 1);
-    const int plane = g % 12, bb = g / 12;
-    const double v = Qr[((long long)(b0 + bb) * 12 + plane) * ntri + t0 + m];
-    double* q = sq + (bb * 6 + plane / 2) * w;
-    if (!(plane & 1))
-      q[m] = v;
-    else if (m > 0)
-      q[n + m] = -v;
+  __syncthreads();
+  const int w = 2 * n + 1, nin = nbh * 12 * (n + 1);
+  const double* Qr = Q64 + (row - row0) * nb * 12 * ntri + (long long)b0 * 12 * ntri + t0;
+  {
+    int e = fix_none;
+    for (int i = threadIdx.x; i < nin; i += blockDim.x)
+      e = max(e, fix_exponent(Qr[(long long)(i / (n + 1)) * ntri + i % (n + 1)]));
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((threadIdx.x & 31) == 0) atomicMax(&emax, e);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < nbh * 6 * (n + 1); i += blockDim.x) {
+  const bool bad = emax == fix_bad;
+  const int e = emax == fix_none || bad ? 0 : emax;
+  for (int i = threadIdx.x; i < nin; i += blockDim.x) {
     const int m = i % (n + 1), g = i / (n + 1);
-    const int bb = g / 6, e = g - bb * 6;
-    const double* q = sq + g * w;
-    const double* c = sC + m * ldC;
-    double re = 0, im = 0;
-    for (int k = 0; k <= n; ++k) re += c[k] * q[k];
-    if (m > 0) {
-      const double* sn = sS + (m - 1) * ldS;
-      for (int k = 1; k <= n; ++k) im += sn[k - 1] * q[n + k];
+    const int plane = g % 12, bb = g / 12;
+    const long long v = bad ? 0 : fix_encode(Qr[(long long)g * ntri + m], e);
+    int2* q = sq + (bb * 6 + plane / 2) * w;
+    if (!(plane & 1))
+      q[m] = fix_split(v);
+    else if (m > 0)
+      q[n + m] = fix_split(-v);
+  }
+  __syncthreads();
+  // units: factors 2^(e-54), blocks 2^-54, sums 2^(e-52) with xb more bits: (n+1) 2^53 2^xb < 2^62
+  const int xb = 9 - ceil_log2(n + 1);
+  for (int i = threadIdx.x; i < nbh * 3 * (n + 1); i += blockDim.x) {
+    const int m = i % (n + 1), g = i / (n + 1) * 2;  // entries g and g + 1 of [bb][e]
+    const int2* q = sq + g * w;
+    const int2* c = sC + m * ldC;
+    long long h[4] = {0, 0, 0, 0}, x[4] = {0, 0, 0, 0};  // real parts of the two entries, then imaginary
+#pragma unroll 2
+    for (int k = 0; k <= n; ++k) {
+      const int2 cv = c[k];
+      fix_mad(h[0], x[0], cv, q[k]);
+      fix_mad(h[1], x[1], cv, q[w + k]);
     }
-    const double co = ph[((long long)m * nb + b0 + bb) * 2], si = ph[((long long)m * nb + b0 + bb) * 2 + 1];
-    const long long o = ((row * nb + b0 + bb) * 6 + e) * ncp + n * (n + 1);
-    const double vr = m > 0 ? re * co + im * si : re;
-    S64[o + m] = vr;
-    S32[o + m] = (float)vr;
     if (m > 0) {
-      const double vi = im * co - re * si;
-      S64[o - m] = vi;
-      S32[o - m] = (float)vi;
-    } else if (n == p) {  // the padding of the row
-      for (int r = p + 1; r < ncp - p * (p + 1); ++r) {
-        S64[o + r] = 0.0;
-        S32[o + r] = 0.0f;
+      const int2* sn = sS + (m - 1) * ldS - 1;
+#pragma unroll 2
+      for (int k = 1; k <= n; ++k) {
+        const int2 sv = sn[k];
+        fix_mad(h[2], x[2], sv, q[n + k]);
+        fix_mad(h[3], x[3], sv, q[w + n + k]);
+      }
+    }
+    const int bb = g / 6, en = g - bb * 6;
+    const double co = ph[((long long)m * nb + b0 + bb) * 2], si = ph[((long long)m * nb + b0 + bb) * 2 + 1];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const double nan = __longlong_as_double(0x7ff8000000000000LL);
+      const double re = bad ? nan : fix_decode(fix_sum(h[u], x[u], xb), e - 52 - xb);
+      const double im = bad ? nan : fix_decode(fix_sum(h[2 + u], x[2 + u], xb), e - 52 - xb);
+      const long long o = ((row * nb + b0 + bb) * 6 + en + u) * ncp + n * (n + 1);
+      const double vr = m > 0 ? re * co + im * si : re;
+      S64[o + m] = vr;
+      S32[o + m] = (float)vr;
+      if (m > 0) {
+        const double vi = im * co - re * si;
+        S64[o - m] = vi;
+        S32[o - m] = (float)vi;
+      } else if (n == p) {  // the padding of the row
+        for (int r = p + 1; r < ncp - p * (p + 1); ++r) {
+          S64[o + r] = 0.0;
+          S32[o + r] = 0.0f;
+        }
       }
     }
   }
@@ -575,8 +646,8 @@ size_t kernel_proj_smem(int p, int pq) {
   return sizeof(double) * ((size_t)kProjPairs * 24 * (pq + 1) + (size_t)kProjPairs * 24 * (p + 1) + 6 * (size_t)(p + 1) * (p + 2));
 }
 
-int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, int pq, const double* cs,
-                       const double* T0, double* Q64, cudaStream_t s) {
+int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, int pq, const int4* CT, const int2* PT,
+                       double* Q64, cudaStream_t s) {
   if (ntarget == 0) return BIE_OK;
   if (ntarget > 0x7fffffffLL) return BIE_EINVAL;
   const size_t smem = kernel_proj_smem(p, pq);
@@ -586,13 +657,13 @@ int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, 
   }
   auto kern = kind == 0 ? k_kernel_proj<0> : k_kernel_proj<1>;
   if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<(unsigned)ntarget, 256, smem, s>>>(cache, pq, p, cs, T0, Q64);
+  kern<<<(unsigned)ntarget, 256, smem, s>>>(cache, pq, p, CT, PT, Q64);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
 }
 
-int launch_unrotate(const double* Q64, long long row0, long long nrow, int p, const double* wblk, long long wstride,
+int launch_unrotate(const double* Q64, long long row0, long long nrow, int p, const int2* wblk, long long wstride,
                     const double* ph, double* S64, float* S32, cudaStream_t s) {
   if (nrow == 0) return BIE_OK;
   const int nbch = (2 * p + 2 + kUnB - 1) / kUnB;

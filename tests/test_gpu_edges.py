@@ -5,6 +5,8 @@ quadruples (a middle longitude exists for an odd P), and a block takes more or f
 orders with the number of fields; the dense self factors pad (p+1)^2 to whole 16-byte loads; the rows of
 the near-singular rule fold the standard and the upsampled grid.  Every parity and remainder is
 compared with the FP64 oracle at the bars of the other parity tests."""
+import math
+
 import numpy as np
 import pytest
 
@@ -74,6 +76,29 @@ def test_dense_self_term_at_every_row_padding(api, p, double):
         for prec, tol in ((0, FP64_TOL), (1, MIXED_TOL), (2, DF_TOL)):
             fn(f, out, precision=prec)
             assert relerr(host(out), r) < tol, (prec,)
+    geo.close()
+    ctx.close()
+
+
+@pytest.mark.parametrize("p, pq, scale, shift", [(5, 5, 1e-9, 0.0), (6, 13, 1e9, 3e9), (36, 36, 1.0, 0.0), (37, 37, 1.0, 7.0),
+                                                  (62, 62, 1.0, 0.0), (63, 63, 1.0, 0.0)])
+def test_self_setup_over_sizes_and_scales(api, p, pq, scale, shift):
+    # the rotated-grid set-up takes two latitude pairs per pass up to degree 36, one up to 62 and goes through
+    # memory above; its fixed-point sums scale with the drop and leave its position out
+    w = inputs.perturbed_drop(p=p, pq=pq, lam=3.0, nmax=min(p, 6))
+    x = w.xcoef.reshape(3, -1) * scale
+    x[:, 0] += shift
+    ctx = api.Context(0)
+    geo = ctx.geometry(w.p, w.pq, dev(x), w.lam)
+    q = layer.SelfQuadrature(x, p, pq)
+    lats = [0, p // 2, p] if p < 60 else [p // 2]
+    f = dev(w.density)
+    out = torch.zeros(3 * (p + 1) * (2 * p + 2), dtype=torch.float64, device="cuda")
+    for kind, fn, wt in (("S", geo.apply_single, -1 / (4 * math.pi)), ("D", geo.apply_double, 2 / (4 * math.pi))):
+        ref = wt * q.apply(w.density, kind, lats=lats)
+        fn(f, out, precision=0, grid_out=True)
+        g = host(out).reshape(3, p + 1, 2 * p + 2)
+        assert relerr(g[:, lats, :], ref[:, lats, :]) < FP64_TOL, (kind,)
     geo.close()
     ctx.close()
 
