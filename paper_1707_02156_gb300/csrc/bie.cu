@@ -82,8 +82,9 @@ struct Plan {
   int p = 0, P = 0;
   DevBuf<double> T0, T1, T2, At, cs, wsin, wsq;
   DevBuf<float> T0f, csf;
-  DevBuf<int4> CT;  // fixed-point tables of the kernel factors (p <= P <= 2p+1): see launch_kernel_proj
-  DevBuf<int2> PT;
+  DevBuf<int4> CT, CM, CP;  // fixed-point tables of the set-up kernels (P <= 2p+1): see launch_kernel_proj, RotGeo
+  DevBuf<int2> PT, LT0, LT1;
+  DevBuf<int> t1;
   template <typename R>
   const R* T0_() const;
   template <typename R>
@@ -117,7 +118,7 @@ struct WigPlan {  // rotation blocks for the p+1 latitudes of the degree-p grid
   int p = 0;
   long long stride = 0;
   DevBuf<double> blk;
-  DevBuf<int2> blkx;  // times 2^54 in fixed point (entries up to 2)
+  DevBuf<int2> blkx;  // times 2^56 in fixed point (entries up to 2)
   DevBuf<float> blkf;
   template <typename R>
   const R* blk_() const;
@@ -208,8 +209,28 @@ static int get_plan(bie_ctx* ctx, int p, int P, Plan** out) {
     for (int n = 0; n <= p; ++n)
       for (int m = 0; m <= n; ++m)
         for (int j = 0; j < nh; ++j)
-          x[(size_t)j * (p + 1) * (p + 2) / 2 + n * (n + 1) / 2 + m] = fix_host(v[leg_row(p, m, n, P + 1) + j], 53);
+          x[(size_t)j * (p + 1) * (p + 2) / 2 + n * (n + 1) / 2 + m] = fix_host(v[leg_row(p, m, n, P + 1) + j], 55);
     BIE_TRY(pl->PT.upload(x));
+    const size_t ntri = (size_t)(p + 1) * (p + 2) / 2;
+    auto diag = [&](int n, int m) { return (size_t)(n - m) * (p + 1) - (n - m) * (n - m - 1) / 2 + m; };
+    std::vector<double> w;
+    legendre_table(p, P, 1, w);
+    std::vector<int> t1(p + 1, 0);
+    std::vector<int2> y(x.size());
+    for (int n = 0; n <= p; ++n) {
+      double mx = 0;
+      for (int m = 0; m <= n; ++m)
+        for (int j = 0; j < nh; ++j) mx = std::max(mx, std::fabs(w[leg_row(p, m, n, P + 1) + j]));
+      while (std::ldexp(mx, -t1[n]) > 2.0) ++t1[n];
+      for (int m = 0; m <= n; ++m)
+        for (int j = 0; j < nh; ++j) {
+          x[j * ntri + diag(n, m)] = fix_host(v[leg_row(p, m, n, P + 1) + j], 56);
+          y[j * ntri + diag(n, m)] = fix_host(w[leg_row(p, m, n, P + 1) + j], 56 - t1[n]);
+        }
+    }
+    BIE_TRY(pl->LT0.upload(x));
+    BIE_TRY(pl->LT1.upload(y));
+    BIE_TRY(pl->t1.upload(t1));
   }
   legendre_table(p, P, 1, v);
   BIE_TRY(pl->T1.upload(v));
@@ -235,6 +256,20 @@ static int get_plan(bie_ctx* ctx, int p, int P, Plan** out) {
         x[(size_t)k * (p + 1) + m] = make_int4(c.x, c.y, sn.x, sn.y);
       }
     BIE_TRY(pl->CT.upload(x));
+    std::vector<int4> y(x.size());
+    for (int m = 0; m <= p; ++m) {
+      int tm = 0;
+      while ((2 << tm) <= m) ++tm;
+      for (int k = 0; k < kn; ++k) {
+        const double* cs = &v[((size_t)m * nk + k) * 2];
+        const int2 c = fix_host(cs[0], 56), sn = fix_host(cs[1], 56);
+        x[(size_t)m * kn + k] = make_int4(c.x, c.y, sn.x, sn.y);
+        const int2 cm = fix_host(cs[0] * m, 55 - tm), sm = fix_host(cs[1] * m, 55 - tm);
+        y[(size_t)m * kn + k] = make_int4(cm.x, cm.y, sm.x, sm.y);
+      }
+    }
+    BIE_TRY(pl->CM.upload(x));
+    BIE_TRY(pl->CP.upload(y));
   }
   BIE_TRY(upload_as(pl->csf, v));
   std::vector<double> t, w, ws;
@@ -270,7 +305,7 @@ static int get_wig(bie_ctx* ctx, int p, WigPlan** out) {
   BIE_TRY(wp->blk.upload(blk));
   {
     std::vector<int2> x(blk.size());
-    for (size_t i = 0; i < blk.size(); ++i) x[i] = fix_host(blk[i], 54);
+    for (size_t i = 0; i < blk.size(); ++i) x[i] = fix_host(blk[i], 56);
     BIE_TRY(wp->blkx.upload(x));
   }
   BIE_TRY(upload_as(wp->blkf, blk));
@@ -694,10 +729,11 @@ static int setup_self(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, DevBuf<doub
   BIE_TRY(get_plan(ctx, p, pq, &pl));
   BIE_TRY(get_plan(ctx, p, p, &pp));
   BIE_TRY(get_wig(ctx, p, &wp));
-  // doubles per target: rotated coefficients, x and its derivatives, and in dense form the cache and the
-  // projected factors of one layer
-  const long long nQ = 6LL * (p + 1) * (p + 2);
-  const long long per = 3 * nc + 9 * nq + (direct ? 0 : 7 * nq + nQ);
+  // doubles per target: where the cache is not made in one kernel (degrees above 62), rotated coefficients, x
+  // and its derivatives; in dense form the cache and the projected factors of one layer
+  const bool fix = rotgeo_fix_fits(p, pq);
+  const long long nQ = 6LL * (p + 1) * (p + 2), nX = fix ? 0 : 3 * nc + 9 * nq;
+  const long long per = std::max(1LL, nX + (direct ? 0 : 7 * nq + nQ));
   const long long fit = std::max<long long>(nb, (2LL << 30) / 8 / per);  // targets at a time
   const int dstep = (int)std::max<long long>(1, std::min<long long>(nd, fit / ng));
   const int astep = (int)std::max<long long>(1, std::min<long long>(p + 1, fit / nb));
@@ -717,15 +753,22 @@ static int setup_self(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, DevBuf<doub
       const long long nt = dn * an * nb, t0 = d0 * ng + a0 * nb;  // targets of the chunk, the group's first one
       double* RC = work.ptr;
       double* X = RC + nt * 3 * nc;
-      double* cache = direct ? G.cache64.ptr + t0 * 7 * nq : X + nt * 9 * nq;
+      double* cache = direct ? G.cache64.ptr + t0 * 7 * nq : work.ptr + nt * nX;
       double* Q = cache + nt * 7 * nq;
       {
         Phase ph(ctx, "setup_rotcache", s);
-        BIE_TRY((launch_rotate<double, double>(g->xcoef.ptr, G.foff3.ptr + 3 * d0, 3, dn, p, wp->blk.ptr + a0 * wp->stride,
-                                               wp->stride, an, (int)nb, pp->cs.ptr, RC, an * nb * 3 * nc, s)));
-        BIE_TRY(synth_xderivs(ctx, RC, nullptr, nc, nt * 3, p, pq, X, s));
-        BIE_TRY(launch_rotgeo<double>(X, X + nt * 3 * nq, X + nt * 6 * nq, dn, (int)(an * nb), (int)(a0 * nb), (int)ng, pq,
-                                      g->rec_std.ptr, G.roff.ptr + d0, pl->wsq.ptr, cache, s));
+        if (fix) {
+          const RotGeo rg{p, pq, (int)(an * nb), (int)(a0 * nb), g->xcoef.ptr, G.foff3.ptr + 3 * d0, pp->cs.ptr,
+                          wp->blkx.ptr, wp->stride, pl->LT0.ptr, pl->LT1.ptr, pl->t1.ptr, pl->CM.ptr, pl->CP.ptr,
+                          g->rec_std.ptr, G.roff.ptr + d0, pl->wsq.ptr};
+          BIE_TRY(launch_rotgeo_fix(rg, dn, cache, s));
+        } else {
+          BIE_TRY((launch_rotate<double, double>(g->xcoef.ptr, G.foff3.ptr + 3 * d0, 3, dn, p, wp->blk.ptr + a0 * wp->stride,
+                                                 wp->stride, an, (int)nb, pp->cs.ptr, RC, an * nb * 3 * nc, s)));
+          BIE_TRY(synth_xderivs(ctx, RC, nullptr, nc, nt * 3, p, pq, X, s));
+          BIE_TRY(launch_rotgeo<double>(X, X + nt * 3 * nq, X + nt * 6 * nq, dn, (int)(an * nb), (int)(a0 * nb), (int)ng, pq,
+                                        g->rec_std.ptr, G.roff.ptr + d0, pl->wsq.ptr, cache, s));
+        }
       }
       if (direct) continue;
       Phase ph(ctx, "kernel_proj", s);

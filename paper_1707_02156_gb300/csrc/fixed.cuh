@@ -1,7 +1,7 @@
 // Sums of products in fixed point on the integer pipe, for set-up contractions whose operation count the FP64
 // pipe bounds: GB300 does 1.7 FP64 multiply-adds per clock and SM, and 30 of the 32 x 32 + 64 bit integer
 // ones.  A value is scaled by a power of two common to the sum's operands, rounded to an integer of at
-// most 56 bits and split into a high and a centred low part of 28 bits; a product is then
+// most 56 bits (tables: 59) and split into a high and a centred low part of 28 bits; a product is then
 //   (a_h 2^28 + a_l)(b_h 2^28 + b_l) = a_h b_h 2^56 + (a_h b_l + a_l b_h) 2^28 + a_l b_l,
 // whose first two terms are accumulated exactly in two 64-bit sums (three multiply-adds a product) and whose
 // last one, below 2^-56 of the largest product, is left out.  Against the largest operand a sum of K products

@@ -91,6 +91,27 @@ int launch_surface(const double* X, const double* Xt, const double* Xp, long lon
 template <typename R>
 int launch_rotgeo(const double* X, const double* Xt, const double* Xp, long long ndrop, int nt, int tl0, int ng, int pq,
                   const double* rec_std, const long long* rec_off, const double* wsq, R* cache, cudaStream_t s);
+// The same cache from the shape coefficients in one kernel (rotgeo.cu), for the degrees whose block fits shared
+// memory.  Fixed-point tables (fixed.cuh) of the degree-pq grid: LT0, LT1[j][diag(n - m) + m] = P~_n^m(t_j) 2^56
+// and its theta derivative times 2^(56 - t1[n]) for the latitudes j <= pq/2, diag(d) the entries with a
+// smaller n - m; CM, CP[m][k] = cos, sin (m phi_k) times 2^56 and times m 2^(55 - floor(log2 m)) for the
+// longitudes k <= (pq+1)/2; wblk the Wigner blocks times 2^56.
+struct RotGeo {
+  int p, pq, nt, tl0;        // nt targets, from tl0 on, of each drop
+  const double* coef;
+  const long long* foff3;    // [drop][3]
+  const double* ph;          // phases of the degree-p grid
+  const int2* wblk;
+  long long wstride;
+  const int2 *LT0, *LT1;
+  const int* t1;
+  const int4 *CM, *CP;
+  const double* rec_std;
+  const long long* rec_off;
+  const double* wsq;
+};
+bool rotgeo_fix_fits(int p, int pq);
+int launch_rotgeo_fix(const RotGeo& A, long long ndrop, double* cache, cudaStream_t s);
 // Singular self interaction (Thm 1, Sec. 2.2), one block per target of ndrop drops of degree p:
 // direct form against the rotated-geometry cache.
 template <typename R>
@@ -100,7 +121,7 @@ int launch_self_direct(int kind, const double* dens, const long long* foff3, lon
                        cudaStream_t s);
 // Projected kernel factors Q[t][12][tri(n,m)] of ntarget targets (see self.cu), from the FP64
 // rotated-geometry cache, with fixed-point tables (fixed.cuh): CT[k][m] = cos, sin (m phi_k) 2^55 for the
-// longitudes k <= (pq+1)/2, PT[j][tri(n, m)] = P~_n^m(t_j) 2^53 for the latitudes j <= pq/2.
+// longitudes k <= (pq+1)/2, PT[j][tri(n, m)] = P~_n^m(t_j) 2^55 for the latitudes j <= pq/2.
 size_t kernel_proj_smem(int p, int pq);
 int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, int pq, const int4* CT, const int2* PT,
                        double* Q64, cudaStream_t s);

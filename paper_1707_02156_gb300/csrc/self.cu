@@ -269,8 +269,9 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
   __syncthreads();
   const int e = emax == fix_none ? 0 : emax;
   // units: folded sums 2^(e-54), of four entries, below 2^56; their phi transforms (tables 2^-55) 2^(e-53), below
-  // 2^(56 + log2 k4n), cut by sh bits to below 2^55; the projections (tables 2^-53) 2^(e-50+sh), accumulated with xb more bits
-  const int sh = ceil_log2(k4n) + 1, xb = 8 - ceil_log2(np);
+  // 2^(56 + log2 k4n), cut by sh bits to below 2^55; the projections (tables 2^-55) 2^(e-52+sh), accumulated with xb more
+  // bits (np <= 64: larger grids take the direct form)
+  const int sh = ceil_log2(k4n) + 1, xb = 6 - ceil_log2(np);
   for (int q0 = 0; q0 < np && e < fix_bad; q0 += kProjPairs) {
     const int qn = min(kProjPairs, np - q0);
     for (int i = threadIdx.x; i < qn * 2 * nk; i += blockDim.x) {
@@ -384,7 +385,7 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
   for (int i = threadIdx.x; i < 12 * ntri; i += blockDim.x) {
     const int it = i % ntri;
     const int n = tri_index_degree(it);
-    const double v = e < fix_bad ? fix_decode(sq[i], e - 50 + sh - xb) : __longlong_as_double(0x7ff8000000000000LL);
+    const double v = e < fix_bad ? fix_decode(sq[i], e - 52 + sh - xb) : __longlong_as_double(0x7ff8000000000000LL);
     o64[i] = (it == n * (n + 1) / 2 ? 1.0 : 2.0) * v;  // c_m
   }
 }
@@ -445,8 +446,8 @@ __global__ void __launch_bounds__(128) k_unrotate(const double* __restrict__ Q64
       q[n + m] = fix_split(-v);
   }
   __syncthreads();
-  // units: factors 2^(e-54), blocks 2^-54, sums 2^(e-52) with xb more bits: (n+1) 2^53 2^xb < 2^62
-  const int xb = 9 - ceil_log2(n + 1);
+  // units: factors 2^(e-54), blocks 2^-56 (up to 2), sums 2^(e-54) with xb more bits: (n+1) 2^55 2^xb <= 2^62
+  const int xb = 7 - ceil_log2(n + 1);
   for (int i = threadIdx.x; i < nbh * 3 * (n + 1); i += blockDim.x) {
     const int m = i % (n + 1), g = i / (n + 1) * 2;  // entries g and g + 1 of [bb][e]
     const int2* q = sq + g * w;
@@ -472,8 +473,8 @@ __global__ void __launch_bounds__(128) k_unrotate(const double* __restrict__ Q64
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const double nan = __longlong_as_double(0x7ff8000000000000LL);
-      const double re = bad ? nan : fix_decode(fix_sum(h[u], x[u], xb), e - 52 - xb);
-      const double im = bad ? nan : fix_decode(fix_sum(h[2 + u], x[2 + u], xb), e - 52 - xb);
+      const double re = bad ? nan : fix_decode(fix_sum(h[u], x[u], xb), e - 54 - xb);
+      const double im = bad ? nan : fix_decode(fix_sum(h[2 + u], x[2 + u], xb), e - 54 - xb);
       const long long o = ((row * nb + b0 + bb) * 6 + en + u) * ncp + n * (n + 1);
       const double vr = m > 0 ? re * co + im * si : re;
       S64[o + m] = vr;
