@@ -1442,6 +1442,8 @@ static int interdrop_apply(bie_geom* g, int kind, bool raw, const double* dens, 
 // interpolation anchored at the exterior limit of the source drop's on-surface values.
 constexpr long long kPtChunk = 32768;  // points per pass at most: 256 tiles
 
+// With both layers asked for, their sum is what the caller gets from the two outputs: the near-singular part of
+// both lies in the first.
 static int eval_layers(bie_ctx* ctx, bie_geom* g, long long npt, const double* pts, const double* const dens[2],
                        double* const out[2], int precision, cudaStream_t s) {
   const bool raw = (precision & BIE_RAW) != 0;
@@ -1649,7 +1651,7 @@ static int eval_layers(bie_ctx* ctx, bie_geom* g, long long npt, const double* p
   tbeg.push_back(npair);
   DevBuf<NearPair> d_pairs;
   DevBuf<int> d_seed, d_tbeg, d_grid, d_tdrop, d_ngd1;
-  DevBuf<double> d_npts, d_cv, c64s, c64u;
+  DevBuf<double> d_npts, d_cv;
   DevBuf<long long> d_tloc, d_voff1;
   BIE_TRY(d_pairs.upload(pairs));
   BIE_TRY(d_seed.alloc(npair));
@@ -1680,33 +1682,54 @@ static int eval_layers(bie_ctx* ctx, bie_geom* g, long long npt, const double* p
   const std::vector<int> ng1{(int)npt};
   BIE_TRY(d_voff1.upload(vo));
   BIE_TRY(d_ngd1.upload(ng1));
-  for (int k : kinds) {
-    const double* wts = weights(k);
-    // the on-surface values of the source drops in this precision, as SH expansions
+  // the on-surface values of the source drops in this precision, as SH expansions
+  auto expansions = [&](int k) -> int {
     if (prec == BIE_MIXED)
       BIE_TRY(self_apply<float>(g, k, raw, dens[k], s));
     else if (prec == BIE_DF)
       BIE_TRY(self_apply<dff>(g, k, raw, dens[k], s));
     else
       BIE_TRY(self_apply<double>(g, k, raw, dens[k], s));
-    BIE_TRY(near_snapshot(g, s));
-    // the check-point values in FP64 (the interpolation amplifies their errors)
-    const double *qs = q64[k][0].ptr, *qu = q64[k][1].ptr;
-    if (prec == BIE_MIXED) {
-      BIE_TRY(c64s.alloc(3 * g->ntarget));
-      BIE_TRY(c64u.alloc(3 * g->nup_total));
-      BIE_TRY(source_densities<double>(g, dens[k], c64s.ptr, c64u.ptr, s));
-      qs = c64s.ptr;
-      qu = c64u.ptr;
+    return near_snapshot(g, s);
+  };
+  // the check-point values in FP64 (the interpolation amplifies their errors)
+  const double *qs[2] = {q64[0][0].ptr, q64[1][0].ptr}, *qu[2] = {q64[0][1].ptr, q64[1][1].ptr};
+  DevBuf<double> c64[2][2], both;
+  if (prec == BIE_MIXED)
+    for (int k : kinds) {
+      BIE_TRY(c64[k][0].alloc(3 * g->ntarget));
+      BIE_TRY(c64[k][1].alloc(3 * g->nup_total));
+      BIE_TRY(source_densities<double>(g, dens[k], c64[k][0].ptr, c64[k][1].ptr, s));
+      qs[k] = c64[k][0].ptr;
+      qu[k] = c64[k][1].ptr;
     }
+  const double* anchor = g->selfcoef.ptr;
+  const int last = kinds.back();
+  BIE_TRY(expansions(kinds[0]));
+  if (kinds.size() == 2) {
+    // both layers are added by the caller (the velocity): their near values go to the first one's output together
+    BIE_TRY(both.alloc(g->ncoef_total));
+    BIE_CUDA_TRY(cudaMemcpyAsync(both.ptr, g->selfcoef.ptr, g->ncoef_total * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    BIE_TRY(expansions(1));
+    BIE_TRY(launch_add(g->selfcoef.ptr, g->ncoef_total, both.ptr, s));
+    anchor = both.ptr;
+  }
+  {
     Phase phc(ctx, "near_checks", s);
-    BIE_TRY(launch_near_checks<double>(k, d_pairs.ptr, npair, L, d_npts.ptr, d_grid.ptr, g->centre_d.ptr,
-                                       g->toff.ptr, g->ngd.ptr, g->up_off_d.ptr, g->up_n_d.ptr, g->sX64.ptr,
-                                       g->sN64.ptr, qs, g->ntarget, g->uX64.ptr, g->uN64.ptr, qu, g->nup_total, wts,
-                                       d_cv.ptr, s));
-    BIE_TRY(launch_near_interp(d_pairs.ptr, d_tbeg.ptr, ntgt, L, k, g->selfcoef.ptr, dens[k], g->coef_off_d.ptr,
-                               g->pdeg_d.ptr, g->hdrop_d.ptr, wts, d_cv.ptr, d_tdrop.ptr, d_tloc.ptr, d_voff1.ptr,
-                               d_ngd1.ptr, out[k], s));
+    if (kinds.size() == 2)
+      BIE_TRY(launch_near_checks_both(d_pairs.ptr, npair, L, d_npts.ptr, d_grid.ptr, g->centre_d.ptr, g->toff.ptr,
+                                      g->ngd.ptr, g->up_off_d.ptr, g->up_n_d.ptr,
+                                      {g->sX64.ptr, g->sN64.ptr, qs[0], qs[1], g->ntarget},
+                                      {g->uX64.ptr, g->uN64.ptr, qu[0], qu[1], g->nup_total}, weights(0), weights(1),
+                                      d_cv.ptr, s));
+    else
+      BIE_TRY(launch_near_checks<double>(last, d_pairs.ptr, npair, L, d_npts.ptr, d_grid.ptr, g->centre_d.ptr,
+                                         g->toff.ptr, g->ngd.ptr, g->up_off_d.ptr, g->up_n_d.ptr, g->sX64.ptr,
+                                         g->sN64.ptr, qs[last], g->ntarget, g->uX64.ptr, g->uN64.ptr, qu[last],
+                                         g->nup_total, weights(last), d_cv.ptr, s));
+    BIE_TRY(launch_near_interp(d_pairs.ptr, d_tbeg.ptr, ntgt, L, last, anchor, dens[last], g->coef_off_d.ptr,
+                               g->pdeg_d.ptr, g->hdrop_d.ptr, weights(last), d_cv.ptr, d_tdrop.ptr, d_tloc.ptr,
+                               d_voff1.ptr, d_ngd1.ptr, out[kinds[0]], s));
   }
   BIE_CUDA_TRY(cudaStreamSynchronize(s));
   return BIE_OK;

@@ -38,6 +38,17 @@ int launch_near_checks(int kind, const NearPair* pairs, int npair, int L, const 
                        const double* centre, const long long* toff, const int* ngd, const long long* up_off,
                        const long long* up_n, const R* Xs, const R* Ns, const R* Qs, long long nstd, const R* Xu,
                        const R* Nu, const R* Qu, long long nup, const double* wts, double* cv, cudaStream_t s);
+// Sources of one grid, [3][ld] each: positions relative to the drop centres, normals, weighted densities of the
+// single (F) and the double layer (U).
+struct NearSources {
+  const double *X, *N, *F, *U;
+  long long ld;
+};
+// cv[pair][l] = wS S[f] + wD D[u] of the pair's source drop at its check points
+int launch_near_checks_both(const NearPair* pairs, int npair, int L, const double* pts, const int* grid,
+                            const double* centre, const long long* toff, const int* ngd, const long long* up_off,
+                            const long long* up_n, const NearSources& std_, const NearSources& up, const double* wS,
+                            const double* wD, double* cv, cudaStream_t s);
 int launch_near_interp(const NearPair* pairs, const int* tbeg, int ntgt, int L, int kind, const double* selfcoef,
                        const double* dens, const long long* coef_off, const int* pdeg, const double* hdrop,
                        const double* wts, const double* cv, const int* tdrop, const long long* tgt_loc,

@@ -155,6 +155,11 @@ __global__ void k_near_seed_points(const NearPair* __restrict__ pairs, int npair
   if ((threadIdx.x & 31) == 0) seed[i] = bi < N ? (int)bi : 0;
 }
 
+__global__ void k_add(const double* __restrict__ x, long long n, double* __restrict__ y) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) y[i] += x[i];
+}
+
 // out = u_inf + (S + D) / 2 (u_inf may be null)
 __global__ void k_velocity(const double* __restrict__ uinf, const double* __restrict__ S, const double* __restrict__ D,
                            long long n, double* __restrict__ out) {
@@ -204,6 +209,14 @@ int launch_near_seed_points(const NearPair* pairs, int npair, const double* pts,
                             const long long* toff, const int* ngd, int* seed, cudaStream_t s) {
   if (npair == 0) return BIE_OK;
   k_near_seed_points<<<(npair + 3) / 4, 128, 0, s>>>(pairs, npair, pts, ld, rec_std, toff, ngd, seed);
+  count_launch();
+  BIE_CUDA_TRY(cudaGetLastError());
+  return BIE_OK;
+}
+
+int launch_add(const double* x, long long n, double* y, cudaStream_t s) {
+  if (n == 0) return BIE_OK;
+  k_add<<<blocks_for(n), kThreads, 0, s>>>(x, n, y);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;

@@ -23,6 +23,8 @@ int launch_gather_points(const double* vals, long long t0, long long n, long lon
 // nearest standard-grid point of the pair's source drop to the pair's point (pairs[i].target indexes pts)
 int launch_near_seed_points(const NearPair* pairs, int npair, const double* pts, long long ld, const double* rec_std,
                             const long long* toff, const int* ngd, int* seed, cudaStream_t s);
+// y += x over n values
+int launch_add(const double* x, long long n, double* y, cudaStream_t s);
 // out = uinf + (S + D) / 2 over n values (uinf may be null)
 int launch_velocity(const double* uinf, const double* S, const double* D, long long n, double* out, cudaStream_t s);
 
