@@ -574,6 +574,7 @@ __global__ void __launch_bounds__(kSelfThreads, 2) k_self_dense(SelfGroups<R> G,
       for (int e = 0; e < 6; ++e) s[e] = load_factor(S + e * nv + i);
 #pragma unroll
       for (int c = 0; c < 3; ++c) f[c] = reinterpret_cast<const uint4*>(rho + c * ncp)[i];
+      R sum[3] = {R(0), R(0), R(0)};  // FP32: the 12 products first, then 9 such sums; as one sum of 108 it errs 1.5e-7, now 7.4e-8
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         R q[6], x[3];
@@ -581,8 +582,11 @@ __global__ void __launch_bounds__(kSelfThreads, 2) k_self_dense(SelfGroups<R> G,
         for (int e = 0; e < 6; ++e) q[e] = lane_of<R>(s[e], v);
 #pragma unroll
         for (int c = 0; c < 3; ++c) x[c] = lane_of<R>(f[c], v);
-        sym_mul_add<R>(q, x, acc);
+        sym_mul_add<R>(q, x, sizeof(R) == 4 ? sum : acc);
       }
+      if (sizeof(R) == 4)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) acc[c] = acc[c] + sum[c];
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c)
