@@ -1431,7 +1431,7 @@ static int interdrop_apply(bie_geom* g, int kind, bool raw, const double* dens, 
   }
   Phase ph(ctx, "interdrop_reduce", s);
   return launch_reduce_tiles(g->partial.ptr, g->tile_blk.ptr, g->tile_t0.ptr, g->tile_n.ptr, g->tile_drop.ptr,
-                             g->tgt_loc.ptr, g->val_off_all.ptr, g->ngd.ptr, g->ntile, g->vals.ptr, s);
+                             g->tgt_loc.ptr, g->val_off_all.ptr, g->ngd.ptr, g->ntile, g->nblk, g->vals.ptr, s);
 }
 
 // ---- layer potentials at points off the surfaces (Sec. 1, with the region rules of Sec. 2.1-2.3) ----
@@ -1629,7 +1629,7 @@ static int eval_layers(bie_ctx* ctx, bie_geom* g, long long npt, const double* p
       Phase ph(ctx, "offsurface_reduce", s);
       BIE_CUDA_TRY(cudaMemsetAsync(d_vals.ptr, 0, (size_t)ntile * 3 * kTile * sizeof(double), s));
       BIE_TRY(launch_reduce_tiles(d_part.ptr, d_tile_blk.ptr, d_t0.ptr, d_n.ptr, d_drop.ptr, d_loc.ptr, d_voff.ptr,
-                                  d_ngd.ptr, ntile, d_vals.ptr, s));
+                                  d_ngd.ptr, ntile, nblk, d_vals.ptr, s));
       BIE_TRY(launch_gather_points(d_vals.ptr, t0, n, npt, out[k], s));
     }
     BIE_CUDA_TRY(cudaStreamSynchronize(s));  // the chunk's host tables are reused

@@ -659,21 +659,33 @@ __global__ void k_tile_masks(const unsigned char* __restrict__ region, int nd, c
   out[idx] = m;
 }
 
-// vals += sum of the partials of the tile's blocks, in block order; one thread per (tile, component, target)
-__global__ void k_reduce_tiles(const double* __restrict__ partial, const int* __restrict__ tile_blk,
-                               const long long* __restrict__ tile_t0, const int* __restrict__ tile_n,
-                               const int* __restrict__ tile_drop, const long long* __restrict__ tgt_loc,
-                               const long long* __restrict__ val_off, const int* __restrict__ ngd, int ntile,
-                               double* __restrict__ vals) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= 3LL * ntile * kTile) return;
+// vals += sum of the partials of the tile's blocks; PARTS threads per (tile, component, target), each on every
+// PARTS-th block.  With one thread a small batch, whose tiles are split over a hundred blocks each, waits for
+// fifteen dependent groups of loads: 8 drops of degree 16 11.4 -> 8.1 us.
+constexpr int kRedThreads = 256, kRedParts = 8;
+
+template <int PARTS>
+__global__ void __launch_bounds__(kRedThreads) k_reduce_tiles(
+    const double* __restrict__ partial, const int* __restrict__ tile_blk, const long long* __restrict__ tile_t0,
+    const int* __restrict__ tile_n, const int* __restrict__ tile_drop, const long long* __restrict__ tgt_loc,
+    const long long* __restrict__ val_off, const int* __restrict__ ngd, int ntile, double* __restrict__ vals) {
+  constexpr int OUT = kRedThreads / PARTS;  // a divisor of kTile: the block's outputs lie in one tile
+  __shared__ double part[PARTS][OUT];
+  const int o = threadIdx.x % OUT, k = threadIdx.x / OUT;
+  const long long idx = (long long)blockIdx.x * OUT + o;
   const int tile = (int)(idx / (3 * kTile)), r = (int)(idx - 3LL * tile * kTile), c = r / kTile, tid = r - c * kTile;
-  if (tid >= tile_n[tile]) return;
-  const int b0 = tile_blk[tile], b1 = tile_blk[tile + 1];
-  if (b0 == b1) return;
+  const bool in = tile < ntile && tid < tile_n[tile];
+  const int b0 = in ? tile_blk[tile] : 0, b1 = in ? tile_blk[tile + 1] : 0;
   double a = 0;
 #pragma unroll 8
-  for (int b = b0; b < b1; ++b) a += partial[3LL * kTile * b + r];
+  for (int b = b0 + k; b < b1; b += PARTS) a += partial[3LL * kTile * b + r];
+  if (PARTS > 1) {
+    part[k][o] = a;
+    __syncthreads();
+    if (k > 0) return;
+    for (int i = 1; i < PARTS; ++i) a += part[i][o];
+  }
+  if (b0 == b1) return;
   const int d = tile_drop[tile];
   vals[val_off[d] + (long long)c * ngd[d] + tgt_loc[tile_t0[tile] + tid]] += a;
 }
@@ -838,11 +850,16 @@ int launch_tile_masks(const unsigned char* region, int nd, const long long* tile
 
 int launch_reduce_tiles(const double* partial, const int* tile_blk, const long long* tile_t0, const int* tile_n,
                         const int* tile_drop, const long long* tgt_loc, const long long* val_off, const int* ngd,
-                        int ntile, double* vals, cudaStream_t s) {
-  long long n = 3LL * ntile * kTile;
-  if (n == 0) return BIE_OK;
-  k_reduce_tiles<<<blocks_for(n), kThreads, 0, s>>>(partial, tile_blk, tile_t0, tile_n, tile_drop, tgt_loc, val_off,
-                                                     ngd, ntile, vals);
+                        int ntile, long long nblk, double* vals, cudaStream_t s) {
+  if (ntile == 0) return BIE_OK;
+  // a long list of blocks per tile is split; short lists (2.6 blocks per tile at 192 drops of degree 24) leave
+  // nothing to split and eight times the threads
+  const bool split = nblk >= 2LL * kRedParts * ntile;
+  const long long out = kRedThreads / (split ? kRedParts : 1), n = (3LL * ntile * kTile + out - 1) / out;
+  if (n > 0x7fffffffLL) return BIE_EINVAL;
+  auto kern = split ? k_reduce_tiles<kRedParts> : k_reduce_tiles<1>;
+  kern<<<(unsigned)n, kRedThreads, 0, s>>>(partial, tile_blk, tile_t0, tile_n, tile_drop, tgt_loc, val_off, ngd, ntile,
+                                           vals);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;

@@ -45,7 +45,7 @@ int launch_interdrop_df(int kind, int nblk, const PairItem* items, const int* bl
                         const double* Qu, long long nup, const double* wts, double* partial, cudaStream_t s);
 int launch_reduce_tiles(const double* partial, const int* tile_blk, const long long* tile_t0, const int* tile_n,
                         const int* tile_drop, const long long* tgt_loc, const long long* val_off, const int* ngd,
-                        int ntile, double* vals, cudaStream_t s);
+                        int ntile, long long nblk, double* vals, cudaStream_t s);
 // per drop i of a group (records of N points at rec + 7 off[i], its number ids[i]): out[i][64][2], the partial sums
 // of x.n wJ and the partial maxima of |x - centre|
 int launch_drop_stats(const double* rec, const long long* off, const int* ids, const double* centre, long long nd,
