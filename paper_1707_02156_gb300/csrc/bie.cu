@@ -648,8 +648,8 @@ static int synth_xderivs(bie_ctx* ctx, const double* coef, const long long* fiel
   Plan* pl;
   BIE_TRY(get_plan(ctx, p, P, &pl));
   const long long N = ngrid(P);
-  return launch_synth<double, double>(7, coef, field_off, coef_stride, nfield, p, P, pl->T0.ptr, pl->T1.ptr,
-                                      (const double*)nullptr, pl->cs.ptr, X, nfield * N, N, ctx->sms, s);
+  return launch_synth(7, coef, field_off, coef_stride, nfield, p, P, pl->T0.ptr, pl->T1.ptr,
+                      (const double*)nullptr, pl->cs.ptr, X, nfield * N, N, ctx->sms, s);
 }
 
 // Surface records of a degree group on its grids of degree P, drop i's at rec + 7 off[i] (off on the device),
@@ -1134,20 +1134,21 @@ template <typename R>
 static int source_densities(bie_geom* g, const double* dens, R* Qs, R* Qu, cudaStream_t s) {
   bie_ctx* ctx = g->ctx;
   Phase ph(ctx, "source_synth", s);
+  std::vector<SynGroup<R>> sg;
   for (auto& Gp : g->groups) {
     auto& G = *Gp;
     const int p = G.p;
     const int Pu = ctx->cfg.upsample * (p + 1) - 1;
-    const long long nd = (long long)G.drops.size();
+    const long long nf = 3 * (long long)G.drops.size();
     Plan *ps, *pu;
     BIE_TRY(get_plan(ctx, p, p, &ps));
     BIE_TRY(get_plan(ctx, p, Pu, &pu));
-    BIE_TRY(launch_synth_sources<R>(dens, G.foff3.ptr, nd, p, p, ps->T0_<R>(), ps->cs_<R>(),
-                                    {g->rec_std.ptr, G.src_off_std.ptr, g->ntarget}, Qs, ctx->sms, s));
-    BIE_TRY(launch_synth_sources<R>(dens, G.foff3.ptr, nd, p, Pu, pu->T0_<R>(), pu->cs_<R>(),
-                                    {g->rec_up.ptr, G.src_off_up.ptr, g->nup_total}, Qu, ctx->sms, s));
+    sg.push_back({nf, G.foff3.ptr, 0, p, p, ps->T0_<R>(), nullptr, nullptr, ps->cs_<R>(), Qs, 0, 0,
+                  {g->rec_std.ptr, G.src_off_std.ptr, g->ntarget}, 0, 0});
+    sg.push_back({nf, G.foff3.ptr, 0, p, Pu, pu->T0_<R>(), nullptr, nullptr, pu->cs_<R>(), Qu, 0, 0,
+                  {g->rec_up.ptr, G.src_off_up.ptr, g->nup_total}, 0, 0});
   }
-  return BIE_OK;
+  return launch_synth_sources<R>(dens, std::move(sg), ctx->sms, s);
 }
 
 // Closest points x* of near pairs (Sec. 2.3): damped Newton in a rotated frame that puts the seed
@@ -2399,6 +2400,7 @@ namespace bie {
 // (x, u: [drop][3] blocks, one offset per component) and of their scalar sets (Gamma: [drop]).
 struct SurfGroup {
   int p = 0, P = 0;
+  long long at = 0;  // first grid point
   Plan* pl = nullptr;
   std::vector<int> drops;
   DevBuf<long long> voff, soff;
@@ -2410,11 +2412,7 @@ struct SurfLayout {
   std::vector<long long> voff, soff;  // per drop: start of its vector / scalar coefficients
   long long nv = 0, ns = 0;           // total lengths
   std::vector<std::unique_ptr<SurfGroup>> groups;
-  long long group_points() const {    // grid points of the largest group
-    long long v = 0;
-    for (const auto& G : groups) v = std::max<long long>(v, (long long)G->drops.size() * ngrid(G->P));
-    return v;
-  }
+  long long points = 0;               // grid points of all groups, one group after another
 };
 
 // P = 2p + 1 (the nonlinear terms of Sec. 1.3) when upsampled, else P = p.
@@ -2438,6 +2436,8 @@ static int surf_layout(bie_ctx* ctx, int ndrop, const int* p, bool upsampled, Su
     G->P = upsampled ? 2 * kv.first + 1 : kv.first;
     BIE_TRY(get_plan(ctx, G->p, G->P, &G->pl));
     G->drops = kv.second;
+    G->at = L.points;
+    L.points += (long long)G->drops.size() * ngrid(G->P);
     std::vector<long long> vo, so;
     for (int d : G->drops) {
       for (int c = 0; c < 3; ++c) vo.push_back(L.voff[d] + c * ncoef(G->p));
@@ -2450,41 +2450,52 @@ static int surf_layout(bie_ctx* ctx, int ndrop, const int* p, bool upsampled, Su
   return BIE_OK;
 }
 
-// Derivative fields of nfield coefficient sets (device offsets off) of the group's degree on its
-// grid: kind k (0 f, 1 t, 2 p, 3 tt, 4 tp, 5 pp) of the mask is written to out + k * nfield * N.
-static int surf_synth(const SurfLayout& L, const SurfGroup& G, const double* coef, const long long* off, long long nfield,
-                      int kinds, double* out, cudaStream_t s) {
-  const Plan* pl = G.pl;
-  const long long N = ngrid(G.P);
-  return launch_synth<double, double>(kinds, coef, off, 0, nfield, G.p, G.P, pl->T0.ptr, pl->T1.ptr, pl->T2.ptr,
-                                      pl->cs.ptr, out + ((kinds & 1) ? 0 : nfield * N), nfield * N, N, L.sms, s);
+// Derivative fields of every drop's vector (ncomp 3) or scalar (1) coefficients on the grids of the groups, one
+// launch: kind k (0 f, 1 t, 2 p, 3 tt, 4 tp, 5 pp) of the mask goes to [6][ncomp nd][N] of each group at out +
+// stride * at, or, with stride 0 (scalars), to [6][points].
+static int surf_synth(const SurfLayout& L, const double* coef, int ncomp, int kinds, double* out, long long stride,
+                      cudaStream_t s) {
+  std::vector<SynGroup<double>> sg;
+  for (auto& Gp : L.groups) {
+    const SurfGroup& G = *Gp;
+    const Plan* pl = G.pl;
+    const long long N = ngrid(G.P), nf = ncomp * (long long)G.drops.size(), ks = stride ? nf * N : L.points;
+    sg.push_back({nf, ncomp == 3 ? G.voff.ptr : G.soff.ptr, 0, G.p, G.P, pl->T0.ptr, pl->T1.ptr, pl->T2.ptr, pl->cs.ptr,
+                  out + (stride ? stride * G.at : G.at) + ((kinds & 1) ? 0 : ks), ks, N, {}, 0, 0});
+  }
+  return launch_synth(kinds, coef, std::move(sg), L.sms, s);
 }
 
-// Projection of nfield grids (N apart) of the group to coefficients at off.
-static int surf_project(const SurfLayout& L, const SurfGroup& G, const double* grid, long long nfield,
-                        const long long* off, double* coef, cudaStream_t s) {
-  return launch_analyze({ana_group(G.pl, nfield, nullptr, ngrid(G.P), off, 0)}, grid, coef, L.sms, s);
+// Projection of one scalar grid per drop, [points], to coefficients.
+static int surf_project(const SurfLayout& L, const double* grid, double* coef, cudaStream_t s) {
+  std::vector<AnaGroup> ag;
+  for (auto& Gp : L.groups) {
+    const SurfGroup& G = *Gp;
+    ag.push_back(ana_group(G.pl, (long long)G.drops.size(), nullptr, ngrid(G.P), G.soff.ptr, 0));
+    ag.back().grid_base = G.at;
+  }
+  return launch_analyze(std::move(ag), grid, coef, L.sms, s);
 }
 
 // Galerkin projections of f_E and (when fi is non-null) f_I = inv_pe lap Gamma, Sec. 3.
 static int surf_rates(const SurfLayout& L, const double* x, const double* u, const double* gam, double inv_pe,
                       double* fe, double* fi, cudaStream_t s) {
-  DevBuf<double> tmp;  // for the largest group; the groups follow one another on the stream
-  BIE_TRY(tmp.alloc(35 * L.group_points()));
+  DevBuf<double> tmp;
+  BIE_TRY(tmp.alloc(35 * L.points));
+  double* X = tmp.ptr;
+  double* U = X + 18 * L.points;
+  double* Gm = U + 9 * L.points;
+  double* out = Gm + 6 * L.points;
+  BIE_TRY(surf_synth(L, x, 3, 62, X, 18, s));
+  BIE_TRY(surf_synth(L, u, 3, 7, U, 9, s));
+  BIE_TRY(surf_synth(L, gam, 1, 63, Gm, 6, s));
   for (auto& Gp : L.groups) {
     const SurfGroup& G = *Gp;
-    const long long nd = (long long)G.drops.size(), N = ngrid(G.P);
-    double* X = tmp.ptr;
-    double* U = X + 18 * nd * N;
-    double* Gm = U + 9 * nd * N;
-    double* out = Gm + 6 * nd * N;
-    BIE_TRY(surf_synth(L, G, x, G.voff.ptr, 3 * nd, 62, X, s));
-    BIE_TRY(surf_synth(L, G, u, G.voff.ptr, 3 * nd, 7, U, s));
-    BIE_TRY(surf_synth(L, G, gam, G.soff.ptr, nd, 63, Gm, s));
-    BIE_TRY(launch_surf_rates(X, U, Gm, nd, N, inv_pe, out, fi ? out + nd * N : nullptr, s));
-    BIE_TRY(surf_project(L, G, out, nd, G.soff.ptr, fe, s));
-    if (fi) BIE_TRY(surf_project(L, G, out + nd * N, nd, G.soff.ptr, fi, s));
+    BIE_TRY(launch_surf_rates(X + 18 * G.at, U + 9 * G.at, Gm + 6 * G.at, (long long)G.drops.size(), ngrid(G.P), inv_pe,
+                              out + G.at, fi ? out + L.points + G.at : nullptr, s));
   }
+  BIE_TRY(surf_project(L, out, fe, s));
+  if (fi) BIE_TRY(surf_project(L, out + L.points, fi, s));
   BIE_CUDA_TRY(cudaStreamSynchronize(s));  // the temporaries are released on return
   return BIE_OK;
 }
@@ -2493,18 +2504,18 @@ static int surf_rates(const SurfLayout& L, const double* x, const double* u, con
 static int surf_integrals(const SurfLayout& L, const double* x, const double* gam, int mode, double* out,
                           cudaStream_t s) {
   DevBuf<double> tmp, res_all;
-  BIE_TRY(tmp.alloc(10 * L.group_points()));
+  BIE_TRY(tmp.alloc(10 * L.points));
   BIE_TRY(res_all.alloc(L.ndrop));
   double* res = res_all.ptr;
   std::vector<double> h(L.ndrop);
+  double* X = tmp.ptr;
+  double* Gm = X + 9 * L.points;
+  BIE_TRY(surf_synth(L, x, 3, mode == 0 ? 7 : 6, X, 9, s));
+  if (mode == 1) BIE_TRY(surf_synth(L, gam, 1, 1, Gm, 1, s));
   for (auto& Gp : L.groups) {
     const SurfGroup& G = *Gp;
-    const long long nd = (long long)G.drops.size(), N = ngrid(G.P);
-    double* X = tmp.ptr;
-    double* Gm = X + 9 * nd * N;
-    BIE_TRY(surf_synth(L, G, x, G.voff.ptr, 3 * nd, mode == 0 ? 7 : 6, X, s));
-    if (mode == 1) BIE_TRY(surf_synth(L, G, gam, G.soff.ptr, nd, 1, Gm, s));
-    BIE_TRY(launch_drop_integral(X, Gm, nd, G.P, G.pl->wsin.ptr, mode, res, s));
+    const long long nd = (long long)G.drops.size();
+    BIE_TRY(launch_drop_integral(X + 9 * G.at, Gm + G.at, nd, G.P, G.pl->wsin.ptr, mode, res, s));
     res += nd;
   }
   BIE_CUDA_TRY(cudaMemcpyAsync(h.data(), res_all.ptr, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -2518,20 +2529,24 @@ static int surf_integrals(const SurfLayout& L, const double* x, const double* ga
 // Per-drop max |value| on the grid of each group of ncomp-component coefficient sets (ncomp 3:
 // vector layout, 1: scalar layout), host out[d].
 static int surf_absmax(const SurfLayout& L, const double* coef, int ncomp, double* out, cudaStream_t s) {
+  DevBuf<double> tmp;
+  BIE_TRY(tmp.alloc(ncomp * L.points + L.ndrop));
+  double* F = tmp.ptr;
+  double* res = F + ncomp * L.points;
+  BIE_TRY(surf_synth(L, coef, ncomp, 1, F, ncomp, s));
+  long long at = 0;
   for (auto& Gp : L.groups) {
     const SurfGroup& G = *Gp;
-    const long long nd = (long long)G.drops.size(), N = ngrid(G.P), nf = ncomp * nd;
-    DevBuf<double> tmp;
-    BIE_TRY(tmp.alloc(nf * N + nd));
-    double* F = tmp.ptr;
-    double* res = F + nf * N;
-    BIE_TRY(surf_synth(L, G, coef, ncomp == 3 ? G.voff.ptr : G.soff.ptr, nf, 1, F, s));
-    BIE_TRY(launch_drop_absmax(F, nd, ncomp, N, res, s));
-    std::vector<double> h(nd);
-    BIE_CUDA_TRY(cudaMemcpyAsync(h.data(), res, nd * sizeof(double), cudaMemcpyDeviceToHost, s));
-    BIE_CUDA_TRY(cudaStreamSynchronize(s));
-    for (long long i = 0; i < nd; ++i) out[G.drops[i]] = h[i];
+    const long long nd = (long long)G.drops.size();
+    BIE_TRY(launch_drop_absmax(F + ncomp * G.at, nd, ncomp, ngrid(G.P), res + at, s));
+    at += nd;
   }
+  std::vector<double> h(L.ndrop);
+  BIE_CUDA_TRY(cudaMemcpyAsync(h.data(), res, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+  BIE_CUDA_TRY(cudaStreamSynchronize(s));
+  at = 0;
+  for (auto& Gp : L.groups)
+    for (int d : Gp->drops) out[d] = h[at++];
   return BIE_OK;
 }
 
@@ -2540,25 +2555,21 @@ static int surf_absmax(const SurfLayout& L, const double* coef, int ncomp, doubl
 struct SurfImplicit {
   const SurfLayout* L = nullptr;
   double a = 0;
-  DevBuf<double> lapc;  // per group [5][nd][N], one after another
+  DevBuf<double> lapc;  // [5][points]
   DevBuf<double> inv_diag, c, work;
 };
 
 static int surf_implicit_setup(const SurfLayout& L, const double* x, double a, SurfImplicit& I, cudaStream_t s) {
   I.L = &L;
   I.a = a;
-  long long total = 0, at = 0;
-  for (auto& Gp : L.groups) total += 5 * (long long)Gp->drops.size() * ngrid(Gp->P);
   DevBuf<double> tmp;
-  BIE_TRY(tmp.alloc(18 * L.group_points()));
-  BIE_TRY(I.lapc.alloc(total));
-  BIE_TRY(I.work.alloc(7 * L.group_points()));
+  BIE_TRY(tmp.alloc(18 * L.points));
+  BIE_TRY(I.lapc.alloc(5 * L.points));
+  BIE_TRY(I.work.alloc(7 * L.points));
+  BIE_TRY(surf_synth(L, x, 3, 62, tmp.ptr, 18, s));
   for (auto& Gp : L.groups) {
     const SurfGroup& G = *Gp;
-    const long long nd = (long long)G.drops.size(), N = ngrid(G.P);
-    BIE_TRY(surf_synth(L, G, x, G.voff.ptr, 3 * nd, 62, tmp.ptr, s));
-    BIE_TRY(launch_lap_coef(tmp.ptr, nd, N, I.lapc.ptr + at, s));
-    at += 5 * nd * N;
+    BIE_TRY(launch_lap_coef(tmp.ptr + 18 * G.at, (long long)G.drops.size(), ngrid(G.P), I.lapc.ptr + G.at, L.points, s));
   }
   std::vector<double> vol(L.ndrop);
   BIE_TRY(surf_integrals(L, x, nullptr, 0, vol.data(), s));
@@ -2576,17 +2587,11 @@ static int surf_implicit_setup(const SurfLayout& L, const double* x, double a, S
 
 static int surf_implicit_apply(SurfImplicit& I, const double* y, double* w, cudaStream_t s) {
   const SurfLayout& L = *I.L;
-  long long at = 0;
-  for (auto& Gp : L.groups) {
-    const SurfGroup& G = *Gp;
-    const long long nd = (long long)G.drops.size(), N = ngrid(G.P);
-    double* S = I.work.ptr;  // [6][nd][N], kinds 1..5 used
-    double* grid = S + 6 * nd * N;
-    BIE_TRY(surf_synth(L, G, y, G.soff.ptr, nd, 62, S, s));
-    BIE_TRY(launch_lap_apply(I.lapc.ptr + at, S, nd, N, grid, s));
-    at += 5 * nd * N;
-    BIE_TRY(surf_project(L, G, grid, nd, G.soff.ptr, I.c.ptr, s));
-  }
+  double* S = I.work.ptr;  // [6][points], kinds 1..5 used
+  double* grid = S + 6 * L.points;
+  BIE_TRY(surf_synth(L, y, 1, 62, S, 0, s));
+  BIE_TRY(launch_lap_apply(I.lapc.ptr, S, 1, L.points, grid, s));
+  BIE_TRY(surf_project(L, grid, I.c.ptr, s));
   return launch_implicit_combine(y, I.c.ptr, I.a, I.inv_diag.ptr, L.ns, w, s);
 }
 
@@ -2774,7 +2779,7 @@ int bie_sh_synthesize(bie_ctx* ctx, int ndrop, const int* p, const int* p_out, i
     for (; e < ndrop && p[e] == p[d] && p_out[e] == p_out[d]; ++e) n += ncomp;
     Plan* pl;
     BIE_TRY(get_plan(ctx, p[d], p_out[d], &pl));
-    BIE_TRY((launch_synth<double, double>(1, coef + co, (const long long*)nullptr, ncoef(p[d]), n, p[d], p_out[d],
+    BIE_TRY((launch_synth(1, coef + co, (const long long*)nullptr, ncoef(p[d]), n, p[d], p_out[d],
                                           pl->T0.ptr, nullptr, nullptr, pl->cs.ptr, grid + go, 0, ngrid(p_out[d]),
                                           ctx->sms, s)));
     go += n * ngrid(p_out[d]);
@@ -2931,9 +2936,9 @@ int bie_interfacial_force(bie_ctx* ctx, const bie_geom* g, const double* gammaco
       double* X = tmp.ptr;           // [5][n][3][N]: t, p, tt, tp, pp
       double* Gm = X + 15 * n * N;   // [3][n][N]: f, t, p
       double* f = Gm + 3 * n * N;    // [n][3][N]
-      BIE_TRY((launch_synth<double, double>(62, g->xcoef.ptr, G.foff3.ptr + 3 * i0, 0, 3 * n, p, P, pl->T0.ptr,
+      BIE_TRY((launch_synth(62, g->xcoef.ptr, G.foff3.ptr + 3 * i0, 0, 3 * n, p, P, pl->T0.ptr,
                                             pl->T1.ptr, pl->T2.ptr, pl->cs.ptr, X, 3 * n * N, N, ctx->sms, s)));
-      BIE_TRY((launch_synth<double, double>(7, gammacoef, G.soff.ptr + i0, 0, n, p, P, pl->T0.ptr, pl->T1.ptr,
+      BIE_TRY((launch_synth(7, gammacoef, G.soff.ptr + i0, 0, n, p, P, pl->T0.ptr, pl->T1.ptr,
                                             nullptr, pl->cs.ptr, Gm, n * N, N, ctx->sms, s)));
       BIE_TRY(launch_force(X, Gm, n, N, elasticity, x_s, f, s));
       BIE_TRY(launch_analyze({ana_group(pl, 3 * n, nullptr, N, G.foff3.ptr + 3 * i0, 0)}, f, fcoef, ctx->sms, s));
@@ -3427,7 +3432,7 @@ static int reparam_group(bie_ctx* ctx, int p, const std::vector<int>& drops, con
     BIE_CUDA_TRY(cudaMemcpyAsync(a_d.ptr, av.data(), av.size() * sizeof(double), cudaMemcpyHostToDevice, s));
     // grad E = 2 sum_n a_n x~_n^m Y_n^m on the grid (Eq. energy_rep), its tangential part at the points
     BIE_TRY(launch_scale_degrees(xt.ptr, a_d.ptr, P, nd, 3, 2.0, sc.ptr, s));
-    BIE_TRY((launch_synth<double, double>(1, sc.ptr, (const long long*)nullptr, nC, nd * 3, P, P, plP->T0.ptr, nullptr,
+    BIE_TRY((launch_synth(1, sc.ptr, (const long long*)nullptr, nC, nd * 3, P, P, plP->T0.ptr, nullptr,
                                           nullptr, plP->cs.ptr, gradE.ptr, 0, N, ctx->sms, s)));
     BIE_TRY(launch_rep_gradient(E.ptr, gradE.ptr, N, nd, gv.ptr, gmax.ptr, s));
     BIE_CUDA_TRY(cudaMemcpyAsync(gm.data(), gmax.ptr, nd * sizeof(double), cudaMemcpyDeviceToHost, s));

@@ -35,24 +35,47 @@ __host__ __device__ inline long long leg_row(int p, int m, int n, int nj) {
 }
 
 // ---- transforms (transforms.cu) ----
-// Synthesis of nfield fields of degree p on the grid of degree P, with the derivative kinds of the mask
-// `kinds` (bit 0 f, 1 t, 2 p, 3 tt, 4 tp, 5 pp; the masks 1, 6, 7, 62, 63): kind
-// number s of the mask of field f goes to out + s * kind_stride + f * field_stride.  Coefficients of
-// field f start at field_off ? field_off[f] : f * coef_stride.  T1, T2 may be null when no kind needs them.
-template <typename CT, typename R>
-int launch_synth(int kinds, const CT* coef, const long long* field_off, long long coef_stride, long long nfield, int p,
-                 int P, const R* T0, const R* T1, const R* T2, const R* cs, R* out, long long kind_stride,
-                 long long field_stride, int sms, cudaStream_t s);
-// Weighted source densities of nd drops, fields [drop][3]: w_s f_c(s) on the degree-P grid to Q[c * ld + off[drop] + s],
+// Weighted source densities, fields [drop][3]: w_s f_c(s) on the degree-P grid to out[c * ld + off[drop] + s],
 // the weights in row 6 of the records rec ([7][N] at 7 off[drop]).
 struct SynthSources {
   const double* rec;
   const long long* off;
   long long ld;
 };
+// A synthesis of nfield fields of degree p on the grid of degree P: the s-th kind asked for of field f goes to
+// out + s * kind_stride + f * field_stride (or to the sources' place).  Coefficients of field f start at
+// field_off ? field_off[f] : f * coef_stride.  T1, T2 may be null when no kind needs them.
 template <typename R>
-int launch_synth_sources(const double* coef, const long long* field_off, long long nd, int p, int P, const R* T0,
-                         const R* cs, const SynthSources& src, R* Q, int sms, cudaStream_t s);
+struct SynGroup {
+  long long nfield;
+  const long long* field_off;
+  long long coef_stride;
+  int p, P;
+  const R *T0, *T1, *T2, *cs;
+  R* out;
+  long long kind_stride, field_stride;
+  SynthSources src;
+  long long begin;  // first block and latitude pairs per block: set by the launcher
+  int jb;
+};
+constexpr int kMaxSynGroups = 8;
+template <typename R>
+struct SynGroups {
+  int n;
+  SynGroup<R> g[kMaxSynGroups];
+};
+// Several of them in one launch, with the derivative kinds of the mask `kinds` (bit 0 f, 1 t, 2 p, 3 tt, 4 tp,
+// 5 pp; the masks 1, 6, 7, 62, 63).
+int launch_synth(int kinds, const double* coef, std::vector<SynGroup<double>> groups, int sms, cudaStream_t s);
+template <typename R>
+int launch_synth_sources(const double* coef, std::vector<SynGroup<R>> groups, int sms, cudaStream_t s);
+inline int launch_synth(int kinds, const double* coef, const long long* field_off, long long coef_stride,
+                        long long nfield, int p, int P, const double* T0, const double* T1, const double* T2,
+                        const double* cs, double* out, long long kind_stride, long long field_stride, int sms,
+                        cudaStream_t s) {
+  return launch_synth(kinds, coef, {{nfield, field_off, coef_stride, p, P, T0, T1, T2, cs, out, kind_stride, field_stride, {}, 0, 0}},
+                      sms, s);
+}
 // analysis: grids (degree P) -> coefficients (degree p <= P), FP64, for several degree groups in one launch.
 // Offsets per field, or null and a stride; begin is set by the launcher.
 struct AnaGroup {
@@ -168,7 +191,7 @@ int launch_to_float(const double* in, float* out, long long n, cudaStream_t s);
 int launch_surf_rates(const double* X, const double* U, const double* Gm, long long nd, long long N, double inv_pe,
                       double* fe, double* fi, cudaStream_t s);
 // coefficients of the surface Laplacian L[5][nd][N] (s_tt, s_tp, s_pp, s_t, s_p) from X [6][nd*3][N]
-int launch_lap_coef(const double* X, long long nd, long long N, double* L, cudaStream_t s);
+int launch_lap_coef(const double* X, long long nd, long long N, double* L, long long ld, cudaStream_t s);
 // out[nd][N] = lap s from L and the fields S [6][nd][N] of s (kinds t..pp used)
 int launch_lap_apply(const double* L, const double* S, long long nd, long long N, double* out, cudaStream_t s);
 // per-drop integral on the grid of degree P (mode 0: volume from X kinds f, t, p; mode 1: mass of

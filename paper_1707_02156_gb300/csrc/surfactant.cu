@@ -110,10 +110,11 @@ __global__ void k_surf_rates(const double* __restrict__ X, const double* __restr
   }
 }
 
-// Coefficients of lap s = a_tt s_tt + a_tp s_tp + a_pp s_pp + b_t s_t + b_p s_p, L[5][nd][N].
+// Coefficients of lap s = a_tt s_tt + a_tp s_tp + a_pp s_pp + b_t s_t + b_p s_p: L[k * ld + d * N + q].
 // With C_t = g^ij x_ij . x_t and C_p = g^ij x_ij . x_p (sum over i, j): b_t = -(g^tt C_t + g^tp C_p),
 // b_p = -(g^tp C_t + g^pp C_p).
-__global__ void k_lap_coef(const double* __restrict__ X, long long nd, long long N, double* __restrict__ L) {
+__global__ void k_lap_coef(const double* __restrict__ X, long long nd, long long N, double* __restrict__ L,
+                           long long ld) {
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= nd * N) return;
   const long long d = idx / N, q = idx - d * N;
@@ -122,12 +123,11 @@ __global__ void k_lap_coef(const double* __restrict__ X, long long nd, long long
   const Metric m = metric(xt, xp);
   const double Ct = m.gtt * dot(xtt, xt) + 2.0 * m.gtp * dot(xtp, xt) + m.gpp * dot(xpp, xt);
   const double Cp = m.gtt * dot(xtt, xp) + 2.0 * m.gtp * dot(xtp, xp) + m.gpp * dot(xpp, xp);
-  const long long s = nd * N;
   L[idx] = m.gtt;
-  L[s + idx] = 2.0 * m.gtp;
-  L[2 * s + idx] = m.gpp;
-  L[3 * s + idx] = -(m.gtt * Ct + m.gtp * Cp);
-  L[4 * s + idx] = -(m.gtp * Ct + m.gpp * Cp);
+  L[ld + idx] = 2.0 * m.gtp;
+  L[2 * ld + idx] = m.gpp;
+  L[3 * ld + idx] = -(m.gtt * Ct + m.gtp * Cp);
+  L[4 * ld + idx] = -(m.gtp * Ct + m.gpp * Cp);
 }
 
 // out = lap s from the coefficients L[5][nd][N] and the fields S[6][nd][N] of s (f, t, p, tt, tp, pp)
@@ -212,9 +212,9 @@ int launch_surf_rates(const double* X, const double* U, const double* Gm, long l
   return BIE_OK;
 }
 
-int launch_lap_coef(const double* X, long long nd, long long N, double* L, cudaStream_t s) {
+int launch_lap_coef(const double* X, long long nd, long long N, double* L, long long ld, cudaStream_t s) {
   if (nd * N == 0) return BIE_OK;
-  k_lap_coef<<<blocks_for(nd * N), kThreads, 0, s>>>(X, nd, N, L);
+  k_lap_coef<<<blocks_for(nd * N), kThreads, 0, s>>>(X, nd, N, L, ld);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;

@@ -49,24 +49,28 @@ constexpr int kSynStageP = BIE_MAX_P;  // coefficients are staged in shared memo
 // the rotated grids of 64 drops of degree 24 56.8 -> 50.3 ms.  Where the block has a thread for every order
 // anyway, each takes one.  With SRC (values only) field 3 d + c is
 // component c of drop d's density, and the weighted source w_s f(s) goes to the sources' place instead of
-// the value to a grid.
-template <typename CT, typename R, int KINDS, bool SRC>
-__global__ void __launch_bounds__(kSynThreads) k_synth(const CT* __restrict__ coef,
-                                                       const long long* __restrict__ field_off, long long coef_stride,
-                                                       int p, int P, const R* __restrict__ T0,
-                                                       const R* __restrict__ T1, const R* __restrict__ T2,
-                                                       const R* __restrict__ cs, R* __restrict__ out,
-                                                       long long kind_stride, long long field_stride, int jb,
-                                                       SynthSources src) {
+// the value to a grid.  Several syntheses (degree groups; the standard and the upsampled grid) share a launch:
+// a small one is as long as its chain of dependent loads, whatever its size, and they have nothing to wait for
+// from one another: an apply's sources on both grids of two drops of degree 32 26 -> 19 us, the five
+// derivatives of 16 fields each of degree 16, 24 and 32 115 -> 88 us.
+template <typename R, int KINDS, bool SRC>
+__global__ void __launch_bounds__(kSynThreads) k_synth(const double* __restrict__ coef, SynGroups<R> G) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int NK = kind_slot(KINDS, 6);
+  SynGroup<R> A = G.g[0];
+#pragma unroll
+  for (int i = 1; i < kMaxSynGroups; ++i)
+    if (i < G.n && (long long)blockIdx.x >= G.g[i].begin) A = G.g[i];
+  const int p = A.p, P = A.P, jb = A.jb;
+  const R* __restrict__ cs = A.cs;
   const int nj = P + 1, nk = 2 * P + 2, half = P + 1, np = (nj + 1) / 2, k4n = half / 2 + 1;
   const int njb = (np + jb - 1) / jb;
-  const long long f = blockIdx.x / njb;
-  const int q0 = (int)(blockIdx.x % njb) * jb, jbn = min(jb, np - q0);
+  const unsigned bl = blockIdx.x - (unsigned)A.begin;
+  const long long f = bl / njb;
+  const int q0 = (int)(bl % njb) * jb, jbn = min(jb, np - q0);
   R* h = reinterpret_cast<R*>(smem_raw);  // [NK][2 jb][p+1][2]
   const long long hk = 2LL * jb * (p + 1) * 2;
-  const CT* cg = coef + (field_off ? field_off[f] : f * coef_stride);
+  const double* __restrict__ cg = coef + (A.field_off ? A.field_off[f] : f * A.coef_stride);
   const bool staged = p <= kSynStageP;
   R* c = h + NK * hk;
   if (staged) {
@@ -82,7 +86,7 @@ __global__ void __launch_bounds__(kSynThreads) k_synth(const CT* __restrict__ co
     int t = i / (jbn * mh);  // the t-th table in use
     if (!(TABS & 1)) ++t;
     if (t > 0 && !(TABS & 2)) ++t;
-    const R* T = t == 0 ? T0 : t == 1 ? T1 : T2;
+    const R* __restrict__ T = t == 0 ? A.T0 : t == 1 ? A.T1 : A.T2;
     for (int half_m = 0; half_m < 2; ++half_m) {
       const int m = half_m ? p - a : a;
       if (half_m && (!both || m == a)) break;
@@ -150,17 +154,17 @@ __global__ void __launch_bounds__(kSynThreads) k_synth(const CT* __restrict__ co
     R* d0;
     R w[4] = {1, 1, 1, 1};  // the weights at k, half + k, 2 half - k, half - k
     if constexpr (SRC) {
-      const long long o = src.off[f / 3], N = (long long)nj * nk;
-      const double* wj = src.rec + 7 * o + 6 * N + (long long)j * nk;
-      d0 = out + (f % 3) * src.ld + o + (long long)j * nk;
+      const long long o = A.src.off[f / 3], N = (long long)nj * nk;
+      const double* __restrict__ wj = A.src.rec + 7 * o + 6 * N + (long long)j * nk;
+      d0 = A.out + (f % 3) * A.src.ld + o + (long long)j * nk;
       w[0] = (R)wj[k];
       if (mir) w[1] = (R)wj[half + k];
       if (rot) w[2] = (R)wj[2 * half - k];
       if (rot && mir) w[3] = (R)wj[half - k];
     } else {
-      d0 = out + f * field_stride + (long long)j * nk;
+      d0 = A.out + f * A.field_stride + (long long)j * nk;
     }
-    R* d = d0 + s * kind_stride;
+    R* d = d0 + s * A.kind_stride;
     const R cp = ce + co, cm = ce - co, sp = se + so, sm = se - so;
     d[k] = w[0] * (cp - sp);
     if (mir) d[half + k] = w[1] * (cm - sm);
@@ -389,39 +393,45 @@ __global__ void k_phase(double* __restrict__ coef, long long nfield, int p, doub
 
 }  // namespace
 
-template <typename CT, typename R, int KINDS, bool SRC = false>
-static int synth_launch(const CT* coef, const long long* field_off, long long coef_stride, long long nfield, int p, int P,
-                        const R* T0, const R* T1, const R* T2, const R* cs, R* out, long long kind_stride,
-                        long long field_stride, int sms, cudaStream_t s, SynthSources src = {}) {
-  if (nfield == 0) return BIE_OK;
-  const int np = (P + 2) / 2;
-  const size_t stage = p <= kSynStageP ? sizeof(R) * (size_t)(p + 1) * (p + 1) : 0;
-  const size_t pair = sizeof(R) * kind_slot(KINDS, 6) * 4 * (size_t)(p + 1);
+template <typename R, int KINDS, bool SRC = false>
+static int synth_launch(const double* coef, std::vector<SynGroup<R>> groups, int sms, cudaStream_t s) {
+  std::sort(groups.begin(), groups.end(), [](const SynGroup<R>& x, const SynGroup<R>& y) { return x.P > y.P; });
+  long long work = 0;  // latitude pairs of all fields
+  for (const auto& g : groups) work += g.nfield * ((g.P + 2) / 2);
+  if (work == 0) return BIE_OK;
   // latitude pairs per block: all of them when there are fields for four blocks per SM (the coefficients
   // are staged once), fewer when not, so that small batches spread over the SMs; at most 64 KB a block
-  const long long want = std::max(1LL, nfield * np / (4LL * sms));
-  const long long fit = std::max<long long>(1, ((64 << 10) - (long long)stage) / (long long)pair);
-  const int jb = (int)std::min<long long>(np, std::min(want, fit));
-  const size_t smem = stage + pair * jb;
-  const long long nblk = nfield * ((np + jb - 1) / jb);
-  if (nblk > 0x7fffffffLL) return BIE_EINVAL;
-  auto kern = k_synth<CT, R, KINDS, SRC>;
-  if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-  kern<<<(unsigned)nblk, kSynThreads, smem, s>>>(coef, field_off, coef_stride, p, P, T0, T1, T2, cs, out, kind_stride,
-                                                 field_stride, jb, src);
-  count_launch();
-  BIE_CUDA_TRY(cudaGetLastError());
+  const long long want = std::max(1LL, work / (4LL * sms));
+  auto kern = k_synth<R, KINDS, SRC>;
+  for (size_t g0 = 0; g0 < groups.size(); g0 += kMaxSynGroups) {
+    SynGroups<R> G{};
+    G.n = (int)std::min<size_t>(kMaxSynGroups, groups.size() - g0);
+    size_t smem = 0;
+    long long nblk = 0;
+    for (int i = 0; i < G.n; ++i) {
+      SynGroup<R>& g = G.g[i] = groups[g0 + i];
+      const int np = (g.P + 2) / 2;
+      const size_t stage = g.p <= kSynStageP ? sizeof(R) * (size_t)(g.p + 1) * (g.p + 1) : 0;
+      const size_t pair = sizeof(R) * kind_slot(KINDS, 6) * 4 * (size_t)(g.p + 1);
+      const long long fit = std::max<long long>(1, ((64 << 10) - (long long)stage) / (long long)pair);
+      g.jb = (int)std::min<long long>(np, std::min(want, fit));
+      g.begin = nblk;
+      nblk += g.nfield * ((np + g.jb - 1) / g.jb);
+      smem = std::max(smem, stage + pair * g.jb);
+    }
+    if (nblk == 0) continue;
+    if (nblk > 0x7fffffffLL) return BIE_EINVAL;
+    if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    kern<<<(unsigned)nblk, kSynThreads, smem, s>>>(coef, G);
+    count_launch();
+    BIE_CUDA_TRY(cudaGetLastError());
+  }
   return BIE_OK;
 }
 
-template <typename CT, typename R>
-int launch_synth(int kinds, const CT* coef, const long long* field_off, long long coef_stride, long long nfield, int p,
-                 int P, const R* T0, const R* T1, const R* T2, const R* cs, R* out, long long kind_stride,
-                 long long field_stride, int sms, cudaStream_t s) {
-#define BIE_SYNTH(K)                                                                                             \
-  if (kinds == K)                                                                                                \
-  return synth_launch<CT, R, K>(coef, field_off, coef_stride, nfield, p, P, T0, T1, T2, cs, out, kind_stride, \
-                                field_stride, sms, s)
+int launch_synth(int kinds, const double* coef, std::vector<SynGroup<double>> groups, int sms, cudaStream_t s) {
+#define BIE_SYNTH(K) \
+  if (kinds == K) return synth_launch<double, K>(coef, std::move(groups), sms, s)
   BIE_SYNTH(1);
   BIE_SYNTH(6);
   BIE_SYNTH(7);
@@ -432,9 +442,8 @@ int launch_synth(int kinds, const CT* coef, const long long* field_off, long lon
 }
 
 template <typename R>
-int launch_synth_sources(const double* coef, const long long* field_off, long long nd, int p, int P, const R* T0,
-                         const R* cs, const SynthSources& src, R* Q, int sms, cudaStream_t s) {
-  return synth_launch<double, R, 1, true>(coef, field_off, 0, 3 * nd, p, P, T0, nullptr, nullptr, cs, Q, 0, 0, sms, s, src);
+int launch_synth_sources(const double* coef, std::vector<SynGroup<R>> groups, int sms, cudaStream_t s) {
+  return synth_launch<R, 1, true>(coef, std::move(groups), sms, s);
 }
 
 int launch_analyze(std::vector<AnaGroup> groups, const double* grid, double* coef, int sms, cudaStream_t s) {
@@ -520,13 +529,8 @@ int launch_phase(double* coef, long long nfield, int p, double gamma, cudaStream
 }
 
 // explicit instantiations
-template int launch_synth<double, double>(int, const double*, const long long*, long long, long long, int, int,
-                                          const double*, const double*, const double*, const double*, double*,
-                                          long long, long long, int, cudaStream_t);
-template int launch_synth_sources<double>(const double*, const long long*, long long, int, int, const double*,
-                                          const double*, const SynthSources&, double*, int, cudaStream_t);
-template int launch_synth_sources<float>(const double*, const long long*, long long, int, int, const float*, const float*,
-                                         const SynthSources&, float*, int, cudaStream_t);
+template int launch_synth_sources<double>(const double*, std::vector<SynGroup<double>>, int, cudaStream_t);
+template int launch_synth_sources<float>(const double*, std::vector<SynGroup<float>>, int, cudaStream_t);
 template int launch_rotate<double, double>(const double*, const long long*, int, long long, int, const double*,
                                            long long, int, int, const double*, double*, long long, cudaStream_t);
 template int launch_rotate<double, float>(const double*, const long long*, int, long long, int, const float*,

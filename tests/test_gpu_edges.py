@@ -13,6 +13,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 from oracle import layer, sh
+from oracle import surfactant as sf
 from paper_1707_02156_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
@@ -122,5 +123,32 @@ def test_near_rows_at_every_grid_parity(api, p, up):
                 out.fill_(float("nan"))
                 fn(f, out, precision=prec)
                 assert relerr(host(out), r) < tol, (prec,)
+    geo.close()
+    ctx.close()
+
+
+def test_more_degree_groups_than_a_launch_takes(api):
+    # transforms of several degrees share a launch, eight syntheses (two grids per degree for sources) at a time
+    ps = [11, 2, 9, 4, 7, 6, 5, 8, 3, 10, 4]
+    rng = np.random.default_rng(21)
+    xs = [inputs.sphere_coef(p, centre=(4.0 * (i % 4), 4.0 * (i // 4), 0.3 * i)) + inputs.perturbation(rng, p, 2, min(p, 4), 0.05)
+          for i, p in enumerate(ps)]
+    fs = [inputs.random_bandlimited(rng, p, 3) for p in ps]
+    gs = [inputs.random_bandlimited(rng, p, 1)[0] * 0.1 for p in ps]
+    lam = np.linspace(0.3, 4.0, len(ps))
+    ctx = api.Context(0)
+    x, f, g = dev(inputs.pack_drops(xs)), dev(inputs.pack_drops(fs)), dev(np.concatenate(gs))
+    geo = ctx.geometry(ps, ps, x, lam)
+    drops = layer.Drops([v.reshape(3, -1) for v in xs], ps, ps, lam)
+    out = torch.full_like(f, float("nan"))
+    for fn, ref in ((geo.apply_single, drops.apply_single), (geo.apply_double, drops.apply_double)):
+        fn(f, out, precision=0)
+        assert relerr(host(out), np.concatenate([v.ravel() for v in ref(fs)])) < FP64_TOL
+    fe, fi, y = torch.full_like(g, float("nan")), torch.full_like(g, float("nan")), torch.full_like(g, float("nan"))
+    api.surfactant_rates(ctx, ps, x, f, g, 0.25, fe, fi)
+    assert relerr(host(fe), np.concatenate([sf.f_explicit(a, u, c, p) for a, u, c, p in zip(xs, fs, gs, ps)])) < 1e-12
+    assert relerr(host(fi), np.concatenate([sf.f_implicit(a, c, p, 4.0) for a, c, p in zip(xs, gs, ps)])) < 1e-12
+    api.surfactant_implicit(ctx, ps, x, g, 0.03, y)
+    assert relerr(host(y), np.concatenate([sf.solve_implicit(a, c, p, 0.03)[0] for a, c, p in zip(xs, gs, ps)])) < 1e-11
     geo.close()
     ctx.close()
