@@ -86,7 +86,9 @@ typedef struct bie_config {
  * on. */
 void bie_config_default(bie_config* cfg);
 
-/* Create a context on cfg->device.  Plan tables are built lazily per degree and cached. */
+/* Create a context on cfg->device.  Plan tables are built lazily per degree and cached.  The library's device
+ * memory comes from a memory pool of the device, which keeps up to a sixteenth of the device's memory for
+ * the next geometry or call and gives it back when the device's last context is destroyed. */
 int bie_create(bie_ctx** ctx, const bie_config* cfg);
 void bie_destroy(bie_ctx* ctx);
 const char* bie_strerror(int status);

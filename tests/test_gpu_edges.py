@@ -6,6 +6,10 @@ orders with the number of fields; the dense self factors pad (p+1)^2 to whole 16
 the near-singular rule fold the standard and the upsampled grid.  Every parity and remainder is
 compared with the FP64 oracle at the bars of the other parity tests."""
 import math
+import os
+import subprocess
+import sys
+import threading
 
 import numpy as np
 import pytest
@@ -152,3 +156,57 @@ def test_more_degree_groups_than_a_launch_takes(api):
     assert relerr(host(y), np.concatenate([sf.solve_implicit(a, c, p, 0.03)[0] for a, c, p in zip(xs, gs, ps)])) < 1e-11
     geo.close()
     ctx.close()
+
+
+def test_buffers_of_several_threads_and_their_return(api):
+    # contexts on threads of their own draw on one memory pool of the device; with the last one gone it is empty
+    w = inputs.two_drops(p=8, gap=0.5, up=2, lam=0.5)
+    got = [[] for _ in range(3)]
+
+    def work(mine):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            ctx = api.Context(0, upsample=2)
+            for _ in range(4):
+                geo = ctx.geometry(w.p, w.pq, dev(w.xcoef), w.lam)
+                f = dev(w.density)
+                out = torch.full_like(f, float("nan"))
+                geo.apply_double(f, out, precision=0)
+                stream.synchronize()
+                mine.append(out.cpu().numpy())
+                geo.close()
+            ctx.close()
+
+    threads = [threading.Thread(target=work, args=(g,)) for g in got]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    nc = 3 * 81
+    xs = [w.xcoef[:nc].reshape(3, -1), w.xcoef[nc:].reshape(3, -1)]
+    fs = [w.density[:nc].reshape(3, -1), w.density[nc:].reshape(3, -1)]
+    ref = np.concatenate([v.ravel() for v in layer.Drops(xs, w.p, w.pq, w.lam, up=2).apply_double(fs)])
+    for g in got:
+        assert len(g) == 4
+        for v in g:
+            assert relerr(v, ref) < FP64_TOL
+    # in a process of its own: contexts of other tests may still hold the pool here
+    code = """
+import torch
+from paper_1707_02156_gb300 import api, inputs
+free = lambda: (torch.cuda.synchronize(), torch.cuda.mem_get_info()[0])[1]
+def run(n, p):
+    w = inputs.deformed_drops(n, p, box=8.0)
+    x = torch.as_tensor(w.xcoef).cuda()
+    ctx = api.Context(0)
+    geo = ctx.geometry(w.p, w.pq, x, w.lam)
+    f = free()
+    geo.close()
+    ctx.close()
+    return f
+run(2, 4)
+before = free()
+used = before - run(8, 20)
+assert used > 200e6 and before - free() < used / 4, (used, before - free())
+"""
+    subprocess.run([sys.executable, "-c", code], check=True, timeout=120, cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
