@@ -1,5 +1,6 @@
 // C ABI entry points: context and plan caches, transforms, geometry set-up, the layer-operator
 // applies (Eq. main_eq) and the GMRES solve (Sec. 6).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1921,24 +1922,10 @@ __device__ inline void kry_slice(long long n, long long* x0, long long* x1) {
   *x1 = min(n, *x0 + chunk);
 }
 
-constexpr int kKrySlice = 64;  // entries of a block whose slice is kept in shared memory
-
-// partial[i][block] = V_i . w over the block's slice for i < nv (V_nv = w itself when with_norm).  A short
-// slice: one warp per vector, with w from shared memory; a long one: every thread of the block on four
-// vectors at a time.
-__device__ void kry_block_dots(const double* V, long long ldv, const double* w, const double* ws, int nv, bool with_norm,
-                               long long x0, long long x1, double* __restrict__ partial) {
+// partial[i][block] = V_i . w over the block's slice for i < nv (V_nv = w itself when with_norm)
+__device__ void kry_block_dots(const double* V, long long ldv, const double* w, int nv, bool with_norm, long long x0,
+                               long long x1, double* __restrict__ partial) {
   const int nt = nv + (with_norm ? 1 : 0);
-  if (x1 - x0 <= kKrySlice) {
-    const int len = (int)(x1 - x0), lane = threadIdx.x & 31;
-    for (int i = threadIdx.x >> 5; i < nt; i += blockDim.x >> 5) {
-      double a = 0;
-      for (int x = lane; x < len; x += 32) a += (i < nv ? V[(long long)i * ldv + x0 + x] : ws[x]) * ws[x];
-      for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-      if (lane == 0) partial[(long long)i * gridDim.x + blockIdx.x] = a;
-    }
-    return;
-  }
   __shared__ double sh[kKryThreads / 32][kKryGroup];
   for (int i0 = 0; i0 < nt; i0 += kKryGroup) {
     double a[kKryGroup];
@@ -1969,32 +1956,12 @@ __device__ void kry_block_dots(const double* V, long long ldv, const double* w, 
   }
 }
 
-// w -= V h (i <= k) on the block's slice, kept in ws when it is short.  A short slice shares the vectors of an
-// entry among four threads, whose sums are added in order.
-__device__ void kry_subtract(double* w, const double* V, long long n, int k, const double* h, long long x0, long long x1,
-                             double* ws) {
-  __shared__ double hs[BIE_MAX_RESTART + 1], ps[4][kKrySlice];
-  if (x1 - x0 <= kKrySlice) {
-    for (int i = threadIdx.x; i <= k; i += blockDim.x) hs[i] = h[i];
-    const int x = threadIdx.x % kKrySlice, part = threadIdx.x / kKrySlice, len = (int)(x1 - x0);
-    const double wx = x < len ? w[x0 + x] : 0.0;
-    __syncthreads();
-    double t = 0;
-    if (x < len)
-#pragma unroll 4
-      for (int i = part; i <= k; i += 4) t += hs[i] * V[(long long)i * n + x0 + x];
-    ps[part][x] = t;
-    __syncthreads();
-    if (part == 0 && x < len) {
-      ws[x] = wx - (((ps[0][x] + ps[1][x]) + ps[2][x]) + ps[3][x]);
-      w[x0 + x] = ws[x];
-    }
-  } else {
-    for (long long x = x0 + threadIdx.x; x < x1; x += blockDim.x) {
-      double t = w[x];
-      for (int i = 0; i <= k; ++i) t -= h[i] * V[(long long)i * n + x];
-      w[x] = t;
-    }
+// w -= V h (i <= k) on the block's slice
+__device__ void kry_subtract(double* w, const double* V, long long n, int k, const double* h, long long x0, long long x1) {
+  for (long long x = x0 + threadIdx.x; x < x1; x += blockDim.x) {
+    double t = w[x];
+    for (int i = 0; i <= k; ++i) t -= h[i] * V[(long long)i * n + x];
+    w[x] = t;
   }
   __syncthreads();
 }
@@ -2035,51 +2002,35 @@ __global__ void __launch_bounds__(kKryThreads) k_kry_sysop_dots(const double* __
                                                                 double* __restrict__ h) {
   long long x0, x1;
   kry_slice(n, &x0, &x1);
-  __shared__ double ws[kKrySlice];
   const double sc = scale ? scale[0] : 1.0;
   for (long long x = x0 + threadIdx.x; x < x1; x += blockDim.x) {
     const double v = sc * u[x];
     if (scale) u[x] = v;
-    const double t = lam ? (lam[x] + 1.0) * v - sc * d[x] : sc * d[x];
-    w[x] = t;
-    if (x - x0 < kKrySlice) ws[x - x0] = t;
+    w[x] = lam ? (lam[x] + 1.0) * v - sc * d[x] : sc * d[x];
   }
   __syncthreads();
-  kry_block_dots(V, n, w, ws, k + 1, false, x0, x1, partial);
+  kry_block_dots(V, n, w, k + 1, false, x0, x1, partial);
   if (kry_last_block(counter)) kry_finish(partial, k + 1, h);
 }
 
-// w -= V h_prev (i <= k), then h = V_i . w for i <= k and h[k+1] = w . w
+// w -= V h_prev (i <= k), then h = V_i . w for i <= k
 __global__ void __launch_bounds__(kKryThreads) k_kry_sub_dots(double* __restrict__ w, const double* __restrict__ V,
                                                               long long n, int k, const double* __restrict__ hprev,
                                                               double* __restrict__ partial, unsigned* counter,
                                                               double* __restrict__ h) {
   long long x0, x1;
   kry_slice(n, &x0, &x1);
-  __shared__ double ws[kKrySlice];
-  kry_subtract(w, V, n, k, hprev, x0, x1, ws);
-  kry_block_dots(V, n, w, ws, k + 1, true, x0, x1, partial);
-  if (kry_last_block(counter)) kry_finish(partial, k + 2, h);
+  kry_subtract(w, V, n, k, hprev, x0, x1);
+  kry_block_dots(V, n, w, k + 1, false, x0, x1, partial);
+  if (kry_last_block(counter)) kry_finish(partial, k + 1, h);
 }
 
-// w -= V h2 (i <= k); |w| by a direct sum; then, in the last block, the end of Arnoldi step k: the
-// Hessenberg column h1 + h2 with subdiagonal |w|, the previous Givens rotations, the new one, the
-// least-squares right-hand side gv, the residual estimate res[k] = |gv[k+1]| and scale = 1/|w|
-// (applied to w at the start of the next step).
-__global__ void __launch_bounds__(kKryThreads) k_kry_sub_tail(double* __restrict__ w, const double* __restrict__ V,
-                                                              long long n, int k, int m,
-                                                              const double* __restrict__ h1,
-                                                              const double* __restrict__ h2,
-                                                              double* __restrict__ partial, unsigned* counter,
-                                                              double* __restrict__ H, double* __restrict__ cs,
-                                                              double* __restrict__ sn, double* __restrict__ gv,
-                                                              double* __restrict__ scale, double* __restrict__ res) {
-  long long x0, x1;
-  kry_slice(n, &x0, &x1);
-  __shared__ double ws[kKrySlice];
-  kry_subtract(w, V, n, k, h2, x0, x1, ws);
-  kry_block_dots(V, n, w, ws, 0, true, x0, x1, partial);
-  if (!kry_last_block(counter)) return;
+// The end of Arnoldi step k, by one block, from |w|^2 = sum of partial[b]: the Hessenberg column h1 + h2 with
+// subdiagonal |w|, the previous Givens rotations, the new one, the least-squares right-hand side gv, the
+// residual estimate res[k] = |gv[k+1]| and scale = 1/|w| (applied to w at the start of the next step).
+__device__ void kry_tail(const double* partial, const double* h1, const double* h2, int k, int m, double* __restrict__ H,
+                         double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ gv,
+                         double* __restrict__ scale, double* __restrict__ res) {
   // the column, the rotations and |w|^2 come in with one round of loads; the recurrence runs in shared memory
   __shared__ double col[BIE_MAX_RESTART + 2], rc[BIE_MAX_RESTART], rs[BIE_MAX_RESTART], wn2;
   kry_finish(partial, 1, &wn2);
@@ -2113,12 +2064,85 @@ __global__ void __launch_bounds__(kKryThreads) k_kry_sub_tail(double* __restrict
   for (int i = threadIdx.x; i <= k; i += blockDim.x) H[(long long)i * m + k] = col[i];
 }
 
-// Blocks of the fused kernels: kKrySlice entries each while kRedBlocks of them cover the vector (19456 entries),
-// then longer slices.  With 256 entries a block and every vector's
-// products reduced by all warps, the three kernels of a step took 30 us on one drop of degree 32, now 24.
-inline int kry_blocks(long long n) {
-  return (int)std::max(1LL, std::min<long long>(kRedBlocks, (n + kKrySlice - 1) / kKrySlice));
+// w -= V h2 (i <= k); |w| by a direct sum; then, in the last block, the end of the step
+__global__ void __launch_bounds__(kKryThreads) k_kry_sub_tail(double* __restrict__ w, const double* __restrict__ V,
+                                                              long long n, int k, int m,
+                                                              const double* __restrict__ h1,
+                                                              const double* __restrict__ h2,
+                                                              double* __restrict__ partial, unsigned* counter,
+                                                              double* __restrict__ H, double* __restrict__ cs,
+                                                              double* __restrict__ sn, double* __restrict__ gv,
+                                                              double* __restrict__ scale, double* __restrict__ res) {
+  long long x0, x1;
+  kry_slice(n, &x0, &x1);
+  kry_subtract(w, V, n, k, h2, x0, x1);
+  kry_block_dots(V, n, w, 0, true, x0, x1, partial);
+  if (kry_last_block(counter)) kry_tail(partial, h1, h2, k, m, H, cs, sn, gv, scale, res);
 }
+
+// The three kernels above in one cooperative launch, for vectors short enough that a block keeps its slice of w
+// (256 / PARTS entries, one per PARTS threads) in shared memory: products of a slice by one warp per basis vector,
+// two grid barriers in the place of the launches, and every block adds the partial sums itself, in the same
+// order.  Bound by the chain of those steps, not by the data (0.2 MB): one drop of degree 32 24 -> 17 us, 48
+// drops of degrees 16 to 32 45 -> 24 us.
+template <int PARTS>
+__global__ void __launch_bounds__(kKryThreads, 2) k_kry_step(const double* __restrict__ lam, double* u,
+                                                             const double* __restrict__ d, double* __restrict__ w,
+                                                             const double* V, long long n, int k, int m, bool normalise,
+                                                             double* partial, unsigned* counter, double* __restrict__ H,
+                                                             double* __restrict__ cs, double* __restrict__ sn,
+                                                             double* __restrict__ gv, double* scale,
+                                                             double* __restrict__ res) {
+  constexpr int SL = kKryThreads / PARTS;
+  __shared__ double ws[SL], ps[PARTS][SL], h1[BIE_MAX_RESTART + 1], h2[BIE_MAX_RESTART + 1];
+  const cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+  long long x0, x1;
+  kry_slice(n, &x0, &x1);
+  const int len = (int)max(0LL, x1 - x0), x = threadIdx.x % SL, part = threadIdx.x / SL, lane = threadIdx.x & 31;
+  if (part == 0 && x < len) {
+    const double sc = normalise ? scale[0] : 1.0, v = sc * u[x0 + x];
+    if (normalise) u[x0 + x] = v;
+    ws[x] = lam ? (lam[x0 + x] + 1.0) * v - sc * d[x0 + x] : sc * d[x0 + x];
+  }
+  __syncthreads();
+  for (int pass = 0; pass < 2; ++pass) {
+    double* P = partial + (long long)pass * (m + 2) * gridDim.x;
+    double* h = pass == 0 ? h1 : h2;
+    for (int i = threadIdx.x >> 5; i <= k; i += kKryThreads >> 5) {
+      double a = 0;
+      for (int q = lane; q < len; q += 32) a += V[(long long)i * n + x0 + q] * ws[q];
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+      if (lane == 0) P[(long long)i * gridDim.x + blockIdx.x] = a;
+    }
+    grid.sync();
+    kry_finish(P, k + 1, h);
+    __syncthreads();
+    double t = 0;
+    if (x < len)
+#pragma unroll 4
+      for (int i = part; i <= k; i += PARTS) t += h[i] * V[(long long)i * n + x0 + x];
+    ps[part][x] = t;
+    __syncthreads();
+    if (part == 0 && x < len) {
+      t = ps[0][x];
+      for (int q = 1; q < PARTS; ++q) t += ps[q][x];
+      ws[x] -= t;
+    }
+    __syncthreads();
+  }
+  if (part == 0 && x < len) w[x0 + x] = ws[x];
+  double* P = partial + 2LL * (m + 2) * gridDim.x;
+  if (threadIdx.x < 32) {
+    double a = 0;
+    for (int q = lane; q < len; q += 32) a += ws[q] * ws[q];
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    if (lane == 0) P[blockIdx.x] = a;
+  }
+  if (kry_last_block(counter)) kry_tail(P, h1, h2, k, m, H, cs, sn, gv, scale, res);
+}
+
+// blocks of the three kernels
+inline int kry_blocks(long long n) { return (int)std::max(1LL, std::min<long long>(kRedBlocks, (n + 63) / 64)); }
 
 // start of a cycle: gv = (beta, 0, ..., 0), V_0 = r / beta
 __global__ void k_cycle_start(const double* __restrict__ r, double beta, double* __restrict__ v0, long long n,
@@ -2150,7 +2174,7 @@ inline unsigned nblk(long long n) { return (unsigned)((n + 255) / 256); }
 
 struct Krylov {
   long long n = 0;
-  int m = 0;
+  int m = 0, sms = 0;
   DevBuf<double> V, w, tmp, partial, hdev, r, dx, t;
   DevBuf<double> Hd, csd, snd, gvd, scale, resd, yd;  // Hessenberg, rotations, rhs, residual estimates
   DevBuf<unsigned> counter;                              // last-block counter of the fused kernels
@@ -2165,12 +2189,13 @@ struct Krylov {
   std::map<long long, StepGraph> steps;  // captured Arnoldi steps by (precision, restart, k)
   bool steps_failed = false;             // a capture failed: step eagerly from then on
   // workspace of restart length mr for vectors of length n_
-  int init(long long n_, int mr) {
+  int init(long long n_, int mr, int sms_) {
     n = n_;
+    sms = sms_;
     m = mr;
     BIE_TRY(V.alloc((size_t)(mr + 1) * n));
     BIE_TRY(tmp.alloc(3 * n));
-    BIE_TRY(partial.alloc((size_t)kRedBlocks * (mr + 2)));
+    BIE_TRY(partial.alloc((size_t)kRedBlocks * (2 * (mr + 2) + 1)));
     BIE_TRY(hdev.alloc(2 * (mr + 2)));
     BIE_TRY(Hd.alloc((size_t)(mr + 1) * mr));
     BIE_TRY(csd.alloc(mr));
@@ -2274,6 +2299,28 @@ static int arnoldi_tail(Krylov& K, const double* lam, const double* t2, long lon
   double* vk1 = V + (long long)(k + 1) * n;
   double* h1 = K.hdev.ptr;
   double* h2d = K.hdev.ptr + (m + 2);
+  // One kernel where 64 or 128 entries a block leave no more than two blocks per SM (up to 38912 entries on 152
+  // SMs), which then are all resident and can wait for one another.
+  const int cap = std::min(kRedBlocks, 2 * K.sms);
+  const int nb1 = (int)std::max(1LL, std::min<long long>((n + 63) / 64, cap));
+  if (n <= 128LL * cap) {
+    auto kern = n <= 64LL * cap ? k_kry_step<4> : k_kry_step<2>;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeCooperative;
+    attr.val.cooperative = 1;
+    cfg.gridDim = dim3((unsigned)nb1);
+    cfg.blockDim = dim3(kKryThreads);
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    BIE_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, lam, vk, t2, vk1, (const double*)V, n, k, m, k > 0, K.partial.ptr,
+                                    K.counter.ptr, K.Hd.ptr, K.csd.ptr, K.snd.ptr, K.gvd.ptr, K.scale.ptr, K.resd.ptr));
+    count_launch();
+    BIE_CUDA_TRY(cudaGetLastError());
+    BIE_CUDA_TRY(cudaMemcpyAsync(K.hpin + k, K.resd.ptr + k, sizeof(double), cudaMemcpyDeviceToHost, s));
+    return BIE_OK;
+  }
   const int nbk = kry_blocks(n);
   k_kry_sysop_dots<<<nbk, kKryThreads, 0, s>>>(lam, vk, t2, vk1, V, n, k, k > 0 ? K.scale.ptr : nullptr, K.partial.ptr,
                                        K.counter.ptr, h1);
@@ -2766,7 +2813,7 @@ static int surf_implicit_solve(const SurfLayout& L, const double* x, const doubl
   BIE_TRY(bp.alloc(L.ns));
   BIE_TRY(launch_mul(b, I.inv_diag.ptr, L.ns, bp.ptr, s));
   Krylov K;
-  BIE_TRY(K.init(L.ns, 60));
+  BIE_TRY(K.init(L.ns, 60, L.sms));
   auto op = [&](const double* in, double* out) { return surf_implicit_apply(I, in, out, s); };
   return surf_gmres(K, op, bp.ptr, y, tol, 600, iters, s);
 }
@@ -3152,7 +3199,7 @@ int bie_solve(bie_ctx* ctx, const bie_geom* g, const double* rhs, double* u, con
     gm->kry = new bie::Krylov();
   }
   bie::Krylov& K = *gm->kry;
-  BIE_TRY(K.init(n, opts->restart));
+  BIE_TRY(K.init(n, opts->restart, ctx->sms));
   double rel = 0;
   int st;
   if ((opts->precision & 0xff) == BIE_FP64) {
