@@ -751,7 +751,7 @@ static int synth_xderivs(bie_ctx* ctx, const double* coef, const long long* fiel
 }
 
 // Surface records of a degree group on its grids of degree P, drop i's at rec + 7 off[i] (off on the device),
-// through temporaries for as many drops at a time as the budget holds.
+// through temporaries for as many drops at a time as the workspace holds.
 static int group_records(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, int P, double* rec, const long long* off,
                          cudaStream_t s) {
   Plan* pl;
@@ -3075,7 +3075,7 @@ int bie_interfacial_force(bie_ctx* ctx, const bie_geom* g, const double* gammaco
   cudaStream_t s = (cudaStream_t)stream;
   Phase phz(ctx, "force", s);
   DevBuf<double> tmp;
-  for (auto& Gp : g->groups) {  // as many drops of a degree at a time as the budget holds
+  for (auto& Gp : g->groups) {  // as many drops of a degree at a time as the workspace holds
     auto& G = *Gp;
     const int p = G.p, P = 2 * p + 1;  // nonlinear terms on the grid of degree 2p+1 (Sec. 1.3)
     Plan* pl;

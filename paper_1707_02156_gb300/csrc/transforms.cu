@@ -9,8 +9,8 @@
 // In FP64, whose rate is 1/76 of FP32's here, the operation count is the bound of every large batch; the
 // symmetries and the plain multiply-adds leave a quarter of the direct sums' operations.  Measured against
 // the direct sums in two kernels: the rotated grids of 64 drops of degree 24 (80000 targets x 3 fields x 3
-// kinds) 103.5 -> 62.7 ms with their rotation, the projection of 192 drops of degree 24 0.52 -> 0.076 ms, the
-// surfactant's rates and implicit stage of 48 drops 10.4 -> 6.2 ms.
+// kinds) 103.5 -> 62.7 ms with their rotation (by now a kernel of their own, rotgeo.cu), the projection of 192
+// drops of degree 24 0.52 -> 0.076 ms, the surfactant's rates and implicit stage of 48 drops 10.4 -> 6.2 ms.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
