@@ -547,7 +547,7 @@ static int analyze_groups(bie_ctx* ctx, bie_geom* g, const double* vals, double*
     ag.push_back(ana_group(pl, (long long)G.drops.size() * 3, G.goff3.ptr, 0, G.foff3.ptr, 0));
   }
   Phase ph(ctx, "analyze", s);
-  return launch_analyze(ag, vals, out, ctx->sms, s);
+  return launch_analyze(ag, vals, out, ctx->sms, s, !ctx->prof.on);
 }
 
 // The direct form serves a group when the configuration asks for it, or when the dense form's

@@ -92,7 +92,10 @@ struct AnaGroups {
   int n, cl, orders;  // groups; blocks per field, or (orders) one block per field and order
   AnaGroup g[kMaxAnaGroups];
 };
-int launch_analyze(std::vector<AnaGroup> groups, const double* grid, double* coef, int sms, cudaStream_t s);
+// early: the launch need not wait until the kernel before it on the stream has been flushed (that one must be a
+// kernel launched in full stream order).
+int launch_analyze(std::vector<AnaGroup> groups, const double* grid, double* coef, int sms, cudaStream_t s,
+                   bool early = false);
 // rotation (App. B): out[ld][a*nb+b][c] = blocks(a) applied to e^{i m alpha_b} coef[ld][c]
 template <typename CT, typename R>
 int launch_rotate(const CT* coef, const long long* field_off, int ncomp, long long ndrop, int p, const R* blocks,
