@@ -159,12 +159,27 @@ struct DevBuf {
     n = count;
     return BIE_OK;
   }
+  // On return the copy has reached the device, so that every stream finds it: on the pool's stream and waited for.
+  // cudaMemcpy from pageable memory returns with its last part still on the way, which only the legacy
+  // stream waits for; the calls' streams needn't be ordered with that one (torch's side streams are not).
   int upload(const T* host, size_t count) {
     BIE_TRY(alloc(count));
-    if (count) BIE_CUDA_TRY(cudaMemcpy(ptr, host, count * sizeof(T), cudaMemcpyHostToDevice));
+    if (!count) return BIE_OK;
+    const cudaStream_t ps = g_pools[dev].stream;
+    BIE_CUDA_TRY(cudaMemcpyAsync(ptr, host, count * sizeof(T), cudaMemcpyHostToDevice, ps));
+    BIE_CUDA_TRY(cudaStreamSynchronize(ps));
     return BIE_OK;
   }
   int upload(const std::vector<T>& v) { return upload(v.data(), v.size()); }
+  // count zeros, in place on return like an upload
+  int zeros(size_t count) {
+    BIE_TRY(alloc(count));
+    if (!count) return BIE_OK;
+    const cudaStream_t ps = g_pools[dev].stream;
+    BIE_CUDA_TRY(cudaMemsetAsync(ptr, 0, count * sizeof(T), ps));
+    BIE_CUDA_TRY(cudaStreamSynchronize(ps));
+    return BIE_OK;
+  }
 };
 
 template <typename T>
@@ -989,7 +1004,8 @@ static int setup_interdrop(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
   const int U = ctx->cfg.upsample;
   // centres from the degree-0 coefficients: x_0^0 = sqrt(4 pi) c
   std::vector<double> xc(g->ncoef_total);
-  BIE_CUDA_TRY(cudaMemcpy(xc.data(), g->xcoef.ptr, xc.size() * sizeof(double), cudaMemcpyDeviceToHost));
+  BIE_CUDA_TRY(cudaMemcpyAsync(xc.data(), g->xcoef.ptr, xc.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+  BIE_CUDA_TRY(cudaStreamSynchronize(s));
   g->centre.assign(3 * nd, 0.0);
   g->bound.assign(nd, 0.0);
   g->hdrop.assign(nd, 0.0);
@@ -1413,7 +1429,8 @@ static int setup_near(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
   if (g->nrow_total) BIE_TRY(g->nrow_off.upload(ro));
   long long npairs_eval = 0;
   std::vector<int> hgrid((size_t)npair * L);
-  BIE_CUDA_TRY(cudaMemcpy(hgrid.data(), g->ngrid_l.ptr, hgrid.size() * sizeof(int), cudaMemcpyDeviceToHost));
+  BIE_CUDA_TRY(cudaMemcpyAsync(hgrid.data(), g->ngrid_l.ptr, hgrid.size() * sizeof(int), cudaMemcpyDeviceToHost, s));
+  BIE_CUDA_TRY(cudaStreamSynchronize(s));
   for (int i = 0; i < npair; ++i)
     for (int l = 0; l < L; ++l) {
       const int j = pairs[i].src_drop;
@@ -2204,10 +2221,7 @@ struct Krylov {
     BIE_TRY(scale.alloc(1));
     BIE_TRY(resd.alloc(mr));
     BIE_TRY(yd.alloc(mr));
-    if (!counter.ptr) {
-      BIE_TRY(counter.alloc(1));
-      BIE_CUDA_TRY(cudaMemset(counter.ptr, 0, sizeof(unsigned)));
-    }
+    if (!counter.ptr) BIE_TRY(counter.zeros(1));
     if (hpin_n < std::max(mr, 2)) {
       if (hpin) cudaFreeHost(hpin);
       hpin = nullptr;
