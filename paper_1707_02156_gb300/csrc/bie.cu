@@ -43,15 +43,22 @@ static const double kPi = 3.14159265358979323846;
 // alloc returns; so the pool knows one stream only.  The pool keeps at most a sixteenth of the device's memory
 // unused; it gives everything unused back when an allocation fails, and when the last context of the device
 // is destroyed.
+//
+// The wait is a cudaFree of a marker made by cudaMalloc (2 us when the device is idle), not a
+// cudaDeviceSynchronize: other threads' streams may be in a graph capture (the library's own, or a caller's), which
+// a device-wide synchronisation breaks and which makes it fail.  When the wait fails all the same (a capture in
+// global mode forbids cudaFree too), the buffer isn't recycled but held until a later wait has succeeded.
 struct DevPool {
   std::once_flag once;
   cudaError_t err = cudaSuccess;
   cudaMemPool_t pool = nullptr;
   cudaStream_t stream = nullptr;
   std::atomic<int> contexts{0};
+  std::mutex mu;
+  std::vector<void*> markers, held;  // made ahead for the next waits; buffers released without a wait
 };
 constexpr int kMaxDevices = 64;
-static DevPool g_pools[kMaxDevices];
+static DevPool* const g_pools = new DevPool[kMaxDevices];  // never destroyed: buffers may be released at exit
 
 // makes a device current for its lifetime
 struct OnDevice {
@@ -65,6 +72,53 @@ struct OnDevice {
   }
 };
 
+static cudaError_t make_marker(DevPool& P) {
+  void* m = nullptr;
+  const cudaError_t e = cudaMalloc(&m, 256);
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // not sticky
+    return e;
+  }
+  std::lock_guard<std::mutex> lk(P.mu);
+  P.markers.push_back(m);
+  return cudaSuccess;
+}
+
+// Waits for everything on the device; buffers held by then return to the pool.
+static cudaError_t device_wait(int dev) {
+  DevPool& P = g_pools[dev];
+  OnDevice on(dev);
+  void* m = nullptr;
+  std::vector<void*> held;
+  for (int tries = 0; !m; ++tries) {
+    {
+      std::lock_guard<std::mutex> lk(P.mu);
+      if (!P.markers.empty()) {
+        m = P.markers.back();
+        P.markers.pop_back();
+        held.swap(P.held);
+        break;
+      }
+    }
+    const cudaError_t e = make_marker(P);
+    if (e != cudaSuccess) {
+      if (tries || !P.pool) return e;
+      cudaMemPoolTrimTo(P.pool, 0);  // room for the marker
+    }
+  }
+  const cudaError_t e = cudaFree(m);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    std::lock_guard<std::mutex> lk(P.mu);
+    P.markers.push_back(m);
+    P.held.insert(P.held.end(), held.begin(), held.end());
+    return e;
+  }
+  for (void* p : held) cudaFreeAsync(p, P.stream);
+  make_marker(P);  // for the next wait; made then if this fails
+  return cudaSuccess;
+}
+
 static cudaError_t pool_init(DevPool& P, int dev) {
   cudaMemPoolProps props{};
   props.allocType = cudaMemAllocationTypePinned;
@@ -77,6 +131,7 @@ static cudaError_t pool_init(DevPool& P, int dev) {
   unsigned long long keep = prop.totalGlobalMem / 16;
   if ((e = cudaMemPoolSetAttribute(P.pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) return e;
   OnDevice on(dev);
+  make_marker(P);
   return cudaStreamCreateWithFlags(&P.stream, cudaStreamNonBlocking);
 }
 
@@ -91,6 +146,7 @@ static cudaError_t dev_malloc(void** ptr, size_t bytes, int* device) {
   e = cudaMallocFromPoolAsync(ptr, bytes, P.pool, P.stream);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();  // not sticky
+    device_wait(dev);    // the buffers held
     cudaStreamSynchronize(P.stream);
     cudaMemPoolTrimTo(P.pool, 0);
     e = cudaMallocFromPoolAsync(ptr, bytes, P.pool, P.stream);
@@ -105,20 +161,20 @@ static cudaError_t dev_malloc(void** ptr, size_t bytes, int* device) {
 static thread_local int g_idle_device = -1;
 
 static void dev_free(void* ptr, int dev) {
-  if (g_idle_device != dev) {
-    OnDevice on(dev);
-    cudaDeviceSynchronize();
+  DevPool& P = g_pools[dev];
+  if (g_idle_device == dev || device_wait(dev) == cudaSuccess) {
+    cudaFreeAsync(ptr, P.stream);
+    return;
   }
-  cudaFreeAsync(ptr, g_pools[dev].stream);
+  std::lock_guard<std::mutex> lk(P.mu);
+  P.held.push_back(ptr);
 }
 
 // Many releases with one wait.
 struct IdleDevice {
   int prev;
   explicit IdleDevice(int dev) : prev(g_idle_device) {
-    OnDevice on(dev);
-    cudaDeviceSynchronize();
-    g_idle_device = dev;
+    if (device_wait(dev) == cudaSuccess) g_idle_device = dev;
   }
   ~IdleDevice() { g_idle_device = prev; }
 };
@@ -127,6 +183,7 @@ static void pool_add_context(int dev, int n) {
   if (dev < 0 || dev >= kMaxDevices) return;
   DevPool& P = g_pools[dev];
   if (P.contexts.fetch_add(n) + n > 0 || !P.pool) return;
+  device_wait(dev);  // the buffers held
   cudaStreamSynchronize(P.stream);
   cudaMemPoolTrimTo(P.pool, 0);
 }
@@ -496,6 +553,7 @@ struct bie_geom {
   std::vector<std::unique_ptr<Group>> groups;
   struct GraphSlot {
     bool warm = false;
+    bool failed = false;  // a capture failed: launched one by one from then on
     cudaGraphExec_t exec = nullptr;
     long long launches = 0;
   };
@@ -700,7 +758,7 @@ static int layer_apply(bie_ctx* ctx, const bie_geom* gc, int kind, const double*
   // Per-phase profiling needs the kernels launched one by one; and a single drop's apply is two kernels
   // (contraction, projection), which cost less launched directly than a replay with its two copies: 51
   // against 36 us a call at degree 16 in FP64.
-  if (!ctx->cfg.use_graphs || ctx->prof.on || g->ndrop == 1) {
+  if (!ctx->cfg.use_graphs || ctx->prof.on || g->ndrop == 1 || slot.failed) {
     BIE_TRY(layer_apply_eager(ctx, g, kind, dens, out, precision, s));
     slot.warm = true;  // every lazy allocation of this key is done
     return BIE_OK;
@@ -725,22 +783,17 @@ static int layer_apply(bie_ctx* ctx, const bie_geom* gc, int kind, const double*
     cudaGraph_t graph = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(g->cap_stream, &graph);
     ctx->prof.on = prof;
-    if (st != BIE_OK) {
-      if (graph) cudaGraphDestroy(graph);
-      return st;
-    }
-    if (ce != cudaSuccess) {
-      set_error(std::string("graph capture: ") + cudaGetErrorString(ce));
-      return BIE_ECUDA;
-    }
     slot.launches = bie_launch_count() - l0;
     count_launch(-(int)slot.launches);  // captured, not run
-    const cudaError_t ie = cudaGraphInstantiate(&slot.exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (ie != cudaSuccess) {
+    cudaError_t ie = cudaErrorUnknown;
+    if (st == BIE_OK && ce == cudaSuccess) ie = cudaGraphInstantiate(&slot.exec, graph, 0);
+    if (graph) cudaGraphDestroy(graph);
+    if (st != BIE_OK || ce != cudaSuccess || ie != cudaSuccess) {
+      // a device-wide synchronisation of another thread breaks a capture, for instance
       slot.exec = nullptr;
-      set_error(std::string("graph instantiate: ") + cudaGetErrorString(ie));
-      return BIE_ECUDA;
+      slot.failed = true;
+      cudaGetLastError();  // clear the capture's error state
+      return layer_apply_eager(ctx, g, kind, dens, out, precision, s);
     }
   }
   Phase ph(ctx, "apply_graph", s);
@@ -2396,14 +2449,14 @@ static int arnoldi_step_graph(bie_ctx* ctx, const bie_geom* gc, Krylov& K, int p
     cudaError_t ie = cudaErrorUnknown;
     if (st == BIE_OK && ce == cudaSuccess) ie = cudaGraphInstantiate(&sg.exec, graph, 0);
     if (graph) cudaGraphDestroy(graph);
+    sg.launches = bie_launch_count() - l0;
+    count_launch(-(int)sg.launches);  // captured, not run
     if (st != BIE_OK || ce != cudaSuccess || ie != cudaSuccess) {
       sg.exec = nullptr;
       K.steps_failed = true;
       cudaGetLastError();  // clear the capture's error state
       return arnoldi_step(ctx, gc, K, prec, k, m, false, s);
     }
-    sg.launches = bie_launch_count() - l0;
-    count_launch(-(int)sg.launches);  // captured, not run
     for (int i = 0; i < 3; ++i) sg.sig[i] = sig[i];
   }
   BIE_CUDA_TRY(cudaGraphLaunch(sg.exec, s));

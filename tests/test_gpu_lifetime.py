@@ -1,0 +1,223 @@
+"""Device memory of the library beside other work: a buffer goes back to the pool only after everything on the
+device that may still use it has ended, whatever the other threads do meanwhile, graph captures included."""
+import ctypes
+import threading
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import layer
+from paper_1707_02156_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+FP64_TOL = 1e-12
+P, UP = 8, 2
+
+
+@pytest.fixture(scope="module")
+def api():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1707_02156_gb300 import api, build
+    build.build()
+    return api
+
+
+@pytest.fixture(scope="module")
+def case():
+    w = inputs.two_drops(p=P, gap=0.5, up=UP, lam=0.5)
+    nc = 3 * (P + 1) ** 2
+    split = lambda v: [v[:nc].reshape(3, -1), v[nc:].reshape(3, -1)]
+    drops = layer.Drops(split(w.xcoef), w.p, w.pq, w.lam, up=UP)
+    ref = np.concatenate([v.ravel() for v in drops.apply_double(split(w.density))])
+    return w, ref, drops
+
+
+def relerr(a, b):
+    a, b = np.asarray(a).ravel(), np.asarray(b).ravel()
+    return max(np.linalg.norm(a - b) / np.linalg.norm(b), np.max(np.abs(a - b)) / np.max(np.abs(b)))
+
+
+class Worker(threading.Thread):
+    """Runs fn on a stream of its own and keeps what it raises."""
+
+    def __init__(self, fn):
+        super().__init__()
+        self.fn, self.error, self.stream = fn, None, torch.cuda.Stream()
+
+    def run(self):
+        try:
+            with torch.cuda.stream(self.stream):
+                self.fn(self.stream)
+        except BaseException as e:  # noqa: BLE001
+            self.error = e
+
+
+def run_all(workers):
+    for t in workers:
+        t.start()
+    for t in workers:
+        t.join()
+    for t in workers:
+        if t.error is not None:
+            raise t.error
+
+
+def tensors(w):
+    x, f = torch.as_tensor(w.xcoef).cuda(), torch.as_tensor(w.density).cuda()
+    return x, f, torch.full_like(f, float("nan"))
+
+
+def test_close_waits_for_the_work_that_uses_the_geometry(api, case):
+    w, ref, _ = case
+    ctx = api.Context(0, upsample=UP)
+    x, f, out = tensors(w)
+    torch.cuda.synchronize()
+    geo = ctx.geometry(w.p, w.pq, x, w.lam)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(100_000_000)  # about 50 ms
+        geo.apply_double(f, out, precision=0)
+    geo.close()
+    assert side.query()
+    assert relerr(out.cpu().numpy(), ref) < FP64_TOL
+    ctx.close()
+
+
+def open_geometry(api, ctx, w, x, f, out):
+    geo = ctx.geometry(w.p, w.pq, x, w.lam)
+    for _ in range(3):  # lazy allocations, capture, replay
+        geo.apply_double(f, out, precision=0)
+    out.fill_(float("nan"))
+    torch.cuda.synchronize()
+    return geo
+
+
+def check_next_geometry(ctx, w, x, f, out, ref):
+    geo = ctx.geometry(w.p, w.pq, x, w.lam)
+    for _ in range(3):
+        out.fill_(float("nan"))
+        geo.apply_double(f, out, precision=0)
+        assert relerr(out.cpu().numpy(), ref) < FP64_TOL
+    geo.close()
+
+
+@pytest.mark.parametrize("mode", ["thread_local", "relaxed"])
+def test_release_beside_another_threads_capture(api, case, mode):
+    # the main thread captures while another one uses and closes a geometry, and makes and closes the next
+    w, ref, _ = case
+    ctx = api.Context(0, upsample=UP)
+    x, f, out = tensors(w)
+    a = torch.ones(1000, device="cuda")
+    b = torch.zeros_like(a)
+    geo = open_geometry(api, ctx, w, x, f, out)
+    got = []
+
+    def work(stream):
+        torch.cuda._sleep(20_000_000)
+        geo.apply_double(f, out, precision=0)
+        geo.close()
+        assert stream.query()
+        ctx2 = api.Context(0, upsample=UP)
+        geo2 = ctx2.geometry(w.p, w.pq, x, w.lam)
+        geo2.apply_double(f, out, precision=0)
+        geo2.close()
+        ctx2.close()
+        got.append(out)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode=mode):
+        b.copy_(a)
+        run_all([Worker(work)])
+        b.add_(a)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert float(b.sum()) == 2000.0
+    assert relerr(got[0].cpu().numpy(), ref) < FP64_TOL
+    check_next_geometry(ctx, w, x, f, out, ref)
+    ctx.close()
+
+
+def test_close_while_a_capture_forbids_the_wait(api, case):
+    # in the capture mode "global" no thread may free memory: the buffers are held, and come back later
+    w, ref, _ = case
+    ctx = api.Context(0, upsample=UP)
+    x, f, out = tensors(w)
+    geo = open_geometry(api, ctx, w, x, f, out)
+    cudart = ctypes.CDLL("libcudart.so.13")
+    other, graph = torch.cuda.Stream(), ctypes.c_void_p()
+    assert cudart.cudaStreamBeginCapture(ctypes.c_void_p(other.cuda_stream), 0) == 0
+    try:
+        def work(stream):
+            torch.cuda._sleep(20_000_000)
+            geo.apply_double(f, out, precision=0)
+            geo.close()
+        t = Worker(work)
+        run_all([t])
+    finally:
+        cudart.cudaStreamEndCapture(ctypes.c_void_p(other.cuda_stream), ctypes.byref(graph))
+        if graph.value:
+            cudart.cudaGraphDestroy(graph)
+        cudart.cudaGetLastError()
+    t.stream.synchronize()
+    assert relerr(out.cpu().numpy(), ref) < FP64_TOL
+    check_next_geometry(ctx, w, x, f, out, ref)
+    ctx.close()
+
+
+@pytest.mark.parametrize("disturb", [False, True])
+def test_threads_capture_and_release_beside_one_another(api, case, disturb):
+    # every geometry's second apply is a capture, its third a replay, and its end a release; with disturb another
+    # thread synchronises the whole device all the time, which breaks captures: their applies run eagerly
+    w, ref, drops = case
+    got, stop = [[] for _ in range(3)], threading.Event()
+
+    def work(k):
+        def fn(stream):
+            x, f, out = tensors(w)
+            ctx = api.Context(0, upsample=UP)
+            for _ in range(6):
+                geo = ctx.geometry(w.p, w.pq, x, w.lam)
+                for _ in range(4):
+                    out.fill_(float("nan"))
+                    geo.apply_double(f, out, precision=0)
+                    stream.synchronize()
+                    got[k].append(out.cpu().numpy())
+                if k == 0:  # the steps of a solve are captures, too
+                    u = torch.zeros_like(f)
+                    info = geo.solve(f, u, precision=0, tol=1e-12)
+                    assert info["converged"]
+                    A = torch.full_like(f, float("nan"))
+                    geo.apply_double(u, A, precision=0)
+                    stream.synchronize()
+                    lam = np.repeat(np.asarray(w.lam), f.numel() // 2)
+                    un = u.cpu().numpy()
+                    r = (lam + 1) * un - A.cpu().numpy() - w.density
+                    assert np.linalg.norm(r) < 1e-11 * np.linalg.norm(w.density)
+                geo.close()
+            ctx.close()
+        return fn
+
+    def sync_all(stream):
+        while not stop.is_set():
+            try:
+                torch.cuda.synchronize()
+            except RuntimeError:  # another thread captures
+                pass
+
+    disturber = Worker(sync_all)
+    if disturb:
+        disturber.start()
+    try:
+        run_all([Worker(work(k)) for k in range(3)])
+    finally:
+        stop.set()
+        if disturb:
+            disturber.join()
+    for g in got:
+        assert len(g) == 24
+        for v in g:
+            assert relerr(v, ref) < FP64_TOL
