@@ -586,6 +586,7 @@ struct bie_geom {
   bie::DevBuf<double> nrows[2];                     // the rule as rows of the operator, S and D (first apply of a kind)
   bie::DevBuf<long long> nrow_off;
   long long nrow_total = 0;                         // doubles per kind; 0: the rows are not used
+  bool no_rows[2] = {false, false};                 // the device had no room for the kind's rows
   bie::DevBuf<long long> coef_off_d, up_off_d, up_n_d;
 };
 
@@ -1499,9 +1500,10 @@ static int near_snapshot(bie_geom* g, cudaStream_t s) {
   return analyze_groups(g->ctx, g, g->vals.ptr, g->selfcoef.ptr, s);
 }
 
-// The rows of one kind, built at its first apply on the geometry (see near.cu).
+// The rows of one kind, built at its first apply on the geometry (see near.cu).  Without room for them on the device
+// the kind keeps the check-point sums, which need none.
 static int ensure_near_rows(bie_geom* g, int kind, cudaStream_t s) {
-  if (g->nrows[kind].ptr) return BIE_OK;
+  if (!g->nrow_total || g->nrows[kind].ptr || g->no_rows[kind]) return BIE_OK;
   bie_ctx* ctx = g->ctx;
   Phase ph(ctx, "near_rows", s);
   std::map<int, std::vector<int>> byp;
@@ -1510,8 +1512,14 @@ static int ensure_near_rows(bie_geom* g, int kind, cudaStream_t s) {
   for (const auto& kv : byp) all.insert(all.end(), kv.second.begin(), kv.second.end());
   DevBuf<int> list;
   DevBuf<double> rows;
-  BIE_TRY(list.upload(all));
-  BIE_TRY(rows.alloc(g->nrow_total));
+  int st = list.upload(all);
+  if (st == BIE_OK) st = rows.alloc(g->nrow_total);
+  if (st == BIE_ENOMEM) {
+    set_error("");
+    g->no_rows[kind] = true;
+    return BIE_OK;
+  }
+  BIE_TRY(st);
   size_t at = 0;
   for (const auto& kv : byp) {
     const int p = kv.first, Pu = ctx->cfg.upsample * (p + 1) - 1, n = (int)kv.second.size();
@@ -1536,8 +1544,8 @@ static int near_apply(bie_geom* g, int kind, bool raw, int prec, const double* d
   bie_ctx* ctx = g->ctx;
   const int npair = (int)g->near.size(), L = ctx->cfg.n_interp;
   const double* wts = kind == 0 ? (raw ? g->wSr_all.ptr : g->wS_all.ptr) : (raw ? g->wDr_all.ptr : g->wD_all.ptr);
-  if (g->nrow_total) {
-    BIE_TRY(ensure_near_rows(g, kind, s));
+  BIE_TRY(ensure_near_rows(g, kind, s));
+  if (g->nrows[kind].ptr) {
     Phase ph(ctx, "near", s);
     return launch_near_rows_apply(g->npairs.ptr, g->ntbeg.ptr, g->nnear_tgt, g->nrows[kind].ptr, g->nrow_off.ptr,
                                   g->selfcoef.ptr, dens, g->coef_off_d.ptr, g->pdeg_d.ptr, wts, g->tdrop.ptr,

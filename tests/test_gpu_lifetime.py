@@ -1,6 +1,9 @@
 """Device memory of the library beside other work: a buffer goes back to the pool only after everything on the
 device that may still use it has ended, whatever the other threads do meanwhile, graph captures included."""
 import ctypes
+import os
+import subprocess
+import sys
 import threading
 
 import numpy as np
@@ -221,3 +224,67 @@ def test_threads_capture_and_release_beside_one_another(api, case, disturb):
         assert len(g) == 24
         for v in g:
             assert relerr(v, ref) < FP64_TOL
+
+
+def test_near_contact_applies_on_a_full_device(api):
+    # 12 contacts of 8 drops: the near rule's rows would take 82 MB, more than the device has left after the set-up.
+    # Rows and check-point sums are the same sum in another order; the bar is its rounding (some 2^-53 a term), which
+    # the interpolation amplifies by up to 1.9e3
+    code = """
+import numpy as np, torch
+from paper_1707_02156_gb300 import api, inputs
+p, d = 32, 2.05
+xs = [inputs.sphere_coef(p, centre=(d * (k & 1), d * (k >> 1 & 1), d * (k >> 2))) for k in range(8)]
+rng = np.random.default_rng(3)
+x = torch.as_tensor(inputs.pack_drops(xs)).cuda()
+f = torch.as_tensor(inputs.pack_drops([inputs.random_bandlimited(rng, p, 3) for _ in xs])).cuda()
+lam = [0.5] * 8
+out = torch.empty_like(f)
+ctx = api.Context(0)
+
+def applies(geo):
+    got = []
+    for fn in (geo.apply_single, geo.apply_double):
+        for prec in (0, 0, 0, 1, 1):
+            out.fill_(float("nan"))
+            fn(f, out, precision=prec)
+            got.append(out.cpu().numpy())
+    return got
+
+geo = ctx.geometry([p] * 8, [p] * 8, x, lam)
+assert geo.info["near_targets"] * 7 * (p + 1) ** 2 * 8 > 80e6, geo.info
+ref = applies(geo)
+geo.close()
+geo = ctx.geometry([p] * 8, [p] * 8, x, lam)
+fill = []
+
+def fill_up(leave):
+    torch.cuda.synchronize()
+    n = torch.cuda.mem_get_info()[0] - leave
+    if n > 4 << 20:
+        fill.append(torch.empty(n >> 21 << 21, dtype=torch.uint8, device="cuda"))
+
+spare = torch.empty(40 << 20, dtype=torch.uint8, device="cuda")
+fill_up(60 << 20)
+kept = []  # what the library keeps for the next geometry goes to small ones, until no room for the smallest is left
+for q in (32, 20, 12, 6):
+    try:
+        while True:
+            kept.append(ctx.geometry([q], [q], torch.as_tensor(inputs.sphere_coef(q).ravel()).cuda(), [0.5]))
+    except api.BIEError as e:
+        assert e.status == 2, e
+del spare
+torch.cuda.empty_cache()
+assert torch.cuda.mem_get_info()[0] < 75e6, torch.cuda.mem_get_info()
+got = applies(geo)
+for k, (a, b) in enumerate(zip(got, ref)):
+    e = np.linalg.norm(a - b) / np.linalg.norm(b)
+    assert e < 1e-11, (k, e)
+for g in [geo] + kept:
+    g.close()
+ctx.close()
+print(len(kept), "ok")
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=180,
+                       cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert r.returncode == 0 and r.stdout.endswith("ok\n"), r.stdout + r.stderr
