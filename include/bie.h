@@ -185,7 +185,11 @@ int bie_interfacial_force(bie_ctx* ctx, const bie_geom* geom, const double* gamm
 int bie_apply_single(bie_ctx* ctx, const bie_geom* geom, const double* fcoef, double* out_coef, int precision,
                      void* stream);
 
-/* Double-layer apply, same layout: out = coefficients of D[u] (the GMRES matvec's operator part). */
+/* Double-layer apply, same layout: out = coefficients of D[u] (the GMRES matvec's operator part).
+ * The first call of a layer with given flags allocates what its precision needs.  On a geometry with pairs in
+ * Omega_2 the second apply of a layer (or the first solve, for the double layer) builds the near rule's rows,
+ * 7 (p+1)^2 doubles per pair, up to 4 GB, and synchronises with the stream; not while the stream is
+ * captured, and not when the device has no room for them.  They count in cache_bytes and go with the geometry. */
 int bie_apply_double(bie_ctx* ctx, const bie_geom* geom, const double* ucoef, double* out_coef, int precision,
                      void* stream);
 

@@ -583,10 +583,11 @@ struct bie_geom {
   bie::DevBuf<bie::NearPair> npairs;
   bie::DevBuf<int> ntbeg, ngrid_l, pdeg_d;
   bie::DevBuf<double> npts, ncv, selfcoef, hdrop_d;
-  bie::DevBuf<double> nrows[2];                     // the rule as rows of the operator, S and D (first apply of a kind)
+  bie::DevBuf<double> nrows[2];                     // the rule as rows of the operator, S and D (ensure_near_rows)
   bie::DevBuf<long long> nrow_off;
   long long nrow_total = 0;                         // doubles per kind; 0: the rows are not used
   bool no_rows[2] = {false, false};                 // the device had no room for the kind's rows
+  bool near_seen[2] = {false, false};               // the kind has been applied
   bie::DevBuf<long long> coef_off_d, up_off_d, up_n_d;
 };
 
@@ -706,6 +707,7 @@ template <typename R>
 static int interdrop_apply(bie_geom* g, int kind, bool raw, const double* dens, cudaStream_t s, bool df = false);
 static int near_apply(bie_geom* g, int kind, bool raw, int prec, const double* dens, cudaStream_t s);
 static int near_snapshot(bie_geom* g, cudaStream_t s);
+static int ensure_near_rows(bie_geom* g, int kind, cudaStream_t s);
 
 static int layer_apply_eager(bie_ctx* ctx, const bie_geom* gc, int kind, const double* dens, double* out,
                              int precision, cudaStream_t s) {
@@ -772,6 +774,7 @@ static int layer_apply(bie_ctx* ctx, const bie_geom* gc, int kind, const double*
       slot.warm = true;
       return BIE_OK;
     }
+    BIE_TRY(ensure_near_rows(g, kind, s));  // of the second apply: they cannot be built in the capture
     BIE_TRY(g->gin.alloc(std::max(g->ncoef_total, 3 * g->ntarget)));
     BIE_TRY(g->gout.alloc(std::max(g->ncoef_total, 3 * g->ntarget)));
     if (!g->cap_stream) BIE_CUDA_TRY(cudaStreamCreateWithFlags(&g->cap_stream, cudaStreamNonBlocking));
@@ -1466,10 +1469,8 @@ static int setup_near(bie_ctx* ctx, bie_geom* g, cudaStream_t s) {
   BIE_TRY(near_points(ctx, g, pairs, g->npairs.ptr, x0, hseed, g->npts, g->ngrid_l, s));
   BIE_TRY(g->ncv.alloc(3 * (size_t)npair * L));
   BIE_TRY(near_tables(g));
-  // The rule becomes rows of the operator unless they would take more than 4 GB per kind, or a block's
-  // sums do not fit in shared memory (degrees above 56): a row costs about 1.3 evaluations of its
-  // check-point sums to build, once, and makes every further apply of the kind read 7 (p+1)^2 doubles
-  // per pair instead.
+  // The rule becomes rows of the operator (at a kind's second apply or a solve, see ensure_near_rows) unless they would
+  // take more than 4 GB per kind, or a block's sums do not fit in shared memory (degrees above 56).
   std::vector<long long> ro(npair);
   long long rtot = 0;
   bool fit = true;
@@ -1500,10 +1501,16 @@ static int near_snapshot(bie_geom* g, cudaStream_t s) {
   return analyze_groups(g->ctx, g, g->vals.ptr, g->selfcoef.ptr, s);
 }
 
-// The rows of one kind, built at its first apply on the geometry (see near.cu).  Without room for them on the device
-// the kind keeps the check-point sums, which need none.
+// The rows of one kind (see near.cu), for a call that applies the kind again: its first apply on a geometry sums the
+// check points, which costs less than building the rows (two drops of degree 32 at gap 0.05: 3.6 against 8.4 to
+// 9.1 ms), and the single layer of a time step is applied once per geometry; from the second apply on, and before
+// the steps of a solve, the rows pay.  Nothing is built in a capture (the apply before it has allocated what the check
+// sums need), and without room on the device the kind keeps the check sums, which need none.
 static int ensure_near_rows(bie_geom* g, int kind, cudaStream_t s) {
   if (!g->nrow_total || g->nrows[kind].ptr || g->no_rows[kind]) return BIE_OK;
+  cudaStreamCaptureStatus cap;
+  BIE_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+  if (cap != cudaStreamCaptureStatusNone) return BIE_OK;
   bie_ctx* ctx = g->ctx;
   Phase ph(ctx, "near_rows", s);
   std::map<int, std::vector<int>> byp;
@@ -1544,7 +1551,8 @@ static int near_apply(bie_geom* g, int kind, bool raw, int prec, const double* d
   bie_ctx* ctx = g->ctx;
   const int npair = (int)g->near.size(), L = ctx->cfg.n_interp;
   const double* wts = kind == 0 ? (raw ? g->wSr_all.ptr : g->wS_all.ptr) : (raw ? g->wDr_all.ptr : g->wD_all.ptr);
-  BIE_TRY(ensure_near_rows(g, kind, s));
+  if (g->near_seen[kind]) BIE_TRY(ensure_near_rows(g, kind, s));
+  g->near_seen[kind] = true;
   if (g->nrows[kind].ptr) {
     Phase ph(ctx, "near", s);
     return launch_near_rows_apply(g->npairs.ptr, g->ntbeg.ptr, g->nnear_tgt, g->nrows[kind].ptr, g->nrow_off.ptr,
@@ -2519,6 +2527,7 @@ static int gmres(bie_ctx* ctx, const bie_geom* g, int prec, const double* b, dou
       BIE_TRY(norm2(K, r, &beta, s));
     *relres = beta / bnorm;
     if (beta / bnorm <= tol || it >= max_iter) return beta / bnorm <= tol ? BIE_OK : BIE_ENOCONV;
+    BIE_TRY(ensure_near_rows(const_cast<bie_geom*>(g), 1, s));
     double* V = K.V.ptr;
     k_cycle_start<<<nblk(std::max<long long>(n, m + 1)), 256, 0, s>>>(r, beta, V, n, K.gvd.ptr, m);
     count_launch();
@@ -3136,6 +3145,7 @@ void bie_geometry_destroy(bie_geom* g) {
 int bie_geometry_info(const bie_geom* g, bie_geom_info* info) {
   if (!g || !info) return BIE_EINVAL;
   *info = g->info;
+  info->cache_bytes += (g->nrows[0].n + g->nrows[1].n) * 8.0;
   return BIE_OK;
 }
 

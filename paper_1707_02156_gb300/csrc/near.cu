@@ -502,10 +502,10 @@ __global__ void k_near_interp(const NearPair* __restrict__ pairs, const int* __r
 // transposed synthesis (phi sums over longitude quadruples, then P~_n^m over latitude pairs).  A row has
 // six symmetric 3x3 planes; for the double layer the jump -4 pi b_0 u(x*) of the exterior limit is part
 // of them.  A seventh plane holds b_0 Y_r(x*), which meets the drop's own on-surface expansion.  Building
-// a row costs about 1.3 evaluations of its check-point sums (31 FP64 operations per check point and source,
-// the projection a quarter of that) and every apply after that reads 7 (p+1)^2 doubles instead.  Two drops of
-// degree 32 at gap 0.05 (U = 4): the near step of an apply 6.1 -> 0.05 ms, a solve with its 15 applies 100 ->
-// 7.2 ms, its first one on a new geometry 27 ms.
+// a row costs about 2.4 evaluations of its check-point sums (31 FP64 operations per check point and source,
+// and the projection), and every apply after that reads 7 (p+1)^2 doubles instead: so a kind's first apply on
+// a geometry sums the check points (k_near_checks), and the rows are built for those after it.  Two drops of
+// degree 32 at gap 0.05 (U = 4): check sums 3.6 ms an apply, rows 8.4 and 9.1 ms (S, D) once and 0.05 ms an apply.
 constexpr int kNearThreads = 256;
 
 template <int KIND>
