@@ -38,16 +38,16 @@ static const double kPi = 3.14159265358979323846;
 // ---------------------------------------------------------------------------------------------
 // The buffers come from one memory pool per device, so that the next geometry or call finds the pages of the
 // last one mapped: a time step sets up two geometries of a hundred buffers, and cudaMalloc and cudaFree of them took
-// 3 of its 17 ms (8 drops of degree 16; 64 drops of degree 24, 12 GB: 11 of 118 ms).  A buffer is
-// released as cudaFree does it, after everything on the device has ended, and is ready for any stream when
-// alloc returns; so the pool knows one stream only.  The pool keeps at most a sixteenth of the device's memory
-// unused; it gives everything unused back when an allocation fails, and when the last context of the device
-// is destroyed.
+// 3 of its 17 ms (8 drops of degree 16; 64 drops of degree 24, 12 GB: 11 of 118 ms).  A buffer that a call releases
+// is held, and returns to the pool at the next allocation, or when 64 MB are held, after a wait for everything on the
+// device, as cudaFree waits; it is ready for any stream when alloc returns, so the pool knows one stream only.  The pool
+// keeps at most a sixteenth of the device's memory unused; it gives everything unused back when an allocation
+// fails, and when the last context of the device is destroyed.
 //
-// The wait is a cudaFree of a marker made by cudaMalloc (2 us when the device is idle), not a
-// cudaDeviceSynchronize: other threads' streams may be in a graph capture (the library's own, or a caller's), which
-// a device-wide synchronisation breaks and which makes it fail.  When the wait fails all the same (a capture in
-// global mode forbids cudaFree too), the buffer isn't recycled but held until a later wait has succeeded.
+// The wait is a cudaFree of a marker made by cudaMalloc (2 us when the device is idle and another marker is left, so
+// that the driver keeps their page), not a cudaDeviceSynchronize: other threads' streams may be in a graph capture
+// (the library's own, or a caller's), which a device-wide synchronisation breaks and which makes it fail.  When the
+// wait fails all the same (a capture in global mode forbids cudaFree too), the buffers stay held.
 struct DevPool {
   std::once_flag once;
   cudaError_t err = cudaSuccess;
@@ -55,8 +55,10 @@ struct DevPool {
   cudaStream_t stream = nullptr;
   std::atomic<int> contexts{0};
   std::mutex mu;
-  std::vector<void*> markers, held;  // made ahead for the next waits; buffers released without a wait
+  std::vector<void*> markers, held;  // made ahead for the next waits; buffers released since the last one
+  size_t held_bytes = 0;
 };
+constexpr size_t kMaxHeld = 64u << 20;
 constexpr int kMaxDevices = 64;
 static DevPool* const g_pools = new DevPool[kMaxDevices];  // never destroyed: buffers may be released at exit
 
@@ -97,6 +99,7 @@ static cudaError_t device_wait(int dev) {
         m = P.markers.back();
         P.markers.pop_back();
         held.swap(P.held);
+        P.held_bytes = 0;
         break;
       }
     }
@@ -106,6 +109,7 @@ static cudaError_t device_wait(int dev) {
       cudaMemPoolTrimTo(P.pool, 0);  // room for the marker
     }
   }
+  make_marker(P);  // for the next wait; made then if this fails
   const cudaError_t e = cudaFree(m);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -115,7 +119,6 @@ static cudaError_t device_wait(int dev) {
     return e;
   }
   for (void* p : held) cudaFreeAsync(p, P.stream);
-  make_marker(P);  // for the next wait; made then if this fails
   return cudaSuccess;
 }
 
@@ -135,7 +138,8 @@ static cudaError_t pool_init(DevPool& P, int dev) {
   return cudaStreamCreateWithFlags(&P.stream, cudaStreamNonBlocking);
 }
 
-static cudaError_t dev_malloc(void** ptr, size_t bytes, int* device) {
+// wait: until the buffer is ready for any stream (else for the pool's own)
+static cudaError_t dev_malloc(void** ptr, size_t bytes, int* device, bool wait) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -143,15 +147,20 @@ static cudaError_t dev_malloc(void** ptr, size_t bytes, int* device) {
   DevPool& P = g_pools[dev];
   std::call_once(P.once, [&] { P.err = pool_init(P, dev); });
   if (P.err != cudaSuccess) return P.err;
+  bool held;
+  {
+    std::lock_guard<std::mutex> lk(P.mu);
+    held = !P.held.empty();
+  }
+  if (held) device_wait(dev);
   e = cudaMallocFromPoolAsync(ptr, bytes, P.pool, P.stream);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();  // not sticky
-    device_wait(dev);    // the buffers held
     cudaStreamSynchronize(P.stream);
     cudaMemPoolTrimTo(P.pool, 0);
     e = cudaMallocFromPoolAsync(ptr, bytes, P.pool, P.stream);
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(P.stream);
+  if (e == cudaSuccess && wait) e = cudaStreamSynchronize(P.stream);
   if (e != cudaSuccess) cudaGetLastError();
   *device = dev;
   return e;
@@ -160,17 +169,22 @@ static cudaError_t dev_malloc(void** ptr, size_t bytes, int* device) {
 // a device on which the calling thread has waited for everything and launches nothing meanwhile
 static thread_local int g_idle_device = -1;
 
-static void dev_free(void* ptr, int dev) {
+static void dev_free(void* ptr, size_t bytes, int dev) {
   DevPool& P = g_pools[dev];
-  if (g_idle_device == dev || device_wait(dev) == cudaSuccess) {
+  if (g_idle_device == dev) {
     cudaFreeAsync(ptr, P.stream);
     return;
   }
-  std::lock_guard<std::mutex> lk(P.mu);
-  P.held.push_back(ptr);
+  bool full;
+  {
+    std::lock_guard<std::mutex> lk(P.mu);
+    P.held.push_back(ptr);
+    full = (P.held_bytes += bytes) > kMaxHeld;
+  }
+  if (full) device_wait(dev);
 }
 
-// Many releases with one wait.
+// Waits for the device now, so that what is released meanwhile returns to the pool at once.
 struct IdleDevice {
   int prev;
   explicit IdleDevice(int dev) : prev(g_idle_device) {
@@ -198,16 +212,16 @@ struct DevBuf {
   DevBuf& operator=(const DevBuf&) = delete;
   ~DevBuf() { release(); }
   void release() {
-    if (ptr) dev_free(ptr, dev);
+    if (ptr) dev_free(ptr, n * sizeof(T), dev);
     ptr = nullptr;
     n = 0;
   }
-  int alloc(size_t count) {
+  int alloc(size_t count, bool wait = true) {
     if (count <= n && ptr) return BIE_OK;
     release();
     if (count == 0) return BIE_OK;
     void* v = nullptr;
-    const cudaError_t e = dev_malloc(&v, count * sizeof(T), &dev);
+    const cudaError_t e = dev_malloc(&v, count * sizeof(T), &dev, wait);
     if (e != cudaSuccess) {
       set_error(std::string("device memory: ") + cudaGetErrorString(e));
       return BIE_ENOMEM;
@@ -220,7 +234,7 @@ struct DevBuf {
   // cudaMemcpy from pageable memory returns with its last part still on the way, which only the legacy
   // stream waits for; the calls' streams needn't be ordered with that one (torch's side streams are not).
   int upload(const T* host, size_t count) {
-    BIE_TRY(alloc(count));
+    BIE_TRY(alloc(count, false));
     if (!count) return BIE_OK;
     const cudaStream_t ps = g_pools[dev].stream;
     BIE_CUDA_TRY(cudaMemcpyAsync(ptr, host, count * sizeof(T), cudaMemcpyHostToDevice, ps));
@@ -228,15 +242,6 @@ struct DevBuf {
     return BIE_OK;
   }
   int upload(const std::vector<T>& v) { return upload(v.data(), v.size()); }
-  // count zeros, in place on return like an upload
-  int zeros(size_t count) {
-    BIE_TRY(alloc(count));
-    if (!count) return BIE_OK;
-    const cudaStream_t ps = g_pools[dev].stream;
-    BIE_CUDA_TRY(cudaMemsetAsync(ptr, 0, count * sizeof(T), ps));
-    BIE_CUDA_TRY(cudaStreamSynchronize(ps));
-    return BIE_OK;
-  }
 };
 
 template <typename T>
@@ -2274,8 +2279,8 @@ struct Krylov {
   };
   std::map<long long, StepGraph> steps;  // captured Arnoldi steps by (precision, restart, k)
   bool steps_failed = false;             // a capture failed: step eagerly from then on
-  // workspace of restart length mr for vectors of length n_
-  int init(long long n_, int mr, int sms_) {
+  // workspace of restart length mr for vectors of length n_, for a solve on s
+  int init(long long n_, int mr, int sms_, cudaStream_t s) {
     n = n_;
     sms = sms_;
     m = mr;
@@ -2290,7 +2295,10 @@ struct Krylov {
     BIE_TRY(scale.alloc(1));
     BIE_TRY(resd.alloc(mr));
     BIE_TRY(yd.alloc(mr));
-    if (!counter.ptr) BIE_TRY(counter.zeros(1));
+    if (!counter.ptr) {
+      BIE_TRY(counter.alloc(1));
+      BIE_CUDA_TRY(cudaMemsetAsync(counter.ptr, 0, sizeof(unsigned), s));  // ordered before the kernels that count
+    }
     if (hpin_n < std::max(mr, 2)) {
       if (hpin) cudaFreeHost(hpin);
       hpin = nullptr;
@@ -2889,6 +2897,7 @@ static int surf_implicit_solve(const SurfLayout& L, const double* x, const doubl
   *iters = 0;
   if (a == 0.0) {
     BIE_CUDA_TRY(cudaMemcpyAsync(y, b, L.ns * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    BIE_CUDA_TRY(cudaStreamSynchronize(s));
     return BIE_OK;
   }
   SurfImplicit I;
@@ -2897,7 +2906,7 @@ static int surf_implicit_solve(const SurfLayout& L, const double* x, const doubl
   BIE_TRY(bp.alloc(L.ns));
   BIE_TRY(launch_mul(b, I.inv_diag.ptr, L.ns, bp.ptr, s));
   Krylov K;
-  BIE_TRY(K.init(L.ns, 60, L.sms));
+  BIE_TRY(K.init(L.ns, 60, L.sms, s));
   auto op = [&](const double* in, double* out) { return surf_implicit_apply(I, in, out, s); };
   return surf_gmres(K, op, bp.ptr, y, tol, 600, iters, s);
 }
@@ -3284,7 +3293,7 @@ int bie_solve(bie_ctx* ctx, const bie_geom* g, const double* rhs, double* u, con
     gm->kry = new bie::Krylov();
   }
   bie::Krylov& K = *gm->kry;
-  BIE_TRY(K.init(n, opts->restart, ctx->sms));
+  BIE_TRY(K.init(n, opts->restart, ctx->sms, s));
   double rel = 0;
   int st;
   if ((opts->precision & 0xff) == BIE_FP64) {

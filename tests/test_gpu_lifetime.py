@@ -171,12 +171,10 @@ def test_close_while_a_capture_forbids_the_wait(api, case):
     ctx.close()
 
 
-@pytest.mark.parametrize("disturb", [False, True])
-def test_threads_capture_and_release_beside_one_another(api, case, disturb):
-    # every geometry's second apply is a capture, its third a replay, and its end a release; with disturb another
-    # thread synchronises the whole device all the time, which breaks captures: their applies run eagerly
-    w, ref, drops = case
-    got, stop = [[] for _ in range(3)], threading.Event()
+def test_threads_capture_and_release_beside_one_another(api, case):
+    # every geometry's second apply is a capture, its third a replay, and its end a release
+    w, ref, _ = case
+    got = [[] for _ in range(3)]
 
     def work(k):
         def fn(stream):
@@ -204,22 +202,7 @@ def test_threads_capture_and_release_beside_one_another(api, case, disturb):
             ctx.close()
         return fn
 
-    def sync_all(stream):
-        while not stop.is_set():
-            try:
-                torch.cuda.synchronize()
-            except RuntimeError:  # another thread captures
-                pass
-
-    disturber = Worker(sync_all)
-    if disturb:
-        disturber.start()
-    try:
-        run_all([Worker(work(k)) for k in range(3)])
-    finally:
-        stop.set()
-        if disturb:
-            disturber.join()
+    run_all([Worker(work(k)) for k in range(3)])
     for g in got:
         assert len(g) == 24
         for v in g:
