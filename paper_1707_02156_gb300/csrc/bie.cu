@@ -633,7 +633,7 @@ static int analyze_groups(bie_ctx* ctx, bie_geom* g, const double* vals, double*
 // The direct form serves a group when the configuration asks for it, or when the dense form's
 // per-target factors would not fit in shared memory while they are built.
 static bool group_uses_direct(const bie_ctx* ctx, const bie_geom::Group& G) {
-  return ctx->cfg.self_direct != 0 || kernel_proj_smem(G.p, G.pq) > 227 * 1024;
+  return ctx->cfg.self_direct != 0 || !self_dense_fits(G.p, G.pq);
 }
 
 // Dense factors of one group in the arithmetic type R (the double-float copy is split from the

@@ -213,14 +213,15 @@ __global__ void __launch_bounds__(256) k_self_direct(
 // For each target, Q[t][e][ri][tri(n,m)] = c_m sum_j Mhat_{e,jm} P~_n^m(cos theta_j), with
 // Mhat_{e,jm} = sum_k M_{e,jk} e^{i m phi_k} the phi transform of entry e of the 3x3 kernel weight
 // over (xx, yy, zz, xy, xz, yz), ri = real / imaginary part, c_0 = 1 and c_m = 2.  Latitudes are
-// processed kProjPairs pairs (q, pq - q) at a time: kernel weights; their sums over the longitude
+// processed NP pairs (q, pq - q) at a time: kernel weights; their sums over the longitude
 // quadruples that share |cos m phi| and |sin m phi|, in place; the phi transform of both rows, whose sum
 // and difference serve even and odd n - m; and the Legendre projection, accumulated in shared memory.
 // The phi transform and the projection (0.15M multiply-adds per target and kind at p = pq = 24) run in
 // fixed point on the integer pipe (fixed.cuh), on one scale per target from a first pass over the kernel
 // weights; the FP64 pipe, which bounded the kernel before, keeps the weights themselves (37k operations).
 // 64 drops of degree 24, both kinds: 127 ms by the direct sums, 62 by the symmetries in FP64, now 32.
-constexpr int kProjPairs = 2;
+// Two pairs a pass where they fit a block's shared memory (fewer barriers: 43.8 ms; three or four 46.9 and 45.1), one
+// at the largest degrees.
 
 __device__ inline int tri_index_degree(int it) {
   int n = (int)((sqrtf(8.0f * it + 1.0f) - 1.0f) * 0.5f);
@@ -237,7 +238,7 @@ __device__ __forceinline__ int weight_exponent(double r2, double wx) {
   return fix_exponent(KIND == 0 ? 2.0001 * wx * ri : 6.0001 * wx * ri * (ri * ri));
 }
 
-template <int KIND>
+template <int KIND, int NP>
 __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ cache, int pq, int p,
                                                      const int4* __restrict__ CT, const int2* __restrict__ PT,
                                                      double* __restrict__ Q64) {
@@ -249,8 +250,8 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
   const int mid = half % 2 == 0 ? half / 2 : -1;
   double* sk = reinterpret_cast<double*>(smem_raw);                                  // [pair][row][6][nk]
   int2* si = reinterpret_cast<int2*>(sk);                                            // the folded sums, in place
-  int2* sd = reinterpret_cast<int2*>(sk + kProjPairs * 12 * nk);                     // [pair][even, odd][12][p+1]
-  long long* sq = reinterpret_cast<long long*>(sd + kProjPairs * 24 * (p + 1));      // [12][ntri]
+  int2* sd = reinterpret_cast<int2*>(sk + NP * 12 * nk);                     // [pair][even, odd][12][p+1]
+  long long* sq = reinterpret_cast<long long*>(sd + NP * 24 * (p + 1));      // [12][ntri]
   const long long nq = (long long)nq_j * nk;
   const double* geo = cache + t * 7 * nq;
   for (int i = threadIdx.x; i < 12 * ntri; i += blockDim.x) sq[i] = 0;
@@ -272,8 +273,8 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
   // 2^(56 + log2 k4n), cut by sh bits to below 2^55; the projections (tables 2^-55) 2^(e-52+sh), accumulated with xb more
   // bits (np <= 64: larger grids take the direct form)
   const int sh = ceil_log2(k4n) + 1, xb = 6 - ceil_log2(np);
-  for (int q0 = 0; q0 < np && e < fix_bad; q0 += kProjPairs) {
-    const int qn = min(kProjPairs, np - q0);
+  for (int q0 = 0; q0 < np && e < fix_bad; q0 += NP) {
+    const int qn = min(NP, np - q0);
     for (int i = threadIdx.x; i < qn * 2 * nk; i += blockDim.x) {
       const int row = i / nk, k = i - row * nk;
       const int q = q0 + row / 2, j = row & 1 ? pq - q : q;
@@ -365,16 +366,16 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
     for (int it = threadIdx.x; it < ntri; it += blockDim.x) {
       const int n = tri_index_degree(it);
       const int m = it - n * (n + 1) / 2;
-      int2 P[kProjPairs];
+      int2 P[NP];
 #pragma unroll
-      for (int pair = 0; pair < kProjPairs; ++pair)
+      for (int pair = 0; pair < NP; ++pair)
         P[pair] = pair < qn ? PT[(long long)(q0 + pair) * ntri + it] : make_int2(0, 0);
       const int2* d = sd + (((n - m) & 1) ? 12 : 0) * (p + 1) + m;
 #pragma unroll
       for (int c = 0; c < 12; ++c) {
         long long h = 0, x = 0;
 #pragma unroll
-        for (int pair = 0; pair < kProjPairs; ++pair)
+        for (int pair = 0; pair < NP; ++pair)
           if (pair < qn) fix_mad(h, x, d[(pair * 24 + c) * (p + 1)], P[pair]);
         sq[c * ntri + it] += fix_sum(h, x, xb);
       }
@@ -647,20 +648,28 @@ int launch_self_direct(int kind, const double* dens, const long long* foff3, lon
   return BIE_OK;
 }
 
-size_t kernel_proj_smem(int p, int pq) {
-  return sizeof(double) * ((size_t)kProjPairs * 24 * (pq + 1) + (size_t)kProjPairs * 24 * (p + 1) + 6 * (size_t)(p + 1) * (p + 2));
+constexpr size_t kMaxSmem = 226 * 1024;  // a block's 227 KB less a kernel's own arrays
+
+// dynamic shared memory of k_kernel_proj with np latitude pairs a pass
+static size_t kernel_proj_smem(int p, int pq, int np) {
+  return sizeof(double) * (24 * (size_t)np * (pq + p + 2) + 6 * (size_t)(p + 1) * (p + 2));
 }
+
+// Degrees up to 62 at pq = p and 59 at pq = 2p + 1.  Above, neither the coefficients of one target (rotgeo.cu) nor twice
+// its projected factors fit a block, and the direct form serves as it always has.
+bool self_dense_fits(int p, int pq) { return 8 * (36 * (size_t)(pq + p + 2) + 6 * (size_t)(p + 1) * (p + 2)) <= 227 * 1024; }
 
 int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, int pq, const int4* CT, const int2* PT,
                        double* Q64, cudaStream_t s) {
   if (ntarget == 0) return BIE_OK;
   if (ntarget > 0x7fffffffLL) return BIE_EINVAL;
-  const size_t smem = kernel_proj_smem(p, pq);
-  if (smem > 227 * 1024) {
+  const bool two = kernel_proj_smem(p, pq, 2) <= kMaxSmem;
+  const size_t smem = kernel_proj_smem(p, pq, two ? 2 : 1);
+  if (smem > kMaxSmem) {
     set_error("degree too large for the dense self form (shared memory)");
     return BIE_ENOTSUP;
   }
-  auto kern = kind == 0 ? k_kernel_proj<0> : k_kernel_proj<1>;
+  auto kern = kind == 0 ? (two ? k_kernel_proj<0, 2> : k_kernel_proj<0, 1>) : (two ? k_kernel_proj<1, 2> : k_kernel_proj<1, 1>);
   if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kern<<<(unsigned)ntarget, 256, smem, s>>>(cache, pq, p, CT, PT, Q64);
   count_launch();
