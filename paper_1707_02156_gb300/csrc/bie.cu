@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "dfloat.cuh"
+#include "fixed.cuh"
 #include "interdrop.h"
 #include "near.h"
 #include "offsurface.h"
@@ -284,9 +285,7 @@ const float* Plan::cs_<float>() const {
 
 // v 2^bits as the two parts of fixed.cuh
 static int2 fix_host(double v, int bits) {
-  const long long f = std::llround(std::ldexp(v, bits));
-  const int h = (int)((f + (1LL << 27)) >> 28);
-  return make_int2(h, (int)(f - ((long long)h << 28)));
+  return fix_split(std::llround(std::ldexp(v, bits)));
 }
 
 struct WigPlan {  // rotation blocks for the p+1 latitudes of the degree-p grid

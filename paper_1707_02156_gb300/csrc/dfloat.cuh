@@ -38,10 +38,10 @@ __device__ inline dff& operator+=(dff& a, dff b) { return a = a + b; }
 __device__ inline float fmad(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ inline double fmad(double a, double b, double c) { return ::fma(a, b, c); }
 __device__ inline dff fmad(dff a, dff b, dff c) { return a * b + c; }
-__device__ inline float shfl_down(float v, int off) { return __shfl_down_sync(0xffffffffu, v, off); }
-__device__ inline double shfl_down(double v, int off) { return __shfl_down_sync(0xffffffffu, v, off); }
-__device__ inline dff shfl_down(dff v, int off) {
-  return dff(__shfl_down_sync(0xffffffffu, v.h, off), __shfl_down_sync(0xffffffffu, v.l, off));
+__device__ inline float shfl_xor(float v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
+__device__ inline double shfl_xor(double v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
+__device__ inline dff shfl_xor(dff v, int off) {
+  return dff(__shfl_xor_sync(0xffffffffu, v.h, off), __shfl_xor_sync(0xffffffffu, v.l, off));
 }
 
 }  // namespace bie

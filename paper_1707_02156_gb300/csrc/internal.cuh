@@ -156,7 +156,7 @@ int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, 
 __host__ __device__ inline int self_row(int p) { return ((p + 1) * (p + 1) + 3) & ~3; }
 // Dense factors S[target][6][self_row(p)] of the latitude rows row0 .. row0 + nrow - 1 (row = drop * (p+1) + a)
 // from their projected factors Q (Q64 starts at row0), written at the rows' places in S64 and S32; wblk: the
-// Wigner blocks times 2^54 in fixed point.
+// Wigner blocks times 2^56 in fixed point.
 int launch_unrotate(const double* Q64, long long row0, long long nrow, int p, const int2* wblk, long long wstride,
                     const double* ph, double* S64, float* S32, cudaStream_t s);
 // One degree group of the dense-form apply (device pointers; begin is set by the launcher).

@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(256) k_self_direct(
 // quadruples that share |cos m phi| and |sin m phi|, in place; the phi transform of both rows, whose sum
 // and difference serve even and odd n - m; and the Legendre projection, accumulated in shared memory.
 // The phi transform and the projection (0.15M multiply-adds per target and kind at p = pq = 24) run in
-// fixed point on the integer pipe (fixed.cuh), on one scale per target from a first pass over the kernel
+// fixed point on the integer pipe (fixed.cuh), on one scale per target and entry from a first pass over the kernel
 // weights; the FP64 pipe, which bounded the kernel before, keeps the weights themselves (37k operations).
 // 64 drops of degree 24, both kinds: 127 ms by the direct sums, 62 by the symmetries in FP64, now 32.
 // Two pairs a pass where they fit a block's shared memory (fewer barriers: 43.8 ms; three or four 46.9 and 45.1), one
@@ -230,12 +230,15 @@ __device__ inline int tri_index_degree(int it) {
   return n;
 }
 
-// a bound on the exponent of the six entries at a point: |entry| <= 2 w / r for the Stokeslet and
-// 6 |x.a| / r^3 for the stresslet
+// Bounds on the exponents of a target's six entries, each on a scale of its own (a drop that is thin along an axis has
+// entries of very different size): with a w/r = the Stokeslet's diagonal part and b_i = c x_i^2 (c = w/r^3 or 6 |x.a| /
+// r^5), |entry ij| = c |x_i x_j| < 2^((E(b_i) + E(b_j))/2), E the exponent of the largest over the points (em their magnitudes); the Stokeslet's
+// diagonal entries are below 2 w/r.
 template <int KIND>
-__device__ __forceinline__ int weight_exponent(double r2, double wx) {
-  const double ri = rsqrt_<double>(r2);
-  return fix_exponent(KIND == 0 ? 2.0001 * wx * ri : 6.0001 * wx * ri * (ri * ri));
+__device__ __forceinline__ int entry_exponent(const int* em, int entry) {
+  const int i = entry < 3 ? entry : entry == 5 ? 1 : 0, j = entry < 3 ? entry : entry == 3 ? 1 : 2;
+  const int ei = fix_exponent(em[KIND == 0 && entry < 3 ? 3 : i]), ej = fix_exponent(em[KIND == 0 && entry < 3 ? 3 : j]);
+  return ei == fix_none || ej == fix_none ? 0 : (ei + ej + 1) >> 1;
 }
 
 template <int KIND, int NP>
@@ -243,7 +246,7 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
                                                      const int4* __restrict__ CT, const int2* __restrict__ PT,
                                                      double* __restrict__ Q64) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int emax;
+  __shared__ int em[4], es[6];
   const long long t = blockIdx.x;
   const int nq_j = pq + 1, nk = 2 * pq + 2, half = pq + 1, np = (nq_j + 1) / 2, k4n = half / 2 + 1;
   const int ntri = (p + 1) * (p + 2) / 2;
@@ -255,25 +258,42 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
   const long long nq = (long long)nq_j * nk;
   const double* geo = cache + t * 7 * nq;
   for (int i = threadIdx.x; i < 12 * ntri; i += blockDim.x) sq[i] = 0;
-  if (threadIdx.x == 0) emax = fix_none;
+  if (threadIdx.x < 4) em[threadIdx.x] = 0;
   __syncthreads();
   {
-    int e = fix_none;
+    int e[4] = {0, 0, 0, 0};
     for (int o = threadIdx.x; o < nq; o += blockDim.x) {
       const double x0 = geo[o], x1 = geo[nq + o], x2 = geo[2 * nq + o];
-      const double wx = KIND == 0 ? geo[6 * nq + o] : x0 * geo[3 * nq + o] + x1 * geo[4 * nq + o] + x2 * geo[5 * nq + o];
-      e = max(e, weight_exponent<KIND>(x0 * x0 + x1 * x1 + x2 * x2, wx));
+      const double y0 = x0 * x0, y1 = x1 * x1, y2 = x2 * x2;
+      const double ri = rsqrt_<double>(y0 + y1 + y2), ri2 = ri * ri;
+      double c;
+      if (KIND == 0) {
+        const double d = geo[6 * nq + o] * ri;
+        e[3] = max(e[3], fix_magnitude(2.0001 * d));
+        c = 1.0001 * (d * ri2);
+      } else {
+        c = (6.0001 * (x0 * geo[3 * nq + o] + x1 * geo[4 * nq + o] + x2 * geo[5 * nq + o])) * (ri * (ri2 * ri2));
+      }
+      e[0] = max(e[0], fix_magnitude(c * y0));
+      e[1] = max(e[1], fix_magnitude(c * y1));
+      e[2] = max(e[2], fix_magnitude(c * y2));
     }
-    e = __reduce_max_sync(0xffffffffu, e);
-    if ((threadIdx.x & 31) == 0) atomicMax(&emax, e);
+#pragma unroll
+    for (int k = 0; k < (KIND == 0 ? 4 : 3); ++k) {
+      e[k] = __reduce_max_sync(0xffffffffu, e[k]);
+      if ((threadIdx.x & 31) == 0) atomicMax(&em[k], e[k]);
+    }
   }
   __syncthreads();
-  const int e = emax == fix_none ? 0 : emax;
-  // units: folded sums 2^(e-54), of four entries, below 2^56; their phi transforms (tables 2^-55) 2^(e-53), below
-  // 2^(56 + log2 k4n), cut by sh bits to below 2^55; the projections (tables 2^-55) 2^(e-52+sh), accumulated with xb more
-  // bits (np <= 64: larger grids take the direct form)
-  const int sh = ceil_log2(k4n) + 1, xb = 6 - ceil_log2(np);
-  for (int q0 = 0; q0 < np && e < fix_bad; q0 += NP) {
+  const bool bad = fix_exponent(max(max(em[0], em[1]), max(em[2], em[3]))) == fix_bad;
+  if (threadIdx.x < 6) es[threadIdx.x] = entry_exponent<KIND>(em, threadIdx.x);  // read after the next barriers
+  // units (e the entry's exponent, lk the bits of k4n): entries 2^(e - 61 + lk), folded sums of four below 2^(63 - lk),
+  // which leaves the phi transform (tables 2^-55) room for its k4n products, and below 2^60 (by the bounds' margin of
+  // 1e-4), so that their high parts are 32-bit; the transforms 2^(e - 57 + lk), the sum of two rows' below 2^60 (the
+  // projection adds NP products of it, and no more); the projections (tables 2^-55) 2^(e - 54 + lk - xb) (np <= 64:
+  // larger grids take the direct form)
+  const int lk = max(3, ceil_log2(k4n)), xb = 3 - ceil_log2(np);
+  for (int q0 = 0; q0 < np && !bad; q0 += NP) {
     const int qn = min(NP, np - q0);
     for (int i = threadIdx.x; i < qn * 2 * nk; i += blockDim.x) {
       const int row = i / nk, k = i - row * nk;
@@ -307,7 +327,7 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
     // cosine sums of the even and odd orders at k and half + k, sine sums at 2 half - k and half - k (a middle
     // k has two longitudes: one cosine sum at k, one sine sum at half + k)
     for (int i = threadIdx.x; i < qn * 12 * k4n; i += blockDim.x) {
-      const int k = i % k4n;
+      const int k = i % k4n, e = es[i / k4n % 6] - 4 + lk;  // 57 - e: 61 - lk bits below the entry's scale
       double* v = sk + (i / k4n) * nk;
       int2* w = si + (i / k4n) * nk;
       const long long a = fix_encode(v[k], e), c = fix_encode(v[half + k], e);
@@ -353,14 +373,13 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
           fix_mad(h[1], x[1], v0[6 * nk + mid], make_int2(cs.x, cs.y));
         }
       }
-      const long long re0 = fix_sum(h[0], x[0], 0), re1 = fix_sum(h[1], x[1], 0), im0 = fix_sum(h[2], x[2], 0),
-                      im1 = fix_sum(h[3], x[3], 0);
-      const long long rnd = 1LL << (sh - 1);
+      const long long re0 = fix_sum(h[0], x[0], -1), re1 = fix_sum(h[1], x[1], -1), im0 = fix_sum(h[2], x[2], -1),
+                      im1 = fix_sum(h[3], x[3], -1);
       int2* d = sd + (pair * 24 + 2 * c) * (p + 1) + m;
-      d[0] = fix_split((re0 + re1 + rnd) >> sh);
-      d[p + 1] = fix_split((im0 + im1 + rnd) >> sh);
-      d[12 * (p + 1)] = fix_split((re0 - re1 + rnd) >> sh);
-      d[13 * (p + 1)] = fix_split((im0 - im1 + rnd) >> sh);
+      d[0] = fix_split(re0 + re1);
+      d[p + 1] = fix_split(im0 + im1);
+      d[12 * (p + 1)] = fix_split(re0 - re1);
+      d[13 * (p + 1)] = fix_split(im0 - im1);
     }
     __syncthreads();
     for (int it = threadIdx.x; it < ntri; it += blockDim.x) {
@@ -386,7 +405,7 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
   for (int i = threadIdx.x; i < 12 * ntri; i += blockDim.x) {
     const int it = i % ntri;
     const int n = tri_index_degree(it);
-    const double v = e < fix_bad ? fix_decode(sq[i], e - 52 + sh - xb) : __longlong_as_double(0x7ff8000000000000LL);
+    const double v = bad ? __longlong_as_double(0x7ff8000000000000LL) : fix_decode(sq[i], es[i / ntri / 2] - 54 + lk - xb);
     o64[i] = (it == n * (n + 1) / 2 ? 1.0 : 2.0) * v;  // c_m
   }
 }
@@ -396,7 +415,7 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
 // and -Q_im(n, m) for the imaginary parts of rho'_n^m, and rho' = (C Re g, S Im g), g = e^{i m phi_b} rho,
 // the transposed rotation is s_re = C^T q_re, s_im = S^T q_im and the transposed phase
 // (s_re cos + s_im sin, s_im cos - s_re sin).  The 2n+1 products per entry and coefficient run in fixed point
-// on the integer pipe (fixed.cuh), on one scale per block; two entries at a time share the reads of the
+// on the integer pipe (fixed.cuh), on one scale per longitude and entry; two entries at a time share the reads of the
 // Wigner block, and the leading dimensions of the staged blocks are odd, so that the strided reads of the
 // transposed products hit every bank.  64 drops of p = 24, both kinds: 20 ms in FP64, now 12.
 constexpr int kUnB = 8;
@@ -406,7 +425,7 @@ __global__ void __launch_bounds__(128) k_unrotate(const double* __restrict__ Q64
                                                   const double* __restrict__ ph, int ncp, double* __restrict__ S64,
                                                   float* __restrict__ S32) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int emax;
+  __shared__ int es[kUnB * 6];
   const int nb = 2 * p + 2, nbch = (nb + kUnB - 1) / kUnB;
   const int b0 = (int)(blockIdx.x % nbch) * kUnB;
   const long long row = row0 + blockIdx.x / nbch;  // latitude row of the group: drop * (p+1) + a
@@ -420,35 +439,39 @@ __global__ void __launch_bounds__(128) k_unrotate(const double* __restrict__ Q64
   int2* sq = sS + n * ldS;                        // [bb][e][re 0..n, im 1..n]
   const int2* blk = wblk + (long long)a * wstride + (long long)n * (n + 1) * (2 * n + 1) / 6 +
                     (long long)(n - 1) * n * (2 * n - 1) / 6;
-  if (threadIdx.x == 0) emax = fix_none;
   for (int i = threadIdx.x; i < (n + 1) * (n + 1); i += blockDim.x) sC[(i / (n + 1)) * ldC + i % (n + 1)] = blk[i];
   for (int i = threadIdx.x; i < n * n; i += blockDim.x) sS[(i / n) * ldS + i % n] = blk[(n + 1) * (n + 1) + i];
-  __syncthreads();
-  const int w = 2 * n + 1, nin = nbh * 12 * (n + 1);
+  const int w = 2 * n + 1;
   const double* Qr = Q64 + (row - row0) * nb * 12 * ntri + (long long)b0 * 12 * ntri + t0;
-  {
-    int e = fix_none;
-    for (int i = threadIdx.x; i < nin; i += blockDim.x)
-      e = max(e, fix_exponent(Qr[(long long)(i / (n + 1)) * ntri + i % (n + 1)]));
-    e = __reduce_max_sync(0xffffffffu, e);
-    if ((threadIdx.x & 31) == 0) atomicMax(&emax, e);
+  // a warp per longitude and entry: the 2 (n + 1) factors (at most 4 per lane, see self_dense_fits) and their scale
+  for (int g = threadIdx.x >> 5; g < nbh * 6; g += 4) {
+    const double* Qg = Qr + (long long)g * 2 * ntri;
+    const int lane = threadIdx.x & 31;
+    double v[4];
+    int e = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int k = lane + 32 * u, im = k > n, m = im ? k - (n + 1) : k;
+      v[u] = k < 2 * (n + 1) ? Qg[im * ntri + m] : 0.0;
+      e = max(e, fix_magnitude(v[u]));
+    }
+    e = fix_exponent(__reduce_max_sync(0xffffffffu, e));
+    if (lane == 0) es[g] = e;
+    const bool bad = e == fix_bad;
+    if (e == fix_none) e = 0;
+    int2* q = sq + g * w;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int k = lane + 32 * u;
+      if (k <= n)
+        q[k] = bad ? make_int2(0, 0) : fix_split(fix_encode(v[u], e));
+      else if (k > n + 1 && k < 2 * (n + 1))  // the imaginary parts m = k - (n + 1) > 0, at n + m
+        q[k - 1] = bad ? make_int2(0, 0) : fix_split(-fix_encode(v[u], e));
+    }
   }
   __syncthreads();
-  const bool bad = emax == fix_bad;
-  const int e = emax == fix_none || bad ? 0 : emax;
-  for (int i = threadIdx.x; i < nin; i += blockDim.x) {
-    const int m = i % (n + 1), g = i / (n + 1);
-    const int plane = g % 12, bb = g / 12;
-    const long long v = bad ? 0 : fix_encode(Qr[(long long)g * ntri + m], e);
-    int2* q = sq + (bb * 6 + plane / 2) * w;
-    if (!(plane & 1))
-      q[m] = fix_split(v);
-    else if (m > 0)
-      q[n + m] = fix_split(-v);
-  }
-  __syncthreads();
-  // units: factors 2^(e-54), blocks 2^-56 (up to 2), sums 2^(e-54) with xb more bits: (n+1) 2^55 2^xb <= 2^62
-  const int xb = 7 - ceil_log2(n + 1);
+  // units: factors 2^(e-57), blocks 2^-56 (up to 2), sums 2^(e-55) with xb more bits: (n+1) 2^56 2^xb <= 2^62
+  const int xb = 6 - ceil_log2(n + 1);
   for (int i = threadIdx.x; i < nbh * 3 * (n + 1); i += blockDim.x) {
     const int m = i % (n + 1), g = i / (n + 1) * 2;  // entries g and g + 1 of [bb][e]
     const int2* q = sq + g * w;
@@ -474,8 +497,10 @@ __global__ void __launch_bounds__(128) k_unrotate(const double* __restrict__ Q64
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const double nan = __longlong_as_double(0x7ff8000000000000LL);
-      const double re = bad ? nan : fix_decode(fix_sum(h[u], x[u], xb), e - 54 - xb);
-      const double im = bad ? nan : fix_decode(fix_sum(h[2 + u], x[2 + u], xb), e - 54 - xb);
+      const bool bad = es[g + u] == fix_bad;
+      const int e = es[g + u] == fix_none ? 0 : es[g + u];
+      const double re = bad ? nan : fix_decode(fix_sum(h[u], x[u], xb), e - 55 - xb);
+      const double im = bad ? nan : fix_decode(fix_sum(h[2 + u], x[2 + u], xb), e - 55 - xb);
       const long long o = ((row * nb + b0 + bb) * 6 + en + u) * ncp + n * (n + 1);
       const double vr = m > 0 ? re * co + im * si : re;
       S64[o + m] = vr;
@@ -567,7 +592,7 @@ __global__ void __launch_bounds__(kSelfThreads, 2) k_self_dense(SelfGroups<R> G,
     const int t = t0 + k * (kSelfThreads / 32) + warp;
     if (t >= ng) break;
     const uint4* S = reinterpret_cast<const uint4*>(A.S + (ld * ng + t) * 6 * (long long)ncp);
-    R acc[3] = {R(0), R(0), R(0)};
+    R acc[3] = {R(0), R(0), R(0)}, odd[3] = {R(0), R(0), R(0)};  // FP64 and double-float: the sums of even and odd entries
 #pragma unroll 2
     for (int i = lane; i < nv; i += 32) {
       uint4 s[6], f[3];
@@ -583,21 +608,24 @@ __global__ void __launch_bounds__(kSelfThreads, 2) k_self_dense(SelfGroups<R> G,
         for (int e = 0; e < 6; ++e) q[e] = lane_of<R>(s[e], v);
 #pragma unroll
         for (int c = 0; c < 3; ++c) x[c] = lane_of<R>(f[c], v);
-        sym_mul_add<R>(q, x, sizeof(R) == 4 ? sum : acc);
+        sym_mul_add<R>(q, x, sizeof(R) == 4 ? sum : (v & 1) ? odd : acc);
       }
       if (sizeof(R) == 4)
 #pragma unroll
         for (int c = 0; c < 3; ++c) acc[c] = acc[c] + sum[c];
     }
+    if (sizeof(R) == 8)
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-      for (int off = 16; off > 0; off >>= 1) acc[c] += shfl_down(acc[c], off);
-    if (lane == 0) {
-      double* v = vals + A.val_off[ld] + t;
-      v[0] = A.wts[ld] * (double)acc[0];
-      v[ng] = A.wts[ld] * (double)acc[1];
-      v[2 * ng] = A.wts[ld] * (double)acc[2];
-    }
+      for (int c = 0; c < 3; ++c) acc[c] = acc[c] + odd[c];
+    // the three sums over the lanes in six additions (fifteen one by one, 2 us of an FP64 apply of one drop of degree 16):
+    // the halves of the warp exchange components first, so that lanes 0, 8 and 16 end up with one each
+    const bool up = lane & 16, mid = lane & 8;
+    const R a0 = (up ? acc[2] : acc[0]) + shfl_xor(up ? acc[0] : acc[2], 16);
+    const R a1 = (up ? R(0) : acc[1]) + shfl_xor(up ? acc[1] : R(0), 16);
+    R a = (mid ? a1 : a0) + shfl_xor(mid ? a0 : a1, 8);
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) a = a + shfl_xor(a, off);
+    if (lane % 8 == 0 && lane < 24) vals[A.val_off[ld] + t + (lane / 8) * (long long)ng] = A.wts[ld] * (double)a;
   }
 }
 
