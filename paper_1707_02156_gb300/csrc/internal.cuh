@@ -29,6 +29,16 @@ int ctx_device(const bie_ctx* ctx);  // CUDA device ordinal of a context
     if (s_ != BIE_OK) return s_;   \
   } while (0)
 
+// Dynamic shared memory of a launch above the default 48 KB.  The attribute belongs to the kernel on its device and all
+// threads of the process share it, so every launch sets the same value: with a value per launch, a thread
+// with a smaller degree could lower it between another thread's setting and its launch, which then failed.
+constexpr size_t kMaxSmem = 226 * 1024;  // a block's 227 KB less a kernel's own arrays
+template <typename K>
+cudaError_t allow_smem(K kern, size_t bytes) {
+  if (bytes <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+}
+
 __host__ __device__ inline long long leg_row(int p, int m, int n, int nj) {
   long long before = (long long)m * (p + 1) - (long long)m * (m - 1) / 2;
   return (before + (n - m)) * nj;

@@ -793,7 +793,7 @@ int launch_near_rows(int kind, const NearPair* pairs, const int* list, int n, in
   if (!n) return BIE_OK;
   const size_t smem = near_rows_smem(p, std_.P > up.P ? std_.P : up.P);
   auto kern = kind == 0 ? k_near_rows<0> : k_near_rows<1>;
-  if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  BIE_CUDA_TRY(allow_smem(kern, smem));
   kern<<<n, kNearThreads, smem, s>>>(pairs, list, p, L, pts, grid, centre, hdrop, std_, up, row_off, rows);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());

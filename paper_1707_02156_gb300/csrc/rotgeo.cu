@@ -318,7 +318,7 @@ int launch_rotgeo_fix(const RotGeo& A, long long ndrop, double* cache, cudaStrea
   const bool two = rotgeo_smem(A.p, A.pq, 2) <= 110 * 1024;
   const size_t smem = rotgeo_smem(A.p, A.pq, two ? 2 : 1);
   auto kern = two ? k_rotgeo_fix<2> : k_rotgeo_fix<1>;
-  BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
+  BIE_CUDA_TRY(allow_smem(kern, smem));
   kern<<<(unsigned)n, kGeoThreads, smem, s>>>(A, cache);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());

@@ -668,15 +668,13 @@ int launch_self_direct(int kind, const double* dens, const long long* foff3, lon
   size_t smem;
   const int jc = pick_jc<R>(p, pq, smem_budget, &smem);
   auto kern = kind == 0 ? k_self_direct<R, 0> : k_self_direct<R, 1>;
-  if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  BIE_CUDA_TRY(allow_smem(kern, smem));
   kern<<<(unsigned)nt, 256, smem, s>>>(dens, foff3, p, pq, wblk, wstride, ph, T0, cs, cache, ng, wts, val_off, vals,
                                        jc);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
 }
-
-constexpr size_t kMaxSmem = 226 * 1024;  // a block's 227 KB less a kernel's own arrays
 
 // dynamic shared memory of k_kernel_proj with np latitude pairs a pass
 static size_t kernel_proj_smem(int p, int pq, int np) {
@@ -698,7 +696,7 @@ int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, 
     return BIE_ENOTSUP;
   }
   auto kern = kind == 0 ? (two ? k_kernel_proj<0, 2> : k_kernel_proj<0, 1>) : (two ? k_kernel_proj<1, 2> : k_kernel_proj<1, 1>);
-  if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  BIE_CUDA_TRY(allow_smem(kern, smem));
   kern<<<(unsigned)ntarget, 256, smem, s>>>(cache, pq, p, CT, PT, Q64);
   count_launch();
   BIE_CUDA_TRY(cudaGetLastError());
@@ -711,8 +709,7 @@ int launch_unrotate(const double* Q64, long long row0, long long nrow, int p, co
   const int nbch = (2 * p + 2 + kUnB - 1) / kUnB;
   if (nrow * nbch > 0x7fffffffLL) return BIE_EINVAL;
   const size_t smem = sizeof(double) * ((size_t)(p + 1) * (p + 2) + (size_t)p * (p + 1) + (size_t)kUnB * 6 * (2 * p + 1));
-  if (smem > 48 * 1024)
-    BIE_CUDA_TRY(cudaFuncSetAttribute(k_unrotate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  BIE_CUDA_TRY(allow_smem(k_unrotate, smem));
   k_unrotate<<<dim3((unsigned)(nrow * nbch), p + 1), 128, smem, s>>>(Q64, row0, p, wblk, wstride, ph, self_row(p), S64,
                                                                      S32);
   count_launch();
@@ -744,7 +741,7 @@ int launch_self_dense(std::vector<SelfGroup<R>> groups, const CT* dens, double* 
     if (nblk == 0) continue;
     if (nblk > 0x7fffffffLL) return BIE_EINVAL;
     auto kern = k_self_dense<R, CT>;
-    if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    BIE_CUDA_TRY(allow_smem(kern, smem));
     kern<<<(unsigned)nblk, kSelfThreads, smem, s>>>(G, per_warp, dens, vals);
     count_launch();
     BIE_CUDA_TRY(cudaGetLastError());

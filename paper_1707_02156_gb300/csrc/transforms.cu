@@ -425,7 +425,7 @@ static int synth_launch(const double* coef, std::vector<SynGroup<R>> groups, int
     }
     if (nblk == 0) continue;
     if (nblk > 0x7fffffffLL) return BIE_EINVAL;
-    if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    BIE_CUDA_TRY(allow_smem(kern, smem));
     kern<<<(unsigned)nblk, kSynThreads, smem, s>>>(coef, G);
     count_launch();
     BIE_CUDA_TRY(cudaGetLastError());
@@ -475,7 +475,7 @@ int launch_analyze(std::vector<AnaGroup> groups, const double* grid, double* coe
     G.cl = 1;
     while (!G.orders && G.cl < 8 && (fields * G.cl < 2LL * sms || bytes(G.cl) > 96 * 1024)) G.cl *= 2;
     const size_t smem = bytes(G.cl);
-    if (smem > 227 * 1024) return BIE_EINVAL;
+    if (smem > kMaxSmem) return BIE_EINVAL;
     long long nblk = 0;
     for (int i = 0; i < G.n; ++i) {
       G.g[i].begin = nblk;
@@ -483,7 +483,7 @@ int launch_analyze(std::vector<AnaGroup> groups, const double* grid, double* coe
     }
     if (nblk == 0) continue;
     if (nblk > 0x7fffffffLL) return BIE_EINVAL;
-    if (smem > 48 * 1024) BIE_CUDA_TRY(cudaFuncSetAttribute(k_analyze, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    BIE_CUDA_TRY(allow_smem(k_analyze, smem));
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[2]{};
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -512,11 +512,7 @@ int launch_rotate(const CT* coef, const long long* field_off, int ncomp, long lo
   long long nblk = ndrop * na * (long long)(p + 1) * nbch;
   if (nblk == 0) return BIE_OK;
   size_t smem = sizeof(R) * ((size_t)(p + 1) * (p + 1) + (size_t)p * p + (size_t)kRotB * ncomp * (2 * p + 1));
-  static thread_local bool attr_set[2] = {false, false};
-  if (smem > 48 * 1024 && !attr_set[sizeof(R) == 8]) {
-    BIE_CUDA_TRY(cudaFuncSetAttribute(k_rotate<CT, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    attr_set[sizeof(R) == 8] = true;
-  }
+  BIE_CUDA_TRY(allow_smem(k_rotate<CT, R>, smem));
   if (nblk > 0x7fffffffLL) return BIE_EINVAL;
   k_rotate<CT, R><<<(unsigned)nblk, 128, smem, s>>>(coef, field_off, ncomp, p, blocks, blk_stride, na, nb, ph, out,
                                                     out_drop_stride);

@@ -209,6 +209,39 @@ def test_threads_capture_and_release_beside_one_another(api, case):
             assert relerr(v, ref) < FP64_TOL
 
 
+def test_threads_with_different_degrees(api):
+    # the kernels of the three threads take different amounts of shared memory above the default
+    ps = [26, 40, 54]
+    shapes = [inputs.perturbed_drop(p=p, pq=p, lam=3.0, nmax=6) for p in ps]
+
+    def run(w, n):
+        got = []
+        ctx = api.Context(0)
+        x, f, out = tensors(w)
+        for _ in range(n):
+            geo = ctx.geometry(w.p, w.pq, x, w.lam)
+            for prec in (0, 1, 2):
+                out.fill_(float("nan"))
+                geo.apply_double(f, out, precision=prec)
+                got.append(out.cpu().numpy())
+            geo.close()
+        ctx.close()
+        return got
+
+    ref = [run(w, 1) for w in shapes]
+    got = [None] * len(ps)
+
+    def work(k):
+        def fn(stream):
+            got[k] = run(shapes[k], 8)
+        return fn
+
+    run_all([Worker(work(k)) for k in range(len(ps))])
+    for r, g in zip(ref, got):
+        for i, v in enumerate(g):
+            assert np.array_equal(v, r[i % 3])
+
+
 def test_near_contact_applies_on_a_full_device(api):
     # 12 contacts of 8 drops: the near rule's rows would take 82 MB, more than the device has left after the set-up.
     # Rows and check-point sums are the same sum in another order; the bar is its rounding (some 2^-53 a term), which
