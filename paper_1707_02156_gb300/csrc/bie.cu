@@ -258,9 +258,11 @@ struct Plan {
   int p = 0, P = 0;
   DevBuf<double> T0, T1, T2, At, cs, wsin, wsq;
   DevBuf<float> T0f, csf;
-  DevBuf<int4> CT, CM, CP;  // fixed-point tables of the set-up kernels (P <= 2p+1): see launch_kernel_proj, RotGeo
+  std::vector<double> hT0, hT1, hcs;  // host copies (P <= 2p+1), for the fixed-point tables of the set-up kernels:
+  DevBuf<int4> CT, CM, CP;            // plan_fixed_tables
   DevBuf<int2> PT, LT0, LT1;
   DevBuf<int> t1;
+  bool fixed_ready = false;
   template <typename R>
   const R* T0_() const;
   template <typename R>
@@ -373,41 +375,15 @@ static int get_plan(bie_ctx* ctx, int p, int P, Plan** out) {
   std::unique_ptr<Plan> pl(new Plan());
   pl->p = p;
   pl->P = P;
+  const bool self = P <= 2 * p + 1 && p <= BIE_MAX_P;  // may become the grid of a self rule
   std::vector<double> v;
   legendre_table(p, P, 0, v);
   BIE_TRY(pl->T0.upload(v));
   BIE_TRY(upload_as(pl->T0f, v));
-  if (P <= 2 * p + 1) {  // a self-rule grid
-    const int nh = P / 2 + 1;
-    std::vector<int2> x((size_t)nh * (p + 1) * (p + 2) / 2);
-    for (int n = 0; n <= p; ++n)
-      for (int m = 0; m <= n; ++m)
-        for (int j = 0; j < nh; ++j)
-          x[(size_t)j * (p + 1) * (p + 2) / 2 + n * (n + 1) / 2 + m] = fix_host(v[leg_row(p, m, n, P + 1) + j], 55);
-    BIE_TRY(pl->PT.upload(x));
-    const size_t ntri = (size_t)(p + 1) * (p + 2) / 2;
-    auto diag = [&](int n, int m) { return (size_t)(n - m) * (p + 1) - (n - m) * (n - m - 1) / 2 + m; };
-    std::vector<double> w;
-    legendre_table(p, P, 1, w);
-    std::vector<int> t1(p + 1, 0);
-    std::vector<int2> y(x.size());
-    for (int n = 0; n <= p; ++n) {
-      double mx = 0;
-      for (int m = 0; m <= n; ++m)
-        for (int j = 0; j < nh; ++j) mx = std::max(mx, std::fabs(w[leg_row(p, m, n, P + 1) + j]));
-      while (std::ldexp(mx, -t1[n]) > 2.0) ++t1[n];
-      for (int m = 0; m <= n; ++m)
-        for (int j = 0; j < nh; ++j) {
-          x[j * ntri + diag(n, m)] = fix_host(v[leg_row(p, m, n, P + 1) + j], 56);
-          y[j * ntri + diag(n, m)] = fix_host(w[leg_row(p, m, n, P + 1) + j], 56 - t1[n]);
-        }
-    }
-    BIE_TRY(pl->LT0.upload(x));
-    BIE_TRY(pl->LT1.upload(y));
-    BIE_TRY(pl->t1.upload(t1));
-  }
+  if (self) pl->hT0 = v;
   legendre_table(p, P, 1, v);
   BIE_TRY(pl->T1.upload(v));
+  if (self) pl->hT1 = v;
   legendre_table(p, P, 2, v);
   BIE_TRY(pl->T2.upload(v));
   analysis_table(p, P, v);
@@ -421,31 +397,8 @@ static int get_plan(bie_ctx* ctx, int p, int P, Plan** out) {
   }
   phase_table(p, P, v);
   BIE_TRY(pl->cs.upload(v));
-  if (P <= 2 * p + 1) {
-    const int kn = (P + 1) / 2 + 1, nk = 2 * P + 2;
-    std::vector<int4> x((size_t)kn * (p + 1));
-    for (int k = 0; k < kn; ++k)
-      for (int m = 0; m <= p; ++m) {
-        const int2 c = fix_host(v[((size_t)m * nk + k) * 2], 55), sn = fix_host(v[((size_t)m * nk + k) * 2 + 1], 55);
-        x[(size_t)k * (p + 1) + m] = make_int4(c.x, c.y, sn.x, sn.y);
-      }
-    BIE_TRY(pl->CT.upload(x));
-    std::vector<int4> y(x.size());
-    for (int m = 0; m <= p; ++m) {
-      int tm = 0;
-      while ((2 << tm) <= m) ++tm;
-      for (int k = 0; k < kn; ++k) {
-        const double* cs = &v[((size_t)m * nk + k) * 2];
-        const int2 c = fix_host(cs[0], 56), sn = fix_host(cs[1], 56);
-        x[(size_t)m * kn + k] = make_int4(c.x, c.y, sn.x, sn.y);
-        const int2 cm = fix_host(cs[0] * m, 55 - tm), sm = fix_host(cs[1] * m, 55 - tm);
-        y[(size_t)m * kn + k] = make_int4(cm.x, cm.y, sm.x, sm.y);
-      }
-    }
-    BIE_TRY(pl->CM.upload(x));
-    BIE_TRY(pl->CP.upload(y));
-  }
   BIE_TRY(upload_as(pl->csf, v));
+  if (self) pl->hcs = v;
   std::vector<double> t, w, ws;
   gauss_legendre(P + 1, t, w);
   singular_weights(P, ws);
@@ -459,6 +412,58 @@ static int get_plan(bie_ctx* ctx, int p, int P, Plan** out) {
   BIE_TRY(pl->wsq.upload(wsq));
   *out = pl.get();
   ctx->plans[key] = std::move(pl);
+  return BIE_OK;
+}
+
+// The fixed-point tables (see launch_kernel_proj, RotGeo) of the plan of a self rule, made at its first set-up: no other
+// plan reads them.
+static int plan_fixed_tables(bie_ctx* ctx, Plan* pl) {
+  std::lock_guard<std::mutex> lk(ctx->mu);
+  if (pl->fixed_ready) return BIE_OK;
+  const int p = pl->p, P = pl->P, nh = P / 2 + 1, kn = (P + 1) / 2 + 1, nk = 2 * P + 2;
+  const size_t ntri = (size_t)(p + 1) * (p + 2) / 2;
+  auto diag = [&](int n, int m) { return (size_t)(n - m) * (p + 1) - (n - m) * (n - m - 1) / 2 + m; };
+  const std::vector<double>&v = pl->hT0, &w = pl->hT1, &cs = pl->hcs;
+  {
+    std::vector<int2> PT(nh * ntri), LT0(nh * ntri), LT1(nh * ntri);
+    std::vector<int> t1(p + 1, 0);
+    for (int n = 0; n <= p; ++n) {
+      double mx = 0;
+      for (int m = 0; m <= n; ++m)
+        for (int j = 0; j < nh; ++j) mx = std::max(mx, std::fabs(w[leg_row(p, m, n, P + 1) + j]));
+      while (std::ldexp(mx, -t1[n]) > 2.0) ++t1[n];
+      for (int m = 0; m <= n; ++m)
+        for (int j = 0; j < nh; ++j) {
+          const long long at = leg_row(p, m, n, P + 1) + j;
+          PT[j * ntri + n * (n + 1) / 2 + m] = fix_host(v[at], 55);
+          LT0[j * ntri + diag(n, m)] = fix_host(v[at], 56);
+          LT1[j * ntri + diag(n, m)] = fix_host(w[at], 56 - t1[n]);
+        }
+    }
+    BIE_TRY(pl->PT.upload(PT));
+    BIE_TRY(pl->LT0.upload(LT0));
+    BIE_TRY(pl->LT1.upload(LT1));
+    BIE_TRY(pl->t1.upload(t1));
+  }
+  std::vector<int4> CT((size_t)kn * (p + 1)), CM(CT.size()), CP(CT.size());
+  auto pair = [](double a, double b, int bits) {
+    const int2 x = fix_host(a, bits), y = fix_host(b, bits);
+    return make_int4(x.x, x.y, y.x, y.y);
+  };
+  for (int m = 0; m <= p; ++m) {
+    int tm = 0;
+    while ((2 << tm) <= m) ++tm;
+    for (int k = 0; k < kn; ++k) {
+      const double c = cs[((size_t)m * nk + k) * 2], s = cs[((size_t)m * nk + k) * 2 + 1];
+      CT[(size_t)k * (p + 1) + m] = pair(c, s, 55);
+      CM[(size_t)m * kn + k] = pair(c, s, 56);
+      CP[(size_t)m * kn + k] = pair(c * m, s * m, 55 - tm);
+    }
+  }
+  BIE_TRY(pl->CT.upload(CT));
+  BIE_TRY(pl->CM.upload(CM));
+  BIE_TRY(pl->CP.upload(CP));
+  pl->fixed_ready = true;
   return BIE_OK;
 }
 
@@ -901,6 +906,7 @@ static int setup_self(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, DevBuf<doub
   Plan *pl, *pp;
   WigPlan* wp;
   BIE_TRY(get_plan(ctx, p, pq, &pl));
+  BIE_TRY(plan_fixed_tables(ctx, pl));
   BIE_TRY(get_plan(ctx, p, p, &pp));
   BIE_TRY(get_wig(ctx, p, &wp));
   // doubles per target: where the cache is not made in one kernel (degrees above 62), rotated coefficients, x
