@@ -49,6 +49,8 @@ static const double kPi = 3.14159265358979323846;
 // that the driver keeps their page), not a cudaDeviceSynchronize: other threads' streams may be in a graph capture
 // (the library's own, or a caller's), which a device-wide synchronisation breaks and which makes it fail.  When the
 // wait fails all the same (a capture in global mode forbids cudaFree too), the buffers stay held.
+//
+// Where a pool cannot be made, the buffers come from cudaMalloc and go back by cudaFree, which waits by itself.
 struct DevPool {
   std::once_flag once;
   cudaError_t err = cudaSuccess;
@@ -87,6 +89,8 @@ static cudaError_t make_marker(DevPool& P) {
   return cudaSuccess;
 }
 
+static cudaError_t recycle(DevPool& P, void* ptr) { return P.pool ? cudaFreeAsync(ptr, P.stream) : cudaFree(ptr); }
+
 // Waits for everything on the device; buffers held by then return to the pool.
 static cudaError_t device_wait(int dev) {
   DevPool& P = g_pools[dev];
@@ -119,24 +123,34 @@ static cudaError_t device_wait(int dev) {
     P.held.insert(P.held.end(), held.begin(), held.end());
     return e;
   }
-  for (void* p : held) cudaFreeAsync(p, P.stream);
+  for (void* p : held) recycle(P, p);
   return cudaSuccess;
 }
 
 static cudaError_t pool_init(DevPool& P, int dev) {
+  OnDevice on(dev);
+  cudaError_t e = cudaStreamCreateWithFlags(&P.stream, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return e;
   cudaMemPoolProps props{};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
   props.location.id = dev;
-  cudaError_t e = cudaMemPoolCreate(&P.pool, &props);
-  if (e != cudaSuccess) return e;
-  cudaDeviceProp prop;
-  if ((e = cudaGetDeviceProperties(&prop, dev)) != cudaSuccess) return e;
-  unsigned long long keep = prop.totalGlobalMem / 16;
-  if ((e = cudaMemPoolSetAttribute(P.pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) return e;
-  OnDevice on(dev);
+  size_t avail = 0, total = 0;
+  if ((e = cudaMemGetInfo(&avail, &total)) != cudaSuccess) return e;
+  unsigned long long keep = total / 16;
+  cudaMemPool_t pool = nullptr;
+  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+    cudaGetLastError();
+    return cudaSuccess;  // without a pool
+  }
+  if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    cudaGetLastError();
+    cudaMemPoolDestroy(pool);
+    return cudaSuccess;
+  }
+  P.pool = pool;
   make_marker(P);
-  return cudaStreamCreateWithFlags(&P.stream, cudaStreamNonBlocking);
+  return cudaSuccess;
 }
 
 // wait: until the buffer is ready for any stream (else for the pool's own)
@@ -154,8 +168,8 @@ static cudaError_t dev_malloc(void** ptr, size_t bytes, int* device, bool wait) 
     held = !P.held.empty();
   }
   if (held) device_wait(dev);
-  e = cudaMallocFromPoolAsync(ptr, bytes, P.pool, P.stream);
-  if (e == cudaErrorMemoryAllocation) {
+  e = P.pool ? cudaMallocFromPoolAsync(ptr, bytes, P.pool, P.stream) : cudaMalloc(ptr, bytes);
+  if (e == cudaErrorMemoryAllocation && P.pool) {
     cudaGetLastError();  // not sticky
     cudaStreamSynchronize(P.stream);
     cudaMemPoolTrimTo(P.pool, 0);
@@ -172,9 +186,9 @@ static thread_local int g_idle_device = -1;
 
 static void dev_free(void* ptr, size_t bytes, int dev) {
   DevPool& P = g_pools[dev];
-  if (g_idle_device == dev) {
-    cudaFreeAsync(ptr, P.stream);
-    return;
+  if (g_idle_device == dev || !P.pool) {  // waited for, or cudaFree waits
+    if (recycle(P, ptr) == cudaSuccess) return;
+    cudaGetLastError();
   }
   bool full;
   {
@@ -197,10 +211,10 @@ struct IdleDevice {
 static void pool_add_context(int dev, int n) {
   if (dev < 0 || dev >= kMaxDevices) return;
   DevPool& P = g_pools[dev];
-  if (P.contexts.fetch_add(n) + n > 0 || !P.pool) return;
+  if (P.contexts.fetch_add(n) + n > 0 || !P.stream) return;
   device_wait(dev);  // the buffers held
   cudaStreamSynchronize(P.stream);
-  cudaMemPoolTrimTo(P.pool, 0);
+  if (P.pool) cudaMemPoolTrimTo(P.pool, 0);
 }
 
 template <typename T>
