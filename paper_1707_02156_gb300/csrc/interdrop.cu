@@ -247,6 +247,11 @@ __device__ __forceinline__ fx2 x2_pack(float lo, float hi) {
 __device__ __forceinline__ void x2_unpack(fx2 v, float& lo, float& hi) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
 }
+__device__ __forceinline__ fx2 x2_add(fx2 a, fx2 b) {
+  fx2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 __device__ __forceinline__ fx2 x2_sub(fx2 a, fx2 b) {
   fx2 d;
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -269,6 +274,10 @@ __device__ __forceinline__ fx2 x2_rsqrt(fx2 v) {
 }
 
 constexpr int kChunkX2 = 64;  // sources staged per pass of the packed kernel
+// Sources per FP32 sum.  One sum per item (up to 4096 terms) was less accurate than the scalar kernel's, since the packed
+// form adds the two parts of a Stokeslet to it one by one: velocity at points among 64 drops of degree 24 3.4e-8
+// (scalar, the tuned variant there once) and 3.7e-8, now 2.7e-8 at the same time (256 sources: 2.5e-8, 0.3 % slower).
+constexpr int kFlushX2 = 512;
 
 // Staged source of the packed kernel: each value duplicated into both lanes, in the order
 // x, y, z, q0, q1, q2, n0, n1, n2 (and one pad), read with 128-bit shared-memory loads (three for
@@ -279,9 +288,8 @@ struct alignas(16) SrcRecX2 {
 
 // Same work list, layout and result as k_interdrop<float, KIND, TPT>; TPT even, the thread's
 // targets tid + u * (128/TPT) taken two by two (u = 2w, 2w + 1 share lane pair w).  The tile's target
-// coordinates (FP32, relative to their drop's centre) and the FP64 accumulators live in shared
-// memory, not in registers, so that more warps fit per SM; the source loop takes two sources per iteration (2 x TPT/2 independent
-// chains per thread).  PF = 1 software-pipelines the staging: the next chunk's sources are loaded
+// coordinates and the FP64 accumulators live in shared memory, not in registers, so that more warps fit per SM; the
+// source loop takes two sources per iteration (2 x TPT/2 independent chains per thread).  PF = 1 software-pipelines the staging: the next chunk's sources are loaded
 // into registers while the current chunk is summed, so the global-memory latency of the staging
 // overlaps the arithmetic.
 template <int KIND, int TPT, int PF, int CH = kChunkX2>
@@ -300,7 +308,7 @@ __global__ void __launch_bounds__(kTile / TPT) k_interdrop_x2(
   static_assert(CH % NT == 0 && CH >= NT, "a chunk is a whole number of sources per thread");
   constexpr int RPT = CH / NT;  // staged sources per thread and chunk
   __shared__ SrcRecX2 src[CH];
-  __shared__ float tgt[3][kTile];   // the tile's targets relative to their own drop's centre (FP32)
+  __shared__ double tgt[3][kTile];  // the tile's targets
   __shared__ double acc[3][kTile];  // per-target sums over the block's items
   const int b = blockIdx.x;
   const int it0 = blk_item[b], it1 = blk_item[b + 1];
@@ -308,24 +316,15 @@ __global__ void __launch_bounds__(kTile / TPT) k_interdrop_x2(
   const int tid = threadIdx.x;
   const int nt = tile_n[tile];
   const int di = tile_drop[tile];
-  const double ox = centre[3 * di], oy = centre[3 * di + 1], oz = centre[3 * di + 2];
   {
     const long long ng = ngd[di];
     const double* ri = rec_std + 7 * toff_std[di];
     for (int k = tid; k < kTile; k += NT) {
-      double x = ox, y = oy, z = oz;
-      if (k < nt) {
-        const long long l = tgt_loc[tile_t0[tile] + k];
-        x = ri[l];
-        y = ri[ng + l];
-        z = ri[2 * ng + l];
+      const long long l = tgt_loc[tile_t0[tile] + (k < nt ? k : 0)];
+      for (int c = 0; c < 3; ++c) {
+        tgt[c][k] = ri[c * ng + l];
+        acc[c][k] = 0.0;
       }
-      // |x - o| is about a drop radius, so its FP32 rounding (2^-24 of it) is far below that of the
-      // target's position relative to a source drop's centre, which the pair sums round to FP32 anyway
-      tgt[0][k] = (float)(x - ox);
-      tgt[1][k] = (float)(y - oy);
-      tgt[2][k] = (float)(z - oz);
-      acc[0][k] = acc[1][k] = acc[2][k] = 0.0;
     }
   }
   // the block's shared arrays are written before any thread reads them (the first staging barrier
@@ -373,15 +372,15 @@ __global__ void __launch_bounds__(kTile / TPT) k_interdrop_x2(
       const int k = tid + u * NT;
       if (k < nt && ((items[it].mask[k >> 5] >> (k & 31)) & 1u)) act |= 1u << u;
     }
-    // target relative to the source drop's centre: (x - o) + (o - c_j), the offset in FP64
-    const double cx = ox - centre[3 * j], cy = oy - centre[3 * j + 1], cz = oz - centre[3 * j + 2];
+    // targets relative to the source drop's centre, rounded to FP32 once
+    const double cx = centre[3 * j], cy = centre[3 * j + 1], cz = centre[3 * j + 2];
     fx2 px[NW], py[NW], pz[NW], s[NW][3];
 #pragma unroll
     for (int w = 0; w < NW; ++w) {
       const int k0 = tid + 2 * w * NT, k1 = k0 + NT;
-      px[w] = x2_pack((float)((double)tgt[0][k0] + cx), (float)((double)tgt[0][k1] + cx));
-      py[w] = x2_pack((float)((double)tgt[1][k0] + cy), (float)((double)tgt[1][k1] + cy));
-      pz[w] = x2_pack((float)((double)tgt[2][k0] + cz), (float)((double)tgt[2][k1] + cz));
+      px[w] = x2_pack((float)(tgt[0][k0] - cx), (float)(tgt[0][k1] - cx));
+      py[w] = x2_pack((float)(tgt[1][k0] - cy), (float)(tgt[1][k1] - cy));
+      pz[w] = x2_pack((float)(tgt[2][k0] - cz), (float)(tgt[2][k1] - cz));
       s[w][0] = s[w][1] = s[w][2] = 0ull;  // +0.0f in both lanes
     }
     const int grid = items[it].grid;
@@ -390,6 +389,22 @@ __global__ void __launch_bounds__(kTile / TPT) k_interdrop_x2(
     const float* Q = grid ? Qu : Qs;
     const long long ld = grid ? nup : nstd;
     const long long s0 = items[it].s0, s1 = items[it].s1;
+    // the FP32 sums go to the FP64 ones of the block after every kFlushX2 sources
+    const double wj = KIND ? -6.0 * wts[j] : wts[j];
+    auto flush = [&]() {
+#pragma unroll
+      for (int w = 0; w < NW; ++w) {
+        const int k0 = tid + 2 * w * NT, k1 = k0 + NT;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          float lo, hi;
+          x2_unpack(s[w][c], lo, hi);
+          if (act & (1u << (2 * w))) acc[c][k0] += wj * (double)lo;
+          if (act & (1u << (2 * w + 1))) acc[c][k1] += wj * (double)hi;
+          s[w][c] = 0ull;
+        }
+      }
+    };
     float pre[RPT][NV];
     if (PF) load_chunk(pre, X, N, Q, ld, s0, s1);
     for (long long c0 = s0; c0 < s1; c0 += CH) {
@@ -432,21 +447,11 @@ __global__ void __launch_bounds__(kTile / TPT) k_interdrop_x2(
             }
           }
         }
+        if ((c0 - s0) % kFlushX2 == kFlushX2 - CH) flush();
       }
       __syncthreads();
     }
-    const double wj = KIND ? -6.0 * wts[j] : wts[j];
-#pragma unroll
-    for (int w = 0; w < NW; ++w) {
-      const int k0 = tid + 2 * w * NT, k1 = k0 + NT;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        float lo, hi;
-        x2_unpack(s[w][c], lo, hi);
-        if (act & (1u << (2 * w))) acc[c][k0] += wj * (double)lo;
-        if (act & (1u << (2 * w + 1))) acc[c][k1] += wj * (double)hi;
-      }
-    }
+    flush();
   }
   double* pp = partial + (long long)b * 3 * kTile;
 #pragma unroll
@@ -478,11 +483,6 @@ struct df2 {
   float h, l;
 };
 
-__device__ __forceinline__ fx2 x2_add(fx2 a, fx2 b) {
-  fx2 d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
 __device__ __forceinline__ fx2 x2_neg(fx2 a) { return a ^ 0x8000000080000000ull; }
 __device__ __forceinline__ fx2 x2_both(float v) { return x2_pack(v, v); }
 __device__ inline df2 df_from(double x) {
