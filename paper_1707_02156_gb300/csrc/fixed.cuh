@@ -36,9 +36,9 @@ __device__ __forceinline__ void fix_mad(long long& h, long long& x, int2 a, int2
   x += (long long)a.x * b.y;
   x += (long long)a.y * b.x;
 }
-// (h + x 2^-29) 2^extra as an integer, extra < 29: the sum in units of 2^(58 - extra) of its products'
+// (h + x 2^-29) 2^extra as an integer, 0 <= extra < 29: the sum in units of 2^(58 - extra) of its products'; half of it
+__device__ __forceinline__ long long fix_half(long long h, long long x) { return (h + (x >> kFixPart) + 1) >> 1; }
 __device__ __forceinline__ long long fix_sum(long long h, long long x, int extra) {
-  if (extra < 0) return (h + (x >> kFixPart) + (1LL << (-extra - 1))) >> -extra;
   return (h << extra) + ((x + (1LL << (kFixPart - 1 - extra))) >> (kFixPart - extra));
 }
 // r 2^u; zero below the normal numbers, infinite above the largest

@@ -55,7 +55,7 @@ __device__ __forceinline__ void block_max(int v, int* out) {
 }
 
 template <int JP>
-__global__ void __launch_bounds__(kGeoThreads) k_rotgeo_fix(RotGeo A, double* __restrict__ cache) {
+__global__ void __launch_bounds__(kGeoThreads, 3) k_rotgeo_fix(RotGeo A, double* __restrict__ cache) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // exponents per component: of the largest coefficient, per table, and per kind in a pass; en: by degree
   __shared__ int emax, bits[2][3], kbits[3][3], en[3][kMaxDeg + 1];

@@ -262,6 +262,7 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
   __syncthreads();
   {
     int e[4] = {0, 0, 0, 0};
+#pragma unroll 2
     for (int o = threadIdx.x; o < nq; o += blockDim.x) {
       const double x0 = geo[o], x1 = geo[nq + o], x2 = geo[2 * nq + o];
       const double y0 = x0 * x0, y1 = x1 * x1, y2 = x2 * x2;
@@ -290,9 +291,10 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
   // units (e the entry's exponent, lk the bits of k4n): entries 2^(e - 61 + lk), folded sums of four below 2^(63 - lk),
   // which leaves the phi transform (tables 2^-55) room for its k4n products, and below 2^60 (by the bounds' margin of
   // 1e-4), so that their high parts are 32-bit; the transforms 2^(e - 57 + lk), the sum of two rows' below 2^60 (the
-  // projection adds NP products of it, and no more); the projections (tables 2^-55) 2^(e - 54 + lk - xb) (np <= 64:
+  // projection adds NP products of it, and no more); the projections (tables 2^-55) 2^(e - 54 + lk + sf) (np <= 64:
   // larger grids take the direct form)
-  const int lk = max(3, ceil_log2(k4n)), xb = 3 - ceil_log2(np);
+  const int lk = max(3, ceil_log2(k4n)), sf = max(0, ceil_log2(np) - 3);
+  const long long rnd = sf > 0 ? 1LL << (sf - 1) : 0, xrnd = sf > 0 ? 0 : 1LL << (kFixPart - 1);  // unbiased
   for (int q0 = 0; q0 < np && !bad; q0 += NP) {
     const int qn = min(NP, np - q0);
     for (int i = threadIdx.x; i < qn * 2 * nk; i += blockDim.x) {
@@ -373,8 +375,8 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
           fix_mad(h[1], x[1], v0[6 * nk + mid], make_int2(cs.x, cs.y));
         }
       }
-      const long long re0 = fix_sum(h[0], x[0], -1), re1 = fix_sum(h[1], x[1], -1), im0 = fix_sum(h[2], x[2], -1),
-                      im1 = fix_sum(h[3], x[3], -1);
+      const long long re0 = fix_half(h[0], x[0]), re1 = fix_half(h[1], x[1]), im0 = fix_half(h[2], x[2]),
+                      im1 = fix_half(h[3], x[3]);
       int2* d = sd + (pair * 24 + 2 * c) * (p + 1) + m;
       d[0] = fix_split(re0 + re1);
       d[p + 1] = fix_split(im0 + im1);
@@ -396,7 +398,7 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
 #pragma unroll
         for (int pair = 0; pair < NP; ++pair)
           if (pair < qn) fix_mad(h, x, d[(pair * 24 + c) * (p + 1)], P[pair]);
-        sq[c * ntri + it] += fix_sum(h, x, xb);
+        sq[c * ntri + it] += (h + ((x + xrnd) >> kFixPart) + rnd) >> sf;
       }
     }
     __syncthreads();
@@ -405,7 +407,7 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
   for (int i = threadIdx.x; i < 12 * ntri; i += blockDim.x) {
     const int it = i % ntri;
     const int n = tri_index_degree(it);
-    const double v = bad ? __longlong_as_double(0x7ff8000000000000LL) : fix_decode(sq[i], es[i / ntri / 2] - 54 + lk - xb);
+    const double v = bad ? __longlong_as_double(0x7ff8000000000000LL) : fix_decode(sq[i], es[i / ntri / 2] - 54 + lk + sf);
     o64[i] = (it == n * (n + 1) / 2 ? 1.0 : 2.0) * v;  // c_m
   }
 }
@@ -443,30 +445,40 @@ __global__ void __launch_bounds__(128) k_unrotate(const double* __restrict__ Q64
   for (int i = threadIdx.x; i < n * n; i += blockDim.x) sS[(i / n) * ldS + i % n] = blk[(n + 1) * (n + 1) + i];
   const int w = 2 * n + 1;
   const double* Qr = Q64 + (row - row0) * nb * 12 * ntri + (long long)b0 * 12 * ntri + t0;
-  // a warp per longitude and entry: the 2 (n + 1) factors (at most 4 per lane, see self_dense_fits) and their scale
-  for (int g = threadIdx.x >> 5; g < nbh * 6; g += 4) {
-    const double* Qg = Qr + (long long)g * 2 * ntri;
-    const int lane = threadIdx.x & 31;
-    double v[4];
-    int e = 0;
+  // a warp per longitude and entry, three of them in flight: the 2 (n + 1) factors (at most 4 per lane, see
+  // self_dense_fits) and their scale
+  constexpr int kFly = 3;
+  const int lane = threadIdx.x & 31, ngr = nbh * 6;
+  for (int g0 = threadIdx.x >> 5; g0 < ngr; g0 += 4 * kFly) {
+    double v[kFly][4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int k = lane + 32 * u, im = k > n, m = im ? k - (n + 1) : k;
-      v[u] = k < 2 * (n + 1) ? Qg[im * ntri + m] : 0.0;
-      e = max(e, fix_magnitude(v[u]));
-    }
-    e = fix_exponent(__reduce_max_sync(0xffffffffu, e));
-    if (lane == 0) es[g] = e;
-    const bool bad = e == fix_bad;
-    if (e == fix_none) e = 0;
-    int2* q = sq + g * w;
+    for (int r = 0; r < kFly; ++r)
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int k = lane + 32 * u;
-      if (k <= n)
-        q[k] = bad ? make_int2(0, 0) : fix_split(fix_encode(v[u], e));
-      else if (k > n + 1 && k < 2 * (n + 1))  // the imaginary parts m = k - (n + 1) > 0, at n + m
-        q[k - 1] = bad ? make_int2(0, 0) : fix_split(-fix_encode(v[u], e));
+      for (int u = 0; u < 4; ++u) {
+        const int g = g0 + 4 * r, k = lane + 32 * u, im = k > n, m = im ? k - (n + 1) : k;
+        v[r][u] = g < ngr && k < 2 * (n + 1) ? Qr[(2LL * g + im) * ntri + m] : 0.0;
+      }
+#pragma unroll
+    for (int r = 0; r < kFly; ++r) {
+      const int g = g0 + 4 * r;
+      if (g >= ngr) break;
+      int e = 0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) e = max(e, fix_magnitude(v[r][u]));
+      e = fix_exponent(__reduce_max_sync(0xffffffffu, e));
+      if (lane == 0) es[g] = e;
+      const bool bad = e == fix_bad;
+      if (e == fix_none) e = 0;
+      int2* q = sq + g * w;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (32 * u >= 2 * (n + 1)) break;
+        const int k = lane + 32 * u;
+        if (k <= n)
+          q[k] = bad ? make_int2(0, 0) : fix_split(fix_encode(v[r][u], e));
+        else if (k > n + 1 && k < 2 * (n + 1))  // the imaginary parts m = k - (n + 1) > 0, at n + m
+          q[k - 1] = bad ? make_int2(0, 0) : fix_split(-fix_encode(v[r][u], e));
+      }
     }
   }
   __syncthreads();
