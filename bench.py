@@ -6,10 +6,9 @@ amplitude 0.1 (degrees 2..8), SH degree p = 24, upsampling factor 2 for the inte
 interfacial force of a random decaying surfactant with sigma = 1 - 0.2 Gamma.
 
 One step = the right-hand side 2 u_inf + S[f] (double-float: FP64-grade) and the mixed-precision
-solve of (lambda + 1) u - D[u] = b: FP32 inner GMRES (FP32 rotation, contraction and pair sums)
+solve of (lambda + 1) u - D[u] = b: FP32 inner GMRES (FP32 self contraction, sources and pair sums)
 inside iterative refinement with double-float residuals, to a relative residual of 1e-10.  Every
-row of the hot path runs in each step: Wigner rotation and contraction of the singular self term,
-source synthesis, inter-drop pair sums by region, Galerkin projection, Krylov kernels.
+row of the hot path runs in each step: contraction of the singular self term, source synthesis, inter-drop pair sums by region, Galerkin projection, Krylov kernels.
 value = Stokes pair interactions evaluated per second: (self-rule + regular + upsampled +
 near-singular pairs of one operator apply) x (operator applies in the step) / step time.
 
@@ -17,7 +16,8 @@ near-singular pairs of one operator apply) x (operator applies in the step) / st
                   [--no-aux] [--timesteps N] [--fp64-solve] [--tensor-rotation] [--coupled c4|c5]
 
 --impl reference times the FP64 CPU oracle on a bounded sample of the same workload, on the host's
-cores.  The other configurations (c1 .. c4) are reported under "also" unless --no-aux.
+cores.  The other configurations (c1 .. c4) are reported under "also" unless --no-aux; the full records
+(phases, set-up, residuals) go to stderr as a second JSON line.
 """
 from __future__ import annotations
 
@@ -52,19 +52,13 @@ WORKLOADS = {
 STEP = ("rhs 2 u_inf + S[f] (double-float S apply) + mixed solve: FP32 inner GMRES inside refinement with "
         "double-float residuals, tol 1e-10")
 
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of a kernel on a workload,
-# from one ncu capture, with the SHA-256 prefix of the kernel's source file at the time of the
-# capture: a capture of an older version of the kernel is not reported (traffic null).
 # bie_config.tensor_rotation of every context the bench makes (--tensor-rotation)
 TENSOR_ROTATION = False
 
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of a kernel on a workload,
+# from one ncu capture, with the SHA-256 prefix of the kernel's source file at the time of the
+# capture: a capture of an older version of the kernel is not reported (traffic null).
 PROFILED_TRAFFIC = {
-    # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum -k regex:k_interdrop_x2
-    #     -s 16 -c 1 python bench.py --no-aux --steps 1 --warmup 3   (one pass; 183.82 MB read, 132.60 MB written)
-    ("interdrop_f32", "c5"): {"bytes": 316.42e6, "source": "interdrop.cu", "sha": "3d31e48d7720c587"},
-    # ncu --set full --kernel-name-base demangled -k regex:"k_self_proj<float" -s 4 -c 1
-    #     python bench.py --workload c2 --no-aux --steps 1 --warmup 3   (60.35 MB read, 0.70 MB written)
-    ("self_proj_f32", "c2"): {"bytes": 61.05e6, "source": "self.cu", "sha": "ea9853933df42712"},
 }
 
 
@@ -891,6 +885,12 @@ def run_reference(args):
     }))
 
 
+def brief(rec):
+    """The headline numbers of an auxiliary record (the whole record goes to stderr)."""
+    keys = ("ms_per_step", "value", "fp64_us", "mixed_us", "ms_mixed", "ms_fp64", "error")
+    return {k: rec[k] for k in keys if k in rec} if isinstance(rec, dict) else rec
+
+
 def run_ours(args):
     import torch
 
@@ -941,10 +941,12 @@ def run_ours(args):
         "clocks": head.get("clocks"),
         "cpu_baseline": cpu,
         "peaks": {"alu_tflops_measured": peaks, "hbm_gbs": bw, "hbm_source": bw_src},
-        "detail": {k: v for k, v in head.items() if k not in ("e2e", "roofline", "clocks", "value", "gpu_launches")},
-        "also": also,
+        "also": {k: brief(v) for k, v in also.items()},
     }
     if rank == 0:
+        # the full records go to stderr: a reader that keeps the last few KB of stdout gets the whole line
+        detail = {k: v for k, v in head.items() if k not in ("e2e", "roofline", "clocks", "value", "gpu_launches")}
+        print(json.dumps({"detail": detail, "also": also}), file=sys.stderr)
         print(json.dumps(res))
     if world > 1:
         torch.distributed.destroy_process_group()
