@@ -52,7 +52,9 @@ enum bie_status {
 
 /* precision flags (the low byte), OR-able with BIE_RAW */
 #define BIE_FP64 0   /* every step in double precision */
-#define BIE_MIXED 1  /* rotation, synthesis and pair sums in FP32; geometry, analysis in FP64 */
+#define BIE_MIXED 1  /* the contraction of the singular self term (dense form; rotation and synthesis in the
+                        direct one), the synthesis of the sources and the pair sums in FP32; geometry, the
+                        near-singular step and the analysis in FP64 */
 #define BIE_DF 2     /* the contraction of the singular self term (dense form) and the
                         inter-drop pair sums (Omega_0, Omega_1) in double-float arithmetic (pairs of
                         FP32 numbers, about 44 significant bits) on the FP32 pipes; geometry, the

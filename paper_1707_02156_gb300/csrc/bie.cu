@@ -2401,8 +2401,8 @@ static int sys_matvec(bie_ctx* ctx, const bie_geom* g, const double* u, double* 
   return BIE_OK;
 }
 
-// The end of Arnoldi step k behind the operator t2 of V_k (not yet normalised for k > 0): the three fused
-// kernels and the copy of the residual estimate to the pinned host array.
+// The end of Arnoldi step k behind the operator t2 of V_k (not yet normalised for k > 0): one cooperative kernel, or
+// three fused ones for long vectors, and the copy of the residual estimate to the pinned host array.
 static int arnoldi_tail(Krylov& K, const double* lam, const double* t2, long long n, int k, int m, cudaStream_t s) {
   double* V = K.V.ptr;
   double* vk = V + (long long)k * n;
@@ -2448,15 +2448,15 @@ static int arnoldi_tail(Krylov& K, const double* lam, const double* t2, long lon
 }
 
 // Arnoldi step k on stream s: the operator apply into the temporary t2 (its kernels launched one by one when
-// eager_apply), the three fused Gram-Schmidt kernels (the first one also normalises V_k, deferred from
-// step k - 1) and the copy of the residual estimate to the pinned host array.
+// eager_apply), then arnoldi_tail: the Gram-Schmidt kernel or kernels (the first also normalises V_k, deferred
+// from step k - 1) and the copy of the residual estimate to the pinned host array.
 static int arnoldi_step(bie_ctx* ctx, const bie_geom* g, Krylov& K, int prec, int k, int m, bool eager_apply,
                         cudaStream_t s) {
   const long long n = g->ncoef_total;
   double* V = K.V.ptr;
   double* t2 = K.tmp.ptr + n;
   double* vk = V + (long long)k * n;
-  // V_k is normalised by k_kry_sysop_dots, behind the apply: the operator is linear
+  // V_k is normalised behind the apply (k_kry_step or k_kry_sysop_dots): the operator is linear
   if (eager_apply)
     BIE_TRY(layer_apply_eager(ctx, g, 1, vk, t2, prec, s));
   else
@@ -2509,8 +2509,8 @@ static int arnoldi_step_graph(bie_ctx* ctx, const bie_geom* gc, Krylov& K, int p
 
 // Restarted GMRES (Sec. 6) with classical Gram-Schmidt and one re-orthogonalisation, FP64 Krylov
 // basis; the operator is applied at precision prec.  x holds the initial guess (zero if x_is_zero).
-// Each Arnoldi step runs as the operator apply and three fused kernels that end on the device
-// (k_kry_sub_tail); the host reads the residual estimate of step k - 1 after it has queued step k,
+// Each Arnoldi step runs as the operator apply and the kernels of arnoldi_tail, which end on the device
+// (kry_tail); the host reads the residual estimate of step k - 1 after it has queued step k,
 // so the device never waits for the host between steps.  A cycle that converges at step k - 1 has
 // computed one more step than it uses.
 //
@@ -2852,7 +2852,7 @@ static int surf_implicit_apply(SurfImplicit& I, const double* y, double* w, cuda
 }
 
 // Restarted GMRES for op x = b from x = 0 on the device kernels of the velocity solve (classical Gram-Schmidt
-// with one re-orthogonalisation, Givens rotations in k_kry_sub_tail); stops on ||b - op x|| <= tol ||b||.
+// with one re-orthogonalisation, Givens rotations in kry_tail); stops on ||b - op x|| <= tol ||b||.
 // The host reads the residual estimate of step k - 1 while step k runs, so an iteration has no
 // synchronisation of its own (five before, each with copies from and to pageable memory).
 static int surf_gmres(Krylov& K, const std::function<int(const double*, double*)>& op, const double* b, double* x,

@@ -90,6 +90,32 @@ __device__ inline void block_sum3(R& a, R& b, R& c, R* sh) {
   }
 }
 
+// The point of the records r [7][N] nearest to x0, scanned by one warp, its lanes striding over the points (the first
+// nearest point wins ties, as in a sequential scan); every lane gets its index and squared distance.
+__device__ inline long long warp_nearest(const double* __restrict__ r, long long N, double x0, double x1, double x2,
+                                         double& d2) {
+  double best = 1e300;
+  long long bi = N;
+  for (long long s = threadIdx.x & 31; s < N; s += 32) {
+    const double d0 = x0 - r[s], d1 = x1 - r[N + s], dz = x2 - r[2 * N + s];
+    const double d = d0 * d0 + d1 * d1 + dz * dz;
+    if (d < best) {
+      best = d;
+      bi = s;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {  // smallest distance, then smallest index
+    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+    const long long oi = __shfl_xor_sync(0xffffffffu, bi, o);
+    if (ob < best || (ob == best && oi < bi)) {
+      best = ob;
+      bi = oi;
+    }
+  }
+  d2 = best;
+  return bi < N ? bi : 0;
+}
+
 // Degree n of the packed index r = n(n+1)+m (0 <= r < (p+1)^2).
 __device__ inline int degree_of(int r) {
   int n = (int)sqrtf((float)r);

@@ -19,8 +19,7 @@ inline unsigned blocks_for(long long n, int t = kThreads) { return (unsigned)((n
 // region[t * ndrop + j]: 0 / 1 / 2 for Omega_0/1/2 of target t w.r.t. drop j, 3 = t inside drop j,
 // 255 for j = own drop.  Distance = nearest point of j's upsampled grid (Sec. 2.3).  A block settles its
 // 256 (target, drop) pairs outside the bounding spheres widened by A h_j and lists the others in shared
-// memory; its warps then scan the upsampled grid for one listed pair each, the lanes striding over the points
-// (the first nearest point wins ties, as in a sequential scan).  The listed pairs of neighbouring targets
+// memory; its warps then scan the upsampled grid for one listed pair each (warp_nearest).  The listed pairs of neighbouring targets
 // come together, so one thread per pair left a few threads with a serial scan each: 8 drops of degree 16,
 // 0.96 -> 0.15 ms.
 __global__ void __launch_bounds__(kThreads) k_classify(
@@ -63,26 +62,9 @@ __global__ void __launch_bounds__(kThreads) k_classify(
     const double x0 = px[k][0], x1 = px[k][1], x2 = px[k][2];
     const long long N = up_n[j];
     const double* r = rec_up + 7 * up_off[j];
-    double best = 1e300;
-    long long bi = N;
-    for (long long s = lane; s < N; s += 32) {
-      const double d0 = x0 - r[s], d1 = x1 - r[N + s], d2 = x2 - r[2 * N + s];
-      const double d = d0 * d0 + d1 * d1 + d2 * d2;
-      if (d < best) {
-        best = d;
-        bi = s;
-      }
-    }
-    for (int o = 16; o > 0; o >>= 1) {  // smallest distance, then smallest index
-      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const long long oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob < best || (ob == best && oi < bi)) {
-        best = ob;
-        bi = oi;
-      }
-    }
+    double best;
+    const long long bi = warp_nearest(r, N, x0, x1, x2, best);
     if (lane) continue;
-    if (bi >= N) bi = 0;
     const double dist = sqrt(best);
     const double side = (x0 - r[bi]) * r[3 * N + bi] + (x1 - r[N + bi]) * r[4 * N + bi] + (x2 - r[2 * N + bi]) * r[5 * N + bi];
     unsigned char code = dist <= h[j] ? 2 : (dist <= a_tilde * h[j] ? 1 : 0);
@@ -474,8 +456,9 @@ __global__ void __launch_bounds__(kTile / TPT) k_interdrop_x2(
 // r^-k = y^k (1 - e)^(-k/2) = y^k (1 + (k/2) e + (k/2)(k/2 + 1)/2 e^2 + O(e^3)).
 // About 170 operations per pair; scalar, the kernel reached 67% of the pipe at 75% of the issue slots.  80
 // drops of degree 24 (1.0e10 pairs): 90.4 -> 68.7 ms.  Rounding the high parts of positions to a common grid,
-// so that their difference is exact in one operation, saved another tenth but lost accuracy where the
-// points of a tile lie at very different distances (4e-11 of the field instead of 1e-11), and was left out.
+// so that their difference is exact in one operation, saved another tenth but lost accuracy where the points of
+// a tile lie at very different distances (3.9e-11 of the field at some fluid points, over the 1e-11 that
+// double-float sums are to keep), and was left out.
 struct d2 {
   fx2 h, l;
 };

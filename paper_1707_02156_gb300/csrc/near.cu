@@ -176,30 +176,6 @@ __device__ void sh_eval3(const double* __restrict__ c, long long cstride, int p,
     for (int o = 16; o > 0; o >>= 1) out[q] += __shfl_xor_sync(0xffffffffu, out[q], o);
 }
 
-// nearest of the N points of records r to x0, scanned by one warp (the first nearest point wins ties, as in
-// a sequential scan); every lane returns it
-__device__ int warp_nearest(const double* __restrict__ r, long long N, double x0, double x1, double x2) {
-  double best = 1e300;
-  long long bi = N;
-  for (long long s = threadIdx.x & 31; s < N; s += 32) {
-    const double d0 = x0 - r[s], d1 = x1 - r[N + s], d2 = x2 - r[2 * N + s];
-    const double d = d0 * d0 + d1 * d1 + d2 * d2;
-    if (d < best) {
-      best = d;
-      bi = s;
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-    const long long oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (ob < best || (ob == best && oi < bi)) {
-      best = ob;
-      bi = oi;
-    }
-  }
-  return bi < N ? (int)bi : 0;
-}
-
 // seed: nearest standard grid point of drop j to the target, one warp per pair
 __global__ void k_near_seed(const NearPair* __restrict__ pairs, int npair, const double* __restrict__ rec_std,
                             const long long* __restrict__ toff, const int* __restrict__ ngd,
@@ -211,8 +187,10 @@ __global__ void k_near_seed(const NearPair* __restrict__ pairs, int npair, const
   const int j = pairs[i].src_drop, di = tdrop[t];
   const long long ngi = ngd[di];
   const double* ri = rec_std + 7 * toff[di];
-  const int bi = warp_nearest(rec_std + 7 * toff[j], ngd[j], ri[tgt_loc[t]], ri[ngi + tgt_loc[t]], ri[2 * ngi + tgt_loc[t]]);
-  if ((threadIdx.x & 31) == 0) seed[i] = bi;
+  double d;
+  const long long bi =
+      warp_nearest(rec_std + 7 * toff[j], ngd[j], ri[tgt_loc[t]], ri[ngi + tgt_loc[t]], ri[2 * ngi + tgt_loc[t]], d);
+  if ((threadIdx.x & 31) == 0) seed[i] = (int)bi;
 }
 
 // Levenberg-Marquardt Newton on F = |x(theta, phi) - x0|^2 / 2 in the rotated frame (seed at the
@@ -905,9 +883,5 @@ template int launch_near_checks<double>(int, const NearPair*, int, int, const do
                                         const double*, const double*, const double*, long long, const double*,
                                         const double*, const double*, long long, const double*, double*,
                                         cudaStream_t);
-template int launch_near_checks<float>(int, const NearPair*, int, int, const double*, const int*, const double*,
-                                       const long long*, const int*, const long long*, const long long*, const float*,
-                                       const float*, const float*, long long, const float*, const float*,
-                                       const float*, long long, const double*, double*, cudaStream_t);
 
 }  // namespace bie

@@ -6,6 +6,7 @@
 // caller's layout and form the velocity.
 #include <cuda_runtime.h>
 
+#include "device.cuh"
 #include "internal.cuh"
 #include "offsurface.h"
 
@@ -20,8 +21,7 @@ inline unsigned blocks_for(long long n, int t = kThreads) { return (unsigned)((n
 // distance to the nearest point of drop j's upsampled grid against h_j and A h_j (after the bounding-
 // sphere test), inside when the point is on the inner side of the tangent plane there.  Two passes:
 // one thread per (point, drop) settles the pairs outside the bounding sphere widened by A h_j and
-// lists the others; then one warp per listed pair scans the upsampled grid, its lanes striding over
-// the points (the first nearest point wins ties, as in a sequential scan).
+// lists the others; then one warp per listed pair scans the upsampled grid (warp_nearest).
 __global__ void k_classify_points_far(const double* __restrict__ pts, long long ld, long long t0, long long n, int nd,
                                       const double* __restrict__ centre, const double* __restrict__ bound,
                                       const double* __restrict__ h, double a_tilde, unsigned char* __restrict__ region,
@@ -55,24 +55,8 @@ __global__ void k_classify_points_near(const double* __restrict__ pts, long long
     const double x0 = pts[t0 + t], x1 = pts[ld + t0 + t], x2 = pts[2 * ld + t0 + t];
     const long long N = up_n[j];
     const double* r = rec_up + 7 * up_off[j];
-    double best = 1e300;
-    long long bi = N;
-    for (long long s = lane; s < N; s += 32) {
-      const double d0 = x0 - r[s], d1 = x1 - r[N + s], d2 = x2 - r[2 * N + s];
-      const double d = d0 * d0 + d1 * d1 + d2 * d2;
-      if (d < best) {
-        best = d;
-        bi = s;
-      }
-    }
-    for (int o = 16; o > 0; o >>= 1) {  // smallest distance, then smallest index
-      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const long long oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob < best || (ob == best && oi < bi)) {
-        best = ob;
-        bi = oi;
-      }
-    }
+    double best;
+    const long long bi = warp_nearest(r, N, x0, x1, x2, best);
     if (lane == 0) {
       const double dist = sqrt(best);
       const double side = (x0 - r[bi]) * r[3 * N + bi] + (x1 - r[N + bi]) * r[4 * N + bi] +
@@ -134,25 +118,9 @@ __global__ void k_near_seed_points(const NearPair* __restrict__ pairs, int npair
   const double x0 = pts[t], x1 = pts[ld + t], x2 = pts[2 * ld + t];
   const long long N = ngd[j];
   const double* r = rec_std + 7 * toff[j];
-  double best = 1e300;
-  long long bi = N;
-  for (long long s = threadIdx.x & 31; s < N; s += 32) {
-    const double d0 = x0 - r[s], d1 = x1 - r[N + s], d2 = x2 - r[2 * N + s];
-    const double d = d0 * d0 + d1 * d1 + d2 * d2;
-    if (d < best) {
-      best = d;
-      bi = s;
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) {  // smallest distance, then smallest index
-    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-    const long long oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (ob < best || (ob == best && oi < bi)) {
-      best = ob;
-      bi = oi;
-    }
-  }
-  if ((threadIdx.x & 31) == 0) seed[i] = bi < N ? (int)bi : 0;
+  double d;
+  const long long bi = warp_nearest(r, N, x0, x1, x2, d);
+  if ((threadIdx.x & 31) == 0) seed[i] = (int)bi;
 }
 
 __global__ void k_add(const double* __restrict__ x, long long n, double* __restrict__ y) {

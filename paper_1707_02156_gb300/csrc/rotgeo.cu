@@ -18,8 +18,8 @@
 //   * Rotated coefficients are stored by (n - m, m), so that neighbouring threads, on neighbouring orders, read
 //     neighbouring entries of them and of the Legendre tables; a thread takes the orders a and p - a, which
 //     makes all sums equally long.
-// 64 drops of degree 24: 59 ms, 50 of them in the synthesis; now 24.  Neither pipe is full any more (FP64 41 %,
-// issue slots 40 % busy): the phases of a pass wait for one another, with three blocks per SM.  Blocks of as
+// 64 drops of degree 24: 59 ms, 50 of them in the synthesis; now 24.  Neither pipe is full any more (FP64 28 %,
+// issue slots 47 % busy): the phases of a pass wait for one another, with three blocks per SM.  Blocks of as
 // many threads as the phases have items (320, 480) are slower (26, 28 ms).
 #include <cuda_runtime.h>
 

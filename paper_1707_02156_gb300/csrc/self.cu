@@ -219,8 +219,8 @@ __global__ void __launch_bounds__(256) k_self_direct(
 // The phi transform and the projection (0.15M multiply-adds per target and kind at p = pq = 24) run in
 // fixed point on the integer pipe (fixed.cuh), on one scale per target and entry from a first pass over the kernel
 // weights; the FP64 pipe, which bounded the kernel before, keeps the weights themselves (37k operations).
-// 64 drops of degree 24, both kinds: 127 ms by the direct sums, 62 by the symmetries in FP64, now 32.
-// Two pairs a pass where they fit a block's shared memory (fewer barriers: 43.8 ms; three or four 46.9 and 45.1), one
+// 64 drops of degree 24, both kinds: 127 ms by the direct sums, 62 by the symmetries in FP64, now 33.
+// Two pairs a pass where they fit a block's shared memory (fewer barriers: 43.8 ms with the rotation below; three or four 46.9 and 45.1), one
 // at the largest degrees.
 
 __device__ inline int tri_index_degree(int it) {
@@ -455,8 +455,10 @@ __global__ void __launch_bounds__(128) k_unrotate(const double* __restrict__ Q64
     for (int r = 0; r < kFly; ++r)
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
+        v[r][u] = 0.0;
+        if (32 * u >= 2 * (n + 1)) continue;
         const int g = g0 + 4 * r, k = lane + 32 * u, im = k > n, m = im ? k - (n + 1) : k;
-        v[r][u] = g < ngr && k < 2 * (n + 1) ? Qr[(2LL * g + im) * ntri + m] : 0.0;
+        if (g < ngr && k < 2 * (n + 1)) v[r][u] = Qr[(2 * g + im) * ntri + m];
       }
 #pragma unroll
     for (int r = 0; r < kFly; ++r) {
