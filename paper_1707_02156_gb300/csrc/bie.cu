@@ -40,10 +40,11 @@ static const double kPi = 3.14159265358979323846;
 // The buffers come from one memory pool per device, so that the next geometry or call finds the pages of the
 // last one mapped: a time step sets up two geometries of a hundred buffers, and cudaMalloc and cudaFree of them took
 // 3 of its 17 ms (8 drops of degree 16; 64 drops of degree 24, 12 GB: 11 of 118 ms).  A buffer that a call releases
-// is held, and returns to the pool at the next allocation, or when 64 MB are held, after a wait for everything on the
-// device, as cudaFree waits; it is ready for any stream when alloc returns, so the pool knows one stream only.  The pool
-// keeps at most a sixteenth of the device's memory unused; it gives everything unused back when an allocation
-// fails, and when the last context of the device is destroyed.
+// is held; when 64 MB are held, a geometry goes or an allocation fails, the held ones return to the pool after a
+// wait for everything on the device, as cudaFree waits.  (A wait at every release or allocation, 27 in a step of 8
+// drops of degree 16, took 0.3 ms of its 13.)  A buffer is ready for any stream when alloc returns, so the pool
+// knows one stream only.  The pool keeps at most a sixteenth of the device's memory unused; it gives everything unused
+// back when an allocation fails, and when the last context of the device is destroyed.
 //
 // The wait is a cudaFree of a marker made by cudaMalloc (2 us when the device is idle and another marker is left, so
 // that the driver keeps their page), not a cudaDeviceSynchronize: other threads' streams may be in a graph capture
@@ -162,15 +163,10 @@ static cudaError_t dev_malloc(void** ptr, size_t bytes, int* device, bool wait) 
   DevPool& P = g_pools[dev];
   std::call_once(P.once, [&] { P.err = pool_init(P, dev); });
   if (P.err != cudaSuccess) return P.err;
-  bool held;
-  {
-    std::lock_guard<std::mutex> lk(P.mu);
-    held = !P.held.empty();
-  }
-  if (held) device_wait(dev);
   e = P.pool ? cudaMallocFromPoolAsync(ptr, bytes, P.pool, P.stream) : cudaMalloc(ptr, bytes);
   if (e == cudaErrorMemoryAllocation && P.pool) {
     cudaGetLastError();  // not sticky
+    device_wait(dev);    // the buffers held
     cudaStreamSynchronize(P.stream);
     cudaMemPoolTrimTo(P.pool, 0);
     e = cudaMallocFromPoolAsync(ptr, bytes, P.pool, P.stream);
