@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "dfloat.cuh"
@@ -445,11 +446,11 @@ __global__ void __launch_bounds__(128) k_unrotate(const double* __restrict__ Q64
   for (int i = threadIdx.x; i < n * n; i += blockDim.x) sS[(i / n) * ldS + i % n] = blk[(n + 1) * (n + 1) + i];
   const int w = 2 * n + 1;
   const double* Qr = Q64 + (row - row0) * nb * 12 * ntri + (long long)b0 * 12 * ntri + t0;
-  // a warp per longitude and entry, three of them in flight: the 2 (n + 1) factors (at most 4 per lane, see
-  // self_dense_fits) and their scale
+  // the 2 (n + 1) factors of a longitude and entry (at most 4 per lane, see self_dense_fits) and their scale, by a warp,
+  // or by a half or a quarter of one where they are no more than that; three at a time, so that their loads overlap
   constexpr int kFly = 3;
-  const int lane = threadIdx.x & 31, ngr = nbh * 6;
-  for (int g0 = threadIdx.x >> 5; g0 < ngr; g0 += 4 * kFly) {
+  const int width = n < 4 ? 8 : n < 8 ? 16 : 32, lane = threadIdx.x & (width - 1), ngr = nbh * 6, step = 128 / width;
+  for (int g0 = threadIdx.x / width; g0 - (int)(threadIdx.x / width) < ngr; g0 += step * kFly) {  // all lanes of a warp
     double v[kFly][4];
 #pragma unroll
     for (int r = 0; r < kFly; ++r)
@@ -457,17 +458,22 @@ __global__ void __launch_bounds__(128) k_unrotate(const double* __restrict__ Q64
       for (int u = 0; u < 4; ++u) {
         v[r][u] = 0.0;
         if (32 * u >= 2 * (n + 1)) continue;
-        const int g = g0 + 4 * r, k = lane + 32 * u, im = k > n, m = im ? k - (n + 1) : k;
+        const int g = g0 + step * r, k = lane + 32 * u, im = k > n, m = im ? k - (n + 1) : k;
         if (g < ngr && k < 2 * (n + 1)) v[r][u] = Qr[(2 * g + im) * ntri + m];
       }
 #pragma unroll
     for (int r = 0; r < kFly; ++r) {
-      const int g = g0 + 4 * r;
-      if (g >= ngr) break;
+      const int g = g0 + step * r;
       int e = 0;
 #pragma unroll
       for (int u = 0; u < 4; ++u) e = max(e, fix_magnitude(v[r][u]));
-      e = fix_exponent(__reduce_max_sync(0xffffffffu, e));
+      if (width == 32) {
+        e = __reduce_max_sync(0xffffffffu, e);
+      } else {
+        for (int o = width / 2; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+      }
+      if (g >= ngr) continue;
+      e = fix_exponent(e);
       if (lane == 0) es[g] = e;
       const bool bad = e == fix_bad;
       if (e == fix_none) e = 0;
@@ -606,7 +612,7 @@ __global__ void __launch_bounds__(kSelfThreads, 2) k_self_dense(SelfGroups<R> G,
     const int t = t0 + k * (kSelfThreads / 32) + warp;
     if (t >= ng) break;
     const uint4* S = reinterpret_cast<const uint4*>(A.S + (ld * ng + t) * 6 * (long long)ncp);
-    R acc[3] = {R(0), R(0), R(0)}, odd[3] = {R(0), R(0), R(0)};  // FP64 and double-float: the sums of even and odd entries
+    R acc[3] = {R(0), R(0), R(0)}, odd[3] = {R(0), R(0), R(0)};  // FP64: the sums of even and odd entries
 #pragma unroll 2
     for (int i = lane; i < nv; i += 32) {
       uint4 s[6], f[3];
@@ -622,13 +628,13 @@ __global__ void __launch_bounds__(kSelfThreads, 2) k_self_dense(SelfGroups<R> G,
         for (int e = 0; e < 6; ++e) q[e] = lane_of<R>(s[e], v);
 #pragma unroll
         for (int c = 0; c < 3; ++c) x[c] = lane_of<R>(f[c], v);
-        sym_mul_add<R>(q, x, sizeof(R) == 4 ? sum : (v & 1) ? odd : acc);
+        sym_mul_add<R>(q, x, sizeof(R) == 4 ? sum : (v & 1) && std::is_same<R, double>::value ? odd : acc);
       }
       if (sizeof(R) == 4)
 #pragma unroll
         for (int c = 0; c < 3; ++c) acc[c] = acc[c] + sum[c];
     }
-    if (sizeof(R) == 8)
+    if (std::is_same<R, double>::value)
 #pragma unroll
       for (int c = 0; c < 3; ++c) acc[c] = acc[c] + odd[c];
     // the three sums over the lanes in six additions (fifteen one by one, 2 us of an FP64 apply of one drop of degree 16):
