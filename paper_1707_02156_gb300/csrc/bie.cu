@@ -962,7 +962,7 @@ static int setup_self(bie_ctx* ctx, bie_geom* g, bie_geom::Group& G, DevBuf<doub
       }
       if (direct) continue;
       Phase ph(ctx, "kernel_proj", s);
-      for (int kind = 0; kind < 2; ++kind) {
+      for (int kind = 1; kind >= 0; --kind) {
         BIE_TRY(launch_kernel_proj(kind, cache, nt, p, pq, pl->CT.ptr, pl->PT.ptr, Q, s));
         BIE_TRY(launch_unrotate(Q, t0 / nb, nt / nb, p, wp->blkx.ptr, wp->stride, pp->cs.ptr, G.qk64[kind].ptr,
                                 G.qk32[kind].ptr, s));

@@ -158,9 +158,10 @@ int launch_self_direct(int kind, const double* dens, const long long* foff3, lon
 // Projected kernel factors Q[t][12][tri(n,m)] of ntarget targets (see self.cu), from the FP64
 // rotated-geometry cache, with fixed-point tables (fixed.cuh): CT[k][m] = cos, sin (m phi_k) 2^55 for the
 // longitudes k <= (pq+1)/2, PT[j][tri(n, m)] = P~_n^m(t_j) 2^55 for the latitudes j <= pq/2.
+// The stresslet (kind 1) first: it leaves its factors in the cache's row 3, the Stokeslet its own in rows 3 and 6.
 // self_dense_fits: whether the dense form serves the degrees.
 bool self_dense_fits(int p, int pq);
-int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, int pq, const int4* CT, const int2* PT,
+int launch_kernel_proj(int kind, double* cache, long long ntarget, int p, int pq, const int4* CT, const int2* PT,
                        double* Q64, cudaStream_t s);
 // Entries per plane of the dense self form: (p+1)^2 rounded up to whole 16-byte loads in every precision.
 __host__ __device__ inline int self_row(int p) { return ((p + 1) * (p + 1) + 3) & ~3; }

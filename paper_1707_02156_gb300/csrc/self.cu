@@ -219,7 +219,8 @@ __global__ void __launch_bounds__(256) k_self_direct(
 // and difference serve even and odd n - m; and the Legendre projection, accumulated in shared memory.
 // The phi transform and the projection (0.15M multiply-adds per target and kind at p = pq = 24) run in
 // fixed point on the integer pipe (fixed.cuh), on one scale per target and entry from a first pass over the kernel
-// weights; the FP64 pipe, which bounded the kernel before, keeps the weights themselves (37k operations).
+// weights, which leaves their factors c and d in the cache for the second; the FP64 pipe, which bounded the kernel before,
+// keeps the weights themselves.
 // 64 drops of degree 24, both kinds: 127 ms by the direct sums, 62 by the symmetries in FP64, now 33.
 // Two pairs a pass where they fit a block's shared memory (fewer barriers: 43.8 ms with the rotation below; three or four 46.9 and 45.1), one
 // at the largest degrees.
@@ -232,9 +233,9 @@ __device__ inline int tri_index_degree(int it) {
 }
 
 // Bounds on the exponents of a target's six entries, each on a scale of its own (a drop that is thin along an axis has
-// entries of very different size): with a w/r = the Stokeslet's diagonal part and b_i = c x_i^2 (c = w/r^3 or 6 |x.a| /
-// r^5), |entry ij| = c |x_i x_j| < 2^((E(b_i) + E(b_j))/2), E the exponent of the largest over the points (em their magnitudes); the Stokeslet's
-// diagonal entries are below 2 w/r.
+// entries of very different size): with d = w/r the Stokeslet's diagonal part and b_i = c x_i^2 (c = w/r^3 or -6 x.a /
+// r^5), |entry ij| = |c x_i x_j| < 2^((E(b_i) + E(b_j))/2), E the exponent of the largest over the points (em their
+// magnitudes); the Stokeslet's diagonal entries are below 2 d.
 template <int KIND>
 __device__ __forceinline__ int entry_exponent(const int* em, int entry) {
   const int i = entry < 3 ? entry : entry == 5 ? 1 : 0, j = entry < 3 ? entry : entry == 3 ? 1 : 2;
@@ -243,7 +244,7 @@ __device__ __forceinline__ int entry_exponent(const int* em, int entry) {
 }
 
 template <int KIND, int NP>
-__global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ cache, int pq, int p,
+__global__ void __launch_bounds__(256) k_kernel_proj(double* cache, int pq, int p,
                                                      const int4* __restrict__ CT, const int2* __restrict__ PT,
                                                      double* __restrict__ Q64) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
   int2* sd = reinterpret_cast<int2*>(sk + NP * 12 * nk);                     // [pair][even, odd][12][p+1]
   long long* sq = reinterpret_cast<long long*>(sd + NP * 24 * (p + 1));      // [12][ntri]
   const long long nq = (long long)nq_j * nk;
-  const double* geo = cache + t * 7 * nq;
+  double* geo = cache + t * 7 * nq;
   for (int i = threadIdx.x; i < 12 * ntri; i += blockDim.x) sq[i] = 0;
   if (threadIdx.x < 4) em[threadIdx.x] = 0;
   __syncthreads();
@@ -267,15 +268,17 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
     for (int o = threadIdx.x; o < nq; o += blockDim.x) {
       const double x0 = geo[o], x1 = geo[nq + o], x2 = geo[2 * nq + o];
       const double y0 = x0 * x0, y1 = x1 * x1, y2 = x2 * x2;
-      const double ri = rsqrt_<double>(y0 + y1 + y2), ri2 = ri * ri;
+      const double r2 = y0 + y1 + y2;
       double c;
       if (KIND == 0) {
-        const double d = geo[6 * nq + o] * ri;
-        e[3] = max(e[3], fix_magnitude(2.0001 * d));
-        c = 1.0001 * (d * ri2);
+        const double ri = rsqrt_<double>(r2), d = geo[6 * nq + o] * ri;
+        c = d * (ri * ri);
+        geo[6 * nq + o] = d;  // for the second pass
+        e[3] = max(e[3], fix_magnitude(d));
       } else {
-        c = (6.0001 * (x0 * geo[3 * nq + o] + x1 * geo[4 * nq + o] + x2 * geo[5 * nq + o])) * (ri * (ri2 * ri2));
+        c = (-6.0 * (x0 * geo[3 * nq + o] + x1 * geo[4 * nq + o] + x2 * geo[5 * nq + o])) * rsqrt5_<double>(r2);
       }
+      geo[3 * nq + o] = c;
       e[0] = max(e[0], fix_magnitude(c * y0));
       e[1] = max(e[1], fix_magnitude(c * y1));
       e[2] = max(e[2], fix_magnitude(c * y2));
@@ -283,7 +286,8 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
 #pragma unroll
     for (int k = 0; k < (KIND == 0 ? 4 : 3); ++k) {
       e[k] = __reduce_max_sync(0xffffffffu, e[k]);
-      if ((threadIdx.x & 31) == 0) atomicMax(&em[k], e[k]);
+      // with a margin of 1e-4 for their rounding (in the magnitude's mantissa); the Stokeslet's diagonal entries are below 2 d
+      if ((threadIdx.x & 31) == 0 && e[k]) atomicMax(&em[k], e[k] + (KIND == 0 && k == 3 ? (1 << 20) + 128 : 128));
     }
   }
   __syncthreads();
@@ -308,16 +312,8 @@ __global__ void __launch_bounds__(256) k_kernel_proj(const double* __restrict__ 
         continue;
       }
       const long long o = (long long)j * nk + k;
-      const double x0 = geo[o], x1 = geo[nq + o], x2 = geo[2 * nq + o];
-      const double r2 = x0 * x0 + x1 * x1 + x2 * x2;
-      double d = 0.0, c;
-      if (KIND == 0) {
-        const double ri = rsqrt_<double>(r2);
-        d = geo[6 * nq + o] * ri;
-        c = d * (ri * ri);
-      } else {
-        c = (-6.0 * (x0 * geo[3 * nq + o] + x1 * geo[4 * nq + o] + x2 * geo[5 * nq + o])) * rsqrt5_<double>(r2);
-      }
+      const double x0 = geo[o], x1 = geo[nq + o], x2 = geo[2 * nq + o], c = geo[3 * nq + o];
+      const double d = KIND == 0 ? geo[6 * nq + o] : 0.0;
       const double a0 = c * x0, a1 = c * x1;
       v[0] = d + a0 * x0;
       v[nk] = d + a1 * x1;
@@ -705,7 +701,7 @@ static size_t kernel_proj_smem(int p, int pq, int np) {
 // its projected factors fit a block, and the direct form serves as it always has.
 bool self_dense_fits(int p, int pq) { return 8 * (36 * (size_t)(pq + p + 2) + 6 * (size_t)(p + 1) * (p + 2)) <= 227 * 1024; }
 
-int launch_kernel_proj(int kind, const double* cache, long long ntarget, int p, int pq, const int4* CT, const int2* PT,
+int launch_kernel_proj(int kind, double* cache, long long ntarget, int p, int pq, const int4* CT, const int2* PT,
                        double* Q64, cudaStream_t s) {
   if (ntarget == 0) return BIE_OK;
   if (ntarget > 0x7fffffffLL) return BIE_EINVAL;
