@@ -59,6 +59,8 @@ TENSOR_ROTATION = False
 # from one ncu capture, with the SHA-256 prefix of the kernel's source file at the time of the
 # capture: a capture of an older version of the kernel is not reported (traffic null).
 PROFILED_TRAFFIC = {
+    ("interdrop_f32", "c5"): {"bytes": 1178150912, "source": "interdrop.cu", "sha": "5b62e7b4e3812873"},
+    ("self_proj_f32", "c2"): {"bytes": 57132032, "source": "self.cu", "sha": "b8dab6b1be9afdcd"},
 }
 
 

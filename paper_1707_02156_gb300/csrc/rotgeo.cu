@@ -106,7 +106,8 @@ __global__ void __launch_bounds__(kGeoThreads, 3) k_rotgeo_fix(RotGeo A, double*
   }
   for (int i = threadIdx.x; i < 3 * (kMaxDeg + 1); i += kGeoThreads) (&en[0][0])[i] = fix_exponent((&en[0][0])[i]);
   __syncthreads();
-  for (int i = threadIdx.x; i < 3 * nc; i += kGeoThreads) gi[i] = fix_split(fix_encode(g[i], en[i / nc][degree_of(i % nc)]));
+  for (int i = threadIdx.x; i < 3 * nc; i += kGeoThreads)
+    gi[i] = fix_split(fix_encode(g[i], en[i / nc][degree_of(i % nc)]));
   __syncthreads();
   // rotation: sums of at most p + 1 <= 64 products of 2^57 and 2^57, in units of 2^(en - 55 - xb)
   const int xb = 6 - ceil_log2(p + 1);
@@ -230,7 +231,8 @@ __global__ void __launch_bounds__(kGeoThreads, 3) k_rotgeo_fix(RotGeo A, double*
       const int tm = 31 - __clz(max(m, 1)), kb0 = max(kbits[0][c], 0), kb1 = max(kbits[1][c], 0), kb2 = max(kbits[2][c], 0);
       long long *o0 = h + 2LL * i, *o1 = h + 2LL * (6 * JP * (p + 1) + i);
       const long long re = o0[0], im = o0[1], re1 = o1[0], im1 = o1[1];
-      const unsigned fr = hf[2 * i], fi = hf[2 * i + 1], fr1 = hf[2 * (6 * JP * (p + 1) + i)], fi1 = hf[2 * (6 * JP * (p + 1) + i) + 1];
+      const unsigned fr = hf[2 * i], fi = hf[2 * i + 1];
+      const unsigned fr1 = hf[2 * (6 * JP * (p + 1) + i)], fi1 = hf[2 * (6 * JP * (p + 1) + i) + 1];
       int2 *w0 = hi + 2LL * i, *w1 = hi + 2LL * (6 * JP * (p + 1) + i), *w2 = hi + 2LL * (12 * JP * (p + 1) + i);
       w0[0] = fix_split(shifted(re, fr, 57 - kb0));
       w0[1] = fix_split(shifted(im, fi, 57 - kb0));
@@ -262,8 +264,10 @@ __global__ void __launch_bounds__(kGeoThreads, 3) k_rotgeo_fix(RotGeo A, double*
       }
       if (m <= p) add(m, 0);
       // units: rotated coefficients 2^(-55 - xb), split 2^(bits - 57) of that, Legendre sums 2^(59 - 56) of that, split
-      // 2^(kbits - 57), tables 2^-56 (2^-55 for kind 2), sums 2^(58 - ext) of their products, which leaves room for four of them
-      const int unit = bits_of(kind == 1, f % 3) - 55 - xb - 57 + 3 + max(kbits[kind][f % 3], 0) - 57 - (kind == 2 ? 55 : 56) + 58 - ext;
+      // 2^(kbits - 57), tables 2^-56 (2^-55 for kind 2), sums 2^(58 - ext) of their products, which leaves room for four
+      // of them
+      const int unit = bits_of(kind == 1, f % 3) - 55 - xb - 57 + 3 + max(kbits[kind][f % 3], 0) - 57 -
+                       (kind == 2 ? 55 : 56) + 58 - ext;
       const bool rot = k > 0, mir = 2 * k < half;
 #pragma unroll
       for (int side = 0; side < 2; ++side) {

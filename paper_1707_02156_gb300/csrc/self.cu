@@ -218,12 +218,12 @@ __global__ void __launch_bounds__(256) k_self_direct(
 // quadruples that share |cos m phi| and |sin m phi|, in place; the phi transform of both rows, whose sum
 // and difference serve even and odd n - m; and the Legendre projection, accumulated in shared memory.
 // The phi transform and the projection (0.15M multiply-adds per target and kind at p = pq = 24) run in
-// fixed point on the integer pipe (fixed.cuh), on one scale per target and entry from a first pass over the kernel
-// weights, which leaves their factors c and d in the cache for the second; the FP64 pipe, which bounded the kernel before,
-// keeps the weights themselves.
-// 64 drops of degree 24, both kinds: 127 ms by the direct sums, 62 by the symmetries in FP64, now 33.
-// Two pairs a pass where they fit a block's shared memory (fewer barriers: 43.8 ms with the rotation below; three or four 46.9 and 45.1), one
-// at the largest degrees.
+// fixed point on the integer pipe (fixed.cuh), on one scale per target and entry from a first pass over the
+// kernel weights, which leaves their factors c and d in the cache for the second; the FP64 pipe, which bounded
+// the kernel before, keeps the weights themselves.  64 drops of degree 24, both kinds: 127 ms by the direct sums,
+// 62 by the symmetries in FP64, now 31.
+// Two pairs a pass where they fit a block's shared memory (fewer barriers: 43.8 ms with the rotation below; three or
+// four 46.9 and 45.1), one at the largest degrees.
 
 __device__ inline int tri_index_degree(int it) {
   int n = (int)((sqrtf(8.0f * it + 1.0f) - 1.0f) * 0.5f);
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(256) k_kernel_proj(double* cache, int pq, int 
 // (s_re cos + s_im sin, s_im cos - s_re sin).  The 2n+1 products per entry and coefficient run in fixed point
 // on the integer pipe (fixed.cuh), on one scale per longitude and entry; two entries at a time share the reads of the
 // Wigner block, and the leading dimensions of the staged blocks are odd, so that the strided reads of the
-// transposed products hit every bank.  64 drops of p = 24, both kinds: 20 ms in FP64, now 12.
+// transposed products hit every bank.  64 drops of p = 24, both kinds: 20 ms in FP64, now 11.
 constexpr int kUnB = 8;
 
 __global__ void __launch_bounds__(128) k_unrotate(const double* __restrict__ Q64, long long row0, int p,
